@@ -153,8 +153,9 @@ int64_t     hat_launch_count(void);
  * path, longer chunks the tile path; long key ranges are cut so that every SM
  * has work, and rows cut into several ranges are merged afterwards.
  * Unless HAT_PLAN_HOST_ONLY is set the schedule is uploaded to the current
- * device (one cudaMalloc + one synchronous copy).  A plan can be reused for
- * every layer of the step and must be destroyed with hat_plan_destroy.
+ * device (into device memory a destroyed plan left, or one cudaMalloc; one small
+ * copy on a stream of the library's own, complete on return).  A plan can be
+ * reused for every layer of the step and must be destroyed with hat_plan_destroy.
  * One call at a time per plan: the plan owns device state that an attention
  * call uses while it runs (the work counter of the persistent tile kernel, the
  * status word, the verify event, the timing recorder).  Calls that take the
@@ -174,6 +175,14 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
 int hat_plan_get_info(const hat_plan* plan, hat_plan_info* out);
 int hat_plan_workspace_bytes(const hat_plan* plan, size_t* out);
 int hat_plan_destroy(hat_plan* plan);   /* NULL is accepted */
+
+/*
+ * A destroyed plan hands its device memory (with the pinned buffer it was
+ * filled from and its events) to later plans; at most 16 such pieces and 64 MiB
+ * wait at any time.  hat_release_cached frees what waits (this synchronises the
+ * device); it is never needed for correctness.  Any thread may call it.
+ */
+int hat_release_cached(void);
 
 /*
  * KV append (Sec. 2.1, KV cache).  For request r, chunk row i and head h the

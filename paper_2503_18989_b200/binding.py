@@ -34,6 +34,7 @@ DTYPE_CODE = {"fp16": HAT_DTYPE_FP16, "bf16": HAT_DTYPE_BF16}
 EXPORTS = [
     "hat_status_string", "hat_version", "hat_last_cuda_error", "hat_launch_count",
     "hat_plan_create", "hat_plan_get_info", "hat_plan_workspace_bytes", "hat_plan_destroy",
+    "hat_release_cached",
     "hat_kv_append", "hat_kv_append_rope", "hat_rope_q", "hat_qkv_rope_append", "hat_chunk_attention", "hat_chunk_attention_out16",
     "hat_plan_staging_bytes",
     "hat_chunk_attention_host",
@@ -111,6 +112,8 @@ def lib() -> C.CDLL:
         L.hat_plan_workspace_bytes.argtypes = [vp, C.POINTER(sz)]
         L.hat_plan_destroy.restype = i32
         L.hat_plan_destroy.argtypes = [vp]
+        L.hat_release_cached.restype = i32
+        L.hat_release_cached.argtypes = []
         L.hat_kv_append.restype = i32
         L.hat_kv_append.argtypes = [C.POINTER(hat_cache_desc), vp, vp, vp, vp]
         L.hat_kv_append_rope.restype = i32
@@ -259,6 +262,10 @@ def hat_plan_staging_bytes(plan) -> int:
 
 def hat_plan_destroy(plan) -> None:
     _check(lib().hat_plan_destroy(_h(plan)), "hat_plan_destroy")
+
+
+def hat_release_cached() -> None:
+    _check(lib().hat_release_cached(), "hat_release_cached")
 
 
 def hat_kv_append(cache: hat_cache_desc, plan, k_new, v_new, stream: int = 0) -> None:

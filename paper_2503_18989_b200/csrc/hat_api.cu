@@ -317,39 +317,35 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
     info.workspace_bytes = p->part_rows ? part_out_bytes + ((p->part_rows * H * 4 + 255) / 256 * 256) : 0;
 }
 
-template <typename T>
-static size_t blob_append(std::vector<char>& blob, const std::vector<T>& v) {
-    size_t off = (blob.size() + 255) / 256 * 256;
-    blob.resize(off + std::max<size_t>(v.size() * sizeof(T), 16));
-    if (!v.empty()) std::memcpy(blob.data() + off, v.data(), v.size() * sizeof(T));
-    return off;
-}
-
 static int upload(hat_plan* p) {
-    std::vector<char> blob;
-    size_t o_cu = blob_append(blob, p->cu_chunk);
-    size_t o_pl = blob_append(blob, p->prefix_len);
-    size_t o_cl = blob_append(blob, p->chunk_len);
-    size_t o_bt = blob_append(blob, p->block_table);
-    size_t o_rr = blob_append(blob, p->row_req);
-    size_t o_vi = blob_append(blob, p->verify_items);
-    size_t o_pi = blob_append(blob, p->prefill_items);
-    size_t o_mr = blob_append(blob, p->merge_rows);
-    size_t o_tu = blob_append(blob, p->tile_units);
-    size_t o_tm = blob_append(blob, p->tree_mask);
-    std::vector<int32_t> status(8, 0);     // status word; (unit counter, finished CTAs) of the tile kernel; the same for a second tile grid; spare
-    size_t o_st = blob_append(blob, status);
+    // the arrays, each at a 256-byte boundary, written straight into the pinned buffer
+    struct Part { const void* src; size_t bytes, off; };
+    std::vector<Part> parts;
+    size_t bytes = 0;
+    auto add = [&](const auto& v) {
+        const size_t off = (bytes + 255) / 256 * 256, n = v.size() * sizeof(v[0]);
+        parts.push_back(Part{v.data(), n, off});
+        bytes = off + std::max<size_t>(n, 16);
+        return off;
+    };
+    const size_t o_cu = add(p->cu_chunk), o_pl = add(p->prefix_len), o_cl = add(p->chunk_len), o_bt = add(p->block_table);
+    const size_t o_rr = add(p->row_req), o_vi = add(p->verify_items), o_pi = add(p->prefill_items), o_mr = add(p->merge_rows);
+    const size_t o_tu = add(p->tile_units), o_tm = add(p->tree_mask);
+    const std::vector<int32_t> status(8, 0);     // status word; (unit counter, finished CTAs) of the tile kernel; the same for a second tile grid; spare
+    const size_t o_st = add(status);
 
     cudaError_t e = cudaGetDevice(&p->device);
     if (e != cudaSuccess) return cuda_fail(e);
     // behind the arrays: room for the (cos, sin) table of the projection epilogue, filled on the device when first used
-    const size_t o_table = (blob.size() + 255) / 256 * 256;
+    const size_t o_table = (bytes + 255) / 256 * 256;
     const size_t table_bytes = (size_t)p->total_rows * (p->head_dim / 2) * sizeof(float2);
-    e = cudaMalloc(&p->dev_blob, o_table + std::max<size_t>(table_bytes, 16));
-    if (e != cudaSuccess) { p->dev_blob = nullptr; return cuda_fail(e); }
-    e = cudaMemcpy(p->dev_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice);
+    e = plan_res_acquire(p->device, o_table + std::max<size_t>(table_bytes, 16), bytes, &p->res);
     if (e != cudaSuccess) return cuda_fail(e);
-    char* base = static_cast<char*>(p->dev_blob);
+    for (const Part& part : parts)
+        if (part.bytes) std::memcpy(static_cast<char*>(p->res.pinned) + part.off, part.src, part.bytes);
+    e = plan_res_upload(p->res, bytes);
+    if (e != cudaSuccess) return cuda_fail(e);
+    char* base = static_cast<char*>(p->res.blob);
     p->rope_table = reinterpret_cast<float2*>(base + o_table);
     DevicePlan& d = p->dev;
     d.cu_chunk = reinterpret_cast<const int32_t*>(base + o_cu);
@@ -468,12 +464,10 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
     p->host_only = (batch->flags & HAT_PLAN_HOST_ONLY) != 0;
     p->device = -1;
     p->part_rows = 0;
-    p->dev_blob = nullptr;
     p->timing = nullptr;
     p->num_verify_merge_rows = 0;
-    p->ev_verify = nullptr;
-    p->ev_done = nullptr;
-    p->ev_table = nullptr;
+    p->captured = p->loose = p->loose_many = false;
+    p->loose_stream = nullptr;
     p->rope_table = nullptr;
     p->rope_theta = 0.f;
     p->table_stream = nullptr;
@@ -570,12 +564,6 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
     if (!p->host_only) {
         st = upload(p);
         if (st != HAT_OK) { hat_plan_destroy(p); return st; }
-        cudaError_t ee = cudaEventCreateWithFlags(&p->ev_verify, cudaEventDisableTiming);
-        if (ee != cudaSuccess) { p->ev_verify = nullptr; hat_plan_destroy(p); return cuda_fail(ee); }
-        ee = cudaEventCreateWithFlags(&p->ev_done, cudaEventDisableTiming);
-        if (ee != cudaSuccess) { p->ev_done = nullptr; hat_plan_destroy(p); return cuda_fail(ee); }
-        ee = cudaEventCreateWithFlags(&p->ev_table, cudaEventDisableTiming);
-        if (ee != cudaSuccess) { p->ev_table = nullptr; hat_plan_destroy(p); return cuda_fail(ee); }
         // Optional throughput mode for a mixed batch on the tcgen05 path (HAT_SIDE_SMS = n > 0): see the launch
         // sequence.  Off by default: it finishes the whole step sooner but the decode-phase rows later.  The side
         // stream has the highest priority so that the tile CTAs are placed before the streaming kernel's many small
@@ -585,7 +573,7 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
             side = std::max(0, std::min(side, p->num_sms - 8));
             if (side > 0) {
                 int lo = 0, hi = 0;
-                ee = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+                cudaError_t ee = cudaDeviceGetStreamPriorityRange(&lo, &hi);
                 if (ee == cudaSuccess) ee = cudaStreamCreateWithPriority(&p->aux_stream, cudaStreamNonBlocking, hi);
                 if (ee == cudaSuccess) ee = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
                 if (ee == cudaSuccess) ee = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
@@ -617,18 +605,22 @@ int hat_plan_destroy(hat_plan* plan) {
         for (cudaEvent_t ev : plan->timing->events) cudaEventDestroy(ev);
         delete plan->timing;
     }
-    if (plan->ev_verify) cudaEventDestroy(plan->ev_verify);
-    if (plan->ev_done) cudaEventDestroy(plan->ev_done);
-    if (plan->ev_table) cudaEventDestroy(plan->ev_table);
     if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
     if (plan->ev_join) cudaEventDestroy(plan->ev_join);
     if (plan->aux_stream) cudaStreamDestroy(plan->aux_stream);
-    if (plan->dev_blob) {
-        cudaError_t e = cudaFree(plan->dev_blob);
+    if (!plan->host_only) {
+        // handed on to a later plan unless a graph may replay a call, or work that ev_done does not cover may still run
+        plan->res.in_use = plan->has_last;
+        const cudaError_t e = plan_res_release(plan->res, !plan->captured && !plan->loose);
         if (e != cudaSuccess) st = cuda_fail(e);
     }
     delete plan;
     return st;
+}
+
+int hat_release_cached(void) {
+    const cudaError_t e = plan_res_trim();
+    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
 }
 
 int hat_kv_append(const hat_cache_desc* cache, const hat_plan* plan, const void* k_new, const void* v_new,
@@ -637,6 +629,7 @@ int hat_kv_append(const hat_cache_desc* cache, const hat_plan* plan, const void*
     if (st != HAT_OK) return st;
     if (plan->total_rows == 0) return HAT_OK;
     if (!k_new || !v_new || !aligned(k_new, 16) || !aligned(v_new, 16)) return HAT_ERR_INVALID_ARG;
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
     cudaError_t e = launch_kv_append(plan, view_of(cache), cache->k_pool, cache->v_pool, k_new, v_new,
                                      static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? HAT_OK : cuda_fail(e);
@@ -650,6 +643,7 @@ int hat_kv_append_rope(const hat_cache_desc* cache, const hat_plan* plan, const 
     if (plan->total_rows == 0) return HAT_OK;
     if (!k_new || !v_new || !aligned(k_new, 16) || !aligned(v_new, 16)) return HAT_ERR_INVALID_ARG;
     const CacheView view = view_of(cache);
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
     cudaError_t e = launch_rope(plan, plan->num_kv_heads, theta, interleaved != 0, k_new, nullptr, &view, cache->k_pool,
                                 cache->v_pool, v_new, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? HAT_OK : cuda_fail(e);
@@ -660,6 +654,7 @@ int hat_rope_q(const hat_plan* plan, const void* q, void* q_out, float theta, in
     if (!(theta > 1.f) || !std::isfinite(theta)) return HAT_ERR_INVALID_ARG;
     if (plan->total_rows == 0) return HAT_OK;
     if (!q || !q_out || !aligned(q, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
     cudaError_t e = launch_rope(plan, plan->num_heads, theta, interleaved != 0, q, q_out, nullptr, nullptr, nullptr, nullptr,
                                 static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? HAT_OK : cuda_fail(e);
@@ -674,6 +669,7 @@ int hat_qkv_rope_append(const hat_cache_desc* cache, const hat_plan* plan, const
     if (hidden % 64 != 0 || (plan->head_dim != 64 && plan->head_dim != 128)) return HAT_ERR_UNSUPPORTED;
     if (plan->total_rows == 0) return HAT_OK;
     if (!x || !w_qkv || !q_out || !aligned(x, 16) || !aligned(w_qkv, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
     cudaError_t e = launch_qkv_gemm(plan, view_of(cache), cache->k_pool, cache->v_pool, x, hidden, w_qkv, q_out, theta,
                                     interleaved != 0, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? HAT_OK : cuda_fail(e);
@@ -708,11 +704,16 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return cuda_fail(e);
     const bool capturing = cap != cudaStreamCaptureStatusNone;
-    if (!capturing && plan->has_last && plan->last_stream != s && (e = cudaStreamWaitEvent(s, plan->ev_done, 0)) != cudaSuccess)
+    if (capturing) mplan->captured = true;
+    else if (plan->loose && !plan->loose_many && plan->loose_stream == s) mplan->loose = false;   // ev_done, recorded on s below, covers it
+    if (!capturing && plan->has_last && plan->last_stream != s && (e = cudaStreamWaitEvent(s, plan->res.ev_done, 0)) != cudaSuccess)
         return cuda_fail(e);
     struct Done {
         hat_plan* p; cudaStream_t s; bool record;
-        ~Done() { if (record && p->ev_done && cudaEventRecord(p->ev_done, s) == cudaSuccess) { p->last_stream = s; p->has_last = true; } }
+        ~Done() {
+            if (record && cudaEventRecord(p->res.ev_done, s) == cudaSuccess) { p->last_stream = s; p->has_last = true; }
+            else if (record) { p->loose = p->loose_many = true; }
+        }
     } done{mplan, s, !capturing};
     // optional event recorder: a start and an end event per slot (append, tile, streaming, merge)
     Timing* tm = plan->timing;
@@ -770,7 +771,7 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
         if (e != cudaSuccess) return cuda_fail(e);
         mark(2, 1);
     }
-    if (plan->ev_verify && (e = cudaEventRecord(plan->ev_verify, s)) != cudaSuccess) return cuda_fail(e);
+    if (plan->res.ev_verify && (e = cudaEventRecord(plan->res.ev_verify, s)) != cudaSuccess) return cuda_fail(e);
     if (side) {
         e = launch_attn_tc5(plan, a, s, plan->side_sms, /*reset_counter=*/false);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, plan->ev_join, 0);
@@ -816,13 +817,13 @@ int hat_chunk_attention_out16(const hat_cache_desc* cache, const hat_plan* plan,
 
 int hat_plan_verify_event(const hat_plan* plan, void** event_out) {
     if (!plan || !event_out || plan->host_only) return HAT_ERR_INVALID_ARG;
-    *event_out = plan->ev_verify;
+    *event_out = plan->res.ev_verify;
     return HAT_OK;
 }
 
 int hat_plan_wait_verify(const hat_plan* plan) {
-    if (!plan || plan->host_only || !plan->ev_verify) return HAT_ERR_INVALID_ARG;
-    cudaError_t e = cudaEventSynchronize(plan->ev_verify);
+    if (!plan || plan->host_only || !plan->res.ev_verify) return HAT_ERR_INVALID_ARG;
+    cudaError_t e = cudaEventSynchronize(plan->res.ev_verify);
     return e == cudaSuccess ? HAT_OK : cuda_fail(e);
 }
 

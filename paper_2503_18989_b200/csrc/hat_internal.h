@@ -163,6 +163,23 @@ struct MapCache {
 cudaError_t smem_attr_once(const void* kernel, int bytes);
 }  // namespace hat
 
+namespace hat {
+// What a plan needs from the driver: one device allocation, the pinned buffer its contents are uploaded from, three
+// events.  Plans live for one inference step, and making these anew costs far more than the step's schedule
+// (cudaMalloc and cudaFree: 270 + 360 us beside 6 GB of pools), so a destroyed plan hands them on (hat_api.cu).
+struct PlanRes {
+    int device = -1;
+    void* blob = nullptr;
+    size_t blob_bytes = 0;
+    void* pinned = nullptr;
+    size_t pinned_bytes = 0;
+    cudaEvent_t ev_verify = nullptr;   // recorded in every attention call once the streaming-class rows are final
+    cudaEvent_t ev_done = nullptr;     // recorded at the end of every attention call: the next call on another stream waits for it
+    cudaEvent_t ev_table = nullptr;    // orders calls on other streams behind the kernel that filled the (cos, sin) table
+    bool in_use = false;               // the last owner's work may still run: ready once ev_done has occurred
+};
+}  // namespace hat
+
 struct hat_plan {
     // geometry the plan was made for
     int32_t dtype, num_pages, num_heads, num_kv_heads, head_dim, max_pages, num_requests, total_rows;   // num_heads: query heads
@@ -181,8 +198,6 @@ struct hat_plan {
     hat_plan_info info;
     hat::Timing* timing;        // null unless hat_plan_enable_timing was called
     int num_verify_merge_rows;  // merge rows of streaming-class requests; they come first in merge_rows
-    cudaEvent_t ev_verify;      // recorded in every attention call once the streaming-class rows are final
-    cudaEvent_t ev_done;        // recorded at the end of every attention call: the next call on another stream waits for it
     cudaStream_t last_stream;   // stream of the previous attention call
     bool has_last;
     // mixed batches: the tile kernel starts on side_sms fewer SMs on a stream of its own while the streaming kernel
@@ -195,12 +210,15 @@ struct hat_plan {
     int withhold_next;          // self test of the bounded waits: applies to the next attention call only
     hat::MapCache maps;         // see MapCache (updated through const_cast by the launchers: one call at a time per plan)
     // rotary position encoding in the projection epilogue: (cos, sin) of every row and pair for base rope_theta
-    // (0: not filled yet), inside dev_blob; ev_table orders calls on other streams behind the kernel that filled it
+    // (0: not filled yet), inside the plan's device memory
     float2* rope_table;
     float rope_theta;
     cudaStream_t table_stream;
-    cudaEvent_t ev_table;
-    void* dev_blob;             // one allocation holding every device array
+    hat::PlanRes res;           // device memory holding every device array, its staging buffer and the plan's events
+    // which work that uses `res` ev_done does not cover (see plan_note_call): decides whether it can be handed on
+    bool captured;              // a call was captured into a graph, which may be replayed at any time
+    bool loose, loose_many;     // calls other than attention since the last ev_done; on more than one stream
+    cudaStream_t loose_stream;
     hat::DevicePlan dev;
 };
 
@@ -231,6 +249,13 @@ cudaError_t launch_attn_stream(const hat_plan* plan, const AttnArgs& args, cudaS
 // Q/K/V projection with the rotation and the cache write in its epilogue (tcgen05); theta <= 0: no rotation
 cudaError_t launch_qkv_gemm(const hat_plan* plan, const CacheView& cache, void* k_pool, void* v_pool, const void* x,
                             int hidden, const void* w, void* q_out, float theta, int interleaved, cudaStream_t stream);
+// the pool of plan resources (plan_pool.cu)
+cudaError_t plan_res_acquire(int device, size_t blob_bytes, size_t pinned_bytes, PlanRes* out);
+cudaError_t plan_res_upload(PlanRes& r, size_t bytes);      // pinned -> blob, complete on return
+cudaError_t plan_res_release(PlanRes& r, bool reusable);    // reusable: ev_done covers every use, or there was none
+cudaError_t plan_res_free(PlanRes& r);
+cudaError_t plan_res_trim();                                // frees what waits for a later plan
+void plan_note_call(hat_plan* p, cudaStream_t s);           // a call other than attention is about to use the plan on s
 void count_launch(int n = 1);
 void set_last_cuda_error(int e);   // what hat_last_cuda_error() returns on this thread
 }  // namespace hat

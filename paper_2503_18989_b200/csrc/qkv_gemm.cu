@@ -480,11 +480,11 @@ cudaError_t launch_qkv_gemm(const hat_plan* plan, const CacheView& cache, void* 
             rope_table_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(plan->dev, d / 2, fr, mp->rope_table);
             count_launch();
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if ((e = cudaEventRecord(mp->ev_table, stream)) != cudaSuccess) return e;
+            if ((e = cudaEventRecord(mp->res.ev_table, stream)) != cudaSuccess) return e;
             mp->rope_theta = theta;
             mp->table_stream = stream;
         } else if (mp->table_stream != stream) {
-            if ((e = cudaStreamWaitEvent(stream, mp->ev_table, 0)) != cudaSuccess) return e;
+            if ((e = cudaStreamWaitEvent(stream, mp->res.ev_table, 0)) != cudaSuccess) return e;
         }
         a.trig = mp->rope_table;
     }
