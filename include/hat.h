@@ -177,10 +177,10 @@ int hat_plan_workspace_bytes(const hat_plan* plan, size_t* out);
 int hat_plan_destroy(hat_plan* plan);   /* NULL is accepted */
 
 /*
- * A destroyed plan hands its device memory (with the pinned buffer it was
- * filled from and its events) to later plans; at most 16 such pieces and 64 MiB
- * wait at any time.  hat_release_cached frees what waits (this synchronises the
- * device); it is never needed for correctness.  Any thread may call it.
+ * A destroyed plan hands its device memory and its events to later plans; at
+ * most 64 such pieces and 64 MiB wait at any time.  hat_release_cached frees
+ * what waits, and the pinned buffer plans are uploaded from (this synchronises
+ * the device); it is never needed for correctness.  Any thread may call it.
  */
 int hat_release_cached(void);
 

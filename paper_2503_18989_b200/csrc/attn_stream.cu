@@ -1,27 +1,62 @@
 // Streaming (verify-class) chunk attention: up to 16 query rows of one request against a long key range, bound by
-// HBM bandwidth.  One CTA = one work item (request, key range) x one head, four warps; warp w owns pages
-// w, w+4, ... of the range and streams them through its own three-slot shared-memory ring.  A page of one head is
-// fetched by TMA as 2 KiB boxes (64 columns x 16 tokens, 128-byte swizzle) whose arrival is counted on the slot's
-// mbarrier, so a page costs the warp a handful of instructions instead of address arithmetic for 32 vector loads.
-// The math is warp-level mma.sync m16n8k16 (queries padded to 16 rows, fp32 accumulate) with an online softmax whose
-// reference maximum only moves when it grows by more than 2^8, so the output accumulator is rarely rescaled.
-// The four warps are combined through shared memory; the result goes to out/lse or, for a cut request, to the
-// partial rows the merge kernel reads.  Waits on the mbarriers are bounded and report through the plan's status word.
+// HBM bandwidth.  One launch appends the chunk's K/V rows, attends, and merges requests whose keys were cut.
+//
+// Persistent kernel, two CTAs per SM (grid = min(units, 2 x SMs)), six warps each.  A unit = one piece of a request's
+// pages x one K/V head x one slab of 16 (chunk row, query head of the group) pairs; units are drawn longest piece
+// first from a counter in the plan.  What a request's rows see is laid out as a list of 16-key pages:
+//   pages 0 .. ceil(P/16)-1   the cached prefix, page by page of the block table (the last one cut at P)
+//   page  ceil(P/16)          the chunk's own rows, gathered: from k_new / v_new when the call appends (the pool then
+//                             need not be written first), else row by row from the pool; rows beyond the chunk are zero
+// so both kinds of call do the same arithmetic in the same order and give the same bits.
+//   warp 4      producer: waits for the end of the stream's previous kernel (no other warp touches what kernels write before
+//               the producer's data reaches it); unit after unit without draining in between, the Q tile (cp.async) and the pages, each by
+//               2 or 4 TMA boxes of 2 KiB (64 columns x 16 tokens, 128-byte swizzle), into a ring of slots on mbarriers
+//   warps 0-3   page j of a unit belongs to warp 3 - j mod 4: mma.sync m16n8k16, fp32 accumulate, online softmax whose
+//               reference maximum only moves when it grows by more than 2^8, so the accumulator is rarely rescaled.
+//               At the end of a unit the partial results pass from warp to warp through one shared-memory buffer; a warp
+//               goes on with the next unit as soon as it has handed over.  The warp that consumed the chunk page copies its
+//               rows from shared memory to the pool.
+//   warp 5      takes the unit's result out of that buffer, normalises and stores it.  A request cut into pieces: every
+//               piece stores partial rows and counts itself in; the CTA with the last piece of a (request, head, slab) merges them
+//               at its end with all warps, in the order of the pieces.  A warp of its own, so that stores, fence and count (2 us
+//               and more) hold up no one, and so that its registers do not weigh on the main loop
+//
+// A unit of 32 pairs (two warps to a page, K/V once instead of twice for grouped heads with more than 16 pairs) measured
+// slower: 16 requests x 8 K/V heads x 16..32 pairs, bf16, 100 us against 89 to 93 in two slabs of 16.  There mma.sync is the limit
+// (96 MMAs a page at 16 cycles), the second pass over K/V comes from L2, and slabs balance better.
+//
+// What bounds it: HBM for large batches (30 requests x 32 heads, 980 MB: 151 us = 6.5 TB/s, which is the measured copy rate; the
+// step of append, this kernel and their gap was 163 us, now 157), the start of the pipeline and the tail for medium ones (12
+// requests, 250 MB: 63 us of append, attention, merge and gaps per layer, now 46), a chain of latencies for one request
+// (4 rows x 700 tokens: 16.4 us a call, now 11.2: 1.5 us to the first request, 0.8 us HBM, 1 us a page, 1 us from warp to
+// warp, 3 us to store, count and merge).
+// Waits on the mbarriers are bounded and report through the plan's status word.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "hat_internal.h"
 #include "tma_desc.h"
+#include "tc5_ptx.cuh"
 
 namespace hat {
 namespace {
+using tc5::fast_exp2;
+using tc5::mbar_arrive;
+using tc5::mbar_expect_tx;
+using tc5::mbar_init;
+using tc5::mbar_try;
+using tc5::smem_u32;
 
-constexpr int kWarps = 4;
-constexpr int kSlots = 3;
+constexpr int kWarps = 4;                   // consumer warps
+constexpr int kThreads = kWarps * 32 + 64;
+constexpr int kCtasPerSm = 2;
+constexpr int kTodo = 48;                   // merges put off to the end of the CTA
+constexpr int kBatch = 4;                   // pages requested at a time
 constexpr float kMoveThreshold = 8.0f;      // log2 units
 
-__device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
@@ -43,23 +78,14 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
     }
 }
 template <bool BF16>
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-    if constexpr (BF16) {
-        __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-        return *reinterpret_cast<uint32_t*>(&v);
-    } else {
-        __half2 v = __floats2half2_rn(lo, hi);
-        return *reinterpret_cast<uint32_t*>(&v);
-    }
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) { return pack_out16(lo, hi, BF16); }
+// 16 bytes global -> shared, asynchronous; zeros when !valid
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
+// the barrier's current phase also waits for this thread's copies so far
+__device__ __forceinline__ void cp_async_on(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // Byte offset of 16-byte vector c of token row `row` in a page as TMA lays it down: two 2 KiB column halves,
@@ -69,324 +95,642 @@ __device__ __forceinline__ uint32_t page_off(int row, int c) {
     if constexpr (D == 128) return (uint32_t)((c >> 3) * 2048 + row * 128 + (((c & 7) ^ (row & 7)) << 4));
     else return (uint32_t)(row * 128 + ((c ^ (row & 7)) << 4));
 }
-// The Q tile is written by ordinary stores: rows of D*2 bytes, vector index XORed with the row.
+// The Q tile is written by ordinary copies: rows of D*2 bytes, vector index XORed with the row.
 template <int D>
 __device__ __forceinline__ uint32_t q_off(int row, int c) { return (uint32_t)(row * (D * 2) + ((c ^ (row & 7)) << 4)); }
 
+// Shared memory of a CTA: ring slots (one page of K, then of V), the Q tile, the hand-over buffer, barriers.
+// Every consumer warp has slots of its own: a parity wait is only sound for a waiter that has seen every earlier phase
+// of the barrier, so a slot must not pass from one warp to another.
+template <int D> struct Geo {
+    static constexpr uint32_t PAGE = 16 * D * 2;                 // K (or V) of one page of one head
+    static constexpr uint32_t SLOT = 2 * PAGE;
+    static constexpr uint32_t Q = 16 * D * 2;
+    static constexpr uint32_t X = (D / 8 + 1) * 512;             // accumulators (and maxima, sums) of one warp
+    // as many slots as let two CTAs share an SM (115712 bytes each)
+    static constexpr int PER = D == 64 ? 4 : 3;                  // slots of each consumer warp
+    static constexpr int SLOTS = kWarps * PER;
+};
+template <int SLOTS> struct __align__(16) Ctl {
+    int4 unit[3];                                                // the unit's StreamItem
+    int hs;                                                      // its head * n_sub + slab; -1: no unit left
+    uint64_t full[SLOTS], empty[SLOTS];
+    uint64_t q_full, q_empty;                                    // Q tile, unit and hs
+    int4 job[3];                                                 // the unit whose result is in the hand-over buffer
+    uint64_t x_free;                                             // the buffer has been read
+    int4 todo[kTodo][2];                                         // merges this CTA owes: it stored the last piece
+    int num_todo;
+    uint64_t todo_full;                                          // every unit is done, the list is final
+    uint64_t hand[kWarps];                                       // warp w has handed over (the last in line: to the output warp)
+    volatile int abort_flag;
+};
+
+template <int SLOTS>
+__device__ __forceinline__ bool wait_for(uint64_t* bar, uint32_t parity, Ctl<SLOTS>* ctl, const AttnArgs& a) {
+    if (mbar_try(bar, parity)) return true;
+    const long long t0 = clock64();
+    while (!mbar_try(bar, parity)) {
+        if (ctl->abort_flag) return false;
+        if (clock64() - t0 > a.wait_cycles) {
+            ctl->abort_flag = 1;
+            atomicOr(a.plan.status, 1);
+            return false;
+        }
+    }
+    return true;
+}
+
 template <bool BF16, int D>
-__global__ void __launch_bounds__(kWarps * 32)
-attn_stream_kernel(AttnArgs a, const WorkItem* __restrict__ items, int n_sub, const __grid_constant__ CUtensorMap map_k,
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, int total_units, int32_t* __restrict__ work_counter,
+                   int32_t* __restrict__ piece_counters, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v) {
-    using T = typename std::conditional<BF16, __nv_bfloat16, __half>::type;
-    constexpr int CH = D / 8, ON = D / 8, HALVES = D / 64;
-    constexpr uint32_t PAGE_BYTES = 16 * D * 2;              // K (or V) of one page of one head
-    constexpr uint32_t SLOT_BYTES = 2 * PAGE_BYTES;          // K then V
-    constexpr uint32_t Q_BYTES = 16 * D * 2;                 // multiple of 1024 for D = 64 and 128
+    using G_ = Geo<D>;
+    constexpr int CH = D / 8, ON = D / 8, SLOTS = G_::SLOTS, PER = G_::PER;
+    constexpr uint32_t PAGE = G_::PAGE, SLOT = G_::SLOT;
+    using Ctl_ = Ctl<SLOTS>;
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Q_BYTES + kWarps * kSlots * SLOT_BYTES);
-    const uint32_t sbase = s_u32(smem);
+    unsigned char* q_buf = smem + SLOTS * SLOT;
+    float4* xbuf = reinterpret_cast<float4*>(q_buf + G_::Q);
+    Ctl_* ctl = reinterpret_cast<Ctl_*>(q_buf + G_::Q + G_::X);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // A CTA serves one K/V head and 16 of the request's (chunk row i, query head gq of the head's group) pairs:
-    // MMA row m of slab `sub` is pair number sub * 16 + m = i * G + gq, so K/V are read once for the whole group.
-    const WorkItem item = items[blockIdx.y];
-    const int h = blockIdx.x / n_sub, sub = blockIdx.x % n_sub;
-    const int H = a.plan.num_heads, G = a.plan.group;
-    const int r = item.req;
-    const int P = a.plan.prefix_len[r];
-    const int C = a.plan.chunk_len[r];
-    if (sub * 16 >= C * G) return;                            // this request has fewer pairs
-    const int row_base = a.plan.cu_chunk[r];
-    const int32_t* __restrict__ table = a.plan.block_table + (int64_t)r * a.plan.max_pages;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
-
-    if (tid < kWarps * kSlots) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(s_u32(bars + tid)));
     if (tid == 0) {
+        for (int s = 0; s < SLOTS; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+        mbar_init(&ctl->q_full, 1);
+        mbar_init(&ctl->q_empty, kWarps);
+        mbar_init(&ctl->x_free, 1);
+        mbar_init(&ctl->todo_full, 1);
+        ctl->num_todo = 0;
+        for (int w = 0; w < kWarps; ++w) mbar_init(&ctl->hand[w], 1);
+        ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    // Q tile (rows >= C are zero)
-    {
-        const T* __restrict__ q = static_cast<const T*>(a.q);
-        for (int idx = tid; idx < 16 * CH; idx += kWarps * 32) {
-            const int row = idx / CH, c = idx % CH;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            const int pair = sub * 16 + row, i = pair / G;
-            if (i < C)
-                v = __ldg(reinterpret_cast<const uint4*>(q + ((int64_t)(row_base + i) * H + h * G + pair % G) * D) + c);
-            *reinterpret_cast<uint4*>(smem + q_off<D>(row, c)) = v;
-        }
-    }
+    tc5::pdl_launch_dependents();
     __syncthreads();
 
-    // ---- this warp's pages and its ring
-    const int n_pages = (item.kv_end - item.kv_begin + kPageSize - 1) / kPageSize;
-    const int n_my = n_pages > warp ? (n_pages - warp + kWarps - 1) / kWarps : 0;
-    const uint32_t ring = sbase + Q_BYTES + warp * (kSlots * SLOT_BYTES);
-    const uint32_t bar0 = s_u32(bars + warp * kSlots);
-    // lanes 0 .. 2*HALVES-1 each move one box: (K or V, column half)
-    auto issue = [&](int ti, int slot) {
-        const int kb = item.kv_begin + ti * kPageSize;
-        const uint32_t bar = bar0 + slot * 8;
-        if (lane == 0)
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(SLOT_BYTES) : "memory");
-        __syncwarp();
-        if (lane < 2 * HALVES) {
-            const int is_v = lane / HALVES, half = lane % HALVES;
-            const int page = HAT_IN_RANGE(__ldg(table + HAT_IN_RANGE(kb / kPageSize, a.plan.max_pages, a.plan.status)), a.plan.num_pages, a.plan.status);
-            const uint32_t dst = ring + slot * SLOT_BYTES + is_v * PAGE_BYTES + half * 2048;
-            const CUtensorMap* map = is_v ? &map_v : &map_k;
-            asm volatile(
-                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n"
-                ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(half * 64), "r"(0), "r"(h), "r"(page), "r"(bar)
-                : "memory");
-        }
-    };
-#pragma unroll
-    for (int s = 0; s < kSlots - 1; ++s)
-        if (s < n_my) issue(warp + s * kWarps, s);
-
-    uint32_t qf[D / 16][4];
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks) {
-        const int mi = lane >> 3;
-        ldsm4(qf[ks], sbase + q_off<D>((mi & 1) * 8 + (lane & 7), ks * 2 + (mi >> 1)));
-    }
-
-    float o[ON][4];
-#pragma unroll
-    for (int n = 0; n < ON; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
-    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // reference maxima (log2 units) and row sums, rows g and g+8
-    // chunk rows of MMA rows g and g+8, and the chunk positions each may see: bit c <=> key P + c.  The causal rule
-    // (Sec. 2.1 / 3.4: a linear draft sequence) is bits 0..i; a token tree supplies its own words
-    const int i0 = (sub * 16 + g) / G, i1 = (sub * 16 + g + 8) / G;
-    uint32_t bits0 = i0 < C ? (2u << i0) - 1u : 0u, bits1 = i1 < C ? (2u << i1) - 1u : 0u;
-    if (a.plan.tree_mask != nullptr) {
-        if (i0 < C) bits0 = __ldg(a.plan.tree_mask + row_base + i0);
-        if (i1 < C) bits1 = __ldg(a.plan.tree_mask + row_base + i1);
-    }
-    const int kend = item.kv_end;
+    const int H = a.plan.num_heads, G = a.plan.group, Hkv = a.plan.num_kv_heads;
+    const int hs_count = Hkv * n_sub;
+    const int4* __restrict__ recs = reinterpret_cast<const int4*>(items);
+    // chunk row of a (row, query head of the group) pair: pair / G, by a multiplication while that is exact (16 G pairs at most)
+    const uint32_t g_inv = ((1u << 20) + G - 1) / G;
+    auto pair_row = [&](int pair) { return G < 256 ? (int)(((uint32_t)pair * g_inv) >> 20) : pair / G; };
     bool ok = true;
 
-    for (int it = 0; it < n_my; ++it) {
-        const int slot = it % kSlots;
-        // the slot that page it+2 goes to was read in the previous iteration: every lane is past those reads here
-        __syncwarp();
-        if (it + kSlots - 1 < n_my) issue(warp + (it + kSlots - 1) * kWarps, (it + kSlots - 1) % kSlots);
-        {
-            const uint32_t bar = bar0 + slot * 8, parity = (it / kSlots) & 1;
-            if (!mbar_try(bar, parity)) {
-                const long long t0 = clock64();
-                while (!mbar_try(bar, parity)) {
-                    if (clock64() - t0 > a.wait_cycles) { ok = false; break; }
+    if (warp == kWarps) {
+        // ------------------------------------------------------------------ producer
+        const uint16_t* __restrict__ q = static_cast<const uint16_t*>(a.q);
+        const bool fused = a.k_new != nullptr;
+        // Pages are requested kBatch at a time, lanes 2 k and 2 k + 1 moving K and V of page k: a page at a time (600 cycles of
+        // waiting and issuing each) held the kernel at 4.8 TB/s.
+        // Page j of a unit goes to way kWarps - 1 - j mod kWarps: where the pages do not come out even, the first in the hand-over line
+        // has the fewest.
+        const int bk = lane < 2 * kBatch ? lane >> 1 : 0, is_v = lane & 1, way = kWarps - 1 - bk % kWarps;
+        int issued = 0;                                           // pages requested for `way` so far
+        int unit = blockIdx.x, un = 0;
+        int hs = 0, page_id = 0;
+        int4 r0, r1, r2;                                          // the unit's StreamItem; page_id: of its first 32 pages, one per lane
+        auto fetch_record = [&](int u, int& hs_, int4& q0, int4& q1, int4& q2) {
+            const int item = u / hs_count;
+            hs_ = u - item * hs_count;
+            q0 = __ldg(recs + item * 3); q1 = __ldg(recs + item * 3 + 1); q2 = __ldg(recs + item * 3 + 2);
+        };
+        auto fetch_ids = [&](const int4& q0, const int4& q1) {
+            const int32_t* __restrict__ t = a.plan.block_table + (int64_t)q0.x * a.plan.max_pages;
+            const int pg = q1.x + lane;
+            return pg < min(q1.y, (q0.w + kPageSize - 1) / kPageSize) ? __ldg(t + pg) : 0;
+        };
+        fetch_record(unit, hs, r0, r1, r2);
+        page_id = fetch_ids(r0, r1);
+        tc5::pdl_wait();                                          // up to here only the plan's own arrays were read
+        for (;;) {
+            const bool done = unit >= total_units;
+            const int row_base = r0.y, C = r0.z, P = r0.w, page0 = r1.x, page1 = r1.y;
+            const int32_t* __restrict__ table = a.plan.block_table + (int64_t)r0.x * a.plan.max_pages;
+            const int npre = (P + kPageSize - 1) / kPageSize;
+            const int h = hs / n_sub, sub = hs - h * n_sub;
+#ifdef HAT_DEBUG_BOUNDS
+            if (!done && (r0.x < 0 || C < 1 || C > 16 || P < 0 || row_base < 0 || row_base + C > a.plan.total_rows || page0 < 0 ||
+                          page1 <= page0 || page1 > npre + 1 || npre > a.plan.max_pages || r2.x < 1 || r2.x > kMaxSplits)) {
+                if (lane == 0) atomicOr(a.plan.status, 2);
+                ctl->abort_flag = 1;
+                ok = false;
+                break;
+            }
+#endif
+            const bool skip = !done && sub * 16 >= C * G;    // this request has fewer pairs
+            if (!skip) {
+                if (un >= 1) ok = wait_for(&ctl->q_empty, (un - 1) & 1, ctl, a);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (!done) {
+                    // this lane copies 16 bytes of every (32 / CH)-th row
+                    const int c = lane % CH;
+#pragma unroll
+                    for (int row = lane / CH; row < 16; row += 32 / CH) {
+                        const int pair = sub * 16 + row, i = pair_row(pair);
+                        const bool in = i < C;
+                        const uint16_t* src = q + (in ? ((int64_t)(row_base + i) * H + h * G + (pair - i * G)) * D + c * 8 : 0);
+                        cp_async16(smem_u32(q_buf) + q_off<D>(row, c), src, in);
+                    }
+                    cp_async_on(&ctl->q_full);
+                }
+                if (lane == 0) { ctl->unit[0] = r0; ctl->unit[1] = r1; ctl->unit[2] = r2; ctl->hs = done ? -1 : hs; }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->q_full);
+                ++un;
+            }
+            if (done) break;
+            // The next unit is drawn, its record and its first page ids are fetched while this unit's last pages are requested,
+            // one step per batch: fetched at the boundary they cost 2 us without a request in flight.
+            int step = 0, drawn = 0, next = 0, next_hs = 0, next_id = 0;
+            int4 n0 = r0, n1 = r1, n2 = r2;
+            auto look_ahead = [&]() {
+                if (step == 0) {
+                    if (lane == 0) drawn = atomicAdd(work_counter, 1);
+                } else if (step == 1) {
+                    next = __shfl_sync(0xffffffffu, drawn, 0) + (int)gridDim.x;
+                    if (next < total_units) fetch_record(next, next_hs, n0, n1, n2);
+                } else {
+                    if (next < total_units) next_id = fetch_ids(n0, n1);
+                }
+                ++step;
+            };
+            if (!skip) {
+                const int n = page1 - page0;
+                int ids = page_id, ids_next = 0;                  // page ids of this and the next 32 pages, one per lane
+                for (int j0 = 0; j0 < n; j0 += kBatch) {
+                    if (step < 3 && n - j0 <= 6 * kBatch) look_ahead();
+                    if ((j0 & 31) == 0) {
+                        if (j0 > 0) ids = ids_next;
+                        const int ahead = page0 + j0 + 32 + lane;
+                        ids_next = ahead < min(page1, npre) ? __ldg(table + ahead) : 0;
+                    }
+                    const int page = HAT_IN_RANGE(__shfl_sync(0xffffffffu, ids, (j0 + bk) & 31), a.plan.num_pages, a.plan.status);
+                    const int turn = issued + bk / kWarps, slot = way * PER + turn % PER;
+                    const bool mine = lane < 2 * kBatch && j0 + bk < n;
+                    if (mine && turn >= PER) ok = wait_for(&ctl->empty[slot], (turn / PER - 1) & 1, ctl, a);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const bool prefix = mine && page0 + j0 + bk < npre;
+                    if (prefix && !is_v) mbar_expect_tx(&ctl->full[slot], SLOT);
+                    __syncwarp();
+                    if (prefix) tc5::tma_load_5d(smem_u32(smem) + slot * SLOT + is_v * PAGE, is_v ? &map_v : &map_k, 0, 0, 0, h, page, &ctl->full[slot]);
+                    if (page1 > npre && j0 + kBatch >= n) {
+                        // the chunk's rows, one after the other from k_new / v_new or from their slots of the pool
+                        const int cslot = __shfl_sync(0xffffffffu, slot, 2 * (n - 1 - j0));
+                        const uint32_t dst = smem_u32(smem) + cslot * SLOT;
+#pragma unroll 4
+                        for (int idx = lane; idx < 16 * CH; idx += 32) {
+                            const int row = idx / CH, c = idx % CH;
+                            const bool in = row < C;
+                            const uint16_t *ks = static_cast<const uint16_t*>(a.cache.k_pool), *vs = static_cast<const uint16_t*>(a.cache.v_pool);
+                            if (in && fused) {
+                                const int64_t off = ((int64_t)(row_base + row) * Hkv + h) * D + c * 8;
+                                ks = static_cast<const uint16_t*>(a.k_new) + off;
+                                vs = static_cast<const uint16_t*>(a.v_new) + off;
+                            } else if (in) {
+                                const int pos = P + row;
+                                const int pp = HAT_IN_RANGE(__ldg(table + HAT_IN_RANGE(pos / kPageSize, a.plan.max_pages, a.plan.status)), a.plan.num_pages, a.plan.status);
+                                const int64_t off = pp * a.cache.stride_page + (pos % kPageSize) * a.cache.stride_token + h * a.cache.stride_head + c * 8;
+                                ks += off; vs += off;
+                            }
+                            cp_async16(dst + page_off<D>(row, c), ks, in);
+                            cp_async16(dst + PAGE + page_off<D>(row, c), vs, in);
+                        }
+                        cp_async_on(&ctl->full[cslot]);
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&ctl->full[cslot]);
+                    }
+                    issued += (min(kBatch, n - j0) + way) / kWarps;
+                }
+                if (!ok) break;
+            }
+            while (step < 3) look_ahead();
+            unit = next; hs = next_hs; page_id = next_id;
+            r0 = n0; r1 = n1; r2 = n2;
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        if (!ok) {
+            // give the copies still in flight a bounded time to land before the CTA's shared memory is released
+            const long long t0 = clock64();
+            while (clock64() - t0 < 2000000) { }
+        }
+        // the last producer to finish leaves the unit counter at zero for the next call
+        if (lane == 0) {
+            __threadfence();
+            if (atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {
+                work_counter[0] = 0;
+                work_counter[1] = 0;
+                __threadfence();
+            }
+        }
+        return;
+    }
+
+    // Merges of cut requests whose last piece this CTA stored: rows first, first + step, ... of the list, two at a time.  They are
+    // put off to the end of the CTA: a round trip to L2 takes 3000 cycles while the pages stream, a merge several of them,
+    // and meanwhile the hand-over buffer would be blocked (spec_verify cut into 135 pieces: 9 us per merge).
+    auto merge_todo = [&](int first, int step) {
+        constexpr int V = D / 32, NP = 8;                         // floats per lane, pieces in flight
+        const int n_todo = ctl->num_todo;
+        int turn = 0;
+        for (int e = 0; e < n_todo; ++e) {
+            const int4 j0 = ctl->todo[e][0], j1 = ctl->todo[e][1];
+            const int part0 = j0.x, nsplit = j0.y, row_base = j0.z, C = j0.w, pair0 = j1.x, pairs = j1.y, h = j1.z;
+            const int64_t hop = (int64_t)C * H;                   // (row, head) pairs from one piece to the next
+            for (int p0 = 0; p0 < pairs; p0 += 2, ++turn) {
+                if (turn % step != first) continue;
+                int64_t at0[2], at[2];
+                float w[2], v[2][NP][V], acc[2][V], mx[2], sum[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int pair = pair0 + min(p0 + u, pairs - 1), i = pair_row(pair), hq = h * G + (pair - i * G);
+                    at0[u] = ((int64_t)part0 + i) * H + hq;
+                    at[u] = (int64_t)(row_base + i) * H + hq;
+                    w[u] = lane < nsplit ? __ldcg(a.part_lse + at0[u] + lane * hop) : -INFINITY;
+                }
+                auto load_pieces = [&](int s0) {
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+#pragma unroll
+                        for (int s = 0; s < NP; ++s)
+                            if (s0 + s < nsplit) {
+                                const float* src = a.part_out + (at0[u] + (s0 + s) * hop) * D + lane * V;
+                                if constexpr (V == 4) { const float4 y = __ldcg(reinterpret_cast<const float4*>(src)); v[u][s][0] = y.x; v[u][s][1] = y.y; v[u][s][2] = y.z; v[u][s][3] = y.w; }
+                                else { const float2 y = __ldcg(reinterpret_cast<const float2*>(src)); v[u][s][0] = y.x; v[u][s][1] = y.y; }
+                            }
+                };
+                load_pieces(0);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) mx[u] = w[u];
+#pragma unroll
+                for (int k = 16; k > 0; k >>= 1)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) mx[u] = fmaxf(mx[u], __shfl_xor_sync(0xffffffffu, mx[u], k));
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    mx[u] = mx[u] == -INFINITY ? 0.f : mx[u];
+                    w[u] = sum[u] = expf(w[u] - mx[u]);           // 0 for empty pieces and idle lanes
+                }
+#pragma unroll
+                for (int k = 16; k > 0; k >>= 1)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], k);
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int k = 0; k < V; ++k) acc[u][k] = 0.f;
+                for (int s0 = 0; s0 < nsplit; s0 += NP) {
+                    if (s0 > 0) load_pieces(s0);
+#pragma unroll
+                    for (int s = 0; s < NP; ++s)
+                        if (s0 + s < nsplit) {
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                const float ws = __shfl_sync(0xffffffffu, w[u], s0 + s);
+#pragma unroll
+                                for (int k = 0; k < V; ++k) acc[u][k] += ws * v[u][s][k];
+                            }
+                        }
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (p0 + u >= pairs) break;
+                    const float inv = sum[u] > 0.f ? 1.f / sum[u] : 0.f;
+#pragma unroll
+                    for (int k = 0; k < V; ++k) acc[u][k] *= inv;
+                    if (a.out16 != nullptr) {
+                        uint16_t* dst = static_cast<uint16_t*>(a.out16) + at[u] * D + lane * V;
+                        if constexpr (V == 4)
+                            *reinterpret_cast<uint2*>(dst) = make_uint2(pack_out16(acc[u][0], acc[u][1], a.out16_bf16), pack_out16(acc[u][2], acc[u][3], a.out16_bf16));
+                        else
+                            *reinterpret_cast<uint32_t*>(dst) = pack_out16(acc[u][0], acc[u][1], a.out16_bf16);
+                    } else if constexpr (V == 4) {
+                        *reinterpret_cast<float4*>(a.out + at[u] * D + lane * V) = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+                    } else {
+                        *reinterpret_cast<float2*>(a.out + at[u] * D + lane * V) = make_float2(acc[u][0], acc[u][1]);
+                    }
+                    if (lane == 0) a.lse[at[u]] = sum[u] > 0.f ? mx[u] + logf(sum[u]) : -INFINITY;
                 }
             }
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
         }
-        const int kb = item.kv_begin + (warp + it * kWarps) * kPageSize;
-        const uint32_t kst = ring + slot * SLOT_BYTES, vst = kst + PAGE_BYTES;
-        if (kb + kPageSize > kend) {
-            // the range ends inside this page: the slots past it hold stale tokens; zero their V rows so that
-            // 0 * garbage cannot produce NaN (their scores are masked below)
-            const int first = kend - kb;
-            for (int idx = lane; idx < (kPageSize - first) * CH; idx += 32) {
-                const int row = first + idx / CH, c = idx % CH;
-                asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};\n" ::"r"(vst + page_off<D>(row, c)), "r"(0));
+    };
+
+    if (warp == kWarps + 1) {
+        // ------------------------------------------------------------------ output, merge of cut requests
+        const int g = lane >> 2, t4 = lane & 3;
+        for (int un = 0;; ++un) {
+            ok = __all_sync(0xffffffffu, wait_for(&ctl->hand[kWarps - 1], un & 1, ctl, a));
+            if (!ok) return;
+            const int4 j0 = ctl->job[0], j1 = ctl->job[1], j2 = ctl->job[2];
+            const int part0 = j0.x, nsplit = j0.y, row_base = j0.w, C = j1.x, pair0 = j1.y, pairs = j1.z, h = j1.w, part = j2.x;
+            if (nsplit < 0) {
+                if (lane == 0) mbar_arrive(&ctl->todo_full);
+                merge_todo(kWarps, kWarps + 1);
+                return;
+            }
+            {
+                float4 o[ON];
+                const float4* x = xbuf + lane;
+                const float4 ml = x[ON * 32];
+#pragma unroll
+                for (int c = 0; c < ON; ++c) o[c] = x[c * 32];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->x_free);
+                // normalise and store: final rows, or partial rows of a cut request
+                constexpr float kLn2 = 0.6931471805599453f;
+                const bool to16 = part < 0 && a.out16 != nullptr;    // final rows in the 16-bit output type
+                float* obase = part < 0 ? a.out : a.part_out;
+                float* lbase = part < 0 ? a.lse : a.part_lse;
+                const int64_t first = part < 0 ? row_base : part;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (e * 8 + g >= pairs) continue;
+                    const int pair = pair0 + e * 8 + g, i = pair_row(pair), hq = h * G + (pair - i * G);
+                    const float m = e ? ml.y : ml.x, sum = e ? ml.w : ml.z, inv = sum > 0.f ? 1.f / sum : 0.f;
+                    const int64_t at = ((first + i) * H + hq) * D + 2 * t4;
+#pragma unroll
+                    for (int c = 0; c < ON; ++c) {
+                        const float v0 = (e ? o[c].z : o[c].x) * inv, v1 = (e ? o[c].w : o[c].y) * inv;
+                        if (to16) *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(a.out16) + at + c * 8) = pack_out16(v0, v1, a.out16_bf16);
+                        else *reinterpret_cast<float2*>(obase + at + c * 8) = make_float2(v0, v1);
+                    }
+                    if (t4 == 0) lbase[(first + i) * H + hq] = sum > 0.f ? (m + log2f(sum)) * kLn2 : -INFINITY;
+                }
+            }
+            if (part < 0) continue;
+            __syncwarp();
+            int arrived = 0;
+            if (lane == 0) {
+                asm volatile("fence.acq_rel.gpu;\n" ::: "memory");   // every lane's partial rows before the count
+                arrived = atomicAdd(piece_counters + j0.z, 1);
+            }
+            if (__shfl_sync(0xffffffffu, arrived, 0) != nsplit - 1) continue;
+            asm volatile("fence.acq_rel.gpu;\n" ::: "memory");
+            if (lane == 0) piece_counters[j0.z] = 0;              // for the next call
+            if (lane == 0) {
+                const int at = ctl->num_todo;
+                ctl->todo[at][0] = make_int4(part0, nsplit, row_base, C);
+                ctl->todo[at][1] = make_int4(pair0, pairs, h, 0);
+                ctl->num_todo = at + 1;
             }
             __syncwarp();
-        }
-
-        // S = Q K^T for the 16 keys of the page
-        float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-            const int mi = lane >> 3;
-            uint32_t b[4];
-            ldsm4(b, kst + page_off<D>((mi >> 1) * 8 + (lane & 7), ks * 2 + (mi & 1)));
-            mma16816<BF16>(s[0], qf[ks], b[0], b[1]);
-            mma16816<BF16>(s[1], qf[ks], b[2], b[3]);
-        }
-        float mx0 = -INFINITY, mx1 = -INFINITY;
-        if (kb + kPageSize > min(P, kend)) {                     // the page holds chunk positions or ends the range
-#pragma unroll
-            for (int n = 0; n < 2; ++n) {
-                const int j = kb + n * 8 + 2 * t4;
-                // key j of the range: everything below P, bit j - P from there on (j < kend <= P + 16 bounds the shift)
-                const bool in0 = j < kend, in1 = j + 1 < kend;
-                const uint32_t sh0 = (uint32_t)min(max(j - P, 0), 31), sh1 = (uint32_t)min(max(j + 1 - P, 0), 31);
-                const bool a0 = in0 && (j < P || ((bits0 >> sh0) & 1u));
-                const bool a1 = in1 && (j + 1 < P || ((bits0 >> sh1) & 1u));
-                const bool b0 = in0 && (j < P || ((bits1 >> sh0) & 1u));
-                const bool b1 = in1 && (j + 1 < P || ((bits1 >> sh1) & 1u));
-                s[n][0] = a0 ? s[n][0] * a.scale_log2 : -INFINITY;
-                s[n][1] = a1 ? s[n][1] * a.scale_log2 : -INFINITY;
-                s[n][2] = b0 ? s[n][2] * a.scale_log2 : -INFINITY;
-                s[n][3] = b1 ? s[n][3] * a.scale_log2 : -INFINITY;
+            if (ctl->num_todo == kTodo) {                         // no room for more: pay now
+                merge_todo(0, 1);
+                __syncwarp();
+                if (lane == 0) ctl->num_todo = 0;
+                __syncwarp();
             }
-        } else {
-#pragma unroll
-            for (int n = 0; n < 2; ++n) {
-                s[n][0] *= a.scale_log2; s[n][1] *= a.scale_log2; s[n][2] *= a.scale_log2; s[n][3] *= a.scale_log2;
-            }
-        }
-#pragma unroll
-        for (int n = 0; n < 2; ++n) {
-            mx0 = fmaxf(mx0, fmaxf(s[n][0], s[n][1]));
-            mx1 = fmaxf(mx1, fmaxf(s[n][2], s[n][3]));
-        }
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-        // move a row's reference maximum only when the new maximum exceeds it by more than the threshold; weights
-        // then stay below 2^8 and the accumulators are rescaled only on the (rare) iterations where some row moved
-        const bool mv0 = mx0 > m0 + kMoveThreshold, mv1 = mx1 > m1 + kMoveThreshold;
-        if (__any_sync(0xffffffffu, mv0 || mv1)) {
-            const float al0 = mv0 ? ((m0 == -INFINITY) ? 0.f : exp2f(m0 - mx0)) : 1.f;
-            const float al1 = mv1 ? ((m1 == -INFINITY) ? 0.f : exp2f(m1 - mx1)) : 1.f;
-            if (mv0) m0 = mx0;
-            if (mv1) m1 = mx1;
-            l0 *= al0; l1 *= al1;
-#pragma unroll
-            for (int n = 0; n < ON; ++n) { o[n][0] *= al0; o[n][1] *= al0; o[n][2] *= al1; o[n][3] *= al1; }
-        }
-        const float r0 = (m0 == -INFINITY) ? 0.f : m0, r1 = (m1 == -INFINITY) ? 0.f : m1;
-#pragma unroll
-        for (int n = 0; n < 2; ++n) {
-            s[n][0] = exp2f(s[n][0] - r0); s[n][1] = exp2f(s[n][1] - r0);
-            s[n][2] = exp2f(s[n][2] - r1); s[n][3] = exp2f(s[n][3] - r1);
-            l0 += s[n][0] + s[n][1];
-            l1 += s[n][2] + s[n][3];
-        }
-        // O += P V
-        uint32_t pa[4], pl[4];
-        pa[0] = pack2<BF16>(s[0][0], s[0][1]); pa[1] = pack2<BF16>(s[0][2], s[0][3]);
-        pa[2] = pack2<BF16>(s[1][0], s[1][1]); pa[3] = pack2<BF16>(s[1][2], s[1][3]);
-        if constexpr (BF16) {
-            // bf16 keeps 8 significant bits: a second operand carries what the rounding of P dropped
-            const float* sf = &s[0][0];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float lo = __uint_as_float(pa[k] << 16), hi = __uint_as_float(pa[k] & 0xffff0000u);
-                pl[k] = pack2<BF16>(sf[2 * k] - lo, sf[2 * k + 1] - hi);
-            }
-        }
-#pragma unroll
-        for (int dn = 0; dn < D / 16; ++dn) {
-            const int mi = lane >> 3;
-            uint32_t b[4];
-            ldsm4t(b, vst + page_off<D>((mi & 1) * 8 + (lane & 7), dn * 2 + (mi >> 1)));
-            mma16816<BF16>(o[2 * dn], pa, b[0], b[1]);
-            mma16816<BF16>(o[2 * dn + 1], pa, b[2], b[3]);
-            if constexpr (BF16) {
-                mma16816<BF16>(o[2 * dn], pl, b[0], b[1]);
-                mma16816<BF16>(o[2 * dn + 1], pl, b[2], b[3]);
-            }
-        }
-    }
-    if (!ok) {
-        // a transfer never arrived: report it, then give the copies still in flight a bounded time to land
-        if (lane == 0) atomicExch(a.plan.status, 1);
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000) { }
-        for (int n = 0; n < ON; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
-        l0 = l1 = 0.f;
-    }
-    l0 += __shfl_xor_sync(0xffffffffu, l0, 1); l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-    l1 += __shfl_xor_sync(0xffffffffu, l1, 1); l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-
-    // ---- combine the four warps through shared memory (fragment positions are identical in each)
-    constexpr int VALS = ON * 4 + 4;
-    static_assert((kWarps - 1) * VALS * 32 * 4 <= kWarps * kSlots * (int)SLOT_BYTES, "exchange buffer must fit in the rings");
-    __syncthreads();                                             // every ring is idle: no load is outstanding
-    float* xbuf = reinterpret_cast<float*>(smem + Q_BYTES);
-    if (warp > 0) {
-        float* dst = xbuf + (warp - 1) * (VALS * 32) + lane;
-#pragma unroll
-        for (int n = 0; n < ON; ++n)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) dst[(n * 4 + k) * 32] = o[n][k];
-        dst[(ON * 4 + 0) * 32] = m0; dst[(ON * 4 + 1) * 32] = m1;
-        dst[(ON * 4 + 2) * 32] = l0; dst[(ON * 4 + 3) * 32] = l1;
-    }
-    __syncthreads();
-    if (warp > 0) return;
-    float mt0 = m0, mt1 = m1;
-#pragma unroll
-    for (int k = 1; k < kWarps; ++k) {
-        const float* src = xbuf + (k - 1) * (VALS * 32) + lane;
-        mt0 = fmaxf(mt0, src[(ON * 4 + 0) * 32]);
-        mt1 = fmaxf(mt1, src[(ON * 4 + 1) * 32]);
-    }
-    const float ms0 = (mt0 == -INFINITY) ? 0.f : mt0, ms1 = (mt1 == -INFINITY) ? 0.f : mt1;
-    {
-        const float w0 = exp2f(m0 - ms0), w1 = exp2f(m1 - ms1);
-        l0 *= w0; l1 *= w1;
-#pragma unroll
-        for (int n = 0; n < ON; ++n) { o[n][0] *= w0; o[n][1] *= w0; o[n][2] *= w1; o[n][3] *= w1; }
-    }
-#pragma unroll
-    for (int k = 1; k < kWarps; ++k) {
-        const float* src = xbuf + (k - 1) * (VALS * 32) + lane;
-        const float w0 = exp2f(src[(ON * 4 + 0) * 32] - ms0), w1 = exp2f(src[(ON * 4 + 1) * 32] - ms1);
-        l0 += w0 * src[(ON * 4 + 2) * 32];
-        l1 += w1 * src[(ON * 4 + 3) * 32];
-#pragma unroll
-        for (int n = 0; n < ON; ++n) {
-            o[n][0] += w0 * src[(n * 4 + 0) * 32]; o[n][1] += w0 * src[(n * 4 + 1) * 32];
-            o[n][2] += w1 * src[(n * 4 + 2) * 32]; o[n][3] += w1 * src[(n * 4 + 3) * 32];
         }
     }
 
-    // ---- normalise and store (final rows, or partial rows for the merge kernel)
-    const float inv0 = l0 > 0.f ? 1.f / l0 : 0.f, inv1 = l1 > 0.f ? 1.f / l1 : 0.f;
-    constexpr float kLn2 = 0.6931471805599453f;
-    const float lse0 = l0 > 0.f ? (mt0 + log2f(l0)) * kLn2 : -INFINITY;
-    const float lse1 = l1 > 0.f ? (mt1 + log2f(l1)) * kLn2 : -INFINITY;
-    const int hq0 = h * G + (sub * 16 + g) % G, hq1 = h * G + (sub * 16 + g + 8) % G;
-    float* obase; float* lbase; int64_t r0, r1;
-    if (item.part < 0) { obase = a.out; lbase = a.lse; r0 = row_base + i0; r1 = row_base + i1; }
-    else { obase = a.part_out; lbase = a.part_lse; r0 = item.part + i0; r1 = item.part + i1; }
-    const bool to16 = item.part < 0 && a.out16 != nullptr;      // final rows in the 16-bit output type
-    if (i0 < C) {
-        const int64_t at = (r0 * H + hq0) * D + 2 * t4;
-        if (to16) {
-#pragma unroll
-            for (int n = 0; n < ON; ++n)
-                *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(a.out16) + at + n * 8) = pack_out16(o[n][0] * inv0, o[n][1] * inv0, a.out16_bf16);
-        } else {
-#pragma unroll
-            for (int n = 0; n < ON; ++n) *reinterpret_cast<float2*>(obase + at + n * 8) = make_float2(o[n][0] * inv0, o[n][1] * inv0);
+    // ---------------------------------------------------------------------- consumers
+    const int g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
+    const bool append = a.k_new != nullptr;
+    const uint32_t k_lane = page_off<D>((mi >> 1) * 8 + (lane & 7), mi & 1), v_lane = page_off<D>((mi & 1) * 8 + (lane & 7), mi >> 1);
+    int taken = 0;                                                // pages this warp has consumed so far
+    for (int un = 0;; ++un) {
+        ok = __all_sync(0xffffffffu, wait_for(&ctl->q_full, un & 1, ctl, a));
+        if (!ok) return;
+        const int hs = ctl->hs;
+        if (hs < 0) {
+            // the end, handed on to the output warp once it has taken the previous result
+            if (warp == kWarps - 1) {
+                if (un > 0) ok = __all_sync(0xffffffffu, wait_for(&ctl->x_free, (un - 1) & 1, ctl, a));
+                if (!ok) return;
+                if (lane == 0) { ctl->job[0] = make_int4(0, -1, 0, 0); mbar_arrive(&ctl->hand[warp]); }
+            }
+            // what is left to merge, with every warp
+            ok = __all_sync(0xffffffffu, wait_for(&ctl->todo_full, 0, ctl, a));
+            if (ok) merge_todo(warp, kWarps + 1);
+            return;
         }
-        if (t4 == 0) lbase[r0 * H + hq0] = lse0;
-    }
-    if (i1 < C) {
-        const int64_t at = (r1 * H + hq1) * D + 2 * t4;
-        if (to16) {
+        const int4 r0 = ctl->unit[0], r1 = ctl->unit[1], r2 = ctl->unit[2];
+        const int row_base = r0.y, C = r0.z, P = r0.w, page0 = r1.x, n = r1.y - r1.x, part = r1.z;
+        const int h = hs / n_sub, sub = hs - h * n_sub;
+        const int npre = (P + kPageSize - 1) / kPageSize;
+        const int pair0 = sub * 16;                                // the unit's pairs: pair0 .. pair0 + pairs - 1
+        const int pairs = min(16, C * G - pair0);                  // at least 1
+        const bool low_rows = pairs <= 8;                          // rows 8..15 of the tile hold nothing
+        const uint32_t qbase = smem_u32(q_buf);
+
+        uint32_t qf[D / 16][4];
 #pragma unroll
-            for (int n = 0; n < ON; ++n)
-                *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(a.out16) + at + n * 8) = pack_out16(o[n][2] * inv1, o[n][3] * inv1, a.out16_bf16);
-        } else {
+        for (int ks = 0; ks < D / 16; ++ks) ldsm4(qf[ks], qbase + q_off<D>((mi & 1) * 8 + (lane & 7), ks * 2 + (mi >> 1)));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->q_empty);
+
+        float o[ON][4];
+        float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};     // reference maxima (log2 units) and row sums, rows g and g+8
 #pragma unroll
-            for (int n = 0; n < ON; ++n) *reinterpret_cast<float2*>(obase + at + n * 8) = make_float2(o[n][2] * inv1, o[n][3] * inv1);
+        for (int k = 0; k < ON; ++k) o[k][0] = o[k][1] = o[k][2] = o[k][3] = 0.f;
+
+        for (int j = kWarps - 1 - warp; j < n; j += kWarps, ++taken) {
+            const int slot = warp * PER + taken % PER;
+            const int pg = page0 + j;
+            const bool chunk_page = pg == npre;
+            // where the rows this lane will copy to the pool go: looked up ahead of the wait
+            int page_a = 0, page_b = 0;
+            if (chunk_page && append && sub == 0) {
+                const int32_t* __restrict__ table = a.plan.block_table + (int64_t)r0.x * a.plan.max_pages;
+                page_a = HAT_IN_RANGE(__ldg(table + HAT_IN_RANGE(P / kPageSize, a.plan.max_pages, a.plan.status)), a.plan.num_pages, a.plan.status);
+                page_b = HAT_IN_RANGE(__ldg(table + HAT_IN_RANGE((P + C - 1) / kPageSize, a.plan.max_pages, a.plan.status)), a.plan.num_pages, a.plan.status);
+            }
+            ok = __all_sync(0xffffffffu, wait_for(&ctl->full[slot], (taken / PER) & 1, ctl, a));
+            if (!ok) return;
+            const uint32_t kst = smem_u32(smem) + slot * SLOT, vst = kst + PAGE;
+            // where this lane's first fragment of K and V lies; the others differ in address bits 5 and 6 and by 2 KiB (page_off)
+            const uint32_t ka = kst + k_lane, va = vst + v_lane;
+            // keys of the page before `cut` hold the prefix (all 16 but in its last page); the chunk page has its own rule
+            const int cut = chunk_page ? kPageSize : min(kPageSize, P - pg * kPageSize);
+            if (cut < kPageSize) {
+                // slots past the prefix hold stale tokens: zero their V rows so that 0 * garbage cannot produce NaN (their
+                // scores are masked below)
+                for (int idx = lane; idx < (kPageSize - cut) * CH; idx += 32) {
+                    const int row = cut + idx / CH, c = idx % CH;
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};\n" ::"r"(vst + page_off<D>(row, c)), "r"(0) : "memory");
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the slot's next TMA write comes after these
+                __syncwarp();
+            }
+
+            // S = Q K^T for the 16 keys of the page, even and odd halves of the sum apart (half as long a chain of MMAs)
+            float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, s2[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+                uint32_t b[4];
+                ldsm4(b, (ka ^ ((ks & 3) << 5)) + (ks >> 2) * 2048);
+                mma16816<BF16>(ks & 1 ? s2[0] : s[0], qf[ks], b[0], b[1]);
+                mma16816<BF16>(ks & 1 ? s2[1] : s[1], qf[ks], b[2], b[3]);
+            }
+            uint32_t pa[4], pl[4];
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[k][e] = (s[k][e] + s2[k][e]) * a.scale_log2;
+            if (chunk_page || cut < kPageSize) {
+                // visible keys of the page, bit c = key c: of the chunk, its causal or tree word; of the prefix, those before `cut`
+                uint32_t bits0 = (1u << cut) - 1u, bits1 = bits0;
+                if (chunk_page) {
+                    const int i0 = pair_row(pair0 + g), i1 = pair_row(pair0 + g + 8);
+                    const uint32_t all = (1u << C) - 1u;
+                    bits0 = i0 < C ? (2u << i0) - 1u : 0u; bits1 = i1 < C ? (2u << i1) - 1u : 0u;
+                    if (a.plan.tree_mask != nullptr) {
+                        if (i0 < C) bits0 = __ldg(a.plan.tree_mask + row_base + i0) & all;
+                        if (i1 < C) bits1 = __ldg(a.plan.tree_mask + row_base + i1) & all;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int c = k * 8 + 2 * t4;
+                    s[k][0] = (bits0 >> c) & 1u ? s[k][0] : -INFINITY;
+                    s[k][1] = (bits0 >> (c + 1)) & 1u ? s[k][1] : -INFINITY;
+                    s[k][2] = (bits1 >> c) & 1u ? s[k][2] : -INFINITY;
+                    s[k][3] = (bits1 >> (c + 1)) & 1u ? s[k][3] : -INFINITY;
+                }
+            }
+            float mx0 = fmaxf(fmaxf(s[0][0], s[0][1]), fmaxf(s[1][0], s[1][1]));
+            float mx1 = low_rows ? -INFINITY : fmaxf(fmaxf(s[0][2], s[0][3]), fmaxf(s[1][2], s[1][3]));
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
+            // move a row's reference maximum only when the new maximum exceeds it by more than the threshold; weights
+            // then stay below 2^8 and the accumulators are rescaled only on the (rare) pages where some row moved
+            const bool mv0 = mx0 > m[0] + kMoveThreshold, mv1 = mx1 > m[1] + kMoveThreshold;
+            if (__any_sync(0xffffffffu, mv0 || mv1)) {
+                const float al0 = mv0 ? ((m[0] == -INFINITY) ? 0.f : fast_exp2(m[0] - mx0)) : 1.f;
+                const float al1 = low_rows ? al0 : mv1 ? ((m[1] == -INFINITY) ? 0.f : fast_exp2(m[1] - mx1)) : 1.f;
+                if (mv0) m[0] = mx0;
+                if (mv1) m[1] = mx1;
+                l[0] *= al0; l[1] *= al1;
+#pragma unroll
+                for (int k = 0; k < ON; ++k) { o[k][0] *= al0; o[k][1] *= al0; o[k][2] *= al1; o[k][3] *= al1; }
+            }
+            const float ref0 = (m[0] == -INFINITY) ? 0.f : m[0], ref1 = (m[1] == -INFINITY) ? 0.f : m[1];
+            // P in the A operand's layout: words 0 and 2 are rows 0..7, words 1 and 3 rows 8..15.  bf16 keeps 8 significant bits,
+            // so what the rounding of P dropped is multiplied as well: in the idle rows 8..15 where those hold nothing
+            // (half the MMAs), else as a second operand.
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                float (&e)[4] = s[k];
+                e[0] = fast_exp2(e[0] - ref0); e[1] = fast_exp2(e[1] - ref0);
+                l[0] += e[0] + e[1];
+                pa[2 * k] = pack2<BF16>(e[0], e[1]);
+                if constexpr (BF16)
+                    pl[2 * k] = pack2<BF16>(e[0] - __uint_as_float(pa[2 * k] << 16), e[1] - __uint_as_float(pa[2 * k] & 0xffff0000u));
+                if (low_rows) {
+                    pa[2 * k + 1] = BF16 ? pl[2 * k] : 0u;
+                    continue;
+                }
+                e[2] = fast_exp2(e[2] - ref1); e[3] = fast_exp2(e[3] - ref1);
+                l[1] += e[2] + e[3];
+                pa[2 * k + 1] = pack2<BF16>(e[2], e[3]);
+                if constexpr (BF16)
+                    pl[2 * k + 1] = pack2<BF16>(e[2] - __uint_as_float(pa[2 * k + 1] << 16), e[3] - __uint_as_float(pa[2 * k + 1] & 0xffff0000u));
+            }
+            // O += P V
+#pragma unroll
+            for (int dn = 0; dn < D / 16; dn += 2) {
+                uint32_t b[4], c[4];
+                ldsm4t(b, (va ^ ((dn & 3) << 5)) + (dn >> 2) * 2048);
+                ldsm4t(c, (va ^ (((dn + 1) & 3) << 5)) + ((dn + 1) >> 2) * 2048);
+                mma16816<BF16>(o[2 * dn], pa, b[0], b[1]);
+                mma16816<BF16>(o[2 * dn + 1], pa, b[2], b[3]);
+                mma16816<BF16>(o[2 * dn + 2], pa, c[0], c[1]);
+                mma16816<BF16>(o[2 * dn + 3], pa, c[2], c[3]);
+                if (BF16 && !low_rows) {
+                    mma16816<BF16>(o[2 * dn], pl, b[0], b[1]);
+                    mma16816<BF16>(o[2 * dn + 1], pl, b[2], b[3]);
+                    mma16816<BF16>(o[2 * dn + 2], pl, c[0], c[1]);
+                    mma16816<BF16>(o[2 * dn + 3], pl, c[2], c[3]);
+                }
+            }
+            if (chunk_page && append && sub == 0) {
+                // the chunk's rows on to their slots of the pool, as they lie in shared memory
+                const int64_t head = (int64_t)h * a.cache.stride_head;
+                for (int idx = lane; idx < C * CH; idx += 32) {
+                    const int row = idx / CH, c = idx % CH, pos = P + row;
+                    const int page = pos / kPageSize == P / kPageSize ? page_a : page_b;
+                    const int64_t at = page * a.cache.stride_page + (pos % kPageSize) * a.cache.stride_token + head + c * 8;
+                    *reinterpret_cast<uint4*>(static_cast<uint16_t*>(a.k_dst) + at) = *reinterpret_cast<const uint4*>(smem + slot * SLOT + page_off<D>(row, c));
+                    *reinterpret_cast<uint4*>(static_cast<uint16_t*>(a.v_dst) + at) = *reinterpret_cast<const uint4*>(smem + slot * SLOT + PAGE + page_off<D>(row, c));
+                }
+            }
+            if (chunk_page) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // written by copies, next by TMA
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->empty[slot]);
         }
-        if (t4 == 0) lbase[r1 * H + hq1] = lse1;
+
+        // ---- the warps' results, from warp to warp in order (fragment positions are identical in each)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            l[e] += __shfl_xor_sync(0xffffffffu, l[e], 1);
+            l[e] += __shfl_xor_sync(0xffffffffu, l[e], 2);
+        }
+        if (BF16 && low_rows) {                                    // the second term of the weights was summed in rows 8..15
+#pragma unroll
+            for (int k = 0; k < ON; ++k) { o[k][0] += o[k][2]; o[k][1] += o[k][3]; }
+        }
+        const bool have = kWarps - 1 - warp < n;                    // this warp worked on the unit
+        float4* x = xbuf + lane;
+        if (warp > 0) ok = wait_for(&ctl->hand[warp - 1], un & 1, ctl, a);
+        else if (un > 0) ok = wait_for(&ctl->x_free, (un - 1) & 1, ctl, a);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) return;
+        if (warp > 0 && have) {
+            const float4 ml = x[ON * 32];
+            const float n0 = fmaxf(m[0], ml.x), n1 = fmaxf(m[1], ml.y);
+            const float f0 = n0 == -INFINITY ? 0.f : n0, f1 = n1 == -INFINITY ? 0.f : n1;
+            const float w0 = fast_exp2(m[0] - f0), w1 = fast_exp2(m[1] - f1), x0 = fast_exp2(ml.x - f0), x1 = fast_exp2(ml.y - f1);
+            m[0] = n0; m[1] = n1;
+            l[0] = l[0] * w0 + ml.z * x0;
+            l[1] = l[1] * w1 + ml.w * x1;
+#pragma unroll
+            for (int k = 0; k < ON; ++k) {
+                if (low_rows) {
+                    const float2 v = *reinterpret_cast<const float2*>(x + k * 32);
+                    o[k][0] = o[k][0] * w0 + v.x * x0; o[k][1] = o[k][1] * w0 + v.y * x0;
+                } else {
+                    const float4 v = x[k * 32];
+                    o[k][0] = o[k][0] * w0 + v.x * x0; o[k][1] = o[k][1] * w0 + v.y * x0;
+                    o[k][2] = o[k][2] * w1 + v.z * x1; o[k][3] = o[k][3] * w1 + v.w * x1;
+                }
+            }
+        }
+        if (have || warp == 0) {
+#pragma unroll
+            for (int k = 0; k < ON; ++k) {
+                if (low_rows) *reinterpret_cast<float2*>(x + k * 32) = make_float2(o[k][0], o[k][1]);
+                else x[k * 32] = make_float4(o[k][0], o[k][1], o[k][2], o[k][3]);
+            }
+            x[ON * 32] = make_float4(m[0], m[1], l[0], l[1]);
+        }
+        if (warp == kWarps - 1 && lane == 0) {
+            ctl->job[0] = make_int4(r1.w, r2.x, r2.y + hs, row_base);
+            ctl->job[1] = make_int4(C, pair0, pairs, h);
+            ctl->job[2] = make_int4(part, 0, 0, 0);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->hand[warp]);
     }
 }
 
 template <bool BF16, int D>
-cudaError_t launch_one(const hat_plan* plan, const AttnArgs& args, const CUtensorMap& mk, const CUtensorMap& mv,
-                       cudaStream_t stream) {
-    constexpr int smem = 1024 + 16 * D * 2 + kWarps * kSlots * 2 * (16 * D * 2) + kWarps * kSlots * 8 + 64;
+cudaError_t launch_one(const hat_plan* plan, const AttnArgs& args, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t stream) {
+    using G_ = Geo<D>;
+    constexpr int smem = 1024 + G_::SLOTS * G_::SLOT + G_::Q + G_::X + (int)sizeof(Ctl<G_::SLOTS>);
+    static_assert(smem <= 115712, "two CTAs share an SM");
     auto kern = attn_stream_kernel<BF16, D>;
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(plan->num_kv_heads * plan->verify_subtiles, (unsigned)plan->verify_items.size()), kWarps * 32, smem, stream>>>(
-        args, plan->dev.verify_items, plan->verify_subtiles, mk, mv);
-    count_launch();
-    return cudaGetLastError();
+    const int units = (int)plan->stream_items.size() * plan->num_kv_heads * plan->verify_subtiles;
+    return launch_pdl(kern, dim3((unsigned)std::min(units, kCtasPerSm * plan->num_sms)), dim3(kThreads), smem, stream, args,
+                      plan->dev.stream_items, plan->verify_subtiles, units, plan->dev.status + 5, plan->dev.piece_counters, mk, mv);
 }
 
 }  // namespace
@@ -395,17 +739,23 @@ bool stream_layout_supported(int dtype, int head_dim, int num_pages, int H, int6
                              int64_t stride_head) {
     CUtensorMap m;
     // the encoder checks alignment and ranges only; any 16-byte aligned address will do for the probe
-    return tma_encode_pool_map(&m, dtype == HAT_DTYPE_BF16, reinterpret_cast<const void*>(uintptr_t(1) << 30), head_dim,
+    return tma_encode_page_map(&m, dtype == HAT_DTYPE_BF16, reinterpret_cast<const void*>(uintptr_t(1) << 30), head_dim,
                                num_pages, H, stride_page, stride_token, stride_head);
 }
 
 cudaError_t launch_attn_stream(const hat_plan* plan, const AttnArgs& args, cudaStream_t stream) {
     const bool bf16 = plan->dtype == HAT_DTYPE_BF16;
     const CUtensorMap *mk = nullptr, *mv = nullptr;
-    if (!plan_pool_maps(plan, args.cache, &mk, &mv)) return cudaErrorInvalidValue;
-    if (plan->head_dim == 128)
-        return bf16 ? launch_one<true, 128>(plan, args, *mk, *mv, stream) : launch_one<false, 128>(plan, args, *mk, *mv, stream);
-    return bf16 ? launch_one<true, 64>(plan, args, *mk, *mv, stream) : launch_one<false, 64>(plan, args, *mk, *mv, stream);
+    if (!plan_page_maps(plan, args.cache, &mk, &mv)) return cudaErrorInvalidValue;
+    auto go = [&](auto b, auto d) -> cudaError_t {
+        constexpr bool B = decltype(b)::value;
+        constexpr int D = decltype(d)::value;
+        return launch_one<B, D>(plan, args, *mk, *mv, stream);
+    };
+    using I128 = std::integral_constant<int, 128>;
+    using I64 = std::integral_constant<int, 64>;
+    if (plan->head_dim == 128) return bf16 ? go(std::true_type{}, I128{}) : go(std::false_type{}, I128{});
+    return bf16 ? go(std::true_type{}, I64{}) : go(std::false_type{}, I64{});
 }
 
 }  // namespace hat

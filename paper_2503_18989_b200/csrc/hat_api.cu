@@ -55,6 +55,25 @@ bool plan_pool_maps(const hat_plan* plan, const CacheView& c, const CUtensorMap*
     return true;
 }
 
+bool plan_page_maps(const hat_plan* plan, const CacheView& c, const CUtensorMap** mk, const CUtensorMap** mv) {
+    MapCache& m = const_cast<hat_plan*>(plan)->maps;
+    if (!m.have_page || m.page_k != c.k_pool || m.page_v != c.v_pool || m.page_strides[0] != c.stride_page ||
+        m.page_strides[1] != c.stride_token || m.page_strides[2] != c.stride_head) {
+        const bool bf16 = plan->dtype == HAT_DTYPE_BF16;
+        m.have_page = false;
+        if (!tma_encode_page_map(&m.mpk, bf16, c.k_pool, plan->head_dim, plan->num_pages, plan->num_kv_heads, c.stride_page,
+                                 c.stride_token, c.stride_head) ||
+            !tma_encode_page_map(&m.mpv, bf16, c.v_pool, plan->head_dim, plan->num_pages, plan->num_kv_heads, c.stride_page,
+                                 c.stride_token, c.stride_head))
+            return false;
+        m.page_k = c.k_pool; m.page_v = c.v_pool;
+        m.page_strides[0] = c.stride_page; m.page_strides[1] = c.stride_token; m.page_strides[2] = c.stride_head;
+        m.have_page = true;
+    }
+    *mk = &m.mpk; *mv = &m.mpv;
+    return true;
+}
+
 const CUtensorMap* plan_q_map(const hat_plan* plan, const void* q) {
     MapCache& m = const_cast<hat_plan*>(plan)->maps;
     if (!m.have_q || m.q != q) {
@@ -181,6 +200,50 @@ static int pick_prefill_split(const hat_plan* p, int num_sms, int tile_rows, int
     return best;
 }
 
+// Key-range length for the streaming-class requests.  The kernel is persistent (two CTAs per SM, units of one piece x one
+// head drawn longest first) and as long as HBM is the limit whole requests are best, however uneven: what remains when the
+// short ones are done still has enough bytes in flight.  A cut costs: the partial rows, a fence and a count per piece and the
+// merge (measured: 12 requests x 32 heads 46 us whole, 50 us in 512-key ranges; 30 requests 151 / 160 us in 768-key ranges).
+// So requests are cut only when the longest one alone would take longer than HBM needs for the batch, and then into as
+// many pieces as the CTAs can take in one round, or in one more round than the whole requests need (16 requests x 8 K/V heads
+// x 2 slabs: 124 us whole, 95 us in 400 units, 93 us in 576, 89 us in 1000, 99 us in 1900).
+static int pick_verify_split(const hat_plan* p, int num_sms) {
+    constexpr int kWhole = 1 << 24, kLeast = 96;       // shorter pieces than 6 pages only add to the merge
+    const double tp = 0.25 * p->head_dim / 128;   // us per page of a CTA that has the SM's share of HBM to itself
+    const double tb = p->head_dim * 64 / 6.45e6;                               // us per page (K and V) at the measured HBM rate
+    constexpr double kCut = 3.0;                       // us
+    const int64_t heads = (int64_t)p->num_kv_heads * p->verify_subtiles;
+    const int64_t slots = 2 * (int64_t)num_sms;
+    int64_t pages = 0, whole_units = 0;
+    int longest = 0;
+    for (int r = 0; r < p->num_requests; ++r) {
+        if (p->chunk_len[r] < 1 || p->chunk_len[r] > 16) continue;
+        const int n = p->prefix_len[r] + p->chunk_len[r];
+        pages += ceil_div(n, kPageSize) + 1;
+        longest = std::max(longest, n);
+        ++whole_units;
+    }
+    pages *= heads; whole_units *= heads;
+    auto time_of = [&](int keys) { return std::max((ceil_div(keys, kPageSize) + 1) * tp, pages * tb); };
+    if (time_of(longest) <= pages * tb + kCut) return kWhole;
+    const int64_t most = 2 * whole_units <= slots ? slots : whole_units + slots;
+    auto units_at = [&](int len) {
+        int64_t n = 0;
+        for (int r = 0; r < p->num_requests; ++r)
+            if (p->chunk_len[r] >= 1 && p->chunk_len[r] <= 16) {
+                const int keys = p->prefix_len[r] + p->chunk_len[r];
+                n += ceil_div(keys, split_len_for(keys, len, kPageSize));
+            }
+        return n * heads;
+    };
+    int lo = kLeast / kPageSize, hi = std::max(lo, ceil_div(longest, kPageSize));
+    while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (units_at(mid * kPageSize) <= most) hi = mid; else lo = mid + 1;
+    }
+    return time_of(lo * kPageSize) + kCut < time_of(longest) ? lo * kPageSize : kWhole;
+}
+
 // tile_kernel: 0 = mma.sync, 1 = tcgen05 with two query tiles per CTA, 3 = tcgen05 by pairs of CTAs (cta_group::2) with a
 // ring of three score buffers; both tcgen05 kernels take 256-row units
 static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
@@ -196,8 +259,8 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
     info.prefill_tile_rows = tile_rows;
     info.prefill_kernel = tile_kernel;
 
-    // ---- streaming (verify-class) requests: fixed-length key ranges, shortened until the SMs are covered.
-    // A CTA of the streaming kernel serves one K/V head and 16 (row, query head of the group) pairs.
+    // ---- streaming (verify-class) requests: key ranges of one length.
+    // A CTA of the streaming kernels serves one K/V head and a slab of (row, query head of the group) pairs.
     const int group = H / p->num_kv_heads;
     int max_verify_rows = 0;
     for (int r = 0; r < R; ++r) {
@@ -209,24 +272,10 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
             info.num_prefill_requests++;
         }
     }
+    const bool stream_tma = info.stream_kernel == 1;
     p->verify_subtiles = std::max(1, ceil_div(max_verify_rows * group, 16));
     int vsplit = env_int("HAT_VERIFY_SPLIT_LEN", 0);
-    if (vsplit <= 0) {
-        // Long ranges stream best (a CTA's pipeline ramp and its cross-warp merge are paid once per range, and an
-        // unsplit request needs no merge pass): start unsplit and halve the range only while the grid would not
-        // give every SM about three rounds of two resident CTAs.
-        vsplit = 16384;
-        const int64_t want_ctas = (int64_t)num_sms * 6;
-        auto ctas_at = [&](int len) {
-            int64_t n = 0;
-            for (int r = 0; r < R; ++r) {
-                const int C = p->chunk_len[r];
-                if (C >= 1 && C <= verify_max_rows) n += ceil_div(p->prefix_len[r] + C, len);
-            }
-            return n * p->num_kv_heads * p->verify_subtiles;
-        };
-        while (vsplit > 256 && ctas_at(vsplit) < want_ctas) vsplit /= 2;
-    }
+    if (vsplit <= 0) vsplit = pick_verify_split(p, num_sms);
     vsplit = std::max(kPageSize, round_up(vsplit, kPageSize));
     info.verify_split_len = vsplit;
 
@@ -255,13 +304,27 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
     if (psplit > 0) psplit = round_up(psplit, key_granule);
     info.prefill_split_len = psplit;
 
+    int stream_merged = 0;                  // rows the streaming kernel merges itself
     // streaming-class requests first: their merge rows form the head of merge_rows, so that they can be merged (and
     // announced through the plan's event) before the tile kernel runs
     for (int r = 0; r < R; ++r) {
         const int C = p->chunk_len[r], P = p->prefix_len[r];
         if (C <= 0 || C > verify_max_rows) continue;
         const int kv_end = P + C;
-        emit_tile(p, p->verify_items, r, 0, C, kv_end, split_len_for(kv_end, vsplit, kPageSize));
+        const int sl = split_len_for(kv_end, vsplit, kPageSize);
+        if (!stream_tma) { emit_tile(p, p->verify_items, r, 0, C, kv_end, sl); continue; }
+        // the TMA kernel: as many pieces as ranges of that length, of (nearly) equal size
+        const int pieces = ceil_div(kv_end, sl), pages = ceil_div(P, kPageSize) + 1;
+        const int32_t part0 = (int32_t)p->part_rows;
+        for (int s = 0; s < pieces; ++s)
+            p->stream_items.push_back(StreamItem{r, p->cu_chunk[r], C, P, (int)((int64_t)pages * s / pieces), (int)((int64_t)pages * (s + 1) / pieces),
+                                                 pieces > 1 ? part0 + s * C : -1, part0, pieces, p->num_piece_counters, 0, 0});
+        if (pieces > 1) {
+            p->part_rows += (int64_t)pieces * C;
+            p->num_piece_counters += p->num_kv_heads * p->verify_subtiles;
+            stream_merged += C;
+            info.max_splits = std::max(info.max_splits, pieces);
+        }
     }
     p->num_verify_merge_rows = (int)p->merge_rows.size();
     for (int r = 0; r < R; ++r) {
@@ -279,6 +342,8 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
         return (a.kv_end - a.kv_begin) > (b.kv_end - b.kv_begin);
     };
     std::stable_sort(p->verify_items.begin(), p->verify_items.end(), longer);
+    std::stable_sort(p->stream_items.begin(), p->stream_items.end(),
+                     [](const StreamItem& a, const StreamItem& b) { return a.page1 - a.page0 > b.page1 - b.page0; });
     std::stable_sort(p->prefill_items.begin(), p->prefill_items.end(), longer);
 
     // Units of the persistent tcgen05 kernels, in the order the CTAs draw them: requests by their longest item first;
@@ -308,9 +373,9 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
         }
     }
 
-    info.num_verify_items = (int32_t)p->verify_items.size();
+    info.num_verify_items = (int32_t)(p->verify_items.size() + p->stream_items.size());
     info.num_prefill_items = (int32_t)p->prefill_items.size();
-    info.num_merge_rows = (int32_t)p->merge_rows.size();
+    info.num_merge_rows = (int32_t)p->merge_rows.size() + stream_merged;
     const int64_t d = p->head_dim;
     int64_t part_out_bytes = p->part_rows * H * d * 4;
     part_out_bytes = (part_out_bytes + 255) / 256 * 256;
@@ -318,20 +383,22 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
 }
 
 static int upload(hat_plan* p) {
-    // the arrays, each at a 256-byte boundary, written straight into the pinned buffer
-    struct Part { const void* src; size_t bytes, off; };
-    std::vector<Part> parts;
+    // the arrays, each at a 256-byte boundary
+    std::vector<UploadPart> parts;
     size_t bytes = 0;
     auto add = [&](const auto& v) {
         const size_t off = (bytes + 255) / 256 * 256, n = v.size() * sizeof(v[0]);
-        parts.push_back(Part{v.data(), n, off});
+        parts.push_back(UploadPart{v.data(), n, off});
         bytes = off + std::max<size_t>(n, 16);
         return off;
     };
     const size_t o_cu = add(p->cu_chunk), o_pl = add(p->prefix_len), o_cl = add(p->chunk_len), o_bt = add(p->block_table);
-    const size_t o_rr = add(p->row_req), o_vi = add(p->verify_items), o_pi = add(p->prefill_items), o_mr = add(p->merge_rows);
+    const size_t o_rr = add(p->row_req), o_vi = add(p->verify_items), o_si = add(p->stream_items), o_pi = add(p->prefill_items), o_mr = add(p->merge_rows);
     const size_t o_tu = add(p->tile_units), o_tm = add(p->tree_mask);
-    const std::vector<int32_t> status(8, 0);     // status word; (unit counter, finished CTAs) of the tile kernel; the same for a second tile grid; spare
+    // status word; (unit counter, finished CTAs) of the tile kernel, of a second tile grid, of the streaming kernel; spare;
+    // finished pieces of the requests the streaming kernel merges
+    p->num_status_words = 8 + p->num_piece_counters;
+    const std::vector<int32_t> status(p->num_status_words, 0);
     const size_t o_st = add(status);
 
     cudaError_t e = cudaGetDevice(&p->device);
@@ -339,11 +406,9 @@ static int upload(hat_plan* p) {
     // behind the arrays: room for the (cos, sin) table of the projection epilogue, filled on the device when first used
     const size_t o_table = (bytes + 255) / 256 * 256;
     const size_t table_bytes = (size_t)p->total_rows * (p->head_dim / 2) * sizeof(float2);
-    e = plan_res_acquire(p->device, o_table + std::max<size_t>(table_bytes, 16), bytes, &p->res);
+    e = plan_res_acquire(p->device, o_table + std::max<size_t>(table_bytes, 16), &p->res);
     if (e != cudaSuccess) return cuda_fail(e);
-    for (const Part& part : parts)
-        if (part.bytes) std::memcpy(static_cast<char*>(p->res.pinned) + part.off, part.src, part.bytes);
-    e = plan_res_upload(p->res, bytes);
+    e = plan_res_upload(p->res, parts.data(), parts.size(), bytes);
     if (e != cudaSuccess) return cuda_fail(e);
     char* base = static_cast<char*>(p->res.blob);
     p->rope_table = reinterpret_cast<float2*>(base + o_table);
@@ -354,10 +419,12 @@ static int upload(hat_plan* p) {
     d.block_table = reinterpret_cast<const int32_t*>(base + o_bt);
     d.row_req = reinterpret_cast<const int32_t*>(base + o_rr);
     d.verify_items = reinterpret_cast<const WorkItem*>(base + o_vi);
+    d.stream_items = reinterpret_cast<const StreamItem*>(base + o_si);
     d.prefill_items = reinterpret_cast<const WorkItem*>(base + o_pi);
     d.merge_rows = reinterpret_cast<const MergeRow*>(base + o_mr);
     d.tile_units = reinterpret_cast<const uint32_t*>(base + o_tu);
     d.status = reinterpret_cast<int32_t*>(base + o_st);
+    d.piece_counters = d.status + 8;
     d.max_pages = p->max_pages;
     d.tree_mask = p->tree_mask.empty() ? nullptr : reinterpret_cast<const uint32_t*>(base + o_tm);
     d.num_heads = p->num_heads;
@@ -451,6 +518,16 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
         }
     }
 
+    // a page that one request writes and another one (or the same one, twice in its table) reads as prefix: then the whole
+    // append has to come first; otherwise a kernel may take the chunk's rows from k_new / v_new
+    bool append_first = false;
+    for (int r = 0; r < R && !append_first; ++r) {
+        if (batch->chunk_len[r] == 0) continue;
+        const int32_t* row = batch->block_table + (int64_t)r * batch->max_pages;
+        for (int j = 0; j < batch->prefix_len[r] / kPageSize; ++j)
+            if (written[row[j]]) { append_first = true; break; }
+    }
+
     hat_plan* p = new (std::nothrow) hat_plan();
     if (!p) return HAT_ERR_INVALID_ARG;
     p->dtype = cache->dtype;
@@ -465,6 +542,8 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
     p->device = -1;
     p->part_rows = 0;
     p->timing = nullptr;
+    p->append_first = append_first;
+    p->num_piece_counters = 0;
     p->num_verify_merge_rows = 0;
     p->captured = p->loose = p->loose_many = false;
     p->loose_stream = nullptr;
@@ -545,7 +624,6 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
         if (use_tc5 && p->head_dim == 128 && std::strcmp(k, "pair") == 0) { tile_kernel = 3; p->pair_takes_all = true; }
         else if (use_tc5 && std::strcmp(k, "tc5") == 0) tile_kernel = 1;
     }
-    schedule(p, num_sms, tile_kernel);
     // the streaming kernel takes its pages by TMA when a descriptor can be built for the pool layout
     bool stream_tma = true;
     if (const char* k = std::getenv("HAT_STREAM_KERNEL"))
@@ -554,8 +632,10 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
         stream_tma = stream_layout_supported(p->dtype, p->head_dim, p->num_pages, p->num_kv_heads, cache->stride_page,
                                              cache->stride_token, cache->stride_head);
     p->info.stream_kernel = stream_tma ? 1 : 0;
+    schedule(p, num_sms, tile_kernel);
     // launch-geometry limits: work items index gridDim.y (65535), partial rows and units are 32-bit
-    if (p->verify_items.size() > 65535 || p->prefill_items.size() > 65535 || p->num_heads > 65535 ||
+    const int64_t verify_count = (int64_t)(p->verify_items.size() + p->stream_items.size());
+    if (verify_count > 65535 || verify_count * p->num_kv_heads * p->verify_subtiles > INT32_MAX / 2 || p->prefill_items.size() > 65535 || p->num_heads > 65535 ||
         p->part_rows > INT32_MAX / 2 || (int64_t)p->prefill_items.size() * p->num_heads > INT32_MAX / 2) {
         delete p;
         return HAT_ERR_TOO_LARGE;
@@ -568,7 +648,7 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
         // sequence.  Off by default: it finishes the whole step sooner but the decode-phase rows later.  The side
         // stream has the highest priority so that the tile CTAs are placed before the streaming kernel's many small
         // CTAs fill the SMs.
-        if (!p->verify_items.empty() && !p->prefill_items.empty() && p->info.prefill_kernel == 1) {
+        if (verify_count > 0 && !p->prefill_items.empty() && p->info.prefill_kernel == 1) {
             int side = env_int("HAT_SIDE_SMS", 0);
             side = std::max(0, std::min(side, p->num_sms - 8));
             if (side > 0) {
@@ -723,7 +803,10 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
         if (call >= 0) cudaEventRecord(tm->events[((size_t)call * HAT_TIMING_SLOTS + slot) * 2 + end], s);
         if (call >= 0 && end) tm->launched[(size_t)call * HAT_TIMING_SLOTS + slot] = 1;
     };
-    if (k_new) {
+    // the streaming kernel appends its own requests' rows; a batch with prompt chunks, or one whose pages are shared, appends first
+    const bool has_verify = plan->info.num_verify_items > 0;
+    const bool stream_appends = k_new && plan->info.stream_kernel == 1 && plan->prefill_items.empty() && !plan->append_first;
+    if (k_new && !stream_appends) {
         mark(0, 0);
         e = launch_kv_append(plan, view_of(cache), cache->k_pool, cache->v_pool, k_new, v_new, s);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -733,6 +816,10 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     a.plan = plan->dev;
     a.cache = view_of(cache);
     a.q = q;
+    a.k_new = stream_appends ? k_new : nullptr;
+    a.v_new = stream_appends ? v_new : nullptr;
+    a.k_dst = cache->k_pool;
+    a.v_dst = cache->v_pool;
     a.out = out;
     a.out16 = out16;
     a.out16_bf16 = plan->dtype == HAT_DTYPE_BF16 ? 1 : 0;
@@ -763,7 +850,7 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
         if (e == cudaSuccess) e = cudaEventRecord(plan->ev_join, plan->aux_stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    if (!plan->verify_items.empty()) {
+    if (has_verify) {
         mark(2, 0);
         e = plan->info.stream_kernel == 1 ? launch_attn_stream(plan, a, s)
                                           : launch_attn_mma(plan, a, /*verify_class=*/true, s);
@@ -923,7 +1010,7 @@ int hat_last_device_status(const hat_plan* plan, void* stream, int* out) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int32_t word = 0;
     cudaError_t e = cudaMemcpyAsync(&word, plan->dev.status, sizeof word, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(plan->dev.status, 0, 8 * sizeof word, s);     // status, unit counters, finished CTAs
+    if (e == cudaSuccess) e = cudaMemsetAsync(plan->dev.status, 0, plan->num_status_words * sizeof word, s);     // status, counters
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e);
     *out = word == 0 ? HAT_OK : (word & 1) ? HAT_ERR_DEVICE_TIMEOUT : HAT_ERR_DEVICE_BOUNDS;

@@ -23,6 +23,19 @@ struct WorkItem {
     int32_t pad0, pad1, pad2;
 };
 
+// One piece of a streaming-class request: pages [page0, page1) of its page list, which is the ceil(P/16) pages of the cached
+// prefix followed by one page that holds the chunk's own rows.  Read by the device as 16-byte words.
+struct StreamItem {
+    int32_t req, row_base, C, P;
+    int32_t page0, page1;
+    int32_t part;     // first partial row of this piece, or -1: it writes the final rows
+    int32_t part0;    // first partial row of the request's first piece; each piece has C rows
+    int32_t nsplit;   // pieces of the request
+    int32_t counter;  // cut request: first of its (head, slab) counters of finished pieces
+    int32_t pad0, pad1;
+};
+static_assert(sizeof(StreamItem) == 48, "three 16-byte words");
+
 // Rows whose result is merged from `nsplit` partial rows part0 + s*stride, s = 0..nsplit-1.
 struct MergeRow {
     int32_t row;      // packed row index t
@@ -38,7 +51,9 @@ struct DevicePlan {
     const int32_t*  chunk_len;
     const int32_t*  block_table;
     const int32_t*  row_req;        // [T] request of each packed row
-    const WorkItem* verify_items;
+    const WorkItem* verify_items;   // mma.sync streaming kernel
+    const StreamItem* stream_items; // TMA streaming kernel, longest first
+    int32_t*        piece_counters; // see StreamItem::counter; zero between calls
     const WorkItem* prefill_items;
     const uint32_t* tile_units;     // tcgen05 tile kernels: unit -> prefill item (low 16 bits) | query head (high 16 bits), in draw order
     const MergeRow* merge_rows;
@@ -62,6 +77,10 @@ struct AttnArgs {
     DevicePlan  plan;
     CacheView   cache;
     const void* q;
+    const void* k_new;        // streaming kernel: the chunk's rows, to be appended to k_dst / v_dst (the pools) as well;
+    const void* v_new;        // null: the rows are in the pools already
+    void*       k_dst;
+    void*       v_dst;
     float*      out;          // [T][H][d]; unused when out16 is set
     void*       out16;        // [T][H][d] in the cache's 16-bit type, or null: final rows go here instead of `out`
     int         out16_bf16;   // type of out16: 0 = fp16, 1 = bf16
@@ -158,21 +177,23 @@ struct MapCache {
     int64_t stride_page = 0, stride_token = 0, stride_head = 0;
     bool have_q = false, have_kv = false;
     CUtensorMap mq, mk, mv;
+    // the streaming kernel's maps of the same pools (boxes of whole pages)
+    const void* page_k = nullptr; const void* page_v = nullptr;
+    int64_t page_strides[3] = {0, 0, 0};
+    bool have_page = false;
+    CUtensorMap mpk, mpv;
 };
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device instead of once per launch
 cudaError_t smem_attr_once(const void* kernel, int bytes);
 }  // namespace hat
 
 namespace hat {
-// What a plan needs from the driver: one device allocation, the pinned buffer its contents are uploaded from, three
-// events.  Plans live for one inference step, and making these anew costs far more than the step's schedule
+// What a plan needs from the driver: one device allocation and three events.  Plans live for one inference step, and making these anew costs far more than the step's schedule
 // (cudaMalloc and cudaFree: 270 + 360 us beside 6 GB of pools), so a destroyed plan hands them on (hat_api.cu).
 struct PlanRes {
     int device = -1;
     void* blob = nullptr;
     size_t blob_bytes = 0;
-    void* pinned = nullptr;
-    size_t pinned_bytes = 0;
     cudaEvent_t ev_verify = nullptr;   // recorded in every attention call once the streaming-class rows are final
     cudaEvent_t ev_done = nullptr;     // recorded at the end of every attention call: the next call on another stream waits for it
     cudaEvent_t ev_table = nullptr;    // orders calls on other streams behind the kernel that filled the (cos, sin) table
@@ -184,12 +205,16 @@ struct hat_plan {
     // geometry the plan was made for
     int32_t dtype, num_pages, num_heads, num_kv_heads, head_dim, max_pages, num_requests, total_rows;   // num_heads: query heads
     int32_t verify_subtiles;    // 16-row slabs of (row, query head of a group) pairs per streaming work item and K/V head
+    bool append_first;          // a page of the batch is written by one request and read as another's prefix (or twice by one): append before anything reads
+    int num_status_words;       // status, counters
     std::vector<uint32_t> tree_mask;
     bool host_only;
     int device;
     int num_sms;
     std::vector<int32_t> cu_chunk, prefix_len, chunk_len, block_table, row_req;
     std::vector<hat::WorkItem> verify_items, prefill_items;
+    std::vector<hat::StreamItem> stream_items;
+    int num_piece_counters;
     std::vector<uint32_t> tile_units;   // (item, head) of every unit of the tcgen05 tile kernels, in the order they are drawn
     bool pair_takes_all;                // HAT_PREFILL_KERNEL=pair: every unit goes to the CTA-pair kernel, narrow ones too (tests)
     int num_pair_units;                 // CTA-pair kernel in use: the first num_pair_units units are its (more than 128 rows each), the rest go to the one-CTA kernel
@@ -214,7 +239,7 @@ struct hat_plan {
     float2* rope_table;
     float rope_theta;
     cudaStream_t table_stream;
-    hat::PlanRes res;           // device memory holding every device array, its staging buffer and the plan's events
+    hat::PlanRes res;           // device memory holding every device array, and the plan's events
     // which work that uses `res` ev_done does not cover (see plan_note_call): decides whether it can be handed on
     bool captured;              // a call was captured into a graph, which may be replayed at any time
     bool loose, loose_many;     // calls other than attention since the last ev_done; on more than one stream
@@ -250,13 +275,29 @@ cudaError_t launch_attn_stream(const hat_plan* plan, const AttnArgs& args, cudaS
 cudaError_t launch_qkv_gemm(const hat_plan* plan, const CacheView& cache, void* k_pool, void* v_pool, const void* x,
                             int hidden, const void* w, void* q_out, float theta, int interleaved, cudaStream_t stream);
 // the pool of plan resources (plan_pool.cu)
-cudaError_t plan_res_acquire(int device, size_t blob_bytes, size_t pinned_bytes, PlanRes* out);
-cudaError_t plan_res_upload(PlanRes& r, size_t bytes);      // pinned -> blob, complete on return
+cudaError_t plan_res_acquire(int device, size_t blob_bytes, PlanRes* out);
+struct UploadPart { const void* src; size_t bytes, off; };
+cudaError_t plan_res_upload(PlanRes& r, const UploadPart* parts, size_t num_parts, size_t bytes);   // complete on return
 cudaError_t plan_res_release(PlanRes& r, bool reusable);    // reusable: ev_done covers every use, or there was none
 cudaError_t plan_res_free(PlanRes& r);
 cudaError_t plan_res_trim();                                // frees what waits for a later plan
 void plan_note_call(hat_plan* p, cudaStream_t s);           // a call other than attention is about to use the plan on s
 void count_launch(int n = 1);
+#ifdef __CUDACC__
+// Launches a kernel that calls tc5::pdl_wait before it touches what earlier kernels of the stream write or read
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    count_launch();
+    return e;
+}
+#endif
 void set_last_cuda_error(int e);   // what hat_last_cuda_error() returns on this thread
 }  // namespace hat
 
@@ -264,5 +305,6 @@ namespace hat {
 // The plan's cached tensor maps for these pools / this q buffer, encoded again only when a pointer or a stride changed.
 // Return null when no map can be built.  (Defined in hat_api.cu.)
 bool plan_pool_maps(const hat_plan* plan, const CacheView& cache, const CUtensorMap** mk, const CUtensorMap** mv);
+bool plan_page_maps(const hat_plan* plan, const CacheView& cache, const CUtensorMap** mk, const CUtensorMap** mv);   // streaming kernel
 const CUtensorMap* plan_q_map(const hat_plan* plan, const void* q);
 }  // namespace hat

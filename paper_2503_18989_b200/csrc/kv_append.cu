@@ -1,5 +1,6 @@
 // KV append: scatter the chunk's new K/V rows into the paged pools (bit-exact 16-byte copies).
 #include "hat_internal.h"
+#include "tc5_ptx.cuh"
 
 namespace hat {
 
@@ -16,6 +17,8 @@ kv_append_kernel(DevicePlan plan, int64_t stride_page, int64_t stride_token, int
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t first = warp * (32 * kVecsPerThread) + (threadIdx.x & 31);
     uint4 kv[kVecsPerThread], vv[kVecsPerThread];
+    tc5::pdl_launch_dependents();
+    tc5::pdl_wait();
 #pragma unroll
     for (int i = 0; i < kVecsPerThread; ++i)
         if (first + 32 * i < total_vecs) kv[i] = __ldg(k_new + first + 32 * i);
@@ -52,12 +55,10 @@ cudaError_t launch_kv_append(const hat_plan* plan, const CacheView& cache, void*
     const int threads = 256;
     const int64_t per_block = (int64_t)threads * kVecsPerThread;
     const int64_t blocks = (total + per_block - 1) / per_block;
-    kv_append_kernel<<<(unsigned)blocks, threads, 0, stream>>>(
-        plan->dev, cache.stride_page, cache.stride_token, cache.stride_head,
-        static_cast<uint4*>(k_pool), static_cast<uint4*>(v_pool),
-        static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), vec_per_head, total);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(kv_append_kernel, dim3((unsigned)blocks), dim3(threads), 0, stream,
+                      plan->dev, cache.stride_page, cache.stride_token, cache.stride_head,
+                      static_cast<uint4*>(k_pool), static_cast<uint4*>(v_pool),
+                      static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), vec_per_head, total);
 }
 
 }  // namespace hat

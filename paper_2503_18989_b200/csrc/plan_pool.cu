@@ -1,4 +1,4 @@
-// What destroyed plans hand on to later ones: device memory, the pinned buffer it is filled from, and events.
+// What destroyed plans hand on to later ones: device memory and events; and the pinned buffer plans are uploaded from.
 //
 // A serving loop makes one plan per inference step.  With a few GB of pools on the device a cudaMalloc / cudaFree pair
 // costs 360 + 270 us of host time (measured beside 6 GB, 12 requests), both synchronise the device, and a pageable
@@ -8,6 +8,7 @@
 // Bounds: at most kMaxIdle entries and kMaxIdleBytes of device memory wait in the list, per process; what does not fit
 // is freed, and hat_release_cached() frees the rest.  Entries are handed on whole under one lock; an entry whose last
 // owner's kernels may still run is taken only after that owner's ev_done has occurred.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -17,13 +18,17 @@
 namespace hat {
 namespace {
 
-constexpr size_t kMaxIdle = 16;
+constexpr size_t kMaxIdle = 64;
 constexpr size_t kMaxIdleBytes = size_t(64) << 20;
 
 struct Pool {
     std::mutex mu;
     std::vector<PlanRes> idle;
-    std::vector<std::pair<int, cudaStream_t>> upload;   // per device: the stream uploads run on
+    // uploads: one at a time, complete before the next, so that one pinned buffer serves all plans
+    std::mutex up_mu;
+    std::vector<std::pair<int, cudaStream_t>> up_streams;   // per device
+    void* up_buf = nullptr;
+    size_t up_bytes = 0;
 };
 Pool& pool() {
     static Pool* p = new Pool();      // never destroyed: plans may outlive static destructors
@@ -44,12 +49,11 @@ cudaError_t plan_res_free(PlanRes& r) {
     if (r.ev_done) cudaEventDestroy(r.ev_done);
     if (r.ev_table) cudaEventDestroy(r.ev_table);
     if (r.blob) e = cudaFree(r.blob);              // waits for the device, so kernels that still use the plan finish first
-    if (r.pinned) cudaFreeHost(r.pinned);
     r = PlanRes{};
     return e;
 }
 
-cudaError_t plan_res_acquire(int device, size_t blob_bytes, size_t pinned_bytes, PlanRes* out) {
+cudaError_t plan_res_acquire(int device, size_t blob_bytes, PlanRes* out) {
     Pool& p = pool();
     {
         std::unique_lock<std::mutex> lock(p.mu);
@@ -57,7 +61,7 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, size_t pinned_bytes,
         for (int i = 0; i < (int)p.idle.size(); ++i) {          // in the order they were given back
             PlanRes& r = p.idle[i];
             // not for a plan that needs a small part of it only: the large ones would all end up with small plans
-            if (r.device != device || r.blob_bytes < blob_bytes || r.pinned_bytes < pinned_bytes || r.blob_bytes / 8 > blob_bytes) continue;
+            if (r.device != device || r.blob_bytes < blob_bytes || r.blob_bytes / 8 > blob_bytes) continue;
             if (oldest < 0) oldest = i;
             if (!r.in_use || cudaEventQuery(r.ev_done) == cudaSuccess) { ready = i; break; }
         }
@@ -80,9 +84,7 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, size_t pinned_bytes,
     }
     PlanRes r;
     r.device = device;
-    auto up = [](size_t n) { size_t m = size_t(64) << 10; while (m < n) m *= 2; return m; };
-    r.blob_bytes = up(blob_bytes);
-    r.pinned_bytes = up(pinned_bytes);
+    for (r.blob_bytes = size_t(64) << 10; r.blob_bytes < blob_bytes;) r.blob_bytes *= 2;
     cudaError_t e = cudaMalloc(&r.blob, r.blob_bytes);
     if (e == cudaErrorMemoryAllocation) {                        // give back what waits in the list and try once more
         cudaGetLastError();
@@ -90,7 +92,6 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, size_t pinned_bytes,
         e = cudaMalloc(&r.blob, r.blob_bytes);
     }
     if (e != cudaSuccess) r.blob = nullptr;
-    if (e == cudaSuccess && (e = cudaMallocHost(&r.pinned, r.pinned_bytes)) != cudaSuccess) r.pinned = nullptr;
     for (cudaEvent_t* ev : {&r.ev_verify, &r.ev_done, &r.ev_table})
         if (e == cudaSuccess && (e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) *ev = nullptr;
     if (e != cudaSuccess) { plan_res_free(r); return e; }
@@ -112,21 +113,26 @@ cudaError_t plan_res_release(PlanRes& r, bool reusable) {
     return plan_res_free(r);
 }
 
-cudaError_t plan_res_upload(PlanRes& r, size_t bytes) {
+cudaError_t plan_res_upload(PlanRes& r, const UploadPart* parts, size_t num_parts, size_t bytes) {
     Pool& p = pool();
+    std::lock_guard<std::mutex> lock(p.up_mu);
     cudaStream_t s = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(p.mu);
-        for (auto& d : p.upload)
-            if (d.first == r.device) s = d.second;
-        if (!s) {
-            const cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-            if (e != cudaSuccess) return e;
-            p.upload.emplace_back(r.device, s);
-        }
+    for (auto& d : p.up_streams)
+        if (d.first == r.device) s = d.second;
+    cudaError_t e = cudaSuccess;
+    if (!s) {
+        if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) != cudaSuccess) return e;
+        p.up_streams.emplace_back(r.device, s);
     }
+    if (p.up_bytes < bytes) {
+        if (p.up_buf) cudaFreeHost(p.up_buf);
+        p.up_bytes = std::max(bytes, size_t(1) << 20);
+        if ((e = cudaMallocHost(&p.up_buf, p.up_bytes)) != cudaSuccess) { p.up_buf = nullptr; p.up_bytes = 0; return e; }
+    }
+    for (size_t i = 0; i < num_parts; ++i)
+        if (parts[i].bytes) std::memcpy(static_cast<char*>(p.up_buf) + parts[i].off, parts[i].src, parts[i].bytes);
     // a stream of its own: the copy does not queue behind the caller's kernels, and the plan is complete on return
-    cudaError_t e = cudaMemcpyAsync(r.blob, r.pinned, bytes, cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(r.blob, p.up_buf, bytes, cudaMemcpyHostToDevice, s);
     return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
@@ -136,6 +142,12 @@ cudaError_t plan_res_trim() {
     {
         std::lock_guard<std::mutex> lock(p.mu);
         gone.swap(p.idle);
+    }
+    {
+        std::lock_guard<std::mutex> lock(p.up_mu);
+        if (p.up_buf) cudaFreeHost(p.up_buf);
+        p.up_buf = nullptr;
+        p.up_bytes = 0;
     }
     cudaError_t first = cudaSuccess;
     int back = 0;

@@ -38,6 +38,21 @@ inline bool tma_encode_pool_map(CUtensorMap* map, bool bf16, const void* pool, i
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same pool with the column halves as a dimension, (column of a half, slot, half, head, page), read in boxes that hold
+// one whole page of one head: the halves land one after the other, 2 KiB each, as two boxes of the map above would.
+inline bool tma_encode_page_map(CUtensorMap* map, bool bf16, const void* pool, int head_dim, int num_pages, int H,
+                                int64_t stride_page, int64_t stride_token, int64_t stride_head) {
+    EncodeTiledFn fn = tma_encode_fn();
+    if (!fn || num_pages <= 0) return false;
+    const cuuint64_t dims[5] = {64, 16, (cuuint64_t)head_dim / 64, (cuuint64_t)H, (cuuint64_t)num_pages};
+    const cuuint64_t strides[4] = {(cuuint64_t)stride_token * 2, 128, (cuuint64_t)stride_head * 2, (cuuint64_t)stride_page * 2};
+    const cuuint32_t box[5] = {64, 16, (cuuint32_t)head_dim / 64, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, const_cast<void*>(pool),
+              dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // The query rows [T][H][d] as a 3-D tensor (column, head, row) read in boxes of 64 columns x 128 rows of one head.
 inline bool tma_encode_q_map(CUtensorMap* map, bool bf16, const void* q, int T, int H, int head_dim) {
     EncodeTiledFn fn = tma_encode_fn();

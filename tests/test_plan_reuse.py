@@ -9,7 +9,7 @@ from common import assert_parity, oracle_replay
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("steps,streams", [(3, 1), (40, 1), (40, 2)])     # below and beyond what waits in the list
+@pytest.mark.parametrize("steps,streams", [(3, 1), (150, 1), (150, 2)])     # below and beyond what waits in the list
 def test_destroyed_plans_hand_their_memory_on(cuda_device, steps, streams):
     """Three batches in turn, a new plan per step, destroyed right after its call was enqueued."""
     import torch
