@@ -54,6 +54,7 @@
 #include "hat_internal.h"
 #include "tma_desc.h"
 #include "tc5_ptx.cuh"
+#include "tile_append.cuh"
 
 namespace hat {
 namespace {
@@ -69,8 +70,9 @@ constexpr int kUnitSlots = 4;   // queue of published units
 constexpr uint32_t kTileBytes = kRows * kD * 2;          // 32 KiB: the Q tile of one CTA
 constexpr uint32_t kSlabBytes = kRows * 64 * 2;          // 16 KiB: 64 columns of 128 rows
 constexpr uint32_t kHalfBytes = kKeys * kD;              // 16 KiB: 64 keys x 128 columns of K, or 128 keys x 64 columns of V
-constexpr uint32_t kKSlabBytes = 64 * 64 * 2;            // 8 KiB: 64 columns of the 64 keys of a K half
-constexpr uint32_t kPageBoxBytes = 16 * 64 * 2;          // 2 KiB: one TMA box (16 tokens x 64 columns)
+constexpr uint32_t kKGroupBytes = 8 * kD * 2;            // 2 KiB: 8 rows of a K half, two blocks of 64 columns
+constexpr uint32_t kKPageBytes = 2 * kKGroupBytes;       // 4 KiB: one page of a K half, one TMA box
+constexpr uint32_t kVPageBytes = 16 * 64 * 2;            // 2 KiB: one page of a V half, one TMA box
 constexpr uint32_t kColO = 384;                          // first TMEM column of the accumulator
 constexpr float kRescaleThreshold = 8.0f;                // log2 units
 
@@ -152,15 +154,13 @@ struct Unit {
 };
 __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* __restrict__ items, int unit) {
     const uint32_t e = __ldg(a.plan.tile_units + unit);      // item | head << 16
-    const WorkItem it = items[e & 0xffffu];
+    const int4* __restrict__ rec = reinterpret_cast<const int4*>(items + (e & 0xffffu));
+    const int4 lo = __ldg(rec), hi = __ldg(rec + 1);
     Unit u;
     u.h = (int)(e >> 16);
     u.hk = u.h / a.plan.group;
-    u.r = it.req;
-    u.P = a.plan.prefix_len[u.r];
-    u.C = a.plan.chunk_len[u.r];
-    u.row_base = a.plan.cu_chunk[u.r];
-    u.row0 = it.row0; u.kv_begin = it.kv_begin; u.kv_end = it.kv_end; u.part = it.part;
+    u.r = lo.x; u.row0 = lo.y; u.kv_begin = lo.z; u.kv_end = lo.w;
+    u.part = hi.x; u.P = hi.y; u.C = hi.z; u.row_base = hi.w;
     u.n = max(1, (u.kv_end - u.kv_begin + kKeys - 1) / kKeys);
     return u;
 }
@@ -169,7 +169,8 @@ template <bool BF16>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units, int32_t* work_counter,
                  const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                 const __grid_constant__ CUtensorMap map_v) {
+                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_k_new,
+                 const __grid_constant__ CUtensorMap map_v_new, int fold) {
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the swizzle pattern and the matrix descriptors assume it.  Both CTAs of a pair must end up
     // with the same offsets (the MMA applies one descriptor to both); the dynamic shared memory of a kernel starts at
@@ -242,7 +243,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
 
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch (CTA 0) + TMA producer (both)
-        int g = 0;                                               // K/V tiles issued so far, over all units
         bool ok = true;
         PH_DECL(8);
         PH_T0(tq0);
@@ -256,7 +256,8 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             }
             int unit = 0;
             if (lane == 0) {
-                unit = atomicAdd(work_counter, 1);
+                // a pair's first unit is its own number: nothing to wait for
+                unit = un == 0 ? (int)(blockIdx.x >> 1) : atomicAdd(work_counter, 1) + (int)(gridDim.x >> 1);
                 if (unit >= total_units) unit = -1;
                 bars->unit_slot[slot] = unit;
                 mbar_arrive(&bars->unit_full[slot]);             // release: the slot is written before the arrival
@@ -266,15 +267,30 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             return __shfl_sync(0xffffffffu, unit, 0);
         };
         int next_unit = rank == 0 ? publish(0) : 0;
+        // K: this CTA's 64 keys = pages 4 rank .. 4 rank + 3 of every tile.  Lane pg + 4 grp moves page pg of them: one box, or its
+        // two 8-row groups where the pool's strides fold neither way and for rows of k_new.
+        const int pg = lane & 3, grp = lane >> 2, kpg = 4 * (int)rank + pg;
+        const int boxes = fold ? 4 : 8, c1 = 8 * grp, s3 = fold == 1 ? 1 : 0, s4 = fold == 2 ? 1 : 0;
+        const uint32_t lane_off = pg * kKPageBytes + grp * kKGroupBytes;
+        int sk = 0;                                              // ring slot of the next tile
+        uint32_t pk = 1;                                         // parity of its "empty" barrier: the first round passes at once
+        // the tile before the one being requested, if this unit is the one that appends its pages: stored from its ring slot
+        bool owes = false, o_whole = false, stored = false;      // stored: a slot may still be read by its store
+        int o_sk = 0, o_page = 0, o_hk = 0;
+        uint32_t o_pk = 0;
+        auto pay = [&]() {
+            if (!owes) return;
+            owes = false;
+            ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_full[o_sk], o_pk, cx));
+            if (ok && o_whole) tma_store_5d(&map_k, smem_u32(k_ring) + o_sk * kHalfBytes + lane_off, 0, c1, 0, o_hk << s3, o_page << s4);
+            tile_append::stores_commit();
+            stored = true;
+        };
         for (int un = 0; ok; ++un) {
             int unit;
             if (rank == 0) {
                 unit = next_unit;
                 if (unit < 0) break;
-                // the unit after this one is published before this one's tiles are requested, so that the MMA thread can
-                // run its score tiles ahead across the unit boundary
-                next_unit = publish(un + 1);
-                if (!ok) break;
             } else {
                 unit = read_unit(un, true);
                 if (unit == -2) { ok = false; break; }
@@ -283,47 +299,106 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             const Unit u = decode_unit(a, items, unit);
             const int32_t* __restrict__ table = a.plan.block_table + (int64_t)u.r * a.plan.max_pages + u.kv_begin / kPageSize;
             const int qs = un & 1;
+            const int total_pages = (u.kv_end - u.kv_begin + kPageSize - 1) / kPageSize;
+            HAT_CHECK(u.kv_begin / kPageSize + total_pages <= a.plan.max_pages, cx.status);
+            // the page id of the NEXT tile is fetched while this tile's boxes are issued
+            auto page_of = [&](int j) -> int {
+                const int at = 8 * j + kpg;
+                return at < total_pages ? HAT_IN_RANGE(__ldg(table + at), a.plan.num_pages, cx.status) : 0;
+            };
+            int page = page_of(0);
+            if (un == 0) { pdl_wait(); pdl_launch_dependents(); }   // up to here only the plan's own arrays were read; the kernel behind may be one that runs beside this one
+            if (rank == 0) {
+                // the unit after this one is published before this one's tiles are requested, so that the MMA thread can
+                // run its score tiles ahead across the unit boundary
+                next_unit = publish(un + 1);
+                if (!ok) break;
+            }
             PH_ADD(0, tq0);
             if (un >= 2) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_empty[qs], ((un >> 1) - 1) & 1, cx));
                 if (!ok) break;
             }
             if (lane == 0) mbar_expect_tx(&bars->q_full[qs], kTileBytes);
-            __syncwarp();
             if (lane < 2)      // lane = column half; this CTA's 128 rows
                 tma_load_3d(smem_u32(q_tiles) + qs * kTileBytes + lane * kSlabBytes, &map_q, lane * 64, u.h,
                             u.row_base + u.row0 + (int)rank * kRows, &bars->q_full[qs]);
             PH_ADD(1, tq0);
-            // K: this CTA's 64 keys = pages 4 rank .. 4 rank + 3 of every tile, both column halves: lane = 2 * page + half.
-            // The page id of the NEXT tile is fetched while this tile's boxes are issued.
-            const int total_pages = (u.kv_end - u.kv_begin + kPageSize - 1) / kPageSize;
-            const int kpg = 4 * (int)rank + (lane >> 1), khalf = lane & 1;
-            HAT_CHECK(u.kv_begin / kPageSize + total_pages <= a.plan.max_pages, cx.status);
-            int page = (lane < 8 && kpg < total_pages) ? HAT_IN_RANGE(__ldg(table + kpg), a.plan.num_pages, cx.status) : 0;
-            for (int j = 0; j < u.n; ++j, ++g) {
-                const int sk = g % kStagesK;
+            // tiles [0, n_plain) hold nothing of the chunk, or the call does not append
+            const int n_plain = a.k_new != nullptr ? min(u.n, max(0, u.P - u.kv_begin) / kKeys) : u.n;
+            const int c3 = u.hk << s3;
+            auto step = [&]() { if (++sk == kStagesK) { sk = 0; pk ^= 1; } };
+            int j = 0;
+            for (; j < n_plain; ++j) {
                 const int npages = min(8, total_pages - 8 * j);                                   // pages of this tile: 1..8
                 const int nk = max(0, min(4, npages - 4 * (int)rank));                            // K pages this CTA loads
-                const int next_pg = 8 * (j + 1) + kpg;
-                const int page_next = (lane < 8 && next_pg < total_pages) ? HAT_IN_RANGE(__ldg(table + next_pg), a.plan.num_pages, cx.status) : 0;
+                const int page_next = page_of(j + 1), c4 = page << s4;
                 HAT_CHECK(sk < kStagesK, cx.status);
                 PH_ADD(2, tq0);
-                if (g >= kStagesK) ok = mbar_wait(&bars->k_empty[sk], ((g / kStagesK) & 1) ^ 1, cx);
-                ok = __all_sync(0xffffffffu, ok);
+                if (stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, cx));
                 if (!ok) break;
                 PH_ADD(3, tq0);
-                if (lane == 0) mbar_expect_tx(&bars->k_full[sk], nk * 2 * kPageBoxBytes);
-                __syncwarp();
-                if (lane < 8 && kpg < npages)
-                    tma_load_4d(smem_u32(k_ring) + sk * kHalfBytes + khalf * kKSlabBytes + (lane >> 1) * kPageBoxBytes, &map_k,
-                                khalf * 64, 0, u.hk, page, &bars->k_full[sk]);
+                if (lane == 0) mbar_expect_tx(&bars->k_full[sk], nk * kKPageBytes);
+                if (lane < boxes && kpg < npages)
+                    tma_load_5d(smem_u32(k_ring) + sk * kHalfBytes + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
                 PH_ADD(4, tq0);
 #ifdef HAT_PHASE_TIMERS
                 ph[7] += 1;
 #endif
+                if (owes) pay();                                 // the previous unit's last tile
                 page = page_next;
+                step();
+            }
+            if (!ok) break;
+            if (j == u.n) continue;
+            // tiles with chunk positions
+            const tile_append::Chunk ck{u.P, u.C, u.row_base, u.hk};
+            // of the units that read a chunk page, the last row block of the group's first query head appends it
+            const bool appends = u.h == u.hk * a.plan.group && u.row0 + 2 * kRows >= u.C;
+            for (; j < u.n; ++j) {
+                const int npages = min(8, total_pages - 8 * j);
+                const int nk = max(0, min(4, npages - 4 * (int)rank));
+                const int page_next = page_of(j + 1);
+                const int kb = u.kv_begin + j * kKeys, key0 = kb + kpg * kPageSize;   // first keys of the tile and of this lane's page
+                // a page with both prefix and chunk rows is gathered and completes the barrier last
+                const int pe = (u.P - kb) / kPageSize;
+                const bool edge = u.P > kb && u.P % kPageSize != 0 && pe < npages && (pe >> 2) == (int)rank;
+                const bool fresh = lane < 8 && kpg < npages && ck.fresh(key0);
+                const bool pool = lane < boxes && kpg < npages && !ck.fresh(key0) && !(edge && kpg == pe);
+                const uint32_t bytes = (nk - (edge ? 1 : 0)) * kKPageBytes;
+                if (stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, cx));
+                if (!ok) break;
+                const uint32_t dst = smem_u32(k_ring) + sk * kHalfBytes;
+                if (lane == 0) { if (edge) mbar_expect_only(&bars->k_full[sk], bytes); else mbar_expect_tx(&bars->k_full[sk], bytes); }
+                if (fresh) tma_load_4d(dst + lane_off, &map_k_new, 0, u.row_base + key0 - u.P + 8 * grp, 0, u.hk, &bars->k_full[sk]);
+                if (pool) tma_load_5d(dst + lane_off, &map_k, 0, c1, 0, c3, page << s4, &bars->k_full[sk]);
+                if (edge) {
+                    tile_append::gather_edge<kD>(a, ck, a.cache.k_pool, a.k_new, kD, 0, __shfl_sync(0xffffffffu, page, pe & 3), kb + pe * kPageSize,
+                                                 dst + (pe & 3) * kKPageBytes, kKGroupBytes, lane);
+                    tile_append::gathered();
+                    if (lane == 0) mbar_arrive(&bars->k_full[sk]);
+                }
+                pay();
+                if (!ok) break;
+                if (appends) {
+                    owes = true;
+                    o_sk = sk; o_pk = pk ^ 1; o_page = page; o_hk = u.hk;
+                    o_whole = lane < boxes && kpg < npages && ck.whole(key0);
+                    // the pages that are not whole, row by row
+                    for (uint32_t left = __ballot_sync(0xffffffffu, lane < 4 && kpg < npages && ck.partly(key0)); left; left &= left - 1) {
+                        const int from = __ffs(left) - 1;
+                        tile_append::store_rows<kD>(a, ck, a.k_dst, a.k_new, kD, 0, __shfl_sync(0xffffffffu, page, from),
+                                                    __shfl_sync(0xffffffffu, key0, from), lane);
+                    }
+                }
+                page = page_next;
+                step();
             }
         }
+        if (ok) pay();
+        tile_append::stores_done();
 #ifdef HAT_PHASE_TIMERS
         if (lane == 0) PH_FLUSH(48 + 8 * (int)rank, 8);
 #endif
@@ -337,8 +412,22 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
         // A warp of its own: the K and the V ring then fill independently (one warp doing both waits for a V slot
         // before it may request the next K tile), and two warps feed the TMA unit.
         // All 8 pages of every tile, this CTA's column half: lane = page.
-        int g = 0;
+        bool withhold = a.withhold;                              // self test: the first V tile never arrives, its consumers give up
         bool ok = true;
+        int sv = 0;                                              // as in the K producer
+        uint32_t pv = 1;
+        bool owes = false, o_whole = false, stored = false;      // stored: a slot may still be read by its store
+        int o_sv = 0, o_page = 0, o_hk = 0;
+        uint32_t o_pv = 0;
+        auto pay = [&]() {
+            if (!owes) return;
+            owes = false;
+            ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_full[o_sv], o_pv, cx));
+            if (ok && o_whole) tma_store_4d(&map_v, smem_u32(v_ring) + o_sv * kHalfBytes + lane * kVPageBytes, (int)rank * 64, 0, o_hk, o_page);
+            tile_append::stores_commit();
+            stored = true;
+        };
+        auto step = [&]() { if (++sv == kStagesV) { sv = 0; pv ^= 1; } };
         for (int un = 0; ok; ++un) {
             const int unit = read_unit(un, true);
             if (unit == -2) { ok = false; break; }
@@ -347,26 +436,78 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             const int32_t* __restrict__ table = a.plan.block_table + (int64_t)u.r * a.plan.max_pages + u.kv_begin / kPageSize;
             const int total_pages = (u.kv_end - u.kv_begin + kPageSize - 1) / kPageSize;
             HAT_CHECK(u.kv_begin / kPageSize + total_pages <= a.plan.max_pages, cx.status);
-            int page = (lane < 8 && lane < total_pages) ? HAT_IN_RANGE(__ldg(table + lane), a.plan.num_pages, cx.status) : 0;
-            for (int j = 0; j < u.n; ++j, ++g) {
-                const int sv = g % kStagesV;
+            auto page_of = [&](int j) -> int {
+                const int at = 8 * j + lane;
+                return lane < 8 && at < total_pages ? HAT_IN_RANGE(__ldg(table + at), a.plan.num_pages, cx.status) : 0;
+            };
+            int page = page_of(0);
+            if (un == 0) pdl_wait();                             // up to here only the plan's own arrays were read
+            const int n_plain = a.k_new != nullptr ? min(u.n, max(0, u.P - u.kv_begin) / kKeys) : u.n;
+            int j = 0;
+            for (; j < n_plain; ++j) {
                 const int npages = min(8, total_pages - 8 * j);
-                const int next_pg = 8 * (j + 1) + lane;
-                const int page_next = (lane < 8 && next_pg < total_pages) ? HAT_IN_RANGE(__ldg(table + next_pg), a.plan.num_pages, cx.status) : 0;
+                const int page_next = page_of(j + 1);
                 HAT_CHECK(sv < kStagesV, cx.status);
-                if (g >= kStagesV) ok = mbar_wait(&bars->v_empty[sv], ((g / kStagesV) & 1) ^ 1, cx);
-                ok = __all_sync(0xffffffffu, ok);
+                if (stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, cx));
                 if (!ok) break;
-                if (!(a.withhold && g == 0)) {               // self test: this V tile never arrives, its consumers give up
-                    if (lane == 0) mbar_expect_tx(&bars->v_full[sv], npages * kPageBoxBytes);
-                    __syncwarp();
-                    if (lane < 8 && lane < npages)
-                        tma_load_4d(smem_u32(v_ring) + sv * kHalfBytes + lane * kPageBoxBytes, &map_v, (int)rank * 64, 0, u.hk, page,
-                                    &bars->v_full[sv]);
+                if (!withhold) {
+                    if (lane == 0) mbar_expect_tx(&bars->v_full[sv], npages * kVPageBytes);
+                    if (lane < npages)
+                        tma_load_4d(smem_u32(v_ring) + sv * kHalfBytes + lane * kVPageBytes, &map_v, (int)rank * 64, 0, u.hk, page, &bars->v_full[sv]);
                 }
+                if (owes) pay();                                 // the previous unit's last tile
+                withhold = false;
                 page = page_next;
+                step();
+            }
+            if (!ok) break;
+            if (j == u.n) continue;
+            const tile_append::Chunk ck{u.P, u.C, u.row_base, u.hk};
+            const bool appends = u.h == u.hk * a.plan.group && u.row0 + 2 * kRows >= u.C;
+            for (; j < u.n; ++j) {
+                const int npages = min(8, total_pages - 8 * j);
+                const int page_next = page_of(j + 1);
+                const int kb = u.kv_begin + j * kKeys, key0 = kb + lane * kPageSize;
+                const int pe = (u.P - kb) / kPageSize;
+                const bool edge = u.P > kb && u.P % kPageSize != 0 && pe < npages;
+                const uint32_t bytes = (npages - (edge ? 1 : 0)) * kVPageBytes;
+                if (stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, cx));
+                if (!ok) break;
+                const uint32_t dst = smem_u32(v_ring) + sv * kHalfBytes;
+                if (!withhold) {
+                    if (lane == 0) { if (edge) mbar_expect_only(&bars->v_full[sv], bytes); else mbar_expect_tx(&bars->v_full[sv], bytes); }
+                    if (lane < npages && ck.fresh(key0))
+                        tma_load_4d(dst + lane * kVPageBytes, &map_v_new, 0, u.row_base + key0 - u.P, (int)rank, u.hk, &bars->v_full[sv]);
+                    else if (lane < npages && !(edge && lane == pe))
+                        tma_load_4d(dst + lane * kVPageBytes, &map_v, (int)rank * 64, 0, u.hk, page, &bars->v_full[sv]);
+                }
+                if (edge) {
+                    tile_append::gather_edge<64>(a, ck, a.cache.v_pool, a.v_new, kD, (int)rank * 64, __shfl_sync(0xffffffffu, page, pe), kb + pe * kPageSize,
+                                                 dst + pe * kVPageBytes, 1024, lane);
+                    tile_append::gathered();
+                    if (lane == 0 && !withhold) mbar_arrive(&bars->v_full[sv]);
+                }
+                pay();
+                if (!ok) break;
+                if (appends && !withhold) {
+                    owes = true;
+                    o_sv = sv; o_pv = pv ^ 1; o_page = page; o_hk = u.hk;
+                    o_whole = lane < npages && ck.whole(key0);
+                    for (uint32_t left = __ballot_sync(0xffffffffu, lane < npages && ck.partly(key0)); left; left &= left - 1) {
+                        const int from = __ffs(left) - 1;
+                        tile_append::store_rows<64>(a, ck, a.v_dst, a.v_new, kD, (int)rank * 64, __shfl_sync(0xffffffffu, page, from),
+                                                    __shfl_sync(0xffffffffu, key0, from), lane);
+                    }
+                }
+                withhold = false;
+                page = page_next;
+                step();
             }
         }
+        if (ok) pay();
+        tile_append::stores_done();
         if (!ok) {
             const long long t0 = clock64();
             while (clock64() - t0 < 2000000) { }
@@ -428,7 +569,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             if (warp == 10) {
                 // ---- S = Q K^T of every tile, up to three tiles ahead of the P V products
                 const uint64_t q_desc0 = smem_desc(smem_u32(q_tiles), 16, 1024);
-                const uint64_t k_desc0 = smem_desc(smem_u32(k_ring), 16, 1024);
+                const uint64_t k_desc0 = smem_desc(smem_u32(k_ring), 16, kKGroupBytes);
                 uint32_t s_col = tmem, s_bar = smem_u32(&bars->s_full[0]), pv_bar = smem_u32(&bars->pv_done[0]), pv_par = 0;
                 int s_buf = 0, k_slot = 0;
                 bool wrapped = false;                       // the buffer about to be written has been used before
@@ -459,9 +600,9 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         tc_fence_after();
 #pragma unroll
                         for (int ks = 0; ks < kD / 16; ++ks) {
-                            // 16 columns = 32 bytes inside a row of a 64-column slab; Q slabs are 16 KiB, K-half slabs 8 KiB apart
+                            // 16 columns = 32 bytes inside a row of 64; the next 64 columns are 16 KiB (Q) or 1 KiB (K) on
                             const uint32_t qoff = ((ks >> 2) * kSlabBytes + (ks & 3) * 32) >> 4;
-                            const uint32_t koff = ((ks >> 2) * kKSlabBytes + (ks & 3) * 32) >> 4;
+                            const uint32_t koff = ((ks >> 2) * 1024 + (ks & 3) * 32) >> 4;
                             mma_ss_pair(s_col, qd + qoff, kd + koff, idesc_s, ks > 0);
                         }
                         commit_addr(s_bar);
@@ -1021,7 +1162,12 @@ cudaError_t launch_attn_pair(const hat_plan* plan, const AttnArgs& args, cudaStr
     const bool bf16 = plan->dtype == HAT_DTYPE_BF16;
     const CUtensorMap *mk = nullptr, *mv = nullptr;
     const CUtensorMap* mq = plan_q_map(plan, args.q);
-    if (!mq || !plan_pool_maps(plan, args.cache, &mk, &mv)) return cudaErrorInvalidValue;
+    // K in boxes of whole pages, V by column halves
+    const CUtensorMap *mk4 = nullptr, *mv5 = nullptr, *mkn = nullptr, *mvn = nullptr, *mvh = nullptr;
+    int fold = 0;
+    if (!mq || !plan_pool_maps(plan, args.cache, &mk4, &mv) || !plan_tile_maps(plan, args.cache, &mk, &mv5, &fold) ||
+        !plan_new_maps(plan, args.k_new, args.v_new, &mkn, &mvn, &mvh))
+        return cudaErrorInvalidValue;
     // the unit counter is zero at this point: the previous call's last CTA cleared it
     const int total_units = num_units >= 0 ? num_units : (int)plan->tile_units.size();
     if (total_units <= 0) return cudaSuccess;
@@ -1033,9 +1179,7 @@ cudaError_t launch_attn_pair(const hat_plan* plan, const AttnArgs& args, cudaStr
     auto kern = bf16 ? attn_pair_kernel<true> : attn_pair_kernel<false>;
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), kSmemBytes);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, kSmemBytes, stream>>>(args, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, dim3(kThreads), kSmemBytes, stream, args, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv, *mkn, *mvh, fold);
 }
 
 #ifdef HAT_PHASE_TIMERS

@@ -43,6 +43,7 @@
 
 namespace hat {
 namespace {
+using tc5::cp_async16;
 using tc5::fast_exp2;
 using tc5::mbar_arrive;
 using tc5::mbar_expect_tx;
@@ -79,10 +80,6 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
 }
 template <bool BF16>
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) { return pack_out16(lo, hi, BF16); }
-// 16 bytes global -> shared, asynchronous; zeros when !valid
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
 // the barrier's current phase also waits for this thread's copies so far
 __device__ __forceinline__ void cp_async_on(uint64_t* bar) {
     asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");

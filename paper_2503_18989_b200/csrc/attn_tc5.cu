@@ -5,7 +5,7 @@
 // tiles of a unit use the same K/V tiles in shared memory, and while one tile's softmax runs the tensor pipe works
 // for the other.  Roles:
 //   warp 0      draws the next unit and publishes it to the other roles; TMA producer: the unit's Q tiles, then K
-//               and V tiles of 128 keys (8 pages x 2 halves of 64 columns, 128-byte swizzle) into a two-slot K ring
+//               and V tiles of 128 keys (8 pages, a box each, 128-byte swizzle) into a two-slot K ring
 //               and a three-slot V ring, completion on mbarriers.  It runs ahead across units: the next unit's Q and
 //               first K/V tiles are already landing while the current unit's last tiles and its output are processed
 //   warp 1      one thread issues tcgen05.mma: S_t = Q_t K^T for query tile t, then O_t += P_t V with P read
@@ -31,6 +31,7 @@
 #include "hat_internal.h"
 #include "tma_desc.h"
 #include "tc5_ptx.cuh"
+#include "tile_append.cuh"
 
 namespace hat {
 namespace {
@@ -44,7 +45,9 @@ constexpr int kStagesV = 3;     // ring slots for V tiles (V is requested later 
 // head_dim / 64 slabs of 64 columns
 template <int D> constexpr uint32_t tile_bytes() { return kKeys * D * 2; }
 constexpr uint32_t kSlabBytes = kKeys * 64 * 2;          // 16 KiB: 64 columns of 128 rows
-constexpr uint32_t kPageBoxBytes = 16 * 64 * 2;          // 2 KiB: one TMA box (16 tokens x 64 columns)
+// K and V tiles: 8-row groups (head_dim / 64 blocks of 1 KiB) one after the other; a page is two groups
+template <int D> constexpr uint32_t group_bytes() { return 8 * D * 2; }
+template <int D> constexpr uint32_t page_bytes() { return 16 * D * 2; }
 constexpr float kRescaleThreshold = 8.0f;                // log2 units
 
 struct __align__(8) Barriers {
@@ -97,15 +100,13 @@ struct Unit {
 };
 __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* __restrict__ items, int unit) {
     const uint32_t e = __ldg(a.plan.tile_units + unit);      // item | head << 16
-    const WorkItem it = items[e & 0xffffu];
+    const int4* __restrict__ rec = reinterpret_cast<const int4*>(items + (e & 0xffffu));
+    const int4 lo = __ldg(rec), hi = __ldg(rec + 1);
     Unit u;
     u.h = (int)(e >> 16);
     u.hk = u.h / a.plan.group;
-    u.r = it.req;
-    u.P = a.plan.prefix_len[u.r];
-    u.C = a.plan.chunk_len[u.r];
-    u.row_base = a.plan.cu_chunk[u.r];
-    u.row0 = it.row0; u.kv_begin = it.kv_begin; u.kv_end = it.kv_end; u.part = it.part;
+    u.r = lo.x; u.row0 = lo.y; u.kv_begin = lo.z; u.kv_end = lo.w;
+    u.part = hi.x; u.P = hi.y; u.C = hi.z; u.row_base = hi.w;
     u.nq = (u.C - u.row0 > kRows) ? 2 : 1;
     u.n_all = (u.kv_end - u.kv_begin + kKeys - 1) / kKeys;
     const int end0 = min(u.kv_end, u.P + u.row0 + kRows);
@@ -120,9 +121,11 @@ template <bool BF16, int kD>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units, int32_t* work_counter,
                 const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                const __grid_constant__ CUtensorMap map_v) {
+                const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_k_new,
+                const __grid_constant__ CUtensorMap map_v_new, int fold) {
     constexpr uint32_t kTileBytes = tile_bytes<kD>();
-    constexpr int kHalves = kD / 64;                             // 64-column slabs (and TMA boxes per page) of a tile
+    constexpr int kHalves = kD / 64;                             // 64-column slabs of a Q tile
+    constexpr uint32_t kGroupBytes = group_bytes<kD>(), kPageBytes = page_bytes<kD>();
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the swizzle pattern and the matrix descriptors assume it
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -162,13 +165,41 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
+    if (!a.overlap) pdl_launch_dependents();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch + TMA producer
-        // lane l < 16 moves box (page l/2 of the tile, column half l%2)
-        const int pg = lane / kHalves, half = lane % kHalves;
-        int kt = 0;                                              // K/V tiles issued so far, over all units
+        // Lane pg + 8 g moves page pg of a tile: one box (g = 0), or its two 8-row groups where the pool's strides fold neither
+        // way and for rows of k_new / v_new.  What this warp does per tile is close to what a tile costs the tensor core, so
+        // the loop over plain tiles holds no more than it must (ring positions are stepped, page ids fetched a tile ahead).
+        const int pg = lane & 7, grp = lane >> 3;
+        const int boxes = fold ? 8 : 16;                         // lanes that move pool pages
+        const int c1 = 8 * grp, s3 = fold == 1 ? 1 : 0, s4 = fold == 2 ? 1 : 0;
+        const uint32_t lane_off = pg * kPageBytes + grp * kGroupBytes;
+        int sk = 0, sv = 0;                                      // ring slots of the next tile
+        uint32_t pk = 1, pv = 1;                                 // parities of their "empty" barriers: the first round passes at once
+        bool withhold = a.withhold;                              // self test: the first V tile never arrives, its consumers give up
         bool ok = true;
+        // the tile before the one being requested, if this unit is the one that appends its pages: stored from its ring slots
+        bool owes = false, o_whole = false, stored = false;      // stored: a slot may still be read by its store
+        int o_sk = 0, o_sv = 0, o_page = 0, o_hk = 0;
+        uint32_t o_pk = 0, o_pv = 0;
+        auto pay = [&]() {
+            if (!owes) return;
+            owes = false;
+            ok = mbar_wait(&bars->k_full[o_sk], o_pk, bars, status) && mbar_wait(&bars->v_full[o_sv], o_pv, bars, status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok && o_whole) {
+                tma_store_5d(&map_k, smem_u32(k_ring) + o_sk * kTileBytes + lane_off, 0, c1, 0, o_hk << s3, o_page << s4);
+                tma_store_5d(&map_v, smem_u32(v_ring) + o_sv * kTileBytes + lane_off, 0, c1, 0, o_hk << s3, o_page << s4);
+            }
+            tile_append::stores_commit();
+            stored = true;
+        };
+        auto step = [&]() {
+            if (++sk == kStagesK) { sk = 0; pk ^= 1; }
+            if (++sv == kStagesV) { sv = 0; pv ^= 1; }
+        };
         for (int un = 0; ok; ++un) {
             const int slot = un & 1;
             if (un >= 2) {
@@ -177,7 +208,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             }
             int unit = 0;
             if (lane == 0) {
-                unit = atomicAdd(work_counter, 1);
+                // a CTA's first unit is its own number: nothing to wait for
+                if (un == 0 && a.static_first) unit = (int)blockIdx.x;
+                else unit = atomicAdd(work_counter, 1) + (a.static_first ? (int)gridDim.x : 0);
                 if (unit >= total_units) unit = -1;
                 bars->unit_slot[slot] = unit;
                 mbar_arrive(&bars->unit_full[slot]);             // release: the slot is written before the arrival
@@ -186,43 +219,109 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             if (unit < 0) break;
             const Unit u = decode_unit(a, items, unit);
             const int32_t* __restrict__ table = a.plan.block_table + (int64_t)u.r * a.plan.max_pages;
+            const int total_pages = (u.kv_end - u.kv_begin + kPageSize - 1) / kPageSize, page0 = u.kv_begin / kPageSize;
+            auto page_of = [&](int j) -> int {
+                const int at = 8 * j + pg;
+                return at < total_pages
+                           ? HAT_IN_RANGE(__ldg(table + HAT_IN_RANGE(page0 + at, a.plan.max_pages, status)), a.plan.num_pages, status) : 0;
+            };
+            int page = page_of(0);
             // Q tiles: the previous unit's last S must have read the old ones
             if (un > 0) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_empty, (un - 1) & 1, bars, status));
                 if (!ok) break;
+            } else if (!a.overlap) {
+                pdl_wait();                                      // up to here only the plan's own arrays were read
             }
             if (lane == 0) mbar_expect_tx(&bars->q_full, u.nq * kTileBytes);
-            __syncwarp();
             if (lane < kHalves * u.nq)      // lane = kHalves * (query tile) + (column half)
                 tma_load_3d(smem_u32(q_tiles) + (lane / kHalves) * kTileBytes + (lane % kHalves) * kSlabBytes, &map_q, (lane % kHalves) * 64, u.h,
                             u.row_base + u.row0 + (lane / kHalves) * kRows, &bars->q_full);
-            for (int j = 0; j < u.n_all; ++j, ++kt) {
-                const int sk = kt % kStagesK, sv = kt % kStagesV;
-                const int kb = u.kv_begin + j * kKeys;
-                const int npages = (min(u.kv_end, kb + kKeys) - kb + kPageSize - 1) / kPageSize;
-                int page = 0;
-                if (lane < 8 * kHalves && pg < npages)
-                    page = HAT_IN_RANGE(__ldg(table + HAT_IN_RANGE(kb / kPageSize + pg, a.plan.max_pages, status)), a.plan.num_pages, status);
+            // tiles [0, n_plain) hold nothing of the chunk, or the call does not append
+            const bool fused = a.k_new != nullptr;
+            const int n_plain = fused ? min(u.n_all, max(0, u.P - u.kv_begin) / kKeys) : u.n_all;
+            const int c3 = u.hk << s3;
+            int j = 0;
+            for (; j < n_plain; ++j) {
+                const int npages = min(8, total_pages - 8 * j);
+                const bool mine = lane < boxes && pg < npages;
+                const int page_next = page_of(j + 1), c4 = page << s4;
                 HAT_CHECK(sk < kStagesK && sv < kStagesV, status);
-                if (kt >= kStagesK) ok = mbar_wait(&bars->k_empty[sk], ((kt / kStagesK) & 1) ^ 1, bars, status);
-                ok = __all_sync(0xffffffffu, ok);
+                if (stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars, status));
                 if (!ok) break;
-                if (lane == 0) mbar_expect_tx(&bars->k_full[sk], npages * kHalves * kPageBoxBytes);
-                __syncwarp();
-                if (lane < 8 * kHalves && pg < npages)
-                    tma_load_4d(smem_u32(k_ring) + sk * kTileBytes + half * kSlabBytes + pg * kPageBoxBytes, &map_k, half * 64, 0,
-                                u.hk, page, &bars->k_full[sk]);
-                if (kt >= kStagesV) ok = mbar_wait(&bars->v_empty[sv], ((kt / kStagesV) & 1) ^ 1, bars, status);
-                ok = __all_sync(0xffffffffu, ok);
+                if (lane == 0) mbar_expect_tx(&bars->k_full[sk], npages * kPageBytes);
+                if (mine) tma_load_5d(smem_u32(k_ring) + sk * kTileBytes + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars, status));
                 if (!ok) break;
-                if (a.withhold && kt == 0) continue;         // self test: this V tile never arrives, its consumers give up
-                if (lane == 0) mbar_expect_tx(&bars->v_full[sv], npages * kHalves * kPageBoxBytes);
-                __syncwarp();
-                if (lane < 8 * kHalves && pg < npages)
-                    tma_load_4d(smem_u32(v_ring) + sv * kTileBytes + half * kSlabBytes + pg * kPageBoxBytes, &map_v, half * 64, 0,
-                                u.hk, page, &bars->v_full[sv]);
+                if (!withhold) {
+                    if (lane == 0) mbar_expect_tx(&bars->v_full[sv], npages * kPageBytes);
+                    if (mine) tma_load_5d(smem_u32(v_ring) + sv * kTileBytes + lane_off, &map_v, 0, c1, 0, c3, c4, &bars->v_full[sv]);
+                }
+                if (owes) pay();                                 // the previous unit's last tile
+                withhold = false;
+                page = page_next;
+                step();
+            }
+            if (!ok) break;
+            if (j == u.n_all) continue;
+            // tiles with chunk positions
+            const tile_append::Chunk ck{u.P, u.C, u.row_base, u.hk};
+            // of the units that read a chunk page, the last row block of the group's first query head appends it
+            const bool appends = u.h == u.hk * a.plan.group && u.row0 + 2 * kRows >= u.C;
+            for (; j < u.n_all; ++j) {
+                const int kb = u.kv_begin + j * kKeys;
+                const int npages = min(8, total_pages - 8 * j);
+                const int page_next = page_of(j + 1);
+                const int key0 = kb + pg * kPageSize;            // of this lane's page
+                // a page with both prefix and chunk rows is gathered and completes the barriers last
+                const int pe = (u.P - kb) / kPageSize;
+                const bool edge = u.P > kb && u.P % kPageSize != 0 && pe < npages;
+                const bool fresh = lane < 16 && pg < npages && ck.fresh(key0);
+                const bool pool = lane < boxes && pg < npages && !ck.fresh(key0) && !(edge && pg == pe);
+                const int row = u.row_base + key0 - u.P + 8 * grp;
+                const uint32_t bytes = (npages - (edge ? 1 : 0)) * kPageBytes;
+                if (stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars, status));
+                if (!ok) break;
+                const uint32_t k_dst = smem_u32(k_ring) + sk * kTileBytes, v_dst = smem_u32(v_ring) + sv * kTileBytes;
+                if (lane == 0) { if (edge) mbar_expect_only(&bars->k_full[sk], bytes); else mbar_expect_tx(&bars->k_full[sk], bytes); }
+                if (fresh) tma_load_4d(k_dst + lane_off, &map_k_new, 0, row, 0, u.hk, &bars->k_full[sk]);
+                if (pool) tma_load_5d(k_dst + lane_off, &map_k, 0, c1, 0, c3, page << s4, &bars->k_full[sk]);
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars, status));
+                if (!ok) break;
+                if (!withhold) {
+                    if (lane == 0) { if (edge) mbar_expect_only(&bars->v_full[sv], bytes); else mbar_expect_tx(&bars->v_full[sv], bytes); }
+                    if (fresh) tma_load_4d(v_dst + lane_off, &map_v_new, 0, row, 0, u.hk, &bars->v_full[sv]);
+                    if (pool) tma_load_5d(v_dst + lane_off, &map_v, 0, c1, 0, c3, page << s4, &bars->v_full[sv]);
+                }
+                if (edge) {
+                    const int at = __shfl_sync(0xffffffffu, page, pe);
+                    tile_append::gather_edge<kD>(a, ck, a.cache.k_pool, a.k_new, kD, 0, at, kb + pe * kPageSize, k_dst + pe * kPageBytes, kGroupBytes, lane);
+                    tile_append::gather_edge<kD>(a, ck, a.cache.v_pool, a.v_new, kD, 0, at, kb + pe * kPageSize, v_dst + pe * kPageBytes, kGroupBytes, lane);
+                    tile_append::gathered();
+                    if (lane == 0) { mbar_arrive(&bars->k_full[sk]); if (!withhold) mbar_arrive(&bars->v_full[sv]); }
+                }
+                pay();
+                if (!ok) break;
+                if (appends && !withhold) {
+                    owes = true;
+                    o_sk = sk; o_sv = sv; o_pk = pk ^ 1; o_pv = pv ^ 1; o_page = page; o_hk = u.hk;
+                    o_whole = lane < boxes && pg < npages && ck.whole(key0);
+                    // the pages that are not whole, row by row
+                    for (uint32_t left = __ballot_sync(0xffffffffu, lane < 8 && pg < npages && ck.partly(key0)); left; left &= left - 1) {
+                        const int from = __ffs(left) - 1, at = __shfl_sync(0xffffffffu, page, from);
+                        tile_append::store_rows<kD>(a, ck, a.k_dst, a.k_new, kD, 0, at, kb + from * kPageSize, lane);
+                        tile_append::store_rows<kD>(a, ck, a.v_dst, a.v_new, kD, 0, at, kb + from * kPageSize, lane);
+                    }
+                }
+                withhold = false;
+                page = page_next;
+                step();
             }
         }
+        if (ok) pay();
+        tile_append::stores_done();
         if (!ok) {
             // give copies already in flight a bounded chance to land before the CTA's shared memory is released
             const long long t0 = clock64();
@@ -236,8 +335,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             constexpr uint32_t idesc_o = make_idesc(fmt, 1, kRows, kD);      // P (TMEM)    x V (MN-major)
             // matrix descriptors of Q tile 0 and of slot 0 of each ring, built once
             const uint64_t q_desc0 = smem_desc(smem_u32(q_tiles), 16, 1024);
-            const uint64_t k_desc0 = smem_desc(smem_u32(k_ring), 16, 1024);
-            const uint64_t v_desc0 = smem_desc(smem_u32(v_ring), kSlabBytes, 1024);
+            const uint64_t k_desc0 = smem_desc(smem_u32(k_ring), 16, kGroupBytes);
+            const uint64_t v_desc0 = smem_desc(smem_u32(v_ring), 1024, kGroupBytes);
             bool ok = true;
             int kt_base = 0;                          // K/V tiles of the units before this one
             int p_cnt[2] = {0, 0};                    // completions of p_ready[t] consumed so far
@@ -272,8 +371,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         tc_fence_after();
 #pragma unroll
                         for (int ks = 0; ks < kD / 16; ++ks) {
-                            const uint32_t off = ((ks >> 2) * kSlabBytes + (ks & 3) * 32) >> 4;   // 16 columns = 32 bytes inside a slab row
-                            mma_ss(tmem + qt * 128, qd + off, kd + off, idesc_s, ks > 0);
+                            // 16 columns = 32 bytes inside a row of 64; the next 64 columns are 16 KiB (Q) or 1 KiB (K) on
+                            const uint32_t q_off = ((ks >> 2) * kSlabBytes + (ks & 3) * 32) >> 4, k_off = ((ks >> 2) * 1024 + (ks & 3) * 32) >> 4;
+                            mma_ss(tmem + qt * 128, qd + q_off, kd + k_off, idesc_s, ks > 0);
                         }
                         tc_commit(&bars->s_full[qt]);
                         if (SPLIT || qt == u.nq - 1) {
@@ -306,8 +406,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         HAT_CHECK((to & 0xffffu) + 128 <= 512 && (tp & 0xffffu) + 128 <= 256, status);
 #pragma unroll
                         for (int ks = 0; ks < kKeys / 16; ++ks) {
-                            // 16 keys = 2048 bytes of every 64-column slab; slabs 16 KiB apart (leading), 8-key groups 1 KiB apart
-                            const uint64_t vdesc = vd + (uint64_t)((ks * 2048) >> 4);
+                            // 16 keys = one page; inside it 64-column blocks 1 KiB apart (leading), then the next 8-key group
+                            const uint64_t vdesc = vd + (uint64_t)((ks * kPageBytes) >> 4);
                             mma_ts(to, tp + ks * 8, vdesc, idesc_o, (sidx > 0) || (ks > 0));
                             if constexpr (BF16) mma_ts(to, tp + 64 + ks * 8, vdesc, idesc_o, true);
                         }
@@ -457,7 +557,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         constexpr int kVecs = kD / 8;                              // 16-byte vectors per row
                         for (int idx = wg_tid; idx < (kKeys - first) * kVecs; idx += 128) {
                             const int row = first + idx / kVecs, part = idx % kVecs;
-                            *reinterpret_cast<uint4*>(vt + (part >> 3) * kSlabBytes + row * 128 + (part & 7) * 16) = make_uint4(0, 0, 0, 0);
+                            *reinterpret_cast<uint4*>(vt + (row >> 3) * kGroupBytes + (part >> 3) * 1024 + (row & 7) * 128 + (part & 7) * 16) = make_uint4(0, 0, 0, 0);
                         }
                         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     }
@@ -574,6 +674,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
     }
     // The last CTA to get here (none draws units any more) leaves the unit counter at zero for the next call, which
     // then needs no memset in front of it.  work_counter[1] counts the CTAs that have finished.
+    if (a.overlap && threadIdx.x == 0) pdl_wait();               // the next kernel takes this one's end for the end of both
     if (a.tail_reset && threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {
@@ -592,16 +693,21 @@ bool tc5_layout_supported(int dtype, int head_dim, int num_pages, int H, int64_t
     if ((head_dim != 64 && head_dim != 128) || num_pages <= 0) return false;
     CUtensorMap m;
     // the encoder checks alignment and ranges only; any 16-byte aligned address will do for the probe
-    return tma_encode_pool_map(&m, dtype == HAT_DTYPE_BF16, reinterpret_cast<const void*>(uintptr_t(1) << 30), head_dim,
-                               num_pages, H, stride_page, stride_token, stride_head);
+    const void* probe = reinterpret_cast<const void*>(uintptr_t(1) << 30);
+    int fold;
+    return tma_encode_pool_map(&m, dtype == HAT_DTYPE_BF16, probe, head_dim, num_pages, H, stride_page, stride_token, stride_head) &&
+           tma_encode_tile_map(&m, dtype == HAT_DTYPE_BF16, probe, head_dim, num_pages, H, stride_page, stride_token, stride_head, &fold);
 }
 
 cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStream_t stream, int grid_limit,
-                            bool reset_counter, int first_unit, int num_units, int counter_word) {
+                            bool reset_counter, int first_unit, int num_units, int counter_word, bool overlap) {
     const bool bf16 = plan->dtype == HAT_DTYPE_BF16;
     const CUtensorMap *mk = nullptr, *mv = nullptr;
     const CUtensorMap* mq = plan_q_map(plan, args.q);
-    if (!mq || !plan_pool_maps(plan, args.cache, &mk, &mv)) return cudaErrorInvalidValue;
+    const CUtensorMap *mkn = nullptr, *mvn = nullptr, *mvh = nullptr;
+    int fold = 0;
+    if (!mq || !plan_tile_maps(plan, args.cache, &mk, &mv, &fold) || !plan_new_maps(plan, args.k_new, args.v_new, &mkn, &mvn, &mvh))
+        return cudaErrorInvalidValue;
     // one CTA per SM draws units from a counter that is zero at this point: the previous call's last CTA cleared it
     // (reset_counter); a grid that joins another one on the same counter leaves it alone
     const int total_units = num_units >= 0 ? num_units : (int)plan->tile_units.size() - first_unit;
@@ -610,6 +716,8 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     AttnArgs a2 = args;
     a2.plan.tile_units = plan->dev.tile_units + first_unit;
     a2.tail_reset = reset_counter ? 1 : 0;
+    a2.static_first = a2.tail_reset;            // a counter of its own
+    a2.overlap = overlap ? 1 : 0;
     int ctas = std::min(total_units, plan->num_sms);
     if (grid_limit > 0) ctas = std::min(ctas, grid_limit);
     const dim3 grid((unsigned)ctas);
@@ -619,9 +727,7 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     const uint32_t smem = d128 ? smem_bytes<128>() : smem_bytes<64>();
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, smem, stream>>>(a2, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, dim3(kThreads), smem, stream, a2, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv, *mkn, *mvn, fold);
 }
 
 }  // namespace hat

@@ -74,6 +74,44 @@ bool plan_page_maps(const hat_plan* plan, const CacheView& c, const CUtensorMap*
     return true;
 }
 
+bool plan_tile_maps(const hat_plan* plan, const CacheView& c, const CUtensorMap** mk, const CUtensorMap** mv, int* fold) {
+    MapCache& m = const_cast<hat_plan*>(plan)->maps;
+    if (!m.have_tile || m.tile_k != c.k_pool || m.tile_v != c.v_pool || m.tile_strides[0] != c.stride_page ||
+        m.tile_strides[1] != c.stride_token || m.tile_strides[2] != c.stride_head) {
+        const bool bf16 = plan->dtype == HAT_DTYPE_BF16;
+        m.have_tile = false;
+        if (!tma_encode_tile_map(&m.mtk, bf16, c.k_pool, plan->head_dim, plan->num_pages, plan->num_kv_heads, c.stride_page,
+                                 c.stride_token, c.stride_head, &m.tile_fold) ||
+            !tma_encode_tile_map(&m.mtv, bf16, c.v_pool, plan->head_dim, plan->num_pages, plan->num_kv_heads, c.stride_page,
+                                 c.stride_token, c.stride_head, &m.tile_fold))
+            return false;
+        m.tile_k = c.k_pool; m.tile_v = c.v_pool;
+        m.tile_strides[0] = c.stride_page; m.tile_strides[1] = c.stride_token; m.tile_strides[2] = c.stride_head;
+        m.have_tile = true;
+    }
+    *mk = &m.mtk; *mv = &m.mtv; *fold = m.tile_fold;
+    return true;
+}
+
+bool plan_new_maps(const hat_plan* plan, const void* k_new, const void* v_new, const CUtensorMap** mk, const CUtensorMap** mv,
+                   const CUtensorMap** mv_half) {
+    MapCache& m = const_cast<hat_plan*>(plan)->maps;
+    if (k_new && (!m.have_new || m.k_new != k_new || m.v_new != v_new)) {
+        const bool bf16 = plan->dtype == HAT_DTYPE_BF16;
+        const int T = plan->total_rows, H = plan->num_kv_heads, d = plan->head_dim;
+        m.have_new = false;
+        if (!tma_encode_new_map(&m.mkn, bf16, k_new, T, H, d, 8, d / 64) || !tma_encode_new_map(&m.mvn, bf16, v_new, T, H, d, 8, d / 64) ||
+            !tma_encode_new_map(&m.mvn_half, bf16, v_new, T, H, d, kPageSize, 1))
+            return false;
+        m.k_new = k_new; m.v_new = v_new;
+        m.have_new = true;
+    }
+    *mk = k_new ? &m.mkn : &m.mq;
+    *mv = k_new ? &m.mvn : &m.mq;
+    *mv_half = k_new ? &m.mvn_half : &m.mq;
+    return true;
+}
+
 const CUtensorMap* plan_q_map(const hat_plan* plan, const void* q) {
     MapCache& m = const_cast<hat_plan*>(plan)->maps;
     if (!m.have_q || m.q != q) {
@@ -121,13 +159,13 @@ static void emit_tile(hat_plan* p, std::vector<WorkItem>& items, int req, int ro
                       int kv_end, int split_len) {
     int nsplit = (split_len > 0) ? ceil_div(kv_end, split_len) : 1;
     if (nsplit <= 1) {
-        items.push_back(WorkItem{req, row0, 0, kv_end, -1, 0, 0, 0});
+        items.push_back(WorkItem{req, row0, 0, kv_end, -1, p->prefix_len[req], p->chunk_len[req], p->cu_chunk[req]});
         return;
     }
     int64_t base = p->part_rows;
     for (int s = 0; s < nsplit; ++s) {
         int b = s * split_len, e = std::min(kv_end, b + split_len);
-        items.push_back(WorkItem{req, row0, b, e, (int32_t)(base + (int64_t)s * rows_valid), 0, 0, 0});
+        items.push_back(WorkItem{req, row0, b, e, (int32_t)(base + (int64_t)s * rows_valid), p->prefix_len[req], p->chunk_len[req], p->cu_chunk[req]});
     }
     int row_base = p->cu_chunk[req] + row0;
     for (int i = 0; i < rows_valid; ++i)
@@ -803,10 +841,12 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
         if (call >= 0) cudaEventRecord(tm->events[((size_t)call * HAT_TIMING_SLOTS + slot) * 2 + end], s);
         if (call >= 0 && end) tm->launched[(size_t)call * HAT_TIMING_SLOTS + slot] = 1;
     };
-    // the streaming kernel appends its own requests' rows; a batch with prompt chunks, or one whose pages are shared, appends first
+    // the attention kernels append on the way, each class its own requests' rows, unless pages are shared between a writer and
+    // a reader or a class runs on the mma.sync kernels
     const bool has_verify = plan->info.num_verify_items > 0;
-    const bool stream_appends = k_new && plan->info.stream_kernel == 1 && plan->prefill_items.empty() && !plan->append_first;
-    if (k_new && !stream_appends) {
+    const bool fused = k_new && !plan->append_first && (!has_verify || plan->info.stream_kernel == 1) &&
+                       (plan->prefill_items.empty() || plan->info.prefill_kernel != 0);
+    if (k_new && !fused) {
         mark(0, 0);
         e = launch_kv_append(plan, view_of(cache), cache->k_pool, cache->v_pool, k_new, v_new, s);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -816,8 +856,8 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     a.plan = plan->dev;
     a.cache = view_of(cache);
     a.q = q;
-    a.k_new = stream_appends ? k_new : nullptr;
-    a.v_new = stream_appends ? v_new : nullptr;
+    a.k_new = fused ? k_new : nullptr;
+    a.v_new = fused ? v_new : nullptr;
     a.k_dst = cache->k_pool;
     a.v_dst = cache->v_pool;
     a.out = out;
@@ -833,6 +873,8 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     a.wait_cycles = plan->wait_cycles;
     a.withhold = plan->withhold_next;
     a.tail_reset = 0;
+    a.static_first = 0;
+    a.overlap = 0;
     const_cast<hat_plan*>(plan)->withhold_next = 0;
 
     // Decode-phase (draft verification) requests first: their rows are final, and announced through the plan's event,
@@ -867,10 +909,10 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     } else if (!plan->prefill_items.empty()) {
         mark(1, 0);
         if (plan->info.prefill_kernel == 3) {
-            // units of more than 128 rows on CTA pairs, the others (if any) on single CTAs behind them
+            // units of more than 128 rows on CTA pairs, the others (if any) on single CTAs that take the SMs as the pairs leave them
             e = launch_attn_pair(plan, a, s, plan->num_pair_units);
             if (e == cudaSuccess)
-                e = launch_attn_tc5(plan, a, s, 0, true, plan->num_pair_units, -1, /*counter_word=*/3);
+                e = launch_attn_tc5(plan, a, s, 0, true, plan->num_pair_units, -1, /*counter_word=*/3, /*overlap=*/plan->num_pair_units > 0);
         } else {
             e = plan->info.prefill_kernel == 1 ? launch_attn_tc5(plan, a, s)
                                                : launch_attn_mma(plan, a, /*verify_class=*/false, s);

@@ -20,8 +20,9 @@ struct WorkItem {
     int32_t kv_begin;
     int32_t kv_end;
     int32_t part;
-    int32_t pad0, pad1, pad2;
+    int32_t P, C, row_base;   // of the request: prefix length, chunk length, first packed row
 };
+static_assert(sizeof(WorkItem) == 32, "two 16-byte words");
 
 // One piece of a streaming-class request: pages [page0, page1) of its page list, which is the ceil(P/16) pages of the cached
 // prefix followed by one page that holds the chunk's own rows.  Read by the device as 16-byte words.
@@ -77,7 +78,7 @@ struct AttnArgs {
     DevicePlan  plan;
     CacheView   cache;
     const void* q;
-    const void* k_new;        // streaming kernel: the chunk's rows, to be appended to k_dst / v_dst (the pools) as well;
+    const void* k_new;        // the chunk's rows, which the kernel appends to k_dst / v_dst (the pools) on the way;
     const void* v_new;        // null: the rows are in the pools already
     void*       k_dst;
     void*       v_dst;
@@ -91,6 +92,8 @@ struct AttnArgs {
     float       scale_log2;   // sm_scale * log2(e)
     long long   wait_cycles;  // bound of every device-side wait, in SM clock cycles
     int         withhold;     // self test: the tile kernel's producer skips its first V tile so that a wait runs out
+    int         static_first; // a CTA's first unit is its own number, the counter gives the ones after the grid's; else all come from the counter
+    int         overlap;      // the grid runs beside the stream's previous kernel (which has waited for everything before it): waits for its end only at its own
     int         tail_reset;   // the last CTA of the persistent tile kernel to finish clears the unit counter for the next call
 };
 
@@ -177,6 +180,15 @@ struct MapCache {
     int64_t stride_page = 0, stride_token = 0, stride_head = 0;
     bool have_q = false, have_kv = false;
     CUtensorMap mq, mk, mv;
+    // the tile kernels' maps of the same pools, and of k_new / v_new
+    const void* tile_k = nullptr; const void* tile_v = nullptr;
+    int64_t tile_strides[3] = {0, 0, 0};
+    bool have_tile = false;
+    int tile_fold = 0;
+    CUtensorMap mtk, mtv;
+    const void* k_new = nullptr; const void* v_new = nullptr;
+    bool have_new = false;
+    CUtensorMap mkn, mvn, mvn_half;
     // the streaming kernel's maps of the same pools (boxes of whole pages)
     const void* page_k = nullptr; const void* page_v = nullptr;
     int64_t page_strides[3] = {0, 0, 0};
@@ -264,7 +276,8 @@ bool tc5_layout_supported(int dtype, int head_dim, int num_pages, int H, int64_t
 // first_unit / num_units (num_units < 0: all) select a part of the plan's unit list; counter_word: which pair of the
 // plan's status words (unit counter, finished CTAs) the grid uses
 cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStream_t stream, int grid_limit = 0,
-                            bool reset_counter = true, int first_unit = 0, int num_units = -1, int counter_word = 1);
+                            bool reset_counter = true, int first_unit = 0, int num_units = -1, int counter_word = 1,
+                            bool overlap = false);
 // tcgen05 tile kernel with 256-row units processed by clusters of two CTAs (cta_group::2), same layout requirements
 cudaError_t launch_attn_pair(const hat_plan* plan, const AttnArgs& args, cudaStream_t stream, int num_units = -1);   // the first num_units units
 // TMA-fed streaming kernel: whether a TMA descriptor can be built for this pool layout, and the launcher
@@ -305,6 +318,11 @@ namespace hat {
 // The plan's cached tensor maps for these pools / this q buffer, encoded again only when a pointer or a stride changed.
 // Return null when no map can be built.  (Defined in hat_api.cu.)
 bool plan_pool_maps(const hat_plan* plan, const CacheView& cache, const CUtensorMap** mk, const CUtensorMap** mv);
+// the tile kernels' maps: pools in boxes of whole pages, 8-row groups one after the other (see tma_encode_tile_map)
+bool plan_tile_maps(const hat_plan* plan, const CacheView& cache, const CUtensorMap** mk, const CUtensorMap** mv, int* fold);
+// k_new / v_new in boxes of 8 rows, and v_new in boxes of 16 rows of one column half; null: some valid map that is not used
+bool plan_new_maps(const hat_plan* plan, const void* k_new, const void* v_new, const CUtensorMap** mk, const CUtensorMap** mv,
+                   const CUtensorMap** mv_half);
 bool plan_page_maps(const hat_plan* plan, const CacheView& cache, const CUtensorMap** mk, const CUtensorMap** mv);   // streaming kernel
 const CUtensorMap* plan_q_map(const hat_plan* plan, const void* q);
 }  // namespace hat

@@ -2,6 +2,7 @@
 // ranges.  One warp per (row, head): lane s holds lse_s, the maximum and the sum of exp are
 // warp-shuffle reductions, and each lane then accumulates its slice of head_dim over the parts.
 #include "hat_internal.h"
+#include "tc5_ptx.cuh"
 
 namespace hat {
 
@@ -12,12 +13,34 @@ merge_kernel(const MergeRow* __restrict__ rows, int num_rows, int H,
              float* __restrict__ out, float* __restrict__ lse, void* __restrict__ out16, int out16_bf16) {
     const int lane = threadIdx.x & 31;
     const int64_t unit = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);     // (row, head) pair
-    if (unit >= (int64_t)num_rows * H) return;
-    const MergeRow mr = rows[unit / H];
+    tc5::pdl_launch_dependents();
+    const bool in = unit < (int64_t)num_rows * H;
+    const MergeRow mr = rows[in ? unit / H : 0];
+    tc5::pdl_wait();                                                       // up to here only the plan's own arrays were read
+    if (!in) return;
     const int h = (int)(unit % H);
 
+    // the values of the first eight parts are on their way while the weights are made
+    constexpr int V = D / 32, NP = 8;                                      // floats per lane
+    float v[NP][V];
+    const float* src = part_out + ((int64_t)mr.part0 * H + h) * D + lane * V;
+    const int64_t hop = (int64_t)mr.stride * H * D;
+    auto load_parts = [&](int s0) {
+#pragma unroll
+        for (int s = 0; s < NP; ++s)
+            if (s0 + s < mr.nsplit) {
+                if constexpr (V == 4) {
+                    const float4 x = __ldcg(reinterpret_cast<const float4*>(src + (s0 + s) * hop));
+                    v[s][0] = x.x; v[s][1] = x.y; v[s][2] = x.z; v[s][3] = x.w;
+                } else {
+                    const float2 x = __ldcg(reinterpret_cast<const float2*>(src + (s0 + s) * hop));
+                    v[s][0] = x.x; v[s][1] = x.y;
+                }
+            }
+    };
     float my = -INFINITY;
-    if (lane < mr.nsplit) my = part_lse[((int64_t)mr.part0 + (int64_t)lane * mr.stride) * H + h];
+    if (lane < mr.nsplit) my = __ldcg(part_lse + ((int64_t)mr.part0 + (int64_t)lane * mr.stride) * H + h);
+    load_parts(0);
     float mx = my;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -29,20 +52,18 @@ merge_kernel(const MergeRow* __restrict__ rows, int num_rows, int H,
     const float inv = sum > 0.f ? 1.f / sum : 0.f;
     w *= inv;
 
-    constexpr int V = D / 32;                                              // floats per lane
     float acc[V];
 #pragma unroll
     for (int k = 0; k < V; ++k) acc[k] = 0.f;
-    for (int s = 0; s < mr.nsplit; ++s) {
-        const float ws = __shfl_sync(0xffffffffu, w, s);
-        const float* src = part_out + (((int64_t)mr.part0 + (int64_t)s * mr.stride) * H + h) * D + lane * V;
-        if constexpr (V == 4) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(src));
-            acc[0] += ws * v.x; acc[1] += ws * v.y; acc[2] += ws * v.z; acc[3] += ws * v.w;
-        } else {
-            const float2 v = __ldg(reinterpret_cast<const float2*>(src));
-            acc[0] += ws * v.x; acc[1] += ws * v.y;
-        }
+    for (int s0 = 0; s0 < mr.nsplit; s0 += NP) {
+        if (s0 > 0) load_parts(s0);
+#pragma unroll
+        for (int s = 0; s < NP; ++s)
+            if (s0 + s < mr.nsplit) {
+                const float ws = __shfl_sync(0xffffffffu, w, s0 + s);
+#pragma unroll
+                for (int k = 0; k < V; ++k) acc[k] += ws * v[s][k];
+            }
     }
     const int64_t at = ((int64_t)mr.row * H + h) * D + lane * V;
     if (out16 != nullptr) {
@@ -65,14 +86,9 @@ cudaError_t launch_merge(const hat_plan* plan, const AttnArgs& args, int first_r
     const int H = plan->num_heads;
     const int64_t units = (int64_t)n * H;
     const unsigned blocks = (unsigned)((units + 3) / 4);
-    if (plan->head_dim == 128)
-        merge_kernel<128><<<blocks, 128, 0, stream>>>(plan->dev.merge_rows + first_row, n, H, args.part_out, args.part_lse,
-                                                      args.out, args.lse, args.out16, args.out16_bf16);
-    else
-        merge_kernel<64><<<blocks, 128, 0, stream>>>(plan->dev.merge_rows + first_row, n, H, args.part_out, args.part_lse,
-                                                     args.out, args.lse, args.out16, args.out16_bf16);
-    count_launch();
-    return cudaGetLastError();
+    auto kern = plan->head_dim == 128 ? merge_kernel<128> : merge_kernel<64>;
+    return launch_pdl(kern, dim3(blocks), dim3(128), 0, stream, plan->dev.merge_rows + first_row, n, H, args.part_out, args.part_lse,
+                      args.out, args.lse, args.out16, args.out16_bf16);
 }
 
 }  // namespace hat

@@ -53,6 +53,41 @@ inline bool tma_encode_page_map(CUtensorMap* map, bool bf16, const void* pool, i
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same pool for the tile kernels: boxes that hold a whole page of one head as the tensor core's 8-row groups, i.e.
+// (column of a half, slot of a group, half, group): 1 KiB blocks, so that a tile of several pages is one operand with a uniform
+// distance of head_dim * 16 bytes between groups.  The group is a dimension beside head or page, whichever stride it
+// divides evenly (*fold = 1: the head coordinate is 2 h; 2: the page coordinate is 2 page); other strides take two boxes per
+// page, by the slot coordinate (*fold = 0).
+inline bool tma_encode_tile_map(CUtensorMap* map, bool bf16, const void* pool, int head_dim, int num_pages, int H,
+                                int64_t stride_page, int64_t stride_token, int64_t stride_head, int* fold) {
+    EncodeTiledFn fn = tma_encode_fn();
+    if (!fn || num_pages <= 0) return false;
+    const cuuint32_t halves = (cuuint32_t)head_dim / 64;
+    *fold = stride_head == 16 * stride_token ? 1 : stride_page == 16 * stride_token ? 2 : 0;
+    const cuuint64_t tok = (cuuint64_t)stride_token * 2, hd = (cuuint64_t)stride_head * 2, pg = (cuuint64_t)stride_page * 2;
+    const cuuint64_t dims[5] = {64, *fold ? 8u : 16u, halves, (cuuint64_t)H * (*fold == 1 ? 2 : 1), (cuuint64_t)num_pages * (*fold == 2 ? 2 : 1)};
+    const cuuint64_t strides[4] = {tok, 128, *fold == 1 ? 8 * tok : hd, *fold == 2 ? 8 * tok : pg};
+    const cuuint32_t box[5] = {64, 8, halves, *fold == 1 ? 2u : 1u, *fold == 2 ? 2u : 1u};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, const_cast<void*>(pool),
+              dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Packed rows k_new / v_new [T][H][d] as (column of a half, row, half, head), read in boxes of box_rows rows and box_halves
+// column halves of one head.
+inline bool tma_encode_new_map(CUtensorMap* map, bool bf16, const void* base, int T, int H, int head_dim, int box_rows, int box_halves) {
+    EncodeTiledFn fn = tma_encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[4] = {64, (cuuint64_t)T, (cuuint64_t)head_dim / 64, (cuuint64_t)H};
+    const cuuint64_t strides[3] = {(cuuint64_t)H * head_dim * 2, 128, (cuuint64_t)head_dim * 2};
+    const cuuint32_t box[4] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_halves, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(base),
+              dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // The query rows [T][H][d] as a 3-D tensor (column, head, row) read in boxes of 64 columns x 128 rows of one head.
 inline bool tma_encode_q_map(CUtensorMap* map, bool bf16, const void* q, int T, int H, int head_dim) {
     EncodeTiledFn fn = tma_encode_fn();
