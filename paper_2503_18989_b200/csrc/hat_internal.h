@@ -209,6 +209,8 @@ struct PlanRes {
     cudaEvent_t ev_verify = nullptr;   // recorded in every attention call once the streaming-class rows are final
     cudaEvent_t ev_done = nullptr;     // recorded at the end of every attention call: the next call on another stream waits for it
     cudaEvent_t ev_table = nullptr;    // orders calls on other streams behind the kernel that filled the (cos, sin) table
+    cudaStream_t copy_in = nullptr, copy_out = nullptr;   // of a plan that takes host buffers, made on its first such call
+    cudaEvent_t ev_copy = nullptr;
     bool in_use = false;               // the last owner's work may still run: ready once ev_done has occurred
 };
 }  // namespace hat
@@ -246,11 +248,16 @@ struct hat_plan {
     long long wait_cycles;      // bound of device-side waits (default: about a second)
     int withhold_next;          // self test of the bounded waits: applies to the next attention call only
     hat::MapCache maps;         // see MapCache (updated through const_cast by the launchers: one call at a time per plan)
-    // rotary position encoding in the projection epilogue: (cos, sin) of every row and pair for base rope_theta
+    // rotary position encoding: (cos, sin) of every row and pair for base rope_theta
     // (0: not filled yet), inside the plan's device memory
     float2* rope_table;
     float rope_theta;
     cudaStream_t table_stream;
+    std::vector<hat_plan*> parts;   // plans of contiguous requests for calls with host buffers (host_step.cu), made on the first one
+    std::vector<int32_t> part_row;  // first packed row of each
+    bool parts_made;
+    bool is_part;                   // one of them: its device memory and events are its owner's part_res
+    hat::PlanRes part_res;
     hat::PlanRes res;           // device memory holding every device array, and the plan's events
     // which work that uses `res` ev_done does not cover (see plan_note_call): decides whether it can be handed on
     bool captured;              // a call was captured into a graph, which may be replayed at any time
@@ -268,6 +275,9 @@ cudaError_t launch_attn_mma(const hat_plan* plan, const AttnArgs& args, bool ver
 // the V rows copied beside them
 cudaError_t launch_rope(const hat_plan* plan, int heads, float theta, int interleaved, const void* src, void* dst,
                         const CacheView* cache, void* k_pool, void* v_pool, const void* v_new, cudaStream_t stream);
+// the plan's table of (cos, sin) per row and pair for base theta, filled if it holds none; holding another base, it is
+// replaced or (replace = false) *table stays null
+cudaError_t plan_rope_table(const hat_plan* plan, float theta, cudaStream_t stream, bool replace, const float2** table);
 cudaError_t launch_merge(const hat_plan* plan, const AttnArgs& args, int first_row, int num_rows, cudaStream_t stream);
 // tcgen05 tile kernel (head_dim 64 or 128): whether a TMA descriptor can be built for this pool layout, and the launcher
 bool tc5_layout_supported(int dtype, int head_dim, int num_pages, int H, int64_t stride_page, int64_t stride_token,
@@ -292,8 +302,20 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, PlanRes* out);
 struct UploadPart { const void* src; size_t bytes, off; };
 cudaError_t plan_res_upload(PlanRes& r, const UploadPart* parts, size_t num_parts, size_t bytes);   // complete on return
 cudaError_t plan_res_release(PlanRes& r, bool reusable);    // reusable: ev_done covers every use, or there was none
+cudaError_t plan_res_copy_streams(PlanRes& r);              // makes copy_in, copy_out and ev_copy if they are missing
 cudaError_t plan_res_free(PlanRes& r);
 cudaError_t plan_res_trim();                                // frees what waits for a later plan
+// hat_plan_create; part = true: nothing is uploaded yet (upload_plans does it for several at once); whole = true: no request
+// is cut into key ranges (no workspace)
+int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool part, bool whole, hat_plan** out);
+int upload_plans(hat_plan* const* plans, size_t count, PlanRes* res);
+// One attention step (see hat_api.cu)
+int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new, const void* v_new, float* out, void* out16,
+                  float* lse, float sm_scale, void* workspace, size_t workspace_bytes, cudaStream_t stream, bool check_alignment = true);
+// The step with host buffers; arguments are checked.  HAT_ERR_CUDA: *err holds the error.
+struct HostBuffers { const void *q, *k, *v; void *out, *lse; };
+int host_step(const hat_cache_desc* cache, const hat_plan* plan, const HostBuffers& host, const HostBuffers& dev, float sm_scale,
+              void* workspace, size_t workspace_bytes, cudaStream_t s, cudaError_t* err);
 void plan_note_call(hat_plan* p, cudaStream_t s);           // a call other than attention is about to use the plan on s
 void count_launch(int n = 1);
 #ifdef __CUDACC__

@@ -115,19 +115,6 @@ __device__ __forceinline__ void store32(unsigned char* dst, const float* v) {
     }
 }
 
-// (cos, sin) of every row and pair: trig[t][c], position of row t = prefix_len[r] + (t - cu_chunk[r])
-__global__ void __launch_bounds__(256) rope_table_kernel(DevicePlan plan, int half, const __grid_constant__ InvFreq fr,
-                                                         float2* __restrict__ trig) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)plan.total_rows * half) return;
-    const int t = (int)(idx / half), c = (int)(idx - (int64_t)t * half);
-    const int r = plan.row_req[t];
-    const int p = plan.prefix_len[r] + (t - plan.cu_chunk[r]);
-    float s, co;
-    rope_sincos(p, fr.f[c], &s, &co);
-    trig[idx] = make_float2(co, s);
-}
-
 // One output row of one tile: the thread's TMEM lane of the accumulator at `acc`, packed row t, feature tile n.
 template <bool BF16, int kTileN>
 __device__ __forceinline__ void epilogue_row(const QkvArgs& a, uint32_t acc, int t, int n, int32_t* status) {
@@ -454,39 +441,7 @@ cudaError_t launch_qkv_gemm(const hat_plan* plan, const CacheView& cache, void* 
     const_cast<hat_plan*>(plan)->withhold_next = 0;
     cudaError_t e;
     if (theta > 0.f) {
-        // the table of cosines and sines depends on the plan's positions and on the base only: every layer of a step
-        // uses the one its first call filled
-        hat_plan* mp = const_cast<hat_plan*>(plan);
-        // Inside a stream capture nothing runs now: the fill becomes part of the captured graph (every replay refills the
-        // table, which is harmless) and the plan does not take the table as filled.
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if ((e = cudaStreamIsCapturing(stream, &cap)) != cudaSuccess) return e;
-        const bool capturing = cap != cudaStreamCaptureStatusNone;
-        if (capturing) {
-            InvFreq fr;
-            for (int c = 0; c < 64; ++c) fr.f[c] = c < d / 2 ? std::pow((double)theta, -2.0 * c / d) : 0.0;
-            const int64_t total = (int64_t)T * (d / 2);
-            rope_table_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(plan->dev, d / 2, fr, mp->rope_table);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            mp->rope_theta = 0.f;                // whoever calls next outside a capture fills it for itself
-        } else if (mp->rope_theta != theta) {
-            InvFreq fr;
-            for (int c = 0; c < 64; ++c) fr.f[c] = c < d / 2 ? std::pow((double)theta, -2.0 * c / d) : 0.0;
-            const int64_t total = (int64_t)T * (d / 2);
-            // a call with the previous base may still be reading the table that is about to be replaced (rare: one
-            // model has one base)
-            if (mp->rope_theta > 0.f && (e = cudaDeviceSynchronize()) != cudaSuccess) return e;
-            rope_table_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(plan->dev, d / 2, fr, mp->rope_table);
-            count_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if ((e = cudaEventRecord(mp->res.ev_table, stream)) != cudaSuccess) return e;
-            mp->rope_theta = theta;
-            mp->table_stream = stream;
-        } else if (mp->table_stream != stream) {
-            if ((e = cudaStreamWaitEvent(stream, mp->res.ev_table, 0)) != cudaSuccess) return e;
-        }
-        a.trig = mp->rope_table;
+        if ((e = plan_rope_table(plan, theta, stream, /*replace=*/true, &a.trig)) != cudaSuccess) return e;
     }
     if (pair) e = bf16 ? launch_form<true, true>(a, mx, mw, plan->num_sms, stream) : launch_form<false, true>(a, mx, mw, plan->num_sms, stream);
     else e = bf16 ? launch_form<true, false>(a, mx, mw, plan->num_sms, stream) : launch_form<false, false>(a, mx, mw, plan->num_sms, stream);
