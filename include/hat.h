@@ -286,8 +286,11 @@ int hat_chunk_attention_out16(const hat_cache_desc* cache, const hat_plan* plan,
 /*
  * The same step for a caller whose activations live in HOST memory (pinned
  * memory makes the copies asynchronous).  Copies q, k_new, v_new to `staging`,
- * appends, attends, copies out and lse back, all on `stream`, and returns
- * without synchronising: the host results are valid once the stream is.
+ * appends, attends, copies out and lse back, all in `stream`'s order, and
+ * returns without synchronising: the host results are valid once the stream is.
+ * A large batch is processed in parts (contiguous requests) so that copies and
+ * kernels overlap, on two more streams that the plan keeps; the first such call
+ * plans the parts.
  *   q_host, k_new_host, v_new_host   host [T][heads][head_dim] 16-bit
  *   out_host [T][heads][head_dim], lse_host [T][heads]   host fp32
  *   staging        device, 256-byte aligned, >= hat_plan_staging_bytes

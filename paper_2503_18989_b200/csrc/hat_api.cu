@@ -284,7 +284,7 @@ static int pick_verify_split(const hat_plan* p, int num_sms) {
 
 // tile_kernel: 0 = mma.sync, 1 = tcgen05 with two query tiles per CTA, 3 = tcgen05 by pairs of CTAs (cta_group::2) with a
 // ring of three score buffers; both tcgen05 kernels take 256-row units
-static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
+static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
     const bool use_tc5 = tile_kernel != 0;
     const int H = p->num_heads;
     const int R = p->num_requests;
@@ -313,7 +313,8 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
     const bool stream_tma = info.stream_kernel == 1;
     p->verify_subtiles = std::max(1, ceil_div(max_verify_rows * group, 16));
     int vsplit = env_int("HAT_VERIFY_SPLIT_LEN", 0);
-    if (vsplit <= 0) vsplit = pick_verify_split(p, num_sms);
+    if (whole) vsplit = 1 << 24;
+    else if (vsplit <= 0) vsplit = pick_verify_split(p, num_sms);
     vsplit = std::max(kPageSize, round_up(vsplit, kPageSize));
     info.verify_split_len = vsplit;
 
@@ -327,7 +328,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
             tile_keys += p->prefix_len[r] + std::min(C, row0 + tile_rows);
         }
     }
-    int psplit = env_int("HAT_PREFILL_SPLIT_LEN", -1);
+    int psplit = whole ? 0 : env_int("HAT_PREFILL_SPLIT_LEN", -1);
     if (psplit < 0) {
         psplit = 0;
         const int64_t want_ctas = (int64_t)num_sms * 2;
@@ -420,56 +421,72 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel) {
     info.workspace_bytes = p->part_rows ? part_out_bytes + ((p->part_rows * H * 4 + 255) / 256 * 256) : 0;
 }
 
-static int upload(hat_plan* p) {
-    // the arrays, each at a 256-byte boundary
+int upload_plans(hat_plan* const* plans, size_t count, PlanRes* res) {
+    // the arrays of all plans, each at a 256-byte boundary, go over in one copy
+    struct Offsets { size_t cu, pl, cl, bt, rr, vi, si, pi, mr, tu, tm, st, table; };
+    std::vector<Offsets> at(count);
     std::vector<UploadPart> parts;
-    size_t bytes = 0;
-    auto add = [&](const auto& v) {
-        const size_t off = (bytes + 255) / 256 * 256, n = v.size() * sizeof(v[0]);
-        parts.push_back(UploadPart{v.data(), n, off});
+    size_t bytes = 0, most_status = 0;
+    // status word; (unit counter, finished CTAs) of the tile kernel, of a second tile grid, of the streaming kernel; spare;
+    // finished pieces of the requests the streaming kernel merges
+    for (size_t i = 0; i < count; ++i) {
+        plans[i]->num_status_words = 8 + plans[i]->num_piece_counters;
+        most_status = std::max(most_status, (size_t)plans[i]->num_status_words);
+    }
+    const std::vector<int32_t> status(most_status, 0);
+    auto place = [&](const void* src, size_t n) {
+        const size_t off = (bytes + 255) / 256 * 256;
+        parts.push_back(UploadPart{src, n, off});
         bytes = off + std::max<size_t>(n, 16);
         return off;
     };
-    const size_t o_cu = add(p->cu_chunk), o_pl = add(p->prefix_len), o_cl = add(p->chunk_len), o_bt = add(p->block_table);
-    const size_t o_rr = add(p->row_req), o_vi = add(p->verify_items), o_si = add(p->stream_items), o_pi = add(p->prefill_items), o_mr = add(p->merge_rows);
-    const size_t o_tu = add(p->tile_units), o_tm = add(p->tree_mask);
-    // status word; (unit counter, finished CTAs) of the tile kernel, of a second tile grid, of the streaming kernel; spare;
-    // finished pieces of the requests the streaming kernel merges
-    p->num_status_words = 8 + p->num_piece_counters;
-    const std::vector<int32_t> status(p->num_status_words, 0);
-    const size_t o_st = add(status);
-
-    cudaError_t e = cudaGetDevice(&p->device);
+    auto add = [&](const auto& v) { return place(v.data(), v.size() * sizeof(v[0])); };
+    for (size_t i = 0; i < count; ++i) {
+        const hat_plan* p = plans[i];
+        at[i] = Offsets{add(p->cu_chunk), add(p->prefix_len), add(p->chunk_len), add(p->block_table), add(p->row_req), add(p->verify_items),
+                        add(p->stream_items), add(p->prefill_items), add(p->merge_rows), add(p->tile_units), add(p->tree_mask),
+                        place(status.data(), p->num_status_words * sizeof(int32_t)), 0};
+    }
+    // behind the arrays: room for the (cos, sin) table of rotation and projection, filled on the device when first used
+    size_t total = bytes;
+    for (size_t i = 0; i < count; ++i) {
+        at[i].table = (total + 255) / 256 * 256;
+        total = at[i].table + (plans[i]->is_part ? 0 : std::max<size_t>((size_t)plans[i]->total_rows * (plans[i]->head_dim / 2) * sizeof(float2), 16));
+    }
+    int device = -1;
+    cudaError_t e = cudaGetDevice(&device);
     if (e != cudaSuccess) return cuda_fail(e);
-    // behind the arrays: room for the (cos, sin) table of the projection epilogue, filled on the device when first used
-    const size_t o_table = (bytes + 255) / 256 * 256;
-    const size_t table_bytes = (size_t)p->total_rows * (p->head_dim / 2) * sizeof(float2);
-    e = plan_res_acquire(p->device, o_table + std::max<size_t>(table_bytes, 16), &p->res);
+    e = plan_res_acquire(device, total, res);
     if (e != cudaSuccess) return cuda_fail(e);
-    e = plan_res_upload(p->res, parts.data(), parts.size(), bytes);
+    e = plan_res_upload(*res, parts.data(), parts.size(), bytes);
     if (e != cudaSuccess) return cuda_fail(e);
-    char* base = static_cast<char*>(p->res.blob);
-    p->rope_table = reinterpret_cast<float2*>(base + o_table);
-    DevicePlan& d = p->dev;
-    d.cu_chunk = reinterpret_cast<const int32_t*>(base + o_cu);
-    d.prefix_len = reinterpret_cast<const int32_t*>(base + o_pl);
-    d.chunk_len = reinterpret_cast<const int32_t*>(base + o_cl);
-    d.block_table = reinterpret_cast<const int32_t*>(base + o_bt);
-    d.row_req = reinterpret_cast<const int32_t*>(base + o_rr);
-    d.verify_items = reinterpret_cast<const WorkItem*>(base + o_vi);
-    d.stream_items = reinterpret_cast<const StreamItem*>(base + o_si);
-    d.prefill_items = reinterpret_cast<const WorkItem*>(base + o_pi);
-    d.merge_rows = reinterpret_cast<const MergeRow*>(base + o_mr);
-    d.tile_units = reinterpret_cast<const uint32_t*>(base + o_tu);
-    d.status = reinterpret_cast<int32_t*>(base + o_st);
-    d.piece_counters = d.status + 8;
-    d.max_pages = p->max_pages;
-    d.tree_mask = p->tree_mask.empty() ? nullptr : reinterpret_cast<const uint32_t*>(base + o_tm);
-    d.num_heads = p->num_heads;
-    d.num_kv_heads = p->num_kv_heads;
-    d.group = p->num_heads / p->num_kv_heads;
-    d.total_rows = p->total_rows;
-    d.num_pages = p->num_pages;
+    char* base = static_cast<char*>(res->blob);
+    for (size_t i = 0; i < count; ++i) {
+        hat_plan* p = plans[i];
+        const Offsets& o = at[i];
+        p->device = device;
+        p->rope_table = p->is_part ? nullptr : reinterpret_cast<float2*>(base + o.table);
+        DevicePlan& d = p->dev;
+        d.cu_chunk = reinterpret_cast<const int32_t*>(base + o.cu);
+        d.prefix_len = reinterpret_cast<const int32_t*>(base + o.pl);
+        d.chunk_len = reinterpret_cast<const int32_t*>(base + o.cl);
+        d.block_table = reinterpret_cast<const int32_t*>(base + o.bt);
+        d.row_req = reinterpret_cast<const int32_t*>(base + o.rr);
+        d.verify_items = reinterpret_cast<const WorkItem*>(base + o.vi);
+        d.stream_items = reinterpret_cast<const StreamItem*>(base + o.si);
+        d.prefill_items = reinterpret_cast<const WorkItem*>(base + o.pi);
+        d.merge_rows = reinterpret_cast<const MergeRow*>(base + o.mr);
+        d.tile_units = reinterpret_cast<const uint32_t*>(base + o.tu);
+        d.status = reinterpret_cast<int32_t*>(base + o.st);
+        d.piece_counters = d.status + 8;
+        d.max_pages = p->max_pages;
+        d.tree_mask = p->tree_mask.empty() ? nullptr : reinterpret_cast<const uint32_t*>(base + o.tm);
+        d.num_heads = p->num_heads;
+        d.num_kv_heads = p->num_kv_heads;
+        d.group = p->num_heads / p->num_kv_heads;
+        d.total_rows = p->total_rows;
+        d.num_pages = p->num_pages;
+    }
     return HAT_OK;
 }
 
@@ -490,32 +507,7 @@ static CacheView view_of(const hat_cache_desc* c) {
     return CacheView{c->k_pool, c->v_pool, c->stride_page, c->stride_token, c->stride_head};
 }
 
-}  // namespace hat
-
-using namespace hat;
-
-extern "C" {
-
-const char* hat_status_string(int status) {
-    switch (status) {
-        case HAT_OK: return "ok";
-        case HAT_ERR_INVALID_ARG: return "invalid argument";
-        case HAT_ERR_UNSUPPORTED: return "unsupported configuration";
-        case HAT_ERR_OUT_OF_RANGE: return "index out of range";
-        case HAT_ERR_WORKSPACE_TOO_SMALL: return "workspace too small";
-        case HAT_ERR_CUDA: return "CUDA error";
-        case HAT_ERR_DEVICE_TIMEOUT: return "device-side wait timed out";
-        case HAT_ERR_TOO_LARGE: return "size exceeds a fixed maximum";
-        case HAT_ERR_DEVICE_BOUNDS: return "device-side index check failed (debug build)";
-        default: return "unknown status";
-    }
-}
-
-int hat_version(void) { return HAT_VERSION; }
-int hat_last_cuda_error(void) { return g_last_cuda_error; }
-int64_t hat_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
-
-int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, hat_plan** out) {
+int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool part, bool whole, hat_plan** out) {
     if (!out) return HAT_ERR_INVALID_ARG;
     *out = nullptr;
     if (!cache || !batch) return HAT_ERR_INVALID_ARG;
@@ -583,6 +575,8 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
     p->append_first = append_first;
     p->num_piece_counters = 0;
     p->num_verify_merge_rows = 0;
+    p->parts_made = false;
+    p->is_part = part;
     p->captured = p->loose = p->loose_many = false;
     p->loose_stream = nullptr;
     p->rope_table = nullptr;
@@ -670,7 +664,7 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
         stream_tma = stream_layout_supported(p->dtype, p->head_dim, p->num_pages, p->num_kv_heads, cache->stride_page,
                                              cache->stride_token, cache->stride_head);
     p->info.stream_kernel = stream_tma ? 1 : 0;
-    schedule(p, num_sms, tile_kernel);
+    schedule(p, num_sms, tile_kernel, whole);
     // launch-geometry limits: work items index gridDim.y (65535), partial rows and units are 32-bit
     const int64_t verify_count = (int64_t)(p->verify_items.size() + p->stream_items.size());
     if (verify_count > 65535 || verify_count * p->num_kv_heads * p->verify_subtiles > INT32_MAX / 2 || p->prefill_items.size() > 65535 || p->num_heads > 65535 ||
@@ -680,7 +674,8 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
     }
 
     if (!p->host_only) {
-        st = upload(p);
+        if (part) { *out = p; return HAT_OK; }               // uploaded with the others
+        st = upload_plans(&p, 1, &p->res);
         if (st != HAT_OK) { hat_plan_destroy(p); return st; }
         // Optional throughput mode for a mixed batch on the tcgen05 path (HAT_SIDE_SMS = n > 0): see the launch
         // sequence.  Off by default: it finishes the whole step sooner but the decode-phase rows later.  The side
@@ -704,106 +699,17 @@ int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, ha
     return HAT_OK;
 }
 
-int hat_plan_get_info(const hat_plan* plan, hat_plan_info* out) {
-    if (!plan || !out) return HAT_ERR_INVALID_ARG;
-    *out = plan->info;
-    return HAT_OK;
-}
-
-int hat_plan_workspace_bytes(const hat_plan* plan, size_t* out) {
-    if (!plan || !out) return HAT_ERR_INVALID_ARG;
-    *out = (size_t)plan->info.workspace_bytes;
-    return HAT_OK;
-}
-
-int hat_plan_destroy(hat_plan* plan) {
-    if (!plan) return HAT_OK;
-    int st = HAT_OK;
-    if (plan->timing) {
-        for (cudaEvent_t ev : plan->timing->events) cudaEventDestroy(ev);
-        delete plan->timing;
-    }
-    if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
-    if (plan->ev_join) cudaEventDestroy(plan->ev_join);
-    if (plan->aux_stream) cudaStreamDestroy(plan->aux_stream);
-    if (!plan->host_only) {
-        // handed on to a later plan unless a graph may replay a call, or work that ev_done does not cover may still run
-        plan->res.in_use = plan->has_last;
-        const cudaError_t e = plan_res_release(plan->res, !plan->captured && !plan->loose);
-        if (e != cudaSuccess) st = cuda_fail(e);
-    }
-    delete plan;
-    return st;
-}
-
-int hat_release_cached(void) {
-    const cudaError_t e = plan_res_trim();
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
-}
-
-int hat_kv_append(const hat_cache_desc* cache, const hat_plan* plan, const void* k_new, const void* v_new,
-                  void* stream) {
-    int st = check_call(cache, plan);
-    if (st != HAT_OK) return st;
-    if (plan->total_rows == 0) return HAT_OK;
-    if (!k_new || !v_new || !aligned(k_new, 16) || !aligned(v_new, 16)) return HAT_ERR_INVALID_ARG;
-    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
-    cudaError_t e = launch_kv_append(plan, view_of(cache), cache->k_pool, cache->v_pool, k_new, v_new,
-                                     static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
-}
-
-int hat_kv_append_rope(const hat_cache_desc* cache, const hat_plan* plan, const void* k_new, const void* v_new,
-                       float theta, int interleaved, void* stream) {
-    int st = check_call(cache, plan);
-    if (st != HAT_OK) return st;
-    if (!(theta > 1.f) || !std::isfinite(theta)) return HAT_ERR_INVALID_ARG;
-    if (plan->total_rows == 0) return HAT_OK;
-    if (!k_new || !v_new || !aligned(k_new, 16) || !aligned(v_new, 16)) return HAT_ERR_INVALID_ARG;
-    const CacheView view = view_of(cache);
-    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
-    cudaError_t e = launch_rope(plan, plan->num_kv_heads, theta, interleaved != 0, k_new, nullptr, &view, cache->k_pool,
-                                cache->v_pool, v_new, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
-}
-
-int hat_rope_q(const hat_plan* plan, const void* q, void* q_out, float theta, int interleaved, void* stream) {
-    if (!plan || plan->host_only) return HAT_ERR_INVALID_ARG;
-    if (!(theta > 1.f) || !std::isfinite(theta)) return HAT_ERR_INVALID_ARG;
-    if (plan->total_rows == 0) return HAT_OK;
-    if (!q || !q_out || !aligned(q, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
-    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
-    cudaError_t e = launch_rope(plan, plan->num_heads, theta, interleaved != 0, q, q_out, nullptr, nullptr, nullptr, nullptr,
-                                static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
-}
-
-int hat_qkv_rope_append(const hat_cache_desc* cache, const hat_plan* plan, const void* x, int hidden, const void* w_qkv,
-                        void* q_out, float theta, int interleaved, void* stream) {
-    int st = check_call(cache, plan);
-    if (st != HAT_OK) return st;
-    if (theta > 0.f && (!(theta > 1.f) || !std::isfinite(theta))) return HAT_ERR_INVALID_ARG;
-    if (hidden <= 0) return HAT_ERR_INVALID_ARG;
-    if (hidden % 64 != 0 || (plan->head_dim != 64 && plan->head_dim != 128)) return HAT_ERR_UNSUPPORTED;
-    if (plan->total_rows == 0) return HAT_OK;
-    if (!x || !w_qkv || !q_out || !aligned(x, 16) || !aligned(w_qkv, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
-    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
-    cudaError_t e = launch_qkv_gemm(plan, view_of(cache), cache->k_pool, cache->v_pool, x, hidden, w_qkv, q_out, theta,
-                                    interleaved != 0, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
-}
-
 // One attention step; the final rows go to `out` (fp32) or, when out16 is given, to out16 in the cache's 16-bit type.
-static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
+int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
                          const void* v_new, float* out, void* out16, float* lse, float sm_scale, void* workspace,
-                         size_t workspace_bytes, void* stream) {
+                         size_t workspace_bytes, cudaStream_t s, bool check_alignment) {
     int st = check_call(cache, plan);
     if (st != HAT_OK) return st;
     if ((k_new == nullptr) != (v_new == nullptr)) return HAT_ERR_INVALID_ARG;
     if (plan->total_rows == 0) return HAT_OK;
     const void* dst = out16 ? out16 : static_cast<const void*>(out);
     if (!q || !dst || !lse) return HAT_ERR_INVALID_ARG;
-    if (!aligned(q, 16) || !aligned(dst, 16) || !aligned(lse, 16)) return HAT_ERR_INVALID_ARG;
+    if (check_alignment && (!aligned(q, 16) || !aligned(dst, 16) || !aligned(lse, 16))) return HAT_ERR_INVALID_ARG;
     if (k_new && (!aligned(k_new, 16) || !aligned(v_new, 16))) return HAT_ERR_INVALID_ARG;
     const size_t need = (size_t)plan->info.workspace_bytes;
     if (need > 0) {
@@ -812,7 +718,6 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     }
     if (!(sm_scale > 0.f) || !std::isfinite(sm_scale)) sm_scale = 1.0f / std::sqrt((float)plan->head_dim);
 
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e;
     // The plan's device state (unit counter, status word) serves one call at a time: a call on another stream than the
     // previous one is ordered behind it.
@@ -929,19 +834,146 @@ static int run_attention(const hat_cache_desc* cache, const hat_plan* plan, cons
     return HAT_OK;
 }
 
+}  // namespace hat
+
+using namespace hat;
+
+extern "C" {
+
+const char* hat_status_string(int status) {
+    switch (status) {
+        case HAT_OK: return "ok";
+        case HAT_ERR_INVALID_ARG: return "invalid argument";
+        case HAT_ERR_UNSUPPORTED: return "unsupported configuration";
+        case HAT_ERR_OUT_OF_RANGE: return "index out of range";
+        case HAT_ERR_WORKSPACE_TOO_SMALL: return "workspace too small";
+        case HAT_ERR_CUDA: return "CUDA error";
+        case HAT_ERR_DEVICE_TIMEOUT: return "device-side wait timed out";
+        case HAT_ERR_TOO_LARGE: return "size exceeds a fixed maximum";
+        case HAT_ERR_DEVICE_BOUNDS: return "device-side index check failed (debug build)";
+        default: return "unknown status";
+    }
+}
+
+int hat_version(void) { return HAT_VERSION; }
+int hat_last_cuda_error(void) { return g_last_cuda_error; }
+int64_t hat_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
+
+int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, hat_plan** out) {
+    return create_plan(cache, batch, /*part=*/false, /*whole=*/false, out);
+}
+
+int hat_plan_get_info(const hat_plan* plan, hat_plan_info* out) {
+    if (!plan || !out) return HAT_ERR_INVALID_ARG;
+    *out = plan->info;
+    return HAT_OK;
+}
+
+int hat_plan_workspace_bytes(const hat_plan* plan, size_t* out) {
+    if (!plan || !out) return HAT_ERR_INVALID_ARG;
+    *out = (size_t)plan->info.workspace_bytes;
+    return HAT_OK;
+}
+
+int hat_plan_destroy(hat_plan* plan) {
+    if (!plan) return HAT_OK;
+    int st = HAT_OK;
+    if (plan->timing) {
+        for (cudaEvent_t ev : plan->timing->events) cudaEventDestroy(ev);
+        delete plan->timing;
+    }
+    if (!plan->parts.empty()) {
+        bool covered = true;                                 // by the parts' common ev_done
+        for (hat_plan* part : plan->parts) {
+            plan->part_res.in_use |= part->has_last;
+            covered &= !part->captured && !part->loose;
+            delete part;
+        }
+        const cudaError_t e = plan_res_release(plan->part_res, covered);
+        if (e != cudaSuccess) st = cuda_fail(e);
+    }
+    if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
+    if (plan->ev_join) cudaEventDestroy(plan->ev_join);
+    if (plan->aux_stream) cudaStreamDestroy(plan->aux_stream);
+    if (!plan->host_only) {
+        // handed on to a later plan unless a graph may replay a call, or work that ev_done does not cover may still run
+        plan->res.in_use = plan->has_last;
+        const cudaError_t e = plan_res_release(plan->res, !plan->captured && !plan->loose);
+        if (e != cudaSuccess) st = cuda_fail(e);
+    }
+    delete plan;
+    return st;
+}
+
+int hat_release_cached(void) {
+    const cudaError_t e = plan_res_trim();
+    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+}
+
+int hat_kv_append(const hat_cache_desc* cache, const hat_plan* plan, const void* k_new, const void* v_new,
+                  void* stream) {
+    int st = check_call(cache, plan);
+    if (st != HAT_OK) return st;
+    if (plan->total_rows == 0) return HAT_OK;
+    if (!k_new || !v_new || !aligned(k_new, 16) || !aligned(v_new, 16)) return HAT_ERR_INVALID_ARG;
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_kv_append(plan, view_of(cache), cache->k_pool, cache->v_pool, k_new, v_new,
+                                     static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+}
+
+int hat_kv_append_rope(const hat_cache_desc* cache, const hat_plan* plan, const void* k_new, const void* v_new,
+                       float theta, int interleaved, void* stream) {
+    int st = check_call(cache, plan);
+    if (st != HAT_OK) return st;
+    if (!(theta > 1.f) || !std::isfinite(theta)) return HAT_ERR_INVALID_ARG;
+    if (plan->total_rows == 0) return HAT_OK;
+    if (!k_new || !v_new || !aligned(k_new, 16) || !aligned(v_new, 16)) return HAT_ERR_INVALID_ARG;
+    const CacheView view = view_of(cache);
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_rope(plan, plan->num_kv_heads, theta, interleaved != 0, k_new, nullptr, &view, cache->k_pool,
+                                cache->v_pool, v_new, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+}
+
+int hat_rope_q(const hat_plan* plan, const void* q, void* q_out, float theta, int interleaved, void* stream) {
+    if (!plan || plan->host_only) return HAT_ERR_INVALID_ARG;
+    if (!(theta > 1.f) || !std::isfinite(theta)) return HAT_ERR_INVALID_ARG;
+    if (plan->total_rows == 0) return HAT_OK;
+    if (!q || !q_out || !aligned(q, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_rope(plan, plan->num_heads, theta, interleaved != 0, q, q_out, nullptr, nullptr, nullptr, nullptr,
+                                static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+}
+
+int hat_qkv_rope_append(const hat_cache_desc* cache, const hat_plan* plan, const void* x, int hidden, const void* w_qkv,
+                        void* q_out, float theta, int interleaved, void* stream) {
+    int st = check_call(cache, plan);
+    if (st != HAT_OK) return st;
+    if (theta > 0.f && (!(theta > 1.f) || !std::isfinite(theta))) return HAT_ERR_INVALID_ARG;
+    if (hidden <= 0) return HAT_ERR_INVALID_ARG;
+    if (hidden % 64 != 0 || (plan->head_dim != 64 && plan->head_dim != 128)) return HAT_ERR_UNSUPPORTED;
+    if (plan->total_rows == 0) return HAT_OK;
+    if (!x || !w_qkv || !q_out || !aligned(x, 16) || !aligned(w_qkv, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
+    plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_qkv_gemm(plan, view_of(cache), cache->k_pool, cache->v_pool, x, hidden, w_qkv, q_out, theta,
+                                    interleaved != 0, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+}
 
 int hat_chunk_attention(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
                         const void* v_new, float* out, float* lse, float sm_scale, void* workspace,
                         size_t workspace_bytes, void* stream) {
     if (!out && plan && plan->total_rows > 0) return HAT_ERR_INVALID_ARG;
-    return run_attention(cache, plan, q, k_new, v_new, out, nullptr, lse, sm_scale, workspace, workspace_bytes, stream);
+    return run_attention(cache, plan, q, k_new, v_new, out, nullptr, lse, sm_scale, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
 }
 
 int hat_chunk_attention_out16(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
                               const void* v_new, void* out16, float* lse, float sm_scale, void* workspace,
                               size_t workspace_bytes, void* stream) {
     if (!out16 && plan && plan->total_rows > 0) return HAT_ERR_INVALID_ARG;
-    return run_attention(cache, plan, q, k_new, v_new, nullptr, out16, lse, sm_scale, workspace, workspace_bytes, stream);
+    return run_attention(cache, plan, q, k_new, v_new, nullptr, out16, lse, sm_scale, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
 }
 
 int hat_plan_verify_event(const hat_plan* plan, void** event_out) {
@@ -1026,8 +1058,12 @@ int hat_chunk_attention_host(const hat_cache_desc* cache, const hat_plan* plan, 
     hat_plan_staging_bytes(plan, &need);
     if (!staging || !aligned(staging, 256)) return HAT_ERR_INVALID_ARG;
     if (staging_bytes < need) return HAT_ERR_WORKSPACE_TOO_SMALL;
+    if (plan->info.workspace_bytes > 0) {
+        if (!workspace || !aligned(workspace, 256)) return HAT_ERR_INVALID_ARG;
+        if (workspace_bytes < (size_t)plan->info.workspace_bytes) return HAT_ERR_WORKSPACE_TOO_SMALL;
+    }
     const size_t T = plan->total_rows, H = plan->num_heads, Hkv = plan->num_kv_heads, d = plan->head_dim;
-    const size_t act_bytes = T * H * d * 2, kv_bytes = T * Hkv * d * 2, out_bytes = T * H * d * 4, lse_bytes = T * H * 4;
+    const size_t act_bytes = T * H * d * 2, kv_bytes = T * Hkv * d * 2, out_bytes = T * H * d * 4;
     const size_t q16 = (act_bytes + 255) / 256 * 256, kv16 = (kv_bytes + 255) / 256 * 256, out32 = (out_bytes + 255) / 256 * 256;
     char* base = static_cast<char*>(staging);
     void* dq = base;
@@ -1035,16 +1071,10 @@ int hat_chunk_attention_host(const hat_cache_desc* cache, const hat_plan* plan, 
     void* dv = base + q16 + kv16;
     float* dout = reinterpret_cast<float*>(base + q16 + 2 * kv16);
     float* dlse = reinterpret_cast<float*>(base + q16 + 2 * kv16 + out32);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(dq, q_host, act_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(dk, k_new_host, kv_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(dv, v_new_host, kv_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail(e);
-    st = hat_chunk_attention(cache, plan, dq, dk, dv, dout, dlse, sm_scale, workspace, workspace_bytes, stream);
-    if (st != HAT_OK) return st;
-    if ((e = cudaMemcpyAsync(out_host, dout, out_bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(lse_host, dlse, lse_bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e);
-    return HAT_OK;
+    cudaError_t e = cudaSuccess;
+    st = host_step(cache, plan, HostBuffers{q_host, k_new_host, v_new_host, out_host, lse_host}, HostBuffers{dq, dk, dv, dout, dlse}, sm_scale,
+                   workspace, workspace_bytes, static_cast<cudaStream_t>(stream), &e);
+    return st == HAT_ERR_CUDA && e != cudaSuccess ? cuda_fail(e) : st;
 }
 
 int hat_last_device_status(const hat_plan* plan, void* stream, int* out) {
@@ -1055,6 +1085,12 @@ int hat_last_device_status(const hat_plan* plan, void* stream, int* out) {
     if (e == cudaSuccess) e = cudaMemsetAsync(plan->dev.status, 0, plan->num_status_words * sizeof word, s);     // status, counters
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e);
+    for (const hat_plan* part : plan->parts) {
+        int st = HAT_OK;
+        const int rc = hat_last_device_status(part, stream, &st);
+        if (rc != HAT_OK) return rc;
+        if (st != HAT_OK) word |= st == HAT_ERR_DEVICE_TIMEOUT ? 1 : 2;
+    }
     *out = word == 0 ? HAT_OK : (word & 1) ? HAT_ERR_DEVICE_TIMEOUT : HAT_ERR_DEVICE_BOUNDS;
     return HAT_OK;
 }

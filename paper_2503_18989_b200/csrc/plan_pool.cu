@@ -48,6 +48,9 @@ cudaError_t plan_res_free(PlanRes& r) {
     if (r.ev_verify) cudaEventDestroy(r.ev_verify);
     if (r.ev_done) cudaEventDestroy(r.ev_done);
     if (r.ev_table) cudaEventDestroy(r.ev_table);
+    if (r.ev_copy) cudaEventDestroy(r.ev_copy);
+    if (r.copy_in) cudaStreamDestroy(r.copy_in);
+    if (r.copy_out) cudaStreamDestroy(r.copy_out);
     if (r.blob) e = cudaFree(r.blob);              // waits for the device, so kernels that still use the plan finish first
     r = PlanRes{};
     return e;
@@ -97,6 +100,14 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, PlanRes* out) {
     if (e != cudaSuccess) { plan_res_free(r); return e; }
     *out = r;
     return cudaSuccess;
+}
+
+cudaError_t plan_res_copy_streams(PlanRes& r) {
+    cudaError_t e = cudaSuccess;
+    for (cudaStream_t* s : {&r.copy_in, &r.copy_out})
+        if (!*s && e == cudaSuccess && (e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking)) != cudaSuccess) *s = nullptr;
+    if (!r.ev_copy && e == cudaSuccess && (e = cudaEventCreateWithFlags(&r.ev_copy, cudaEventDisableTiming)) != cudaSuccess) r.ev_copy = nullptr;
+    return e;
 }
 
 cudaError_t plan_res_release(PlanRes& r, bool reusable) {

@@ -1,0 +1,53 @@
+"""Calls with host buffers that are large enough to be split into parts (copies overlap the kernels)."""
+import numpy as np
+import pytest
+
+from paper_2503_18989_b200 import workloads as W
+
+from common import assert_parity, oracle_replay
+from test_stream_kernel import _batch
+
+pytestmark = pytest.mark.gpu
+
+# heads odd in number, so that the parts' lse rows are not 16-byte aligned; an empty chunk; requests of every class
+_PREFIX = [300, 0, 77, 1000, 16, 640, 5, 129, 900, 33]
+_CHUNK = [400, 3, 512, 16, 129, 0, 300, 7, 256, 200]
+
+
+@pytest.mark.parametrize("dtype,group,tree,pinned", [("fp16", 1, False, True), ("bf16", 2, True, True), ("fp16", 1, False, False)])
+def test_parts_of_a_host_call(cuda_device, dtype, group, tree, pinned):
+    import torch
+    from paper_2503_18989_b200 import binding as B, runner
+    H, d = 5, 128
+    sc = _batch(dtype, H, d, _PREFIX, _CHUNK, 301, group)
+    st = sc.steps[0]
+    if tree:
+        st.tree_mask = W.random_tree_masks(5, _CHUNK)
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, st)
+    T, Hq = st.total_rows, H * group
+    host = lambda a: torch.from_numpy(a.view(np.int16)).pin_memory() if pinned else torch.from_numpy(a.view(np.int16).copy())
+    q, k, v = host(st.q), host(st.k_new), host(st.v_new)
+    nbytes = B.hat_plan_staging_bytes(ds.plan)
+    streams = [torch.cuda.Stream(cuda_device) for _ in range(2)]
+    sets = []
+    for _ in streams:
+        o, l = torch.full((T, Hq, d), float("nan")), torch.full((T, Hq), float("nan"))
+        sets.append((o.pin_memory() if pinned else o, l.pin_memory() if pinned else l,
+                     torch.empty(nbytes, dtype=torch.uint8, device=cuda_device)))
+    torch.cuda.synchronize()
+    before = B.hat_launch_count()
+    for i in range(6):                                       # alternate streams, two calls in flight
+        o, l, stg = sets[i % 2]
+        B.hat_chunk_attention_host(cache.desc, ds.plan, q, k, v, o, l, 0.0, stg, nbytes, ds.workspace, ds.workspace_bytes,
+                                   streams[i % 2].cuda_stream)
+    assert B.hat_launch_count() - before >= 6 * 4             # several parts, a streaming and a tile kernel in most
+    torch.cuda.synchronize()
+    assert B.hat_last_device_status(ds.plan) == B.HAT_OK
+    kp, vp, want = oracle_replay(sc)
+    for o, l, _ in sets:
+        assert_parity(o.numpy(), want[0][0], "out")
+        assert_parity(l.numpy(), want[0][1], "lse")
+    gk, gv = cache.pools_to_host()
+    assert np.array_equal(gk, kp) and np.array_equal(gv, vp) and ds.canaries_intact()
+    ds.close()
