@@ -163,19 +163,19 @@ def lib() -> C.CDLL:
 
 
 def _check(status: int, where: str) -> None:
-    if status != HAT_OK:
+    if status:                              # HAT_OK is 0
         raise HatError(status, where)
 
 
 def _ptr(x) -> Optional[int]:
     """Raw address of a torch tensor, numpy array, int or None."""
-    if x is None:
-        return None
-    if isinstance(x, int):
+    try:
+        return x.data_ptr()                 # the common case first: this runs six times per call
+    except AttributeError:
+        pass
+    if x is None or isinstance(x, int):
         return x
-    if isinstance(x, np.ndarray):
-        return x.ctypes.data
-    return int(x.data_ptr())
+    return x.ctypes.data
 
 
 def hat_status_string(status: int) -> str:
