@@ -326,8 +326,8 @@ int hat_plan_read_timing(hat_plan* plan, float* ms, int capacity_calls, int* num
  * Inference": long prefills delay the decode requests of the same batch; Sec.
  * 3.3).  hat_chunk_attention computes the streaming-class chunks (draft
  * verification, chunk_len <= 16) first and records an event owned by the plan
- * as soon as their out/lse rows are final, before the tile kernel for the
- * prompt chunks of the same batch starts.
+ * as soon as their out/lse rows are final; the tile kernel for the prompt chunks
+ * of the same batch only takes the SMs that they leave.
  *   hat_plan_verify_event   the cudaEvent_t (as void*), e.g. for cudaStreamWaitEvent on the caller's own stream
  *                           that returns those rows to the devices; it is re-recorded by every attention call
  *   hat_plan_wait_verify    blocks the host until the event of the latest call has occurred

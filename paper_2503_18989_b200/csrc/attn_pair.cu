@@ -307,7 +307,10 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 return at < total_pages ? HAT_IN_RANGE(__ldg(table + at), a.plan.num_pages, cx.status) : 0;
             };
             int page = page_of(0);
-            if (un == 0) { pdl_wait(); pdl_launch_dependents(); }   // up to here only the plan's own arrays were read; the kernel behind may be one that runs beside this one
+            if (un == 0) {
+                if (!a.overlap) pdl_wait();                      // up to here only the plan's own arrays were read
+                pdl_launch_dependents();                         // the kernel behind may be one that runs beside this one
+            }
             if (rank == 0) {
                 // the unit after this one is published before this one's tiles are requested, so that the MMA thread can
                 // run its score tiles ahead across the unit boundary
@@ -441,7 +444,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 return lane < 8 && at < total_pages ? HAT_IN_RANGE(__ldg(table + at), a.plan.num_pages, cx.status) : 0;
             };
             int page = page_of(0);
-            if (un == 0) pdl_wait();                             // up to here only the plan's own arrays were read
+            if (un == 0 && !a.overlap) pdl_wait();               // up to here only the plan's own arrays were read
             const int n_plain = a.k_new != nullptr ? min(u.n, max(0, u.P - u.kv_begin) / kKeys) : u.n;
             int j = 0;
             for (; j < n_plain; ++j) {
@@ -1146,6 +1149,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
     }
     // The last CTA to get here (none draws units any more) leaves the unit counter at zero for the next call, which
     // then needs no memset in front of it.  work_counter[1] counts the CTAs that have finished.
+    if (a.overlap && threadIdx.x == 0) pdl_wait();               // the next kernel takes this one's end for the end of both
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {

@@ -166,7 +166,6 @@ attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, 
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    tc5::pdl_launch_dependents();
     __syncthreads();
 
     const int H = a.plan.num_heads, G = a.plan.group, Hkv = a.plan.num_kv_heads;
@@ -203,6 +202,8 @@ attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, 
         fetch_record(unit, hs, r0, r1, r2);
         page_id = fetch_ids(r0, r1);
         tc5::pdl_wait();                                          // up to here only the plan's own arrays were read
+        // the kernel behind may be one that runs beside this one (tile kernels of the same call): what precedes both has ended
+        tc5::pdl_launch_dependents();
         for (;;) {
             const bool done = unit >= total_units;
             const int row_base = r0.y, C = r0.z, P = r0.w, page0 = r1.x, page1 = r1.y;

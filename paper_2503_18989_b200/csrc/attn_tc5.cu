@@ -165,7 +165,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
-    if (!a.overlap) pdl_launch_dependents();
+    pdl_launch_dependents();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch + TMA producer
@@ -717,7 +717,7 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     a2.plan.tile_units = plan->dev.tile_units + first_unit;
     a2.tail_reset = reset_counter ? 1 : 0;
     a2.static_first = a2.tail_reset;            // a counter of its own
-    a2.overlap = overlap ? 1 : 0;
+    a2.overlap = overlap || args.overlap ? 1 : 0;
     int ctas = std::min(total_units, plan->num_sms);
     if (grid_limit > 0) ctas = std::min(ctas, grid_limit);
     const dim3 grid((unsigned)ctas);

@@ -805,7 +805,12 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
         if (e != cudaSuccess) return cuda_fail(e);
         mark(2, 1);
     }
-    if (plan->res.ev_verify && (e = cudaEventRecord(plan->res.ev_verify, s)) != cudaSuccess) return cuda_fail(e);
+    // a batch without such rows has nothing to announce (an event that was never recorded counts as occurred); a part's are
+    // announced with the whole batch
+    if (has_verify && !plan->is_part && (e = cudaEventRecord(plan->res.ev_verify, s)) != cudaSuccess) return cuda_fail(e);
+    // The tile kernels depend on nothing the streaming kernel does: they take the SMs as it leaves them.  (Not under the timing
+    // recorder, which wants the kernels one after the other.)
+    a.overlap = has_verify && plan->info.stream_kernel == 1 && !side && call < 0 ? 1 : 0;
     if (side) {
         e = launch_attn_tc5(plan, a, s, plan->side_sms, /*reset_counter=*/false);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, plan->ev_join, 0);
