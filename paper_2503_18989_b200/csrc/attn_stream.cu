@@ -56,6 +56,7 @@ constexpr int kThreads = kWarps * 32 + 64;
 constexpr int kCtasPerSm = 2;
 constexpr int kTodo = 48;                   // merges put off to the end of the CTA
 constexpr int kBatch = 4;                   // pages requested at a time
+constexpr int kAhead = 32;                  // pages prefetched to L2 before the previous kernel's end (a lane has one page id)
 constexpr float kMoveThreshold = 8.0f;      // log2 units
 
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
@@ -201,6 +202,16 @@ attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, 
         };
         fetch_record(unit, hs, r0, r1, r2);
         page_id = fetch_ids(r0, r1);
+        {
+            // CTAs of this kernel start as those of the one before run out of work: its tail brings their first pages to L2
+            // (eight calls of 12 requests x 32 heads one after the other: 376 us without, 366 us with; 12 pages 368)
+            const int npre = (r0.w + kPageSize - 1) / kPageSize, h = hs / n_sub;
+            if (lane < kAhead && r1.x + lane < min(r1.y, npre)) {
+                const int page = HAT_IN_RANGE(page_id, a.plan.num_pages, a.plan.status);
+                tc5::tma_prefetch_5d(&map_k, 0, 0, 0, h, page);
+                tc5::tma_prefetch_5d(&map_v, 0, 0, 0, h, page);
+            }
+        }
         tc5::pdl_wait();                                          // up to here only the plan's own arrays were read
         // the kernel behind may be one that runs beside this one (tile kernels of the same call): what precedes both has ended
         tc5::pdl_launch_dependents();
