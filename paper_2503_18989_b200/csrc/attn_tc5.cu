@@ -107,7 +107,7 @@ __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* _
     u.hk = u.h / a.plan.group;
     u.r = lo.x; u.row0 = lo.y; u.kv_begin = lo.z; u.kv_end = lo.w;
     u.part = hi.x; u.P = hi.y; u.C = hi.z; u.row_base = hi.w;
-    u.nq = (u.C - u.row0 > kRows) ? 2 : 1;
+    u.nq = min(u.C - u.row0, a.plan.tile_rows) > kRows ? 2 : 1;
     u.n_all = (u.kv_end - u.kv_begin + kKeys - 1) / kKeys;
     const int end0 = min(u.kv_end, u.P + u.row0 + kRows);
     u.n_q0 = u.nq == 1 ? u.n_all : max(0, (end0 - u.kv_begin + kKeys - 1) / kKeys);
@@ -268,7 +268,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             // tiles with chunk positions
             const tile_append::Chunk ck{u.P, u.C, u.row_base, u.hk};
             // of the units that read a chunk page, the last row block of the group's first query head appends it
-            const bool appends = u.h == u.hk * a.plan.group && u.row0 + 2 * kRows >= u.C;
+            const bool appends = u.h == u.hk * a.plan.group && u.row0 + a.plan.tile_rows >= u.C;
             for (; j < u.n_all; ++j) {
                 const int kb = u.kv_begin + j * kKeys;
                 const int npages = min(8, total_pages - 8 * j);

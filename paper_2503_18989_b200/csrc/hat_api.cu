@@ -8,6 +8,7 @@
 #include <mutex>
 #include <new>
 #include <vector>
+#include <limits>
 #include <queue>
 
 #include "hat_internal.h"
@@ -185,26 +186,34 @@ static int split_len_for(int kv_end, int wanted, int granule) {
 // step of a 256-row unit (two query tiles) or of a unit of at most 128 rows (two chains share it), the fixed cost of a
 // unit (its Q tiles, refilling the rings, storing its rows), and the merge pass (its launch plus reading every partial
 // row).  Units go to the CTAs longest first, as the kernel draws them.  Returns 0 for "leave every request whole".
-static int pick_prefill_split(const hat_plan* p, int num_sms, int tile_rows, int key_granule) {
+// `tile_rows` says how many rows a unit may have; given 0, both forms are priced and it is set to the cheaper one's: units of
+// 128 rows take about as long per row and key, and twice as many units need half as many key ranges, that is less to merge or
+// nothing (one request of 256 rows x 32 heads, fp16, us with units of 256 / 128 rows: prefix 0 13.2 / 10.8, 512 20.0 / 15.8 (now
+// uncut), 1280 22.8 / 21.5, 4000 42.6 / 38.9; 512 rows at 1000 32.8 / 24.4; but two of 200 rows x 40 heads at 500, where 128-row
+// units need a second round, 22.9 / 26.5).
+static int pick_prefill_split(const hat_plan* p, int num_sms, int* tile_rows, int key_granule) {
     constexpr int64_t kStepWide = 4000, kStepNarrow = 2200, kUnit = 10000, kMergeLaunch = 5700;
     constexpr int64_t kMergeBytesPerCycle = 3000;
     struct Tile { int keys, rows; };
     std::vector<Tile> tiles;
     int max_keys = 0;
-    for (int r = 0; r < p->num_requests; ++r) {
-        const int C = p->chunk_len[r];
-        if (C <= 16) continue;
-        for (int row0 = 0; row0 < C; row0 += tile_rows) {
-            const int rows = std::min(tile_rows, C - row0);
-            tiles.push_back(Tile{p->prefix_len[r] + row0 + rows, rows});
-            max_keys = std::max(max_keys, tiles.back().keys);
+    auto cut_rows = [&](int unit_rows) {
+        tiles.clear();
+        for (int r = 0; r < p->num_requests; ++r) {
+            const int C = p->chunk_len[r];
+            if (C <= 16) continue;
+            for (int row0 = 0; row0 < C; row0 += unit_rows) {
+                const int rows = std::min(unit_rows, C - row0);
+                tiles.push_back(Tile{p->prefix_len[r] + row0 + rows, rows});
+                max_keys = std::max(max_keys, tiles.back().keys);
+            }
         }
-    }
+    };
     const int H = p->num_heads;
     std::vector<int64_t> units;
-    auto price = [&](int len) -> int64_t {
+    auto price = [&](int len, int64_t least) -> int64_t {      // exact only below `least`
         units.clear();
-        int64_t part_rows = 0;
+        int64_t part_rows = 0, work = 0;
         for (const Tile& t : tiles) {
             const int sl = len > 0 ? split_len_for(t.keys, len, key_granule) : t.keys;
             const int n = ceil_div(t.keys, sl);
@@ -212,9 +221,13 @@ static int pick_prefill_split(const hat_plan* p, int num_sms, int tile_rows, int
             for (int s = 0; s < n; ++s) {
                 const int keys = std::min(t.keys, (s + 1) * sl) - s * sl;
                 units.push_back(ceil_div(keys, 128) * (t.rows > 128 ? kStepWide : kStepNarrow) + kUnit);
+                work += units.back();
             }
         }
+        const int64_t merge = part_rows > 0 ? kMergeLaunch + part_rows * H * (p->head_dim + 1) * 4 / kMergeBytesPerCycle : 0;
         std::sort(units.begin(), units.end(), std::greater<int64_t>());
+        if ((int64_t)units.size() * H <= num_sms) return units[0] + merge;
+        if (work * H / num_sms + merge >= least) return least;
         std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> sms;
         for (int i = 0; i < num_sms; ++i) sms.push(0);
         int64_t makespan = 0;
@@ -226,15 +239,19 @@ static int pick_prefill_split(const hat_plan* p, int num_sms, int tile_rows, int
                 makespan = std::max(makespan, t);
             }
         }
-        if (part_rows > 0) makespan += kMergeLaunch + part_rows * H * (p->head_dim + 1) * 4 / kMergeBytesPerCycle;
-        return makespan;
+        return makespan + merge;
     };
-    int best = 0;
-    int64_t best_cost = price(0);
-    for (int len = 256; len < max_keys; len += (len < 1024 ? 128 : len < 4096 ? 512 : 2048)) {
-        const int64_t c = price(len);
-        if (c < best_cost) { best_cost = c; best = len; }
+    int best = 0, best_rows = *tile_rows;
+    int64_t best_cost = std::numeric_limits<int64_t>::max();
+    for (int unit_rows : {256, 128}) {
+        if (*tile_rows != 0 && unit_rows != *tile_rows) continue;
+        cut_rows(unit_rows);
+        for (int len = 0; len < max_keys; len += (len == 0 ? 256 : len < 1024 ? 128 : len < 4096 ? 512 : 2048)) {
+            const int64_t c = price(len, best_cost);
+            if (c < best_cost) { best_cost = c; best = len; best_rows = unit_rows; }
+        }
     }
+    *tile_rows = best_rows;
     return best;
 }
 
@@ -292,9 +309,8 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
 
     const int verify_max_rows = 16;
     // tile kernel: tcgen05 with 256-row tiles (two 128-row MMA tiles) and 128-key steps, or mma.sync with 4 warps x 16 rows and 64-key steps
-    const int tile_rows = use_tc5 ? 256 : 64;
+    int tile_rows = use_tc5 ? 256 : 64;
     const int key_granule = use_tc5 ? 128 : 64;
-    info.prefill_tile_rows = tile_rows;
     info.prefill_kernel = tile_kernel;
 
     // ---- streaming (verify-class) requests: key ranges of one length.
@@ -329,11 +345,13 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
         }
     }
     int psplit = whole ? 0 : env_int("HAT_PREFILL_SPLIT_LEN", -1);
+    int want_rows = tile_kernel == 1 && !whole ? env_int("HAT_PREFILL_TILE_ROWS", 0) : tile_rows;   // 0: whichever is cheaper
+    if (want_rows != 128 && want_rows != 0) want_rows = tile_rows;
     if (psplit < 0) {
         psplit = 0;
         const int64_t want_ctas = (int64_t)num_sms * 2;
         if (tiles > 0 && tiles * H < want_ctas && use_tc5) {
-            psplit = pick_prefill_split(p, num_sms, tile_rows, key_granule);
+            psplit = pick_prefill_split(p, num_sms, &want_rows, key_granule);
         } else if (tiles > 0 && tiles * H < want_ctas) {
             // aim for want_ctas pieces of equal length, not shorter than 256 keys
             const int pieces = ceil_div((int)want_ctas, H);
@@ -342,6 +360,8 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
     }
     if (psplit > 0) psplit = round_up(psplit, key_granule);
     info.prefill_split_len = psplit;
+    if (want_rows > 0) tile_rows = want_rows;
+    info.prefill_tile_rows = tile_rows;
 
     int stream_merged = 0;                  // rows the streaming kernel merges itself
     // streaming-class requests first: their merge rows form the head of merge_rows, so that they can be merged (and
@@ -485,6 +505,7 @@ int upload_plans(hat_plan* const* plans, size_t count, PlanRes* res) {
         d.num_kv_heads = p->num_kv_heads;
         d.group = p->num_heads / p->num_kv_heads;
         d.total_rows = p->total_rows;
+        d.tile_rows = p->info.prefill_tile_rows;
         d.num_pages = p->num_pages;
     }
     return HAT_OK;

@@ -65,6 +65,7 @@ struct DevicePlan {
     int32_t         num_kv_heads;   // K/V heads (pools, k_new, v_new)
     int32_t         group;          // query heads per K/V head
     int32_t         total_rows;
+    int32_t         tile_rows;      // query rows of a prefill item, its last one of a chunk may have fewer
     int32_t         num_pages;      // pages in the pools (index checks of the debug build)
 };
 
@@ -94,7 +95,7 @@ struct AttnArgs {
     int         withhold;     // self test: the tile kernel's producer skips its first V tile so that a wait runs out
     int         static_first; // a CTA's first unit is its own number, the counter gives the ones after the grid's; else all come from the counter
     int         overlap;      // the grid runs beside the stream's previous kernel (which has waited for everything before it): waits for its end only at its own
-    int         tail_reset;   // the last CTA of the persistent tile kernel to finish clears the unit counter for the next call
+    int         tail_reset;   // the last producer of the persistent tile kernel to finish clears the unit counter for the next call
 };
 
 // Key range of one split of the allocation-free streaming entry point, from lengths that nobody validated (they are
