@@ -54,6 +54,7 @@
 #include "hat_internal.h"
 #include "tma_desc.h"
 #include "tc5_ptx.cuh"
+#include "out_rows.cuh"
 #include "tile_append.cuh"
 
 namespace hat {
@@ -400,6 +401,12 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 step();
             }
         }
+        // The last pair whose producer draws no more leaves the unit counter at zero for the next call, which then needs no
+        // memset in front of it.  work_counter[1] counts them.  (Every draw has returned: no fence is needed.)
+        if (rank == 0 && lane == 0 && atomicAdd(work_counter + 1, 1) == (int)(gridDim.x >> 1) - 1) {
+            work_counter[0] = 0;
+            work_counter[1] = 0;
+        }
         if (ok) pay();
         tile_append::stores_done();
 #ifdef HAT_PHASE_TIMERS
@@ -706,7 +713,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             const uint32_t tm_o = tmem + kColO + lane_sel;
             const int wg_tid = (int)threadIdx.x - 64 - w * 128;
             const float sc = a.scale_log2;
-            const bool wide_stores = ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.part_out)) & 31) == 0;
             const uint32_t lead_o_free = lead(&bars->o_free), lead_p_ready = lead(&bars->p_ready[0]);
             int g0 = 0;                                         // global index of the unit's first tile
             int px = 0;                                         // meetings of this warp with its partner so far
@@ -872,44 +878,11 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_remote(lead_o_free);
-                if (i_row < u.C) {
-                    const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
-                    float* obase; float* lbase; int64_t orow;
-                    if (u.part < 0) { obase = a.out; lbase = a.lse; orow = u.row_base + i_row; }
-                    else { obase = a.part_out; lbase = a.part_lse; orow = u.part + (i_row - u.row0); }
-                    HAT_CHECK(orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows), cx.status);
-                    if (u.part < 0 && a.out16 != nullptr) {
-                        // final rows in the 16-bit output type: 128 bytes per row and warpgroup
-                        uint16_t* dst16 = static_cast<uint16_t*>(a.out16) + (orow * H + u.h) * kD + w * 64;
-                        const bool wide16 = (reinterpret_cast<uintptr_t>(a.out16) & 31) == 0;
-#pragma unroll
-                        for (int k = 0; k < 64; k += 16) {
-                            uint32_t wd[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) wd[e] = pack_out16(o[k + 2 * e] * inv, o[k + 2 * e + 1] * inv, a.out16_bf16);
-                            if (wide16) {
-                                asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
-                                             ::"l"(dst16 + k), "r"(wd[0]), "r"(wd[1]), "r"(wd[2]), "r"(wd[3]), "r"(wd[4]), "r"(wd[5]), "r"(wd[6]), "r"(wd[7]) : "memory");
-                            } else {
-                                *reinterpret_cast<uint4*>(dst16 + k) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                                *reinterpret_cast<uint4*>(dst16 + k + 8) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-                            }
-                        }
-                    } else {
-                        float* dst = obase + (orow * H + u.h) * kD + w * 64;
-                        if (wide_stores) {
-#pragma unroll
-                            for (int k = 0; k < 64; k += 8)
-                                st_global_v8(dst + k, o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv, o[k + 4] * inv,
-                                             o[k + 5] * inv, o[k + 6] * inv, o[k + 7] * inv);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 64; k += 4)
-                                *reinterpret_cast<float4*>(dst + k) = make_float4(o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv);
-                        }
-                    }
-                    if (w == 0) lbase[orow * H + u.h] = l_tot > 0.f ? (m_fin + log2f(l_tot)) * 0.6931471805599453f : -INFINITY;
-                }
+                const int64_t orow = u.part < 0 ? u.row_base + i_row : u.part + (i_row - u.row0);
+                HAT_CHECK(i_row >= u.C || (orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows)), cx.status);
+                out_rows::store<64, kD, false>(a, o, l_tot > 0.f ? 1.f / l_tot : 0.f, u.part < 0, orow, u.C - i_row, u.h, w * 64, lane);
+                if (w == 0 && i_row < u.C)
+                    (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l_tot > 0.f ? (m_fin + log2f(l_tot)) * 0.6931471805599453f : -INFINITY;
                 g0 += u.n;
                 PH_ADD(9, tw0);
 #ifdef HAT_PHASE_TIMERS
@@ -927,7 +900,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             const uint32_t tm_o = tmem + kColO + lane_sel;
             const int wg_tid = (int)threadIdx.x - 64 - w * 128;
             const float sc = a.scale_log2;
-            const bool wide_stores = ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.part_out)) & 31) == 0;
             const uint32_t lead_o_free = lead(&bars->o_free), lead_p_ready = lead(&bars->p_ready[0]);
             int g0 = 0;                                         // global index of the unit's first tile
             bool ok = true;
@@ -1088,44 +1060,11 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_remote(lead_o_free);
-                if (i_row < u.C) {
-                    const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
-                    float* obase; float* lbase; int64_t orow;
-                    if (u.part < 0) { obase = a.out; lbase = a.lse; orow = u.row_base + i_row; }
-                    else { obase = a.part_out; lbase = a.part_lse; orow = u.part + (i_row - u.row0); }
-                    HAT_CHECK(orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows), cx.status);
-                    if (u.part < 0 && a.out16 != nullptr) {
-                        // final rows in the 16-bit output type: 128 bytes per row and warpgroup
-                        uint16_t* dst16 = static_cast<uint16_t*>(a.out16) + (orow * H + u.h) * kD + w * 64;
-                        const bool wide16 = (reinterpret_cast<uintptr_t>(a.out16) & 31) == 0;
-#pragma unroll
-                        for (int k = 0; k < 64; k += 16) {
-                            uint32_t wd[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) wd[e] = pack_out16(o[k + 2 * e] * inv, o[k + 2 * e + 1] * inv, a.out16_bf16);
-                            if (wide16) {
-                                asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
-                                             ::"l"(dst16 + k), "r"(wd[0]), "r"(wd[1]), "r"(wd[2]), "r"(wd[3]), "r"(wd[4]), "r"(wd[5]), "r"(wd[6]), "r"(wd[7]) : "memory");
-                            } else {
-                                *reinterpret_cast<uint4*>(dst16 + k) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                                *reinterpret_cast<uint4*>(dst16 + k + 8) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-                            }
-                        }
-                    } else {
-                        float* dst = obase + (orow * H + u.h) * kD + w * 64;
-                        if (wide_stores) {
-#pragma unroll
-                            for (int k = 0; k < 64; k += 8)
-                                st_global_v8(dst + k, o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv, o[k + 4] * inv,
-                                             o[k + 5] * inv, o[k + 6] * inv, o[k + 7] * inv);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 64; k += 4)
-                                *reinterpret_cast<float4*>(dst + k) = make_float4(o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv);
-                        }
-                    }
-                    if (took_last) lbase[orow * H + u.h] = l_tot > 0.f ? (m_fin + log2f(l_tot)) * 0.6931471805599453f : -INFINITY;
-                }
+                const int64_t orow = u.part < 0 ? u.row_base + i_row : u.part + (i_row - u.row0);
+                HAT_CHECK(i_row >= u.C || (orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows)), cx.status);
+                out_rows::store<64, kD, false>(a, o, l_tot > 0.f ? 1.f / l_tot : 0.f, u.part < 0, orow, u.C - i_row, u.h, w * 64, lane);
+                if (took_last && i_row < u.C)
+                    (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l_tot > 0.f ? (m_fin + log2f(l_tot)) * 0.6931471805599453f : -INFINITY;
                 g0 += u.n;
                 PH_ADD(9, tw0);
 #ifdef HAT_PHASE_TIMERS
@@ -1147,17 +1086,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
     }
-    // The last CTA to get here (none draws units any more) leaves the unit counter at zero for the next call, which
-    // then needs no memset in front of it.  work_counter[1] counts the CTAs that have finished.
     if (a.overlap && threadIdx.x == 0) pdl_wait();               // the next kernel takes this one's end for the end of both
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {
-            work_counter[0] = 0;
-            work_counter[1] = 0;
-            __threadfence();
-        }
-    }
 }
 
 }  // namespace

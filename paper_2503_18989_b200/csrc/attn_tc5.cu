@@ -31,6 +31,7 @@
 #include "hat_internal.h"
 #include "tma_desc.h"
 #include "tc5_ptx.cuh"
+#include "out_rows.cuh"
 #include "tile_append.cuh"
 
 namespace hat {
@@ -56,7 +57,7 @@ struct __align__(8) Barriers {
     uint64_t v_full[kStagesV], v_empty[kStagesV];
     uint64_t s_full[2], p_ready[2], o_done[2], o_free[2];   // per query tile
     uint64_t unit_full[2], unit_empty[2];                   // two-slot queue of work units, producer -> other roles
-    uint64_t x_ready;                                       // split units: chain 1's (reference maximum, row sum) are in xchg
+    uint64_t x_ready, x_ready0;                             // split units: (reference maximum, row sum) of chain 1 are in xchg, chain 0's too
     uint64_t drain;
     long long wait_cycles;                                  // bound of every wait below
     uint32_t tmem_base;
@@ -117,7 +118,9 @@ __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* _
     return u;
 }
 
-template <bool BF16, int kD>
+// ONE: no CTA has more than one unit (head_dim 128; rows of 64 columns store as fast as they are).  A template parameter
+// because the softmax loop's registers are tight: as a branch, the other output form cost it 2 %.
+template <bool BF16, int kD, bool ONE>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units, int32_t* work_counter,
                 const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -151,6 +154,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             mbar_init(&bars->unit_empty[s], 1 + 8);              // the MMA thread and every softmax warp
         }
         mbar_init(&bars->x_ready, 4);
+        mbar_init(&bars->x_ready0, 4);
         mbar_init(&bars->drain, 1);
         bars->abort_flag = 0;
         bars->wait_cycles = a.wait_cycles;
@@ -210,6 +214,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             if (lane == 0) {
                 // a CTA's first unit is its own number: nothing to wait for
                 if (un == 0 && a.static_first) unit = (int)blockIdx.x;
+                else if (ONE) unit = -1;
                 else unit = atomicAdd(work_counter, 1) + (a.static_first ? (int)gridDim.x : 0);
                 if (unit >= total_units) unit = -1;
                 bars->unit_slot[slot] = unit;
@@ -319,6 +324,13 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 page = page_next;
                 step();
             }
+        }
+        // The last CTA whose producer draws no more leaves the unit counter at zero for the next call, which then needs no
+        // memset in front of it.  work_counter[1] counts them.  (Every draw has returned, so no fence is needed; at the CTA's end, behind
+        // one, this held up the next kernel of the stream by about 1 us.)
+        if (!ONE && a.tail_reset && lane == 0 && atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {
+            work_counter[0] = 0;
+            work_counter[1] = 0;
         }
         if (ok) pay();
         tile_append::stores_done();
@@ -452,7 +464,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         const int wg_tid = (int)threadIdx.x - 64 - qt * 128;
         const float sc = a.scale_log2;
         // rows are 512 bytes apart at least, so a 32-byte aligned base keeps every 32-byte store aligned
-        const bool wide_stores = ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.part_out)) & 31) == 0;
+        const bool wide_stores = !ONE && ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.part_out)) & 31) == 0;
         int kt_base = 0;                                    // K/V tiles of the units before this one
         int s_cnt = 0, o_cnt = 0, x_cnt = 0;                // completions of s_full[qt] / o_done[qt] / x_ready consumed so far
         bool ok = true;
@@ -567,15 +579,65 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     if (lane == 0) mbar_arrive(&bars->p_ready[qt]);
                 }
                 if (!ok) break;
-                // ---- output of the unit: pull O into registers, hand the accumulator back, then store
-                float o[kD];
+                // ---- output of the unit
                 if (n_mine > 0) {                            // uniform over the warpgroup
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done[qt], o_cnt & 1, bars, status));
                     ++o_cnt;
                     if (!ok) break;
                     tc_fence_after();
                 }
-                if (u.split && qt == 1) {
+                if constexpr (ONE) {
+                    // 64 columns at a time, stored with the lanes' halves exchanged (out_rows.cuh).  A split unit: the chains (disjoint keys)
+                    // are merged, weights 2^(m_t - m), sums and accumulators add up; each chain's warpgroup does half of the columns
+                    const bool have0 = u.split ? u.n_t0 > 0 : n_mine > 0, have1 = u.split && u.n_t1 > 0;
+                    float w0 = 1.f, w1 = 0.f;
+                    if (have1) {
+                        float2* x0 = reinterpret_cast<float2*>(q_tiles + kTileBytes);   // the second query tile's place is free
+                        (qt == 0 ? x0 : bars->xchg)[t] = make_float2(m_used, l);
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(qt == 0 ? &bars->x_ready0 : &bars->x_ready);
+                        ok = __all_sync(0xffffffffu, mbar_wait(qt == 0 ? &bars->x_ready : &bars->x_ready0, 0, bars, status));
+                        if (!ok) break;
+                        tc_fence_after();
+                        const float2 c0 = x0[t], c1 = bars->xchg[t];
+                        m_used = fmaxf(c0.x, c1.x);
+                        w0 = (c0.x == -INFINITY) ? 0.f : fast_exp2(c0.x - m_used);
+                        w1 = (c1.x == -INFINITY) ? 0.f : fast_exp2(c1.x - m_used);
+                        l = c0.y * w0 + c1.y * w1;
+                    }
+                    const float inv = l > 0.f ? 1.f / l : 0.f;
+                    const int64_t orow = u.part < 0 ? u.row_base + i_row : u.part + (i_row - u.row0);
+                    HAT_CHECK(i_row >= u.C || (orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows)), status);
+                    const uint32_t tm_a = u.split ? tmem + 256 + lane_sel : tm_o;
+#pragma unroll
+                    for (int c0 = 0; c0 < kD; c0 += 64) {
+                        // without a second chain its warpgroup knows nothing of the rows: the first one stores them whole
+                        if (u.split && (have1 ? c0 != 64 * qt : qt != 0)) continue;
+                        float o[64];
+                        if (have0) {
+                            tmem_ld32(tm_a + c0, reinterpret_cast<uint32_t*>(o));
+                            tmem_ld32(tm_a + c0 + 32, reinterpret_cast<uint32_t*>(o) + 32);
+                            tmem_ld_wait();
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 64; ++k) o[k] = 0.f;
+                        }
+                        if (have1) {
+#pragma unroll
+                            for (int c = 0; c < 64; c += 32) {
+                                uint32_t o1[32];
+                                tmem_ld32(tm_a + 128 + c0 + c, o1);      // the second chain's accumulator: next 128 columns
+                                tmem_ld_wait();
+#pragma unroll
+                                for (int k = 0; k < 32; ++k) o[c + k] = o[c + k] * w0 + __uint_as_float(o1[k]) * w1;
+                            }
+                        }
+                        out_rows::store<64, kD, true>(a, o, inv, u.part < 0, orow, u.C - i_row, u.h, c0, lane);
+                    }
+                    if (i_row < u.C && !(u.split && qt == 1))
+                        (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
+                } else if (u.split && qt == 1) {
                     // second chain of a split unit: its accumulator is complete; publish the row's reference maximum
                     // and sum, the first chain's warpgroup reads the accumulator itself (same TMEM lanes) and stores
                     if (n_mine > 0) {
@@ -585,6 +647,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         if (lane == 0) mbar_arrive(&bars->x_ready);
                     }
                 } else {
+                    // pull O into registers, hand the accumulator back, then store
+                    float o[kD];
                     if (n_mine > 0) {
 #pragma unroll
                         for (int c = 0; c < kD / 32; ++c) tmem_ld32(tm_o + c * 32, reinterpret_cast<uint32_t*>(o) + c * 32);
@@ -672,17 +736,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
     }
-    // The last CTA to get here (none draws units any more) leaves the unit counter at zero for the next call, which
-    // then needs no memset in front of it.  work_counter[1] counts the CTAs that have finished.
     if (a.overlap && threadIdx.x == 0) pdl_wait();               // the next kernel takes this one's end for the end of both
-    if (a.tail_reset && threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {
-            work_counter[0] = 0;
-            work_counter[1] = 0;
-            __threadfence();
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------------------------- host side
@@ -722,8 +776,10 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     if (grid_limit > 0) ctas = std::min(ctas, grid_limit);
     const dim3 grid((unsigned)ctas);
     const bool d128 = plan->head_dim == 128;
-    auto kern = d128 ? (bf16 ? attn_tc5_kernel<true, 128> : attn_tc5_kernel<false, 128>)
-                     : (bf16 ? attn_tc5_kernel<true, 64> : attn_tc5_kernel<false, 64>);
+    const bool one = d128 && total_units <= ctas && a2.static_first;
+    auto kern = !d128 ? (bf16 ? attn_tc5_kernel<true, 64, false> : attn_tc5_kernel<false, 64, false>)
+                : one ? (bf16 ? attn_tc5_kernel<true, 128, true> : attn_tc5_kernel<false, 128, true>)
+                      : (bf16 ? attn_tc5_kernel<true, 128, false> : attn_tc5_kernel<false, 128, false>);
     const uint32_t smem = d128 ? smem_bytes<128>() : smem_bytes<64>();
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), (int)smem);
     if (e != cudaSuccess) return e;
