@@ -58,6 +58,7 @@ struct __align__(8) Barriers {
     uint64_t s_full[2], p_ready[2], o_done[2], o_free[2];   // per query tile
     uint64_t unit_full[2], unit_empty[2];                   // two-slot queue of work units, producer -> other roles
     uint64_t x_ready, x_ready0;                             // split units: (reference maximum, row sum) of chain 1 are in xchg, chain 0's too
+    uint64_t peer_ready[8];                                 // kHalves: the softmax warp of the same number in the other CTA has its rows ready
     uint64_t drain;
     long long wait_cycles;                                  // bound of every wait below
     uint32_t tmem_base;
@@ -74,6 +75,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Barrie
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try(bar, parity)) {
+        if (b->abort_flag) return false;
+        if (clock64() - t0 > b->wait_cycles) {
+            b->abort_flag = 1;
+            atomicOr(status, 1);
+            return false;
+        }
+    }
+    return true;
+}
+
+// The same for a barrier the cluster's other CTA arrives on, acquiring what it wrote before.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, Barriers* b, int32_t* status) {
+    const long long t0 = clock64();
+    while (!mbar_try_cluster(bar, parity)) {
         if (b->abort_flag) return false;
         if (clock64() - t0 > b->wait_cycles) {
             b->abort_flag = 1;
@@ -118,14 +133,22 @@ __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* _
     return u;
 }
 
-// ONE: no CTA has more than one unit (head_dim 128; rows of 64 columns store as fast as they are).  A template parameter
-// because the softmax loop's registers are tight: as a branch, the other output form cost it 2 %.
-template <bool BF16, int kD, bool ONE>
+// How the units lie on the CTAs.  A template parameter because the softmax loop's registers are tight: as a branch, the other
+// output form cost it 2 %.
+//   kMany    CTAs draw units
+//   kOne     no CTA has more than one unit (head_dim 128; rows of 64 columns store as fast as they are)
+//   kHalves  the same, and the CTAs of a cluster of two have the two key ranges of one tile of at most 128 rows: they merge them
+//            through each other's shared memory, 32 columns to a warpgroup, instead of through global memory and a launch
+//            (one request of 256 rows x 32 heads, us a call: prefix 768
+//            19.4 -> 13.4, 1792 23.9 -> 17.9, 4000 38.9 -> 32.3)
+enum Form { kMany, kOne, kHalves };
+template <bool BF16, int kD, int FORM>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units, int32_t* work_counter,
                 const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_k_new,
                 const __grid_constant__ CUtensorMap map_v_new, int fold) {
+    constexpr bool ONE = FORM != kMany;
     constexpr uint32_t kTileBytes = tile_bytes<kD>();
     constexpr int kHalves = kD / 64;                             // 64-column slabs of a Q tile
     constexpr uint32_t kGroupBytes = group_bytes<kD>(), kPageBytes = page_bytes<kD>();
@@ -155,6 +178,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         }
         mbar_init(&bars->x_ready, 4);
         mbar_init(&bars->x_ready0, 4);
+        for (int w = 0; w < 8; ++w) mbar_init(&bars->peer_ready[w], 1);
         mbar_init(&bars->drain, 1);
         bars->abort_flag = 0;
         bars->wait_cycles = a.wait_cycles;
@@ -167,6 +191,10 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (FORM == kHalves) {
+        cluster_arrive();                                        // the other CTA's barriers are initialised
+        cluster_wait();
+    }
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     pdl_launch_dependents();
@@ -589,9 +617,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 if constexpr (ONE) {
                     // 64 columns at a time, stored with the lanes' halves exchanged (out_rows.cuh).  A split unit: the chains (disjoint keys)
                     // are merged, weights 2^(m_t - m), sums and accumulators add up; each chain's warpgroup does half of the columns
-                    const bool have0 = u.split ? u.n_t0 > 0 : n_mine > 0, have1 = u.split && u.n_t1 > 0;
+                    const bool have0 = u.split || n_mine > 0, have1 = u.split && u.n_t1 > 0;
                     float w0 = 1.f, w1 = 0.f;
-                    if (have1) {
+                    if (u.split) {
                         float2* x0 = reinterpret_cast<float2*>(q_tiles + kTileBytes);   // the second query tile's place is free
                         (qt == 0 ? x0 : bars->xchg)[t] = make_float2(m_used, l);
                         tc_fence_before();
@@ -606,15 +634,10 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         w1 = (c1.x == -INFINITY) ? 0.f : fast_exp2(c1.x - m_used);
                         l = c0.y * w0 + c1.y * w1;
                     }
-                    const float inv = l > 0.f ? 1.f / l : 0.f;
                     const int64_t orow = u.part < 0 ? u.row_base + i_row : u.part + (i_row - u.row0);
                     HAT_CHECK(i_row >= u.C || (orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows)), status);
                     const uint32_t tm_a = u.split ? tmem + 256 + lane_sel : tm_o;
-#pragma unroll
-                    for (int c0 = 0; c0 < kD; c0 += 64) {
-                        // without a second chain its warpgroup knows nothing of the rows: the first one stores them whole
-                        if (u.split && (have1 ? c0 != 64 * qt : qt != 0)) continue;
-                        float o[64];
+                    auto load64 = [&](float (&o)[64], int c0) {
                         if (have0) {
                             tmem_ld32(tm_a + c0, reinterpret_cast<uint32_t*>(o));
                             tmem_ld32(tm_a + c0 + 32, reinterpret_cast<uint32_t*>(o) + 32);
@@ -633,10 +656,56 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                                 for (int k = 0; k < 32; ++k) o[c + k] = o[c + k] * w0 + __uint_as_float(o1[k]) * w1;
                             }
                         }
-                        out_rows::store<64, kD, true>(a, o, inv, u.part < 0, orow, u.C - i_row, u.h, c0, lane);
+                    };
+                    if constexpr (FORM == kHalves) {
+                        // this CTA finishes columns 64 qt + 32 rank ..; the other 32 of the warpgroup's 64 go where the Q tile was (every
+                        // product that read it has ended), the maximum and sum behind chain 0's
+                        const uint32_t rank = cluster_ctarank();
+                        float o[64], mine[32];
+                        load64(o, 64 * qt);
+                        float4* give = reinterpret_cast<float4*>(q_tiles) + qt * (8 * kRows) + t;
+                        float2* ml = reinterpret_cast<float2*>(q_tiles + kTileBytes) + (1 + qt) * kRows + t;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const float* lo = o + 4 * k; const float* hi = o + 32 + 4 * k;
+                            give[k * kRows] = rank == 0 ? make_float4(hi[0], hi[1], hi[2], hi[3]) : make_float4(lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) mine[4 * k + e] = rank == 0 ? lo[e] : hi[e];
+                        }
+                        *ml = make_float2(m_used, l);
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bars->peer_ready[warp - 2]), rank ^ 1u));
+                        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&bars->peer_ready[warp - 2], 0, bars, status));
+                        if (!ok) break;
+                        const float2 other = ld_cluster_f2(map_to_cta(smem_u32(ml), rank ^ 1u));
+                        const uint32_t from = map_to_cta(smem_u32(give), rank ^ 1u);
+                        const float m_new = fmaxf(m_used, other.x);
+                        const float wm = (m_used == -INFINITY) ? 0.f : fast_exp2(m_used - m_new);
+                        const float wo = (other.x == -INFINITY) ? 0.f : fast_exp2(other.x - m_new);
+                        // the same in both CTAs, whichever piece is its own
+                        l = __fadd_rn(__fmul_rn(l, wm), __fmul_rn(other.y, wo));
+                        m_used = m_new;
+                        const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const float4 v = ld_cluster_f4(from + k * kRows * 16);
+                            mine[4 * k] = mine[4 * k] * wm + v.x * wo; mine[4 * k + 1] = mine[4 * k + 1] * wm + v.y * wo;
+                            mine[4 * k + 2] = mine[4 * k + 2] * wm + v.z * wo; mine[4 * k + 3] = mine[4 * k + 3] * wm + v.w * wo;
+                        }
+                        out_rows::store<32, kD, true>(a, mine, inv, true, orow, u.C - i_row, u.h, 64 * qt + 32 * (int)rank, lane);
+                        if (i_row < u.C && qt == 0 && rank == 0) a.lse[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
+                    } else {
+                        const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+                        for (int c0 = 0; c0 < kD; c0 += 64) {
+                            if (u.split && c0 != 64 * qt) continue;
+                            float o[64];
+                            load64(o, c0);
+                            out_rows::store<64, kD, true>(a, o, inv, u.part < 0, orow, u.C - i_row, u.h, c0, lane);
+                        }
+                        if (i_row < u.C && !(u.split && qt == 1))
+                            (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
                     }
-                    if (i_row < u.C && !(u.split && qt == 1))
-                        (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
                 } else if (u.split && qt == 1) {
                     // second chain of a split unit: its accumulator is complete; publish the row's reference maximum
                     // and sum, the first chain's warpgroup reads the accumulator itself (same TMEM lanes) and stores
@@ -732,6 +801,10 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (FORM == kHalves) {
+        cluster_arrive();                                        // the other CTA has read what it needs of this one's shared memory
+        cluster_wait();
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
@@ -777,13 +850,15 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     const dim3 grid((unsigned)ctas);
     const bool d128 = plan->head_dim == 128;
     const bool one = d128 && total_units <= ctas && a2.static_first;
-    auto kern = !d128 ? (bf16 ? attn_tc5_kernel<true, 64, false> : attn_tc5_kernel<false, 64, false>)
-                : one ? (bf16 ? attn_tc5_kernel<true, 128, true> : attn_tc5_kernel<false, 128, true>)
-                      : (bf16 ? attn_tc5_kernel<true, 128, false> : attn_tc5_kernel<false, 128, false>);
+    if (plan->tile_clusters && !one) return cudaErrorInvalidValue;
+    auto kern = !d128 ? (bf16 ? attn_tc5_kernel<true, 64, kMany> : attn_tc5_kernel<false, 64, kMany>)
+                : plan->tile_clusters ? (bf16 ? attn_tc5_kernel<true, 128, kHalves> : attn_tc5_kernel<false, 128, kHalves>)
+                : one ? (bf16 ? attn_tc5_kernel<true, 128, kOne> : attn_tc5_kernel<false, 128, kOne>)
+                      : (bf16 ? attn_tc5_kernel<true, 128, kMany> : attn_tc5_kernel<false, 128, kMany>);
     const uint32_t smem = d128 ? smem_bytes<128>() : smem_bytes<64>();
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, grid, dim3(kThreads), smem, stream, a2, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv, *mkn, *mvn, fold);
+    return launch_pdl_clusters(plan->tile_clusters ? 2 : 1, kern, grid, dim3(kThreads), smem, stream, a2, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv, *mkn, *mvn, fold);
 }
 
 }  // namespace hat

@@ -181,6 +181,13 @@ static int split_len_for(int kv_end, int wanted, int granule) {
     return std::max(wanted, least);
 }
 
+// Whether the two halves of every cut tile are merged inside the one-CTA tile kernel, by clusters of two CTAs: every tile is
+// cut in two, has at most 128 rows, and the pieces are one round of the CTAs.  (Side by side with another grid on one
+// counter, HAT_SIDE_SMS, a unit has no CTA of its own.)
+static bool pieces_meet_in_clusters(const hat_plan* p, int num_sms, int64_t units, bool all_in_two, bool all_narrow) {
+    return p->head_dim == 128 && all_in_two && all_narrow && units <= num_sms / 2 * 2 && env_int("HAT_SIDE_SMS", 0) <= 0;
+}
+
 // Key-range length for the tile-class requests of a batch that is too small to fill the persistent tcgen05 kernel.
 // Every candidate length is priced with a small model of that kernel, in SM clock cycles measured on B200: a 128-key
 // step of a 256-row unit (two query tiles) or of a unit of at most 128 rows (two chains share it), the fixed cost of a
@@ -188,11 +195,11 @@ static int split_len_for(int kv_end, int wanted, int granule) {
 // row).  Units go to the CTAs longest first, as the kernel draws them.  Returns 0 for "leave every request whole".
 // `tile_rows` says how many rows a unit may have; given 0, both forms are priced and it is set to the cheaper one's: units of
 // 128 rows take about as long per row and key, and twice as many units need half as many key ranges, that is less to merge or
-// nothing (one request of 256 rows x 32 heads, fp16, us with units of 256 / 128 rows: prefix 0 13.2 / 10.8, 512 20.0 / 15.8 (now
-// uncut), 1280 22.8 / 21.5, 4000 42.6 / 38.9; 512 rows at 1000 32.8 / 24.4; but two of 200 rows x 40 heads at 500, where 128-row
-// units need a second round, 22.9 / 26.5).
-static int pick_prefill_split(const hat_plan* p, int num_sms, int* tile_rows, int key_granule) {
-    constexpr int64_t kStepWide = 4000, kStepNarrow = 2200, kUnit = 10000, kMergeLaunch = 5700;
+// nothing, and two ranges are merged by clusters (one request of 256 rows x 32 heads, fp16, us with units of 256 / 128 rows: prefix
+// 0 11.4 / 8.7, 512 18.0 / 12.5, 1280 20.7 / 15.5, 4000 40.6 / 32.3; 512 rows at 1000 31.6 / 23.3; but two of 200 rows x 40
+// heads at 500, where 128-row units need a second round, 21.9 / 25.5).
+static int pick_prefill_split(const hat_plan* p, int num_sms, int* tile_rows, int key_granule, bool clusters) {
+    constexpr int64_t kStepWide = 4000, kStepNarrow = 2200, kUnit = 10000, kMergeLaunch = 5700, kMergeCluster = 2500;
     constexpr int64_t kMergeBytesPerCycle = 3000;
     struct Tile { int keys, rows; };
     std::vector<Tile> tiles;
@@ -214,17 +221,20 @@ static int pick_prefill_split(const hat_plan* p, int num_sms, int* tile_rows, in
     auto price = [&](int len, int64_t least) -> int64_t {      // exact only below `least`
         units.clear();
         int64_t part_rows = 0, work = 0;
+        bool in_two = clusters, narrow = true;
         for (const Tile& t : tiles) {
             const int sl = len > 0 ? split_len_for(t.keys, len, key_granule) : t.keys;
             const int n = ceil_div(t.keys, sl);
             if (n > 1) part_rows += (int64_t)n * t.rows;
+            in_two &= n == 2; narrow &= t.rows <= 128;
             for (int s = 0; s < n; ++s) {
                 const int keys = std::min(t.keys, (s + 1) * sl) - s * sl;
                 units.push_back(ceil_div(keys, 128) * (t.rows > 128 ? kStepWide : kStepNarrow) + kUnit);
                 work += units.back();
             }
         }
-        const int64_t merge = part_rows > 0 ? kMergeLaunch + part_rows * H * (p->head_dim + 1) * 4 / kMergeBytesPerCycle : 0;
+        const int64_t merge = pieces_meet_in_clusters(p, num_sms, (int64_t)units.size() * H, in_two, narrow) ? kMergeCluster
+                              : part_rows > 0 ? kMergeLaunch + part_rows * H * (p->head_dim + 1) * 4 / kMergeBytesPerCycle : 0;
         std::sort(units.begin(), units.end(), std::greater<int64_t>());
         if ((int64_t)units.size() * H <= num_sms) return units[0] + merge;
         if (work * H / num_sms + merge >= least) return least;
@@ -351,7 +361,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
         psplit = 0;
         const int64_t want_ctas = (int64_t)num_sms * 2;
         if (tiles > 0 && tiles * H < want_ctas && use_tc5) {
-            psplit = pick_prefill_split(p, num_sms, &want_rows, key_granule);
+            psplit = pick_prefill_split(p, num_sms, &want_rows, key_granule, tile_kernel == 1);
         } else if (tiles > 0 && tiles * H < want_ctas) {
             // aim for want_ctas pieces of equal length, not shorter than 256 keys
             const int pieces = ceil_div((int)want_ctas, H);
@@ -386,16 +396,33 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
         }
     }
     p->num_verify_merge_rows = (int)p->merge_rows.size();
-    for (int r = 0; r < R; ++r) {
-        const int C = p->chunk_len[r], P = p->prefix_len[r];
-        if (C <= verify_max_rows) continue;
-        for (int row0 = 0; row0 < C; row0 += tile_rows) {
-            const int rows_valid = std::min(tile_rows, C - row0);
-            const int kv_end = P + row0 + rows_valid;
-            const int sl = psplit > 0 ? split_len_for(kv_end, psplit, key_granule) : 0;
-            emit_tile(p, p->prefill_items, r, row0, rows_valid, kv_end, sl);
+    int cluster_merged = 0;                 // rows the one-CTA tile kernel merges itself
+    auto each_tile = [&](auto&& f) {
+        for (int r = 0; r < R; ++r) {
+            const int C = p->chunk_len[r];
+            if (C <= verify_max_rows) continue;
+            for (int row0 = 0; row0 < C; row0 += tile_rows) {
+                const int rows_valid = std::min(tile_rows, C - row0), kv_end = p->prefix_len[r] + row0 + rows_valid;
+                f(r, row0, rows_valid, kv_end, psplit > 0 ? split_len_for(kv_end, psplit, key_granule) : 0);
+            }
         }
-    }
+    };
+    bool in_two = tile_kernel == 1, narrow = true;
+    int64_t pieces = 0;
+    each_tile([&](int, int, int rows, int kv_end, int sl) {
+        in_two &= sl > 0 && ceil_div(kv_end, sl) == 2;
+        narrow &= rows <= 128;
+        pieces += 2;
+    });
+    p->tile_clusters = pieces > 0 && pieces_meet_in_clusters(p, num_sms, pieces * H, in_two, narrow);
+    each_tile([&](int r, int row0, int rows, int kv_end, int sl) {
+        if (!p->tile_clusters) { emit_tile(p, p->prefill_items, r, row0, rows, kv_end, sl); return; }
+        // one piece behind the other: the CTAs of a cluster
+        for (int b = 0; b < kv_end; b += sl)
+            p->prefill_items.push_back(WorkItem{r, row0, b, std::min(kv_end, b + sl), -1, p->prefix_len[r], p->chunk_len[r], p->cu_chunk[r]});
+        cluster_merged += rows;
+        info.max_splits = std::max(info.max_splits, 2);
+    });
     // longest pieces first so the tail of the grid is made of short ones
     auto longer = [](const WorkItem& a, const WorkItem& b) {
         return (a.kv_end - a.kv_begin) > (b.kv_end - b.kv_begin);
@@ -403,7 +430,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
     std::stable_sort(p->verify_items.begin(), p->verify_items.end(), longer);
     std::stable_sort(p->stream_items.begin(), p->stream_items.end(),
                      [](const StreamItem& a, const StreamItem& b) { return a.page1 - a.page0 > b.page1 - b.page0; });
-    std::stable_sort(p->prefill_items.begin(), p->prefill_items.end(), longer);
+    if (!p->tile_clusters) std::stable_sort(p->prefill_items.begin(), p->prefill_items.end(), longer);
 
     // Units of the persistent tcgen05 kernels, in the order the CTAs draw them: requests by their longest item first;
     // inside a request head by head, and for each head all items of the request one after the other, so that the row
@@ -434,7 +461,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
 
     info.num_verify_items = (int32_t)(p->verify_items.size() + p->stream_items.size());
     info.num_prefill_items = (int32_t)p->prefill_items.size();
-    info.num_merge_rows = (int32_t)p->merge_rows.size() + stream_merged;
+    info.num_merge_rows = (int32_t)p->merge_rows.size() + stream_merged + cluster_merged;
     const int64_t d = p->head_dim;
     int64_t part_out_bytes = p->part_rows * H * d * 4;
     part_out_bytes = (part_out_bytes + 255) / 256 * 256;
@@ -596,6 +623,7 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     p->append_first = append_first;
     p->num_piece_counters = 0;
     p->num_verify_merge_rows = 0;
+    p->tile_clusters = false;
     p->parts_made = false;
     p->is_part = part;
     p->captured = p->loose = p->loose_many = false;

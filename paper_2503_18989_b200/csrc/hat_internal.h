@@ -237,6 +237,7 @@ struct hat_plan {
     int64_t part_rows;          // partial rows in the workspace
     hat_plan_info info;
     hat::Timing* timing;        // null unless hat_plan_enable_timing was called
+    bool tile_clusters;         // tile units are pieces of tiles cut in two, in pairs that clusters of two CTAs merge
     int num_verify_merge_rows;  // merge rows of streaming-class requests; they come first in merge_rows
     cudaStream_t last_stream;   // stream of the previous attention call
     bool has_last;
@@ -322,16 +323,22 @@ void count_launch(int n = 1);
 #ifdef __CUDACC__
 // Launches a kernel that calls tc5::pdl_wait before it touches what earlier kernels of the stream write or read
 template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
+cudaError_t launch_pdl_clusters(unsigned cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
     count_launch();
     return e;
+}
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
+    return launch_pdl_clusters(1, kern, grid, block, smem, stream, args...);
 }
 #endif
 void set_last_cuda_error(int e);   // what hat_last_cuda_error() returns on this thread

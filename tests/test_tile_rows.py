@@ -16,6 +16,17 @@ def test_one_request(cuda_device, dtype, prefix, chunk, rows, monkeypatch):
     _check(_batch(dtype, 3, 128, [prefix], [chunk], 11), cuda_device)
 
 
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("split", ["128", "256", "896"])     # both halves in a cluster, ragged halves, more pieces than two
+@pytest.mark.parametrize("prefix,chunk", [(0, 129), (0, 256), (255, 100), (383, 128), (700, 256), (1000, 17), (1663, 300)])
+def test_tiles_cut_in_two(cuda_device, dtype, prefix, chunk, split, monkeypatch):
+    """Calls follow without a wait, so that a cluster's shared memory is in use when the next one starts."""
+    monkeypatch.setenv("HAT_PREFILL_KERNEL", "tc5")
+    monkeypatch.setenv("HAT_PREFILL_TILE_ROWS", "128")
+    monkeypatch.setenv("HAT_PREFILL_SPLIT_LEN", split)
+    _check(_batch(dtype, 5, 128, [prefix], [chunk], 17), cuda_device, repeat=5)
+
+
 @pytest.mark.parametrize("chunk", [129, 256, 301])
 def test_output_in_the_cache_type(cuda_device, chunk):
     import torch
