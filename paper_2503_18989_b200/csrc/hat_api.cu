@@ -272,7 +272,9 @@ static int pick_prefill_split(const hat_plan* p, int num_sms, int* tile_rows, in
 // So requests are cut only when the longest one alone would take longer than HBM needs for the batch, and then into as
 // many pieces as the CTAs can take in one round, or in one more round than the whole requests need (16 requests x 8 K/V heads
 // x 2 slabs: 124 us whole, 95 us in 400 units, 93 us in 576, 89 us in 1000, 99 us in 1900).
+static int pick_verify_split_slabs(const hat_plan* p, int num_sms);
 static int pick_verify_split(const hat_plan* p, int num_sms) {
+    if (p->verify_subtiles > 1) return pick_verify_split_slabs(p, num_sms);
     constexpr int kWhole = 1 << 24, kLeast = 96;       // shorter pieces than 6 pages only add to the merge
     const double tp = 0.25 * p->head_dim / 128;   // us per page of a CTA that has the SM's share of HBM to itself
     const double tb = p->head_dim * 64 / 6.45e6;                               // us per page (K and V) at the measured HBM rate
@@ -307,6 +309,53 @@ static int pick_verify_split(const hat_plan* p, int num_sms) {
         if (units_at(mid * kPageSize) <= most) hi = mid; else lo = mid + 1;
     }
     return time_of(lo * kPageSize) + kCut < time_of(longest) ? lo * kPageSize : kWhole;
+}
+
+// The same for batches with more than one slab of 16 pairs a K/V head.  There mma.sync is the limit, not HBM: a page takes a slab
+// about the same time however many CTAs run, so what counts is how evenly the units fill the CTAs.  Every candidate
+// length (the longest request in 1, 1.5, 2 ... 8 pieces) is priced by placing its units, longest first, on the CTAs; all heads of a piece are
+// alike, so as many as divide evenly are placed as one.  Measured, us, rule above / this, bf16: 16 requests of 1300 to 7800 tokens x 8 K/V
+// heads x 16..32 pairs 92.4 / 86.3, 10 x 16 heads 119.7 / 91.2, 12 of up to 2048 tokens 33.1 / 27.4, 16 x 8 heads x 8..64 pairs 129.2 /
+// 103.7, 8 x 8 heads 51.9 / 52.8.
+static int pick_verify_split_slabs(const hat_plan* p, int num_sms) {
+    const double page = 0.26 * p->head_dim / 128, unit = 0.8, cut = 3.0;       // us: a page, a unit, a piece of a cut request
+    const int group = p->num_heads / p->num_kv_heads;
+    int alike = 1;
+    for (int g = 2; g <= 8; ++g) if (p->num_kv_heads % g == 0) alike = g;
+    const int copies = p->num_kv_heads / alike, slots = std::max(1, 2 * num_sms / alike);
+    int longest = 0;
+    for (int r = 0; r < p->num_requests; ++r)
+        if (p->chunk_len[r] >= 1 && p->chunk_len[r] <= 16) longest = std::max(longest, p->prefix_len[r] + p->chunk_len[r]);
+    std::vector<double> times, load;
+    auto price = [&](int len) {
+        times.clear();
+        for (int r = 0; r < p->num_requests; ++r) {
+            const int C = p->chunk_len[r];
+            if (C < 1 || C > 16) continue;
+            const int keys = p->prefix_len[r] + C, n = ceil_div(keys, split_len_for(keys, len, kPageSize));
+            const int pages = ceil_div(p->prefix_len[r], kPageSize) + 1;
+            times.insert(times.end(), (size_t)n * copies * ceil_div(C * group, 16), (double)pages / n * page + unit + (n > 1 ? cut : 0.0));
+        }
+        std::sort(times.begin(), times.end(), std::greater<double>());
+        load.assign(slots, 0.0);                                       // a heap, least loaded first
+        double most = 0.0;
+        for (double t : times) {
+            std::pop_heap(load.begin(), load.end(), std::greater<double>());
+            load.back() += t;
+            most = std::max(most, load.back());
+            std::push_heap(load.begin(), load.end(), std::greater<double>());
+        }
+        return most;
+    };
+    int best = 1 << 24;
+    double least = price(best);
+    for (int halves = 3; halves <= 16; ++halves) {
+        const int len = std::max(96, round_up(ceil_div(2 * longest, halves), kPageSize));
+        const double t = price(len);
+        if (t < 0.98 * least) { least = t; best = len; }
+        if (len == 96) break;
+    }
+    return best;
 }
 
 // tile_kernel: 0 = mma.sync, 1 = tcgen05 with two query tiles per CTA, 3 = tcgen05 by pairs of CTAs (cta_group::2) with a
