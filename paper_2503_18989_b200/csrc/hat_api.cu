@@ -797,6 +797,16 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     return HAT_OK;
 }
 
+cudaError_t plan_begin(hat_plan* p, cudaStream_t s) {
+    if (p->loose && !p->loose_many && p->loose_stream == s) p->loose = false;      // ev_done, recorded on s by plan_end, covers it
+    return p->has_last && p->last_stream != s ? cudaStreamWaitEvent(s, p->res.ev_done, 0) : cudaSuccess;
+}
+
+void plan_end(hat_plan* p, cudaStream_t s) {
+    if (cudaEventRecord(p->res.ev_done, s) == cudaSuccess) { p->last_stream = s; p->has_last = true; }
+    else p->loose = p->loose_many = true;
+}
+
 // One attention step; the final rows go to `out` (fp32) or, when out16 is given, to out16 in the cache's 16-bit type.
 int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
                          const void* v_new, float* out, void* out16, float* lse, float sm_scale, void* workspace,
@@ -826,15 +836,10 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return cuda_fail(e);
     const bool capturing = cap != cudaStreamCaptureStatusNone;
     if (capturing) mplan->captured = true;
-    else if (plan->loose && !plan->loose_many && plan->loose_stream == s) mplan->loose = false;   // ev_done, recorded on s below, covers it
-    if (!capturing && plan->has_last && plan->last_stream != s && (e = cudaStreamWaitEvent(s, plan->res.ev_done, 0)) != cudaSuccess)
-        return cuda_fail(e);
+    else if ((e = plan_begin(mplan, s)) != cudaSuccess) return cuda_fail(e);
     struct Done {
         hat_plan* p; cudaStream_t s; bool record;
-        ~Done() {
-            if (record && cudaEventRecord(p->res.ev_done, s) == cudaSuccess) { p->last_stream = s; p->has_last = true; }
-            else if (record) { p->loose = p->loose_many = true; }
-        }
+        ~Done() { if (record) plan_end(p, s); }
     } done{mplan, s, !capturing};
     // optional event recorder: a start and an end event per slot (append, tile, streaming, merge)
     Timing* tm = plan->timing;

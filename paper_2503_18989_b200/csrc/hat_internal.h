@@ -319,6 +319,11 @@ struct HostBuffers { const void *q, *k, *v; void *out, *lse; };
 int host_step(const hat_cache_desc* cache, const hat_plan* plan, const HostBuffers& host, const HostBuffers& dev, float sm_scale,
               void* workspace, size_t workspace_bytes, cudaStream_t s, cudaError_t* err);
 void plan_note_call(hat_plan* p, cudaStream_t s);           // a call other than attention is about to use the plan on s
+// The plan's device state and the caller's workspace serve one attention call at a time.  plan_begin: what follows on s runs
+// behind the plan's previous call, wherever that was enqueued; plan_end: what was enqueued on s so far is the previous call
+// from now on.  Not for calls inside a stream capture.
+cudaError_t plan_begin(hat_plan* p, cudaStream_t s);
+void plan_end(hat_plan* p, cudaStream_t s);
 void count_launch(int n = 1);
 #ifdef __CUDACC__
 // Launches a kernel that calls tc5::pdl_wait before it touches what earlier kernels of the stream write or read

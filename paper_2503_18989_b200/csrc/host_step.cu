@@ -127,6 +127,14 @@ int host_step(const hat_cache_desc* cache, const hat_plan* plan, const HostBuffe
         return e == cudaSuccess;
     };
     if (!edge(s, in) || !edge(s, out)) return HAT_ERR_CUDA;
+    // The parts' kernels run behind the plan's previous call and its next one behind them, like those of a call in one part;
+    // the copies in (to the caller's staging memory) need not wait for that.
+    if ((e = plan_begin(p, s)) != cudaSuccess) return HAT_ERR_CUDA;
+    struct Done {
+        hat_plan* p; cudaStream_t s;
+        void now() { if (p) plan_end(p, s); p = nullptr; }
+        ~Done() { now(); }
+    } done{p, s};
     const size_t n = p->parts.size();
     for (size_t i = 0; i < n; ++i) {
         hat_plan* part = p->parts[i];
@@ -141,6 +149,7 @@ int host_step(const hat_cache_desc* cache, const hat_plan* plan, const HostBuffe
         if (!edge(s, out)) return HAT_ERR_CUDA;
     }
     if ((e = cudaEventRecord(p->res.ev_verify, s)) != cudaSuccess) return HAT_ERR_CUDA;
+    done.now();                                              // before the last copies back: they are no one's business but the caller's
     if (!copy_out(p->part_row[n - 1], p->parts[n - 1]->total_rows, out) || !edge(out, s)) return HAT_ERR_CUDA;
     return HAT_OK;
 }

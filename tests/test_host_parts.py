@@ -51,3 +51,59 @@ def test_parts_of_a_host_call(cuda_device, dtype, group, tree, pinned):
     gk, gv = cache.pools_to_host()
     assert np.array_equal(gk, kp) and np.array_equal(gv, vp) and ds.canaries_intact()
     ds.close()
+
+
+@pytest.mark.parametrize("first,second", [("host", "device"), ("device", "host"), ("host", "host")])
+def test_a_call_in_parts_and_the_plans_other_calls_are_ordered(cuda_device, first, second):
+    """Two calls of one plan on two streams: the second one's kernels wait for the first, whichever of them copies from host
+    buffers in parts.  The first call is held back by a kernel in front of it; some requests are cut, so that both calls use
+    the plan's workspace."""
+    import torch
+    from paper_2503_18989_b200 import binding as B, runner
+    H, d = 5, 128
+    sc = _batch("fp16", H, d, _PREFIX + [30000], _CHUNK + [4], 302)
+    st = sc.steps[0]
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, st)
+    assert ds.info["max_splits"] > 1 and ds.workspace_bytes > 0
+    T = st.total_rows
+    q, k, v = (torch.from_numpy(a.view(np.int16)).pin_memory() for a in (st.q, st.k_new, st.v_new))
+    nbytes = B.hat_plan_staging_bytes(ds.plan)
+    bufs = [(torch.full((T, H, d), float("nan")).pin_memory(), torch.full((T, H), float("nan")).pin_memory(),
+             torch.empty(nbytes, dtype=torch.uint8, device=cuda_device)) for _ in range(2)]
+    streams = [torch.cuda.Stream(cuda_device) for _ in range(2)]
+
+    def call(kind, i):
+        if kind == "device":
+            ds.attend(stream=streams[i].cuda_stream)
+        else:
+            o, l, stg = bufs[i]
+            B.hat_chunk_attention_host(cache.desc, ds.plan, q, k, v, o, l, 0.0, stg, nbytes, ds.workspace, ds.workspace_bytes,
+                                       streams[i].cuda_stream)
+
+    before = B.hat_launch_count()
+    call("host", 0)                                                   # the parts are planned, everything is loaded
+    assert B.hat_launch_count() - before >= 4
+    torch.cuda.synchronize()
+    for t in (ds.out, ds.lse, *(x for o, l, _ in bufs for x in (o, l))):
+        t.fill_(float("nan"))
+    torch.cuda.synchronize()
+    held, done = torch.cuda.Event(), torch.cuda.Event()
+    with torch.cuda.stream(streams[0]):
+        torch.cuda._sleep(1_000_000_000)                              # about half a second
+        held.record()
+    call(first, 0)
+    call(second, 1)
+    done.record(streams[1])
+    while not held.query():
+        assert not done.query() or held.query(), "the second call did not wait for the first"
+    torch.cuda.synchronize()
+    assert B.hat_last_device_status(ds.plan) == B.HAT_OK
+    kp, vp, want = oracle_replay(sc)
+    got = [(bufs[i][0].numpy(), bufs[i][1].numpy()) if kind == "host" else ds.results() for i, kind in enumerate((first, second))]
+    for o, l in got:
+        assert_parity(o, want[0][0], "out")
+        assert_parity(l, want[0][1], "lse")
+    gk, gv = cache.pools_to_host()
+    assert np.array_equal(gk, kp) and np.array_equal(gv, vp) and ds.canaries_intact()
+    ds.close()
