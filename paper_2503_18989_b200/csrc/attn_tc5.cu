@@ -70,32 +70,27 @@ template <int D> constexpr uint32_t smem_bytes() { return 1024 /*alignment slack
 static_assert(smem_bytes<128>() <= 227 * 1024, "shared memory of one CTA");
 constexpr int kThreads = 320;   // producer warp, MMA warp, two softmax warpgroups
 
-// Bounded wait.  Returns false if the wait gave up or another role already did.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Barriers* b, int32_t* status) {
+// Bounded wait.  Returns false if the wait gave up or another role already did.  It is inlined some thirty times, so it holds no more
+// than it must: the CTA reports to the status word once, at its end (see "Code size" at the kernel).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Barriers* b) {
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
-    while (!mbar_try(bar, parity)) {
-        if (b->abort_flag) return false;
-        if (clock64() - t0 > b->wait_cycles) {
+    while (!mbar_try(bar, parity))
+        if (b->abort_flag || clock64() - t0 > b->wait_cycles) {
             b->abort_flag = 1;
-            atomicOr(status, 1);
             return false;
         }
-    }
     return true;
 }
 
 // The same for a barrier the cluster's other CTA arrives on, acquiring what it wrote before.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, Barriers* b, int32_t* status) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, Barriers* b) {
     const long long t0 = clock64();
-    while (!mbar_try_cluster(bar, parity)) {
-        if (b->abort_flag) return false;
-        if (clock64() - t0 > b->wait_cycles) {
+    while (!mbar_try_cluster(bar, parity))
+        if (b->abort_flag || clock64() - t0 > b->wait_cycles) {
             b->abort_flag = 1;
-            atomicOr(status, 1);
             return false;
         }
-    }
     return true;
 }
 
@@ -142,7 +137,11 @@ __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* _
 //            (one request of 256 rows x 32 heads, us a call: prefix 768
 //            19.4 -> 13.4, 1792 23.9 -> 17.9, 4000 38.9 -> 32.3)
 enum Form { kMany, kOne, kHalves };
-template <bool BF16, int kD, int FORM>
+// Code size: the loops of the roles run side by side and have to share the instruction cache; what else the kernel holds, executed or
+// not, costs misses.  Calls that append nothing therefore get a kernel without the code for it (APPEND = false), and a wait is
+// as short as it can be.  One call of 30 ragged chunks x 32 heads, fp16, nothing appended: 124 KB of code 417 us, 97 KB 387 us (64 columns:
+// 358 -> 327 us); instruction cache misses of 12 chunks 1.0 M -> 0.6 M, 133 -> 124 us.
+template <bool BF16, int kD, int FORM, bool APPEND>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units, int32_t* work_counter,
                 const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -219,7 +218,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         auto pay = [&]() {
             if (!owes) return;
             owes = false;
-            ok = mbar_wait(&bars->k_full[o_sk], o_pk, bars, status) && mbar_wait(&bars->v_full[o_sv], o_pv, bars, status);
+            ok = mbar_wait(&bars->k_full[o_sk], o_pk, bars) && mbar_wait(&bars->v_full[o_sv], o_pv, bars);
             ok = __all_sync(0xffffffffu, ok);
             if (ok && o_whole) {
                 tma_store_5d(&map_k, smem_u32(k_ring) + o_sk * kTileBytes + lane_off, 0, c1, 0, o_hk << s3, o_page << s4);
@@ -235,7 +234,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         for (int un = 0; ok; ++un) {
             const int slot = un & 1;
             if (un >= 2) {
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->unit_empty[slot], ((un >> 1) - 1) & 1, bars, status));
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->unit_empty[slot], ((un >> 1) - 1) & 1, bars));
                 if (!ok) break;
             }
             int unit = 0;
@@ -261,7 +260,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             int page = page_of(0);
             // Q tiles: the previous unit's last S must have read the old ones
             if (un > 0) {
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_empty, (un - 1) & 1, bars, status));
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_empty, (un - 1) & 1, bars));
                 if (!ok) break;
             } else if (!a.overlap) {
                 pdl_wait();                                      // up to here only the plan's own arrays were read
@@ -271,81 +270,65 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 tma_load_3d(smem_u32(q_tiles) + (lane / kHalves) * kTileBytes + (lane % kHalves) * kSlabBytes, &map_q, (lane % kHalves) * 64, u.h,
                             u.row_base + u.row0 + (lane / kHalves) * kRows, &bars->q_full);
             // tiles [0, n_plain) hold nothing of the chunk, or the call does not append
-            const bool fused = a.k_new != nullptr;
-            const int n_plain = fused ? min(u.n_all, max(0, u.P - u.kv_begin) / kKeys) : u.n_all;
+            const int n_plain = APPEND ? min(u.n_all, max(0, u.P - u.kv_begin) / kKeys) : u.n_all;
             const int c3 = u.hk << s3;
-            int j = 0;
-            for (; j < n_plain; ++j) {
-                const int npages = min(8, total_pages - 8 * j);
-                const bool mine = lane < boxes && pg < npages;
-                const int page_next = page_of(j + 1), c4 = page << s4;
-                HAT_CHECK(sk < kStagesK && sv < kStagesV, status);
-                if (stored) { tile_append::stores_read(); stored = false; }
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars, status));
-                if (!ok) break;
-                if (lane == 0) mbar_expect_tx(&bars->k_full[sk], npages * kPageBytes);
-                if (mine) tma_load_5d(smem_u32(k_ring) + sk * kTileBytes + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars, status));
-                if (!ok) break;
-                if (!withhold) {
-                    if (lane == 0) mbar_expect_tx(&bars->v_full[sv], npages * kPageBytes);
-                    if (mine) tma_load_5d(smem_u32(v_ring) + sv * kTileBytes + lane_off, &map_v, 0, c1, 0, c3, c4, &bars->v_full[sv]);
-                }
-                if (owes) pay();                                 // the previous unit's last tile
-                withhold = false;
-                page = page_next;
-                step();
-            }
-            if (!ok) break;
-            if (j == u.n_all) continue;
-            // tiles with chunk positions
             const tile_append::Chunk ck{u.P, u.C, u.row_base, u.hk};
             // of the units that read a chunk page, the last row block of the group's first query head appends it
-            const bool appends = u.h == u.hk * a.plan.group && u.row0 + a.plan.tile_rows >= u.C;
-            for (; j < u.n_all; ++j) {
-                const int kb = u.kv_begin + j * kKeys;
+            const bool appends = APPEND && u.h == u.hk * a.plan.group && u.row0 + a.plan.tile_rows >= u.C;
+            for (int j = 0; j < u.n_all; ++j) {
                 const int npages = min(8, total_pages - 8 * j);
-                const int page_next = page_of(j + 1);
-                const int key0 = kb + pg * kPageSize;            // of this lane's page
-                // a page with both prefix and chunk rows is gathered and completes the barriers last
-                const int pe = (u.P - kb) / kPageSize;
-                const bool edge = u.P > kb && u.P % kPageSize != 0 && pe < npages;
-                const bool fresh = lane < 16 && pg < npages && ck.fresh(key0);
-                const bool pool = lane < boxes && pg < npages && !ck.fresh(key0) && !(edge && pg == pe);
-                const int row = u.row_base + key0 - u.P + 8 * grp;
-                const uint32_t bytes = (npages - (edge ? 1 : 0)) * kPageBytes;
-                if (stored) { tile_append::stores_read(); stored = false; }
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars, status));
-                if (!ok) break;
+                const int page_next = page_of(j + 1), c4 = page << s4;
+                const bool plain = !APPEND || j < n_plain;
                 const uint32_t k_dst = smem_u32(k_ring) + sk * kTileBytes, v_dst = smem_u32(v_ring) + sv * kTileBytes;
-                if (lane == 0) { if (edge) mbar_expect_only(&bars->k_full[sk], bytes); else mbar_expect_tx(&bars->k_full[sk], bytes); }
-                if (fresh) tma_load_4d(k_dst + lane_off, &map_k_new, 0, row, 0, u.hk, &bars->k_full[sk]);
-                if (pool) tma_load_5d(k_dst + lane_off, &map_k, 0, c1, 0, c3, page << s4, &bars->k_full[sk]);
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars, status));
+                // in a tile with chunk positions: pages of the chunk alone come from k_new / v_new; a page with both prefix and
+                // chunk rows is gathered and completes the barriers last
+                const int kb = u.kv_begin + j * kKeys, key0 = kb + pg * kPageSize, pe = (u.P - kb) / kPageSize;
+                bool edge = false, fresh = false, pool = lane < boxes && pg < npages;
+                uint32_t bytes = npages * kPageBytes;
+                if (APPEND && !plain) {
+                    edge = u.P > kb && u.P % kPageSize != 0 && pe < npages;
+                    fresh = lane < 16 && pg < npages && ck.fresh(key0);
+                    pool = pool && !ck.fresh(key0) && !(edge && pg == pe);
+                    if (edge) bytes -= kPageBytes;
+                }
+                const int row = u.row_base + key0 - u.P + 8 * grp;
+                HAT_CHECK(sk < kStagesK && sv < kStagesV, status);
+                if (APPEND && stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars));
+                if (!ok) break;
+                if (lane == 0) { if (APPEND && edge) mbar_expect_only(&bars->k_full[sk], bytes); else mbar_expect_tx(&bars->k_full[sk], bytes); }
+                if (pool) tma_load_5d(k_dst + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
+                if (APPEND && fresh) tma_load_4d(k_dst + lane_off, &map_k_new, 0, row, 0, u.hk, &bars->k_full[sk]);
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars));
                 if (!ok) break;
                 if (!withhold) {
-                    if (lane == 0) { if (edge) mbar_expect_only(&bars->v_full[sv], bytes); else mbar_expect_tx(&bars->v_full[sv], bytes); }
-                    if (fresh) tma_load_4d(v_dst + lane_off, &map_v_new, 0, row, 0, u.hk, &bars->v_full[sv]);
-                    if (pool) tma_load_5d(v_dst + lane_off, &map_v, 0, c1, 0, c3, page << s4, &bars->v_full[sv]);
+                    if (lane == 0) { if (APPEND && edge) mbar_expect_only(&bars->v_full[sv], bytes); else mbar_expect_tx(&bars->v_full[sv], bytes); }
+                    if (pool) tma_load_5d(v_dst + lane_off, &map_v, 0, c1, 0, c3, c4, &bars->v_full[sv]);
+                    if (APPEND && fresh) tma_load_4d(v_dst + lane_off, &map_v_new, 0, row, 0, u.hk, &bars->v_full[sv]);
                 }
-                if (edge) {
-                    const int at = __shfl_sync(0xffffffffu, page, pe);
-                    tile_append::gather_edge<kD>(a, ck, a.cache.k_pool, a.k_new, kD, 0, at, kb + pe * kPageSize, k_dst + pe * kPageBytes, kGroupBytes, lane);
-                    tile_append::gather_edge<kD>(a, ck, a.cache.v_pool, a.v_new, kD, 0, at, kb + pe * kPageSize, v_dst + pe * kPageBytes, kGroupBytes, lane);
-                    tile_append::gathered();
-                    if (lane == 0) { mbar_arrive(&bars->k_full[sk]); if (!withhold) mbar_arrive(&bars->v_full[sv]); }
-                }
-                pay();
-                if (!ok) break;
-                if (appends && !withhold) {
-                    owes = true;
-                    o_sk = sk; o_sv = sv; o_pk = pk ^ 1; o_pv = pv ^ 1; o_page = page; o_hk = u.hk;
-                    o_whole = lane < boxes && pg < npages && ck.whole(key0);
-                    // the pages that are not whole, row by row
-                    for (uint32_t left = __ballot_sync(0xffffffffu, lane < 8 && pg < npages && ck.partly(key0)); left; left &= left - 1) {
-                        const int from = __ffs(left) - 1, at = __shfl_sync(0xffffffffu, page, from);
-                        tile_append::store_rows<kD>(a, ck, a.k_dst, a.k_new, kD, 0, at, kb + from * kPageSize, lane);
-                        tile_append::store_rows<kD>(a, ck, a.v_dst, a.v_new, kD, 0, at, kb + from * kPageSize, lane);
+                if constexpr (APPEND) {
+                    if (edge) {
+                        const int at = __shfl_sync(0xffffffffu, page, pe);
+#pragma unroll 1
+                        for (int kv = 0; kv < 2; ++kv)
+                            tile_append::gather_edge<kD>(a, ck, kv ? a.cache.v_pool : a.cache.k_pool, kv ? a.v_new : a.k_new, kD, 0, at, kb + pe * kPageSize,
+                                                         (kv ? v_dst : k_dst) + pe * kPageBytes, kGroupBytes, lane);
+                        tile_append::gathered();
+                        if (lane == 0) { mbar_arrive(&bars->k_full[sk]); if (!withhold) mbar_arrive(&bars->v_full[sv]); }
+                    }
+                    pay();                                       // the tile before, or the previous unit's last
+                    if (!ok) break;
+                    if (appends && !plain && !withhold) {
+                        owes = true;
+                        o_sk = sk; o_sv = sv; o_pk = pk ^ 1; o_pv = pv ^ 1; o_page = page; o_hk = u.hk;
+                        o_whole = lane < boxes && pg < npages && ck.whole(key0);
+                        // the pages that are not whole, row by row
+                        for (uint32_t left = __ballot_sync(0xffffffffu, lane < 8 && pg < npages && ck.partly(key0)); left; left &= left - 1) {
+                            const int from = __ffs(left) - 1, at = __shfl_sync(0xffffffffu, page, from);
+#pragma unroll 1
+                            for (int kv = 0; kv < 2; ++kv)
+                                tile_append::store_rows<kD>(a, ck, kv ? a.v_dst : a.k_dst, kv ? a.v_new : a.k_new, kD, 0, at, kb + from * kPageSize, lane);
+                        }
                     }
                 }
                 withhold = false;
@@ -360,8 +343,10 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             work_counter[0] = 0;
             work_counter[1] = 0;
         }
-        if (ok) pay();
-        tile_append::stores_done();
+        if constexpr (APPEND) {
+            if (ok) pay();
+            tile_append::stores_done();
+        }
         if (!ok) {
             // give copies already in flight a bounded chance to land before the CTA's shared memory is released
             const long long t0 = clock64();
@@ -384,13 +369,13 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             bool o_busy[2] = {false, false};          // O_t holds a finished unit that its warpgroup may still be reading
             for (int un = 0; ok; ++un) {
                 const int slot = un & 1;
-                ok = mbar_wait(&bars->unit_full[slot], (un >> 1) & 1, bars, status);
+                ok = mbar_wait(&bars->unit_full[slot], (un >> 1) & 1, bars);
                 if (!ok) break;
                 const int unit = bars->unit_slot[slot];
                 mbar_arrive(&bars->unit_empty[slot]);
                 if (unit < 0) break;
                 const Unit u = decode_unit(a, items, unit);
-                ok = mbar_wait(&bars->q_full, un & 1, bars, status);
+                ok = mbar_wait(&bars->q_full, un & 1, bars);
                 if (!ok) break;
                 // the two kinds of unit get their own copy of the issue loop: every instruction of this thread counts
                 auto run_unit = [&](auto split_tag) {
@@ -401,7 +386,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         const int j = SPLIT ? 2 * sidx + qt : sidx;
                         const int kt = kt_base + j, st = kt % kStagesK;
                         if (k_ready < j) {
-                            ok = mbar_wait(&bars->k_full[st], (kt / kStagesK) & 1, bars, status);
+                            ok = mbar_wait(&bars->k_full[st], (kt / kStagesK) & 1, bars);
                             k_ready = j;
                             if (!ok) return;
                         }
@@ -426,18 +411,18 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         const int j = SPLIT ? 2 * sidx + qt : sidx;
                         const int kt = kt_base + j, st = kt % kStagesV;
                         if (v_ready < j) {
-                            ok = mbar_wait(&bars->v_full[st], (kt / kStagesV) & 1, bars, status);
+                            ok = mbar_wait(&bars->v_full[st], (kt / kStagesV) & 1, bars);
                             v_ready = j;
                             if (!ok) return;
                         }
                         if (sidx == 0 && o_busy[qt]) {
                             // the accumulator still holds the previous unit: wait until its rows are in registers
-                            ok = mbar_wait(&bars->o_free[qt], f_cnt[qt] & 1, bars, status);
+                            ok = mbar_wait(&bars->o_free[qt], f_cnt[qt] & 1, bars);
                             ++f_cnt[qt];
                             o_busy[qt] = false;
                             if (!ok) return;
                         }
-                        ok = mbar_wait(&bars->p_ready[qt], p_cnt[qt] & 1, bars, status);
+                        ok = mbar_wait(&bars->p_ready[qt], p_cnt[qt] & 1, bars);
                         ++p_cnt[qt];
                         if (!ok) return;
                         tc_fence_after();
@@ -498,7 +483,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         bool ok = true;
         for (int un = 0; ok; ++un) {
             const int slot = un & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(&bars->unit_full[slot], (un >> 1) & 1, bars, status));
+            ok = __all_sync(0xffffffffu, mbar_wait(&bars->unit_full[slot], (un >> 1) & 1, bars));
             if (!ok) break;
             const int unit = bars->unit_slot[slot];
             __syncwarp();                                    // every lane has read the slot
@@ -513,7 +498,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 for (int sidx = 0; sidx < n_mine; ++sidx) {
                     const int j = u.tile_of(qt, sidx);       // key tile of this step
                     const int kb = u.kv_begin + j * kKeys;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&bars->s_full[qt], s_cnt & 1, bars, status));
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bars->s_full[qt], s_cnt & 1, bars));
                     ++s_cnt;
                     if (!ok) break;
                     tc_fence_after();
@@ -569,7 +554,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     // O may only be rescaled once the previous P V product has finished; waiting here every tile (it
                     // has long completed by now) also keeps this thread's count of the barrier's phases exact
                     if (sidx > 0) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done[qt], o_cnt & 1, bars, status));
+                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done[qt], o_cnt & 1, bars));
                         ++o_cnt;
                         if (!ok) break;
                         tc_fence_after();
@@ -590,7 +575,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     // slots); zero them so that 0 * garbage cannot produce NaN (both warpgroups may do it: same zeros)
                     if (kb + kKeys > u.kv_end) {
                         const int kt = kt_base + j;
-                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_full[kt % kStagesV], (kt / kStagesV) & 1, bars, status));
+                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_full[kt % kStagesV], (kt / kStagesV) & 1, bars));
                         if (!ok) break;
                         unsigned char* vt = v_ring + (kt % kStagesV) * kTileBytes;
                         const int first = u.kv_end - kb;
@@ -609,7 +594,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 if (!ok) break;
                 // ---- output of the unit
                 if (n_mine > 0) {                            // uniform over the warpgroup
-                    ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done[qt], o_cnt & 1, bars, status));
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done[qt], o_cnt & 1, bars));
                     ++o_cnt;
                     if (!ok) break;
                     tc_fence_after();
@@ -625,7 +610,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(qt == 0 ? &bars->x_ready0 : &bars->x_ready);
-                        ok = __all_sync(0xffffffffu, mbar_wait(qt == 0 ? &bars->x_ready : &bars->x_ready0, 0, bars, status));
+                        ok = __all_sync(0xffffffffu, mbar_wait(qt == 0 ? &bars->x_ready : &bars->x_ready0, 0, bars));
                         if (!ok) break;
                         tc_fence_after();
                         const float2 c0 = x0[t], c1 = bars->xchg[t];
@@ -675,7 +660,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         *ml = make_float2(m_used, l);
                         __syncwarp();
                         if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bars->peer_ready[warp - 2]), rank ^ 1u));
-                        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&bars->peer_ready[warp - 2], 0, bars, status));
+                        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&bars->peer_ready[warp - 2], 0, bars));
                         if (!ok) break;
                         const float2 other = ld_cluster_f2(map_to_cta(smem_u32(ml), rank ^ 1u));
                         const uint32_t from = map_to_cta(smem_u32(give), rank ^ 1u);
@@ -728,7 +713,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     }
                     if (u.split && u.n_t1 > 0) {
                         // merge the second chain (disjoint keys): weights 2^(m_t - m), sums and accumulators add up
-                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->x_ready, x_cnt & 1, bars, status));
+                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->x_ready, x_cnt & 1, bars));
                         ++x_cnt;
                         if (!ok) break;
                         tc_fence_after();
@@ -801,6 +786,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
 
     tc_fence_before();
     __syncthreads();
+    if (threadIdx.x == 0 && bars->abort_flag) atomicOr(status, 1);
     if constexpr (FORM == kHalves) {
         cluster_arrive();                                        // the other CTA has read what it needs of this one's shared memory
         cluster_wait();
@@ -851,10 +837,14 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     const bool d128 = plan->head_dim == 128;
     const bool one = d128 && total_units <= ctas && a2.static_first;
     if (plan->tile_clusters && !one) return cudaErrorInvalidValue;
-    auto kern = !d128 ? (bf16 ? attn_tc5_kernel<true, 64, kMany> : attn_tc5_kernel<false, 64, kMany>)
-                : plan->tile_clusters ? (bf16 ? attn_tc5_kernel<true, 128, kHalves> : attn_tc5_kernel<false, 128, kHalves>)
-                : one ? (bf16 ? attn_tc5_kernel<true, 128, kOne> : attn_tc5_kernel<false, 128, kOne>)
-                      : (bf16 ? attn_tc5_kernel<true, 128, kMany> : attn_tc5_kernel<false, 128, kMany>);
+    auto form = [&](auto b, auto app) {
+        constexpr bool B = decltype(b)::value, A = decltype(app)::value;
+        return !d128 ? attn_tc5_kernel<B, 64, kMany, A> : plan->tile_clusters ? attn_tc5_kernel<B, 128, kHalves, A>
+               : one ? attn_tc5_kernel<B, 128, kOne, A> : attn_tc5_kernel<B, 128, kMany, A>;
+    };
+    using Yes = std::true_type;
+    using No = std::false_type;
+    auto kern = args.k_new ? (bf16 ? form(Yes{}, Yes{}) : form(No{}, Yes{})) : (bf16 ? form(Yes{}, No{}) : form(No{}, No{}));
     const uint32_t smem = d128 ? smem_bytes<128>() : smem_bytes<64>();
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), (int)smem);
     if (e != cudaSuccess) return e;

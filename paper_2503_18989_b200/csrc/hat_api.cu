@@ -358,6 +358,20 @@ static int pick_verify_split_slabs(const hat_plan* p, int num_sms) {
     return best;
 }
 
+// Whether the chunk's rows are appended by a kernel in front of the one-CTA tile kernel instead of inside it.  Inside, the append costs
+// no launch and no second read, but the instructions for it crowd the kernel's loops out of the instruction cache and its producer
+// works on units with chunk pages longer; in front, it costs a launch and the bytes once more.  So in front where CTAs have
+// several units each and a unit is short work: 64 columns, or on average at most one query tile.  Measured, us inside / in front, fp16, 32
+// heads: 30 chunks of 32 to 128 rows at up to 512 90 / 77, at up to 2048 147 / 128, 64 columns 72 / 56 and 117 / 93; 30 of 64 to 512 at up to
+// 4096 365 / 368, 64 columns 311 / 296; 30 of 64 to 256 at up to 512 115 / 120; with less than two units a CTA 8 of 64 to 256 50 / 54.  The
+// CTA-pair kernel, whose loops are smaller, appends inside (30 chunks, bf16, 433 / 441).
+static bool append_is_apart(const hat_plan* p, int num_sms, int tile_rows) {
+    int64_t tiles = 0, rows = 0;
+    for (int r = 0; r < p->num_requests; ++r)
+        if (p->chunk_len[r] > 16) { tiles += ceil_div(p->chunk_len[r], tile_rows); rows += p->chunk_len[r]; }
+    return tiles * p->num_heads > 2 * (int64_t)num_sms && (p->head_dim == 64 || rows <= 128 * tiles);
+}
+
 // tile_kernel: 0 = mma.sync, 1 = tcgen05 with two query tiles per CTA, 3 = tcgen05 by pairs of CTAs (cta_group::2) with a
 // ring of three score buffers; both tcgen05 kernels take 256-row units
 static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
@@ -464,6 +478,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
         pieces += 2;
     });
     p->tile_clusters = pieces > 0 && pieces_meet_in_clusters(p, num_sms, pieces * H, in_two, narrow);
+    p->append_apart = tile_kernel == 1 && append_is_apart(p, num_sms, tile_rows);
     each_tile([&](int r, int row0, int rows, int kv_end, int sl) {
         if (!p->tile_clusters) { emit_tile(p, p->prefill_items, r, row0, rows, kv_end, sl); return; }
         // one piece behind the other: the CTAs of a cluster
@@ -673,6 +688,7 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     p->num_piece_counters = 0;
     p->num_verify_merge_rows = 0;
     p->tile_clusters = false;
+    p->append_apart = false;
     p->parts_made = false;
     p->is_part = part;
     p->captured = p->loose = p->loose_many = false;
@@ -850,9 +866,9 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
         if (call >= 0 && end) tm->launched[(size_t)call * HAT_TIMING_SLOTS + slot] = 1;
     };
     // the attention kernels append on the way, each class its own requests' rows, unless pages are shared between a writer and
-    // a reader or a class runs on the mma.sync kernels
+    // a reader, a class runs on the mma.sync kernels, or a kernel in front is cheaper
     const bool has_verify = plan->info.num_verify_items > 0;
-    const bool fused = k_new && !plan->append_first && (!has_verify || plan->info.stream_kernel == 1) &&
+    const bool fused = k_new && !plan->append_first && !plan->append_apart && (!has_verify || plan->info.stream_kernel == 1) &&
                        (plan->prefill_items.empty() || plan->info.prefill_kernel != 0);
     if (k_new && !fused) {
         mark(0, 0);

@@ -238,6 +238,7 @@ struct hat_plan {
     hat_plan_info info;
     hat::Timing* timing;        // null unless hat_plan_enable_timing was called
     bool tile_clusters;         // tile units are pieces of tiles cut in two, in pairs that clusters of two CTAs merge
+    bool append_apart;          // calls that append do so in a kernel of their own (see append_is_apart)
     int num_verify_merge_rows;  // merge rows of streaming-class requests; they come first in merge_rows
     cudaStream_t last_stream;   // stream of the previous attention call
     bool has_last;

@@ -5,8 +5,8 @@
 // so that nothing has to be appended before the kernel starts.  The pool is written on the way: one unit per (request, K/V
 // head, page) stores the page from the ring slot it was loaded into (TMA store, no registers, no second read).  A page that
 // the chunk shares with the prefix (prefix not a multiple of 16) is gathered row by row, and a page that the chunk shares or
-// does not fill is stored row by row.  A kernel of its own in front took 34 us on 30 ragged chunks (218 MB) and 4 us plus a
-// gap of 2 us on a single 256-row chunk.
+// does not fill is stored row by row.  A kernel of its own in front takes 34 us on 30 ragged chunks (218 MB) and 2 to 4 us on a
+// single 256-row chunk; append_is_apart (hat_api.cu) says where that is the cheaper way all the same.
 #pragma once
 #include "hat_internal.h"
 #include "tc5_ptx.cuh"

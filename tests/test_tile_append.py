@@ -76,3 +76,22 @@ def test_wide_and_narrow_units_together_back_to_back(cuda_device):
     chunk = rng.choice([17, 64, 100, 128, 200, 256, 300, 512], size=9).tolist()
     prefix = rng.integers(0, 1500, size=9).tolist()
     _check(_batch("bf16", 8, 128, prefix, chunk, 81), cuda_device, repeat=20)
+
+
+@pytest.mark.parametrize("d,drafts", [(128, False), (128, True), (64, False)])
+@pytest.mark.parametrize("requests,apart", [(37, False), (38, True)])     # 8 heads: two units a CTA at most, and just above
+def test_append_in_front_of_many_short_units(cuda_device, d, drafts, requests, apart):
+    """Above two units a CTA of the one-CTA kernel, short ones, a kernel in front appends; the launches tell which way it went."""
+    from paper_2503_18989_b200 import binding as B, runner
+    rng = np.random.default_rng(requests)
+    prefix = rng.integers(0, 400, size=requests).tolist() + ([700, 33] if drafts else [])
+    chunk = rng.integers(17, 128, size=requests).tolist() + ([4, 16] if drafts else [])
+    sc = _batch("fp16", 8, d, prefix, chunk, 95)
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, sc.steps[0])
+    assert ds.info["prefill_kernel"] == 1 and ds.info["prefill_split_len"] == 0      # (cut drafts are merged without a launch)
+    before = B.hat_launch_count()
+    ds.attend()
+    assert B.hat_launch_count() - before == 1 + drafts + apart
+    ds.close()
+    _check(sc, cuda_device, repeat=2)
