@@ -109,20 +109,6 @@ constexpr int kThreads = 384;   // K producer, P V issuer / forwarder, two softm
 constexpr int kQueueReaders0 = 2 + 8 + 1;    // CTA 0: the two MMA threads, softmax warps, V producer (the K producer drew the unit itself)
 constexpr int kQueueReaders1 = 2 + 1 + 8;    // CTA 1: both producer warps, forwarding thread, softmax warps
 
-#ifdef HAT_PHASE_TIMERS
-// Diagnostic build only: cycles spent per phase, summed over all CTAs (clock64 stamps around the phases).
-__device__ unsigned long long g_phase[80];
-#define PH_T0(v) long long v = clock64()
-#define PH_ADD(slot, v) do { const long long now_ = clock64(); ph[slot] += now_ - v; v = now_; } while (0)
-#define PH_DECL(n) long long ph[n] = {0}
-#define PH_FLUSH(base, n) do { for (int i_ = 0; i_ < n; ++i_) atomicAdd(&g_phase[base + i_], (unsigned long long)ph[i_]); } while (0)
-#else
-#define PH_T0(v)
-#define PH_ADD(slot, v)
-#define PH_DECL(n)
-#define PH_FLUSH(base, n)
-#endif
-
 struct Ctx {
     Barriers* bars;
     int32_t* status;
@@ -245,8 +231,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch (CTA 0) + TMA producer (both)
         bool ok = true;
-        PH_DECL(8);
-        PH_T0(tq0);
         // CTA 0: draw a unit and publish it in slot un % 4 of both CTAs' queues (all lanes return it); the slot is free
         // once every reader in both CTAs has read the unit published four draws earlier
         auto publish = [&](int un) -> int {
@@ -318,7 +302,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 next_unit = publish(un + 1);
                 if (!ok) break;
             }
-            PH_ADD(0, tq0);
             if (un >= 2) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_empty[qs], ((un >> 1) - 1) & 1, cx));
                 if (!ok) break;
@@ -327,7 +310,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             if (lane < 2)      // lane = column half; this CTA's 128 rows
                 tma_load_3d(smem_u32(q_tiles) + qs * kTileBytes + lane * kSlabBytes, &map_q, lane * 64, u.h,
                             u.row_base + u.row0 + (int)rank * kRows, &bars->q_full[qs]);
-            PH_ADD(1, tq0);
             // tiles [0, n_plain) hold nothing of the chunk, or the call does not append
             const int n_plain = a.k_new != nullptr ? min(u.n, max(0, u.P - u.kv_begin) / kKeys) : u.n;
             const int c3 = u.hk << s3;
@@ -338,18 +320,12 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 const int nk = max(0, min(4, npages - 4 * (int)rank));                            // K pages this CTA loads
                 const int page_next = page_of(j + 1), c4 = page << s4;
                 HAT_CHECK(sk < kStagesK, cx.status);
-                PH_ADD(2, tq0);
                 if (stored) { tile_append::stores_read(); stored = false; }
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, cx));
                 if (!ok) break;
-                PH_ADD(3, tq0);
                 if (lane == 0) mbar_expect_tx(&bars->k_full[sk], nk * kKPageBytes);
                 if (lane < boxes && kpg < npages)
                     tma_load_5d(smem_u32(k_ring) + sk * kHalfBytes + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
-                PH_ADD(4, tq0);
-#ifdef HAT_PHASE_TIMERS
-                ph[7] += 1;
-#endif
                 if (owes) pay();                                 // the previous unit's last tile
                 page = page_next;
                 step();
@@ -409,9 +385,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
         }
         if (ok) pay();
         tile_append::stores_done();
-#ifdef HAT_PHASE_TIMERS
-        if (lane == 0) PH_FLUSH(48 + 8 * (int)rank, 8);
-#endif
         if (!ok) {
             // give copies already in flight a bounded chance to land before the CTA's shared memory is released
             const long long t0 = clock64();
@@ -527,31 +500,21 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
         if (lane == 0) {
             int g = 0;
             bool ok = true;
-            PH_DECL(8);
-            PH_T0(tf0);
             for (int un = 0; ok; ++un) {
                 const int unit = read_unit(un, false);
-                PH_ADD(0, tf0);
                 if (unit < 0) break;
                 const Unit u = decode_unit(a, items, unit);
                 const int qs = un & 1;
                 ok = mbar_wait(&bars->q_full[qs], (un >> 1) & 1, cx);
                 if (!ok) break;
                 mbar_arrive_remote(lead(&bars->q_full[qs]));
-                PH_ADD(1, tf0);
                 for (int j = 0; j < u.n && ok; ++j, ++g) {
                     const int sk = g % kStagesK;
                     ok = mbar_wait(&bars->k_full[sk], (g / kStagesK) & 1, cx);
                     if (!ok) break;
-                    PH_ADD(2, tf0);
                     mbar_arrive_remote(lead(&bars->k_full[sk]));
-                    PH_ADD(3, tf0);
-#ifdef HAT_PHASE_TIMERS
-                    ph[7] += 1;
-#endif
                 }
             }
-            PH_FLUSH(64, 8);
         }
         __syncwarp();
     } else if (warp == 1 || warp == 10) {
@@ -574,8 +537,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n"
                              ::"r"(bar_addr), "h"((uint16_t)3) : "memory");
             };
-            PH_DECL(16);
-            PH_T0(tl0);
             if (warp == 10) {
                 // ---- S = Q K^T of every tile, up to three tiles ahead of the P V products
                 const uint64_t q_desc0 = smem_desc(smem_u32(q_tiles), 16, 1024);
@@ -598,15 +559,12 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     const uint64_t qd = q_desc0 + (uint64_t)(qs * (kTileBytes >> 4));
                     ok = mbar_wait(&bars->q_full[qs], (un >> 1) & 1, cx);
                     for (int j = 0; j < n && ok; ++j) {
-                        PH_T0(ts0);
                         ok = wait_addr(k_bar, k_par);
                         if (!ok) break;
-                        PH_ADD(0, ts0);
                         if (wrapped) {                      // the P V product that read this buffer three tiles ago
                             ok = wait_addr(pv_bar, pv_par);
                             if (!ok) break;
                         }
-                        PH_ADD(1, ts0);
                         tc_fence_after();
 #pragma unroll
                         for (int ks = 0; ks < kD / 16; ++ks) {
@@ -625,17 +583,8 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         } else { s_col += 128; s_bar += 8; pv_bar += 8; }
                         if (++k_slot == kStagesK) { k_slot = 0; kd = k_desc0; k_bar = smem_u32(&bars->k_full[0]); ke_bar = smem_u32(&bars->k_empty[0]); k_par ^= 1; }
                         else { kd += kHalfBytes >> 4; k_bar += 8; ke_bar += 8; }
-                        PH_ADD(2, ts0);
-#ifdef HAT_PHASE_TIMERS
-                        ph[6] += 1;
-#endif
                     }
                 }
-                PH_ADD(5, tl0);
-#ifdef HAT_PHASE_TIMERS
-                ph[7] = 1;
-#endif
-                PH_FLUSH(0, 8);
             } else {
                 // ---- O (+)= P V of every tile
                 const uint64_t v_desc0 = smem_desc(smem_u32(v_ring), kSlabBytes, 1024);
@@ -656,10 +605,8 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     // the accumulators still hold the previous unit until its rows are in registers
                     if (un > 0) ok = mbar_wait(&bars->o_free, (un - 1) & 1, cx);
                     for (int j = 0; j < n && ok; ++j) {
-                        PH_T0(tp0);
                         ok = wait_addr(p_bar, p_par);
                         if (!ok) break;
-                        PH_ADD(0, tp0);
                         tc_fence_after();
 #pragma unroll
                         for (int ks = 0; ks < kKeys / 16; ++ks) {
@@ -675,17 +622,8 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         else { p_col += 128; p_bar += 8; pv_bar += 8; }
                         if (++v_slot == kStagesV) { v_slot = 0; vd = v_desc0; ve_bar = smem_u32(&bars->v_empty[0]); }
                         else { vd += kHalfBytes >> 4; ve_bar += 8; }
-                        PH_ADD(2, tp0);
-#ifdef HAT_PHASE_TIMERS
-                        ph[6] += 1;
-#endif
                     }
                 }
-                PH_ADD(5, tl0);
-#ifdef HAT_PHASE_TIMERS
-                ph[7] = 1;
-#endif
-                PH_FLUSH(8, 8);
             }
             if (!ok) {
                 // gave up: let the MMAs this thread issued finish (bounded) before TMEM is released
@@ -726,11 +664,8 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 ++px;
                 return met;
             };
-            PH_DECL(16);
-            PH_T0(tw0);
             for (int un = 0; ok; ++un) {
                 const int unit = read_unit(un, true);
-                PH_ADD(0, tw0);
                 if (unit == -2) { ok = false; break; }
                 if (unit < 0) break;
                 const Unit u = decode_unit(a, items, unit);
@@ -744,7 +679,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     const uint32_t tm_s = tmem + b * 128 + lane_sel;
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->s_full[b], (g / kSBuf) & 1, cx));
                     if (!ok) break;
-                    PH_ADD(1, tw0);
                     tc_fence_after();
                     float s[64];
 #pragma unroll
@@ -764,14 +698,12 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         for (int v = 0; v < 4; ++v) mx4[v] = fmaxf(mx4[v], fmaxf(s[k + 2 * v], s[k + 2 * v + 1]));
                     }
                     const float mx_half = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                    PH_ADD(2, tw0);
                     // the other half's maximum.  After this meeting both threads also have their scores in registers, so P
                     // (which overwrites the score columns of BOTH halves) may be written
                     bars->mx_x[g & 1][w][t] = mx_half;
                     ok = pair_sync();
                     if (!ok) break;
                     const float mx = fmaxf(mx_half, bars->mx_x[g & 1][w ^ 1][t]) * sc;
-                    PH_ADD(3, tw0);
                     // the reference moves only when this tile's maximum exceeds it by more than the threshold (same decision in
                     // both threads of the row: same inputs)
                     const float m_new = (mx > m_ref + kRescaleThreshold) ? mx : m_ref;
@@ -811,7 +743,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         sum4[0] = a0 + a1; sum4[1] = b0 + b1; sum4[2] = c0 + c1; sum4[3] = d0 + d1;
                     }
                     l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-                    PH_ADD(4, tw0);
 
                     if (__any_sync(0xffffffffu, rescale)) {
                         // O holds the tiles before this one in units of the old reference; the previous tile's P V must have
@@ -830,7 +761,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         }
                     }
                     tmem_st_wait();
-                    PH_ADD(5, tw0);
                     // this CTA's half of V tile g must have landed before the P V product may be issued (the MMA thread does
                     // not look at the V ring itself)
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_full[g % kStagesV], (g / kStagesV) & 1, cx));
@@ -850,10 +780,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote(lead_p_ready + b * 8);
-                    PH_ADD(6, tw0);
-#ifdef HAT_PHASE_TIMERS
-                    ph[15] += 1;
-#endif
                 }
                 if (!ok) break;
                 // ---- end of the unit: the two threads of a row add their row sums (both in units of the same reference),
@@ -865,11 +791,9 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 if (!ok) break;
                 const float l_tot = l + bars->lsum2[up][w ^ 1][t];
                 const float m_fin = m_ref;
-                PH_ADD(7, tw0);
                 // the last P V of the unit
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->pv_done[g_last % kSBuf], (g_last / kSBuf) & 1, cx));
                 if (!ok) break;
-                PH_ADD(8, tw0);
                 tc_fence_after();
                 float o[64];                                    // this warpgroup's half of the columns
 #pragma unroll
@@ -884,14 +808,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 if (w == 0 && i_row < u.C)
                     (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l_tot > 0.f ? (m_fin + log2f(l_tot)) * 0.6931471805599453f : -INFINITY;
                 g0 += u.n;
-                PH_ADD(9, tw0);
-#ifdef HAT_PHASE_TIMERS
-                ph[14] += 1;
-#endif
             }
-#ifdef HAT_PHASE_TIMERS
-            if (lane == 0 && quarter == 0) PH_FLUSH(16 + 16 * w, 16);
-#endif
         } else {
             const int w = (warp - 2) >> 2;                      // warpgroup: takes the tiles with g % 2 == w
             const int quarter = warp & 3;                       // TMEM lanes this warp may touch
@@ -903,11 +820,8 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             const uint32_t lead_o_free = lead(&bars->o_free), lead_p_ready = lead(&bars->p_ready[0]);
             int g0 = 0;                                         // global index of the unit's first tile
             bool ok = true;
-            PH_DECL(16);
-            PH_T0(tw0);
             for (int un = 0; ok; ++un) {
                 const int unit = read_unit(un, true);
-                PH_ADD(0, tw0);
                 if (unit == -2) { ok = false; break; }
                 if (unit < 0) break;
                 const Unit u = decode_unit(a, items, unit);
@@ -921,7 +835,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     const uint32_t tm_s = tmem + b * 128 + lane_sel;
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->s_full[b], (g / kSBuf) & 1, cx));
                     if (!ok) break;
-                    PH_ADD(1, tw0);
                     tc_fence_after();
                     float s[kKeys];
 #pragma unroll
@@ -941,7 +854,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         for (int v = 0; v < 4; ++v) mx4[v] = fmaxf(mx4[v], fmaxf(s[k + 2 * v], s[k + 2 * v + 1]));
                     }
                     const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sc;
-                    PH_ADD(2, tw0);
                     // the reference the previous tile (the other warpgroup's) left behind
                     float m_prev = -INFINITY;
                     if (j > 0) {
@@ -949,7 +861,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         if (!ok) break;
                         m_prev = bars->mref[t];
                     }
-                    PH_ADD(3, tw0);
                     // move it only when this tile's maximum exceeds it by more than the threshold
                     const float m_new = (mx > m_prev + kRescaleThreshold) ? mx : m_prev;
                     const bool rescale = (m_new != m_prev) && (m_prev != -INFINITY);
@@ -978,7 +889,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         m_mine = m_new;
                     }
                     l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-                    PH_ADD(4, tw0);
 
                     if (__any_sync(0xffffffffu, rescale)) {
                         // O holds the tiles before this one in units of m_prev; the previous tile's P V must have finished
@@ -997,7 +907,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                         }
                     }
                     tmem_st_wait();
-                    PH_ADD(5, tw0);
                     // this CTA's half of V tile g must have landed before the P V product may be issued (the MMA thread does
                     // not look at the V ring itself)
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_full[g % kStagesV], (g / kStagesV) & 1, cx));
@@ -1017,10 +926,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote(lead_p_ready + b * 8);
-                    PH_ADD(6, tw0);
-#ifdef HAT_PHASE_TIMERS
-                    ph[15] += 1;
-#endif
                 }
                 if (!ok) break;
                 // ---- end of the unit.  The warpgroup that did not take the last tile hands its row sum over (it is in units
@@ -1047,11 +952,9 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bars->fin_ready[w][quarter]);
                 }
-                PH_ADD(7, tw0);
                 // the last P V of the unit
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->pv_done[g_last % kSBuf], (g_last / kSBuf) & 1, cx));
                 if (!ok) break;
-                PH_ADD(8, tw0);
                 tc_fence_after();
                 float o[64];                                    // this warpgroup's half of the columns
 #pragma unroll
@@ -1066,14 +969,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
                 if (took_last && i_row < u.C)
                     (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l_tot > 0.f ? (m_fin + log2f(l_tot)) * 0.6931471805599453f : -INFINITY;
                 g0 += u.n;
-                PH_ADD(9, tw0);
-#ifdef HAT_PHASE_TIMERS
-                ph[14] += 1;
-#endif
             }
-#ifdef HAT_PHASE_TIMERS
-            if (lane == 0 && quarter == 0) PH_FLUSH(16 + 16 * w, 16);
-#endif
         }
     }
 
@@ -1114,17 +1010,5 @@ cudaError_t launch_attn_pair(const hat_plan* plan, const AttnArgs& args, cudaStr
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, grid, dim3(kThreads), kSmemBytes, stream, args, plan->dev.prefill_items, total_units, counter, *mq, *mk, *mv, *mkn, *mvh, fold);
 }
-
-#ifdef HAT_PHASE_TIMERS
-extern "C" int hat_debug_phase_read(unsigned long long* out, int n, int clear) {
-    if (n > 80) n = 80;
-    cudaError_t e = cudaMemcpyFromSymbol(out, g_phase, sizeof(unsigned long long) * n);
-    if (e == cudaSuccess && clear) {
-        unsigned long long z[80] = {0};
-        e = cudaMemcpyToSymbol(g_phase, z, sizeof z);
-    }
-    return e == cudaSuccess ? 0 : -1;
-}
-#endif
 
 }  // namespace hat
