@@ -239,7 +239,8 @@ int hat_rope_q(const hat_plan* plan, const void* q, void* q_out, float theta, in
  * INVALID_ARG, UNSUPPORTED (hidden not a multiple of 64, other head_dim), CUDA;
  * a device-side wait that ran out shows in hat_last_device_status.  The table of
  * cosines and sines is kept with the plan and filled by the first call with a
- * given theta (one more small kernel in that call); a call captured into a CUDA
+ * given theta (one more small kernel in that call, and in each call outside of
+ * graphs once one has been captured with this plan); a call captured into a CUDA
  * graph carries its own fill.  Like the attention calls, one call per plan at a time.
  */
 int hat_qkv_rope_append(const hat_cache_desc* cache, const hat_plan* plan, const void* x, int hidden, const void* w_qkv,

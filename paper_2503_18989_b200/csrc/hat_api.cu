@@ -695,6 +695,7 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     p->loose_stream = nullptr;
     p->rope_table = nullptr;
     p->rope_theta = 0.f;
+    p->table_in_graph = false;
     p->table_stream = nullptr;
     p->last_stream = nullptr;
     p->has_last = false;

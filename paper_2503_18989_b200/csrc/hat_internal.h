@@ -255,6 +255,7 @@ struct hat_plan {
     // (0: not filled yet), inside the plan's device memory
     float2* rope_table;
     float rope_theta;
+    bool table_in_graph;        // a captured graph fills the table whenever it is replayed
     cudaStream_t table_stream;
     std::vector<hat_plan*> parts;   // plans of contiguous requests for calls with host buffers (host_step.cu), made on the first one
     std::vector<int32_t> part_row;  // first packed row of each
@@ -278,8 +279,8 @@ cudaError_t launch_attn_mma(const hat_plan* plan, const AttnArgs& args, bool ver
 // the V rows copied beside them
 cudaError_t launch_rope(const hat_plan* plan, int heads, float theta, int interleaved, const void* src, void* dst,
                         const CacheView* cache, void* k_pool, void* v_pool, const void* v_new, cudaStream_t stream);
-// the plan's table of (cos, sin) per row and pair for base theta, filled if it holds none; holding another base, it is
-// replaced or (replace = false) *table stays null
+// the plan's table of (cos, sin) per row and pair for base theta, filled if it holds none; where it holds another base, a graph may
+// refill it or the call is being captured, it is filled again or (replace = false) *table stays null
 cudaError_t plan_rope_table(const hat_plan* plan, float theta, cudaStream_t stream, bool replace, const float2** table);
 cudaError_t launch_merge(const hat_plan* plan, const AttnArgs& args, int first_row, int num_rows, cudaStream_t stream);
 // tcgen05 tile kernel (head_dim 64 or 128): whether a TMA descriptor can be built for this pool layout, and the launcher

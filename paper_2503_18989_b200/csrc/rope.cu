@@ -155,17 +155,18 @@ cudaError_t plan_rope_table(const hat_plan* plan, float theta, cudaStream_t stre
         return cudaGetLastError();
     };
     if (cap != cudaStreamCaptureStatusNone) {
-        // Inside a stream capture nothing runs now: the fill becomes part of the captured graph (every replay refills the
-        // table, which is harmless) and the plan does not take the table as filled.
-        if (mp->rope_theta > 0.f && mp->rope_theta != theta && !replace) return cudaSuccess;
+        // Inside a stream capture nothing runs now: the fill becomes part of the captured graph, ahead of the call that needs it,
+        // and every replay refills the table at a time the plan does not know of.
+        if (!replace) return cudaSuccess;
         if ((e = fill()) != cudaSuccess) return e;
-        mp->rope_theta = 0.f;                    // whoever calls next outside a capture fills it for itself
-    } else if (mp->rope_theta != theta) {
-        if (mp->rope_theta > 0.f) {
+        mp->table_in_graph = true;
+    } else if (mp->table_in_graph || mp->rope_theta != theta) {
+        // (a table that a replay may have refilled since is not trusted)
+        if (mp->rope_theta > 0.f || mp->table_in_graph) {
             if (!replace) return cudaSuccess;
             // a call with the previous base may still be reading the table that is about to be replaced (rare: one model
             // has one base)
-            if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+            if (mp->rope_theta > 0.f && mp->rope_theta != theta && (e = cudaDeviceSynchronize()) != cudaSuccess) return e;
         }
         if ((e = fill()) != cudaSuccess) return e;
         if ((e = cudaEventRecord(mp->res.ev_table, stream)) != cudaSuccess) return e;
