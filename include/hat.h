@@ -146,6 +146,10 @@ int         hat_last_cuda_error(void);
 /* Number of kernels this library has launched in this process (all threads). */
 int64_t     hat_launch_count(void);
 
+/* Number of device allocations this library has made for plans in this process (all threads).  It stands still in a loop that makes,
+   uses and destroys plans once such plans have been through it (see hat_release_cached). */
+int64_t     hat_device_alloc_count(void);
+
 /*
  * Validate a batch and schedule it (Sec. 2.1 "Batched Inference": the batch
  * mixes prefill chunks and decode-phase requests; cost follows the batched
@@ -178,7 +182,8 @@ int hat_plan_destroy(hat_plan* plan);   /* NULL is accepted */
 
 /*
  * A destroyed plan hands its device memory and its events to later plans; at
- * most 64 such pieces and 64 MiB wait at any time.  hat_release_cached frees
+ * most 64 such pieces and 64 MiB wait at any time (the oldest make room for
+ * newer ones).  hat_release_cached frees
  * what waits, and the pinned buffer plans are uploaded from (this synchronises
  * the device); it is never needed for correctness.  Any thread may call it.
  */

@@ -32,7 +32,7 @@ HAT_PLAN_HOST_ONLY = 1
 DTYPE_CODE = {"fp16": HAT_DTYPE_FP16, "bf16": HAT_DTYPE_BF16}
 
 EXPORTS = [
-    "hat_status_string", "hat_version", "hat_last_cuda_error", "hat_launch_count",
+    "hat_status_string", "hat_version", "hat_last_cuda_error", "hat_launch_count", "hat_device_alloc_count",
     "hat_plan_create", "hat_plan_get_info", "hat_plan_workspace_bytes", "hat_plan_destroy",
     "hat_release_cached",
     "hat_kv_append", "hat_kv_append_rope", "hat_rope_q", "hat_qkv_rope_append", "hat_chunk_attention", "hat_chunk_attention_out16",
@@ -104,6 +104,8 @@ def lib() -> C.CDLL:
         L.hat_last_cuda_error.argtypes = []
         L.hat_launch_count.restype = C.c_int64
         L.hat_launch_count.argtypes = []
+        L.hat_device_alloc_count.restype = C.c_int64
+        L.hat_device_alloc_count.argtypes = []
         L.hat_plan_create.restype = i32
         L.hat_plan_create.argtypes = [C.POINTER(hat_cache_desc), C.POINTER(hat_batch_desc), C.POINTER(vp)]
         L.hat_plan_get_info.restype = i32
@@ -192,6 +194,10 @@ def hat_last_cuda_error() -> int:
 
 def hat_launch_count() -> int:
     return int(lib().hat_launch_count())
+
+
+def hat_device_alloc_count() -> int:
+    return int(lib().hat_device_alloc_count())
 
 
 def make_cache_desc(dtype, num_pages, num_kv_heads, head_dim, stride_page, stride_token, stride_head,

@@ -984,6 +984,8 @@ int hat_version(void) { return HAT_VERSION; }
 int hat_last_cuda_error(void) { return g_last_cuda_error; }
 int64_t hat_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
+int64_t hat_device_alloc_count(void) { return plan_res_allocs(); }
+
 int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, hat_plan** out) {
     return create_plan(cache, batch, /*part=*/false, /*whole=*/false, out);
 }

@@ -201,8 +201,9 @@ cudaError_t smem_attr_once(const void* kernel, int bytes);
 }  // namespace hat
 
 namespace hat {
-// What a plan needs from the driver: one device allocation and three events.  Plans live for one inference step, and making these anew costs far more than the step's schedule
-// (cudaMalloc and cudaFree: 270 + 360 us beside 6 GB of pools), so a destroyed plan hands them on (hat_api.cu).
+// What a plan needs from the driver: one device allocation and its events, and two streams and an event more where it takes host
+// buffers.  Plans live for one inference step, and making these anew costs far more than the step's schedule (cudaMalloc and
+// cudaFree: 360 + 270 us beside 6 GB of pools), so a destroyed plan hands them on (plan_pool.cu).
 struct PlanRes {
     int device = -1;
     void* blob = nullptr;
@@ -308,6 +309,7 @@ cudaError_t plan_res_upload(PlanRes& r, const UploadPart* parts, size_t num_part
 cudaError_t plan_res_release(PlanRes& r, bool reusable);    // reusable: ev_done covers every use, or there was none
 cudaError_t plan_res_copy_streams(PlanRes& r);              // makes copy_in, copy_out and ev_copy if they are missing
 cudaError_t plan_res_free(PlanRes& r);
+int64_t plan_res_allocs();                                  // blocks of device memory allocated so far
 cudaError_t plan_res_trim();                                // frees what waits for a later plan
 // hat_plan_create; part = true: nothing is uploaded yet (upload_plans does it for several at once); whole = true: no request
 // is cut into key ranges (no workspace)

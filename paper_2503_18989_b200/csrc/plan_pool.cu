@@ -5,10 +5,11 @@
 // cudaMemcpy on the legacy stream waits for the previous step's kernels: together more than the eight layers of the
 // step take on the GPU.  The pool turns that into a search of a short list and one small asynchronous copy.
 //
-// Bounds: at most kMaxIdle entries and kMaxIdleBytes of device memory wait in the list, per process; what does not fit
-// is freed, and hat_release_cached() frees the rest.  Entries are handed on whole under one lock; an entry whose last
-// owner's kernels may still run is taken only after that owner's ev_done has occurred.
+// Bounds: at most kMaxIdle entries and kMaxIdleBytes of device memory wait in the list, per process; the oldest that are no
+// longer in use make room for what is given back, and hat_release_cached() frees the rest.  Entries are handed on whole under one
+// lock; an entry whose last owner's kernels may still run is taken (or freed for room) only after that owner's ev_done has occurred.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -20,6 +21,14 @@ namespace {
 
 constexpr size_t kMaxIdle = 64;
 constexpr size_t kMaxIdleBytes = size_t(64) << 20;
+std::atomic<int64_t> g_allocs{0};
+
+// what a plan that needs n bytes is given where nothing waits for it: a power of two, 64 KiB at least
+size_t block_size(size_t n) {
+    size_t b = size_t(64) << 10;
+    while (b < n) b *= 2;
+    return b;
+}
 
 struct Pool {
     std::mutex mu;
@@ -63,8 +72,8 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, PlanRes* out) {
         int ready = -1, oldest = -1;
         for (int i = 0; i < (int)p.idle.size(); ++i) {          // in the order they were given back
             PlanRes& r = p.idle[i];
-            // not for a plan that needs a small part of it only: the large ones would all end up with small plans
-            if (r.device != device || r.blob_bytes < blob_bytes || r.blob_bytes / 8 > blob_bytes) continue;
+            // not for a plan that would need much less: the large ones would all end up with small plans
+            if (r.device != device || r.blob_bytes < blob_bytes || r.blob_bytes / 8 > block_size(blob_bytes)) continue;
             if (oldest < 0) oldest = i;
             if (!r.in_use || cudaEventQuery(r.ev_done) == cudaSuccess) { ready = i; break; }
         }
@@ -87,7 +96,8 @@ cudaError_t plan_res_acquire(int device, size_t blob_bytes, PlanRes* out) {
     }
     PlanRes r;
     r.device = device;
-    for (r.blob_bytes = size_t(64) << 10; r.blob_bytes < blob_bytes;) r.blob_bytes *= 2;
+    r.blob_bytes = block_size(blob_bytes);
+    g_allocs.fetch_add(1, std::memory_order_relaxed);
     cudaError_t e = cudaMalloc(&r.blob, r.blob_bytes);
     if (e == cudaErrorMemoryAllocation) {                        // give back what waits in the list and try once more
         cudaGetLastError();
@@ -111,18 +121,38 @@ cudaError_t plan_res_copy_streams(PlanRes& r) {
 }
 
 cudaError_t plan_res_release(PlanRes& r, bool reusable) {
-    if (!r.blob) return plan_res_free(r);
-    if (reusable) {
-        Pool& p = pool();
+    if (!r.blob || !reusable || r.blob_bytes > kMaxIdleBytes) return plan_res_free(r);
+    Pool& p = pool();
+    std::vector<PlanRes> gone;
+    {
         std::lock_guard<std::mutex> lock(p.mu);
-        if (p.idle.size() < kMaxIdle && idle_bytes(p.idle) + r.blob_bytes <= kMaxIdleBytes) {
+        size_t bytes = idle_bytes(p.idle);
+        bool queried = false;
+        for (size_t i = 0; i < p.idle.size() && (p.idle.size() >= kMaxIdle || bytes + r.blob_bytes > kMaxIdleBytes);) {
+            PlanRes& old = p.idle[i];
+            if (old.in_use) {
+                queried = true;
+                if (cudaEventQuery(old.ev_done) != cudaSuccess) { ++i; continue; }
+            }
+            bytes -= old.blob_bytes;
+            gone.push_back(old);
+            p.idle.erase(p.idle.begin() + i);
+        }
+        if (queried) cudaGetLastError();                         // cudaErrorNotReady of a query is no error
+        if (p.idle.size() < kMaxIdle && bytes + r.blob_bytes <= kMaxIdleBytes) {
             p.idle.push_back(r);
             r = PlanRes{};
-            return cudaSuccess;
         }
     }
-    return plan_res_free(r);
+    cudaError_t first = plan_res_free(r);                        // nothing, if it waits in the list
+    for (PlanRes& old : gone) {
+        const cudaError_t e = plan_res_free(old);
+        if (first == cudaSuccess) first = e;
+    }
+    return first;
 }
+
+int64_t plan_res_allocs() { return g_allocs.load(std::memory_order_relaxed); }
 
 cudaError_t plan_res_upload(PlanRes& r, const UploadPart* parts, size_t num_parts, size_t bytes) {
     Pool& p = pool();
