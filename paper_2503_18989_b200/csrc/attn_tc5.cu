@@ -248,7 +248,11 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 mbar_arrive(&bars->unit_full[slot]);             // release: the slot is written before the arrival
             }
             unit = __shfl_sync(0xffffffffu, unit, 0);
-            if (unit < 0) break;
+            if (unit < 0) {
+                // a grid that joins another one may find nothing left: its end still stands for the end of what precedes it
+                if (un == 0 && !a.overlap) pdl_wait();
+                break;
+            }
             const Unit u = decode_unit(a, items, unit);
             const int32_t* __restrict__ table = a.plan.block_table + (int64_t)u.r * a.plan.max_pages;
             const int total_pages = (u.kv_end - u.kv_begin + kPageSize - 1) / kPageSize, page0 = u.kv_begin / kPageSize;

@@ -506,6 +506,33 @@ def test_mixed_batch_with_the_tile_kernel_on_a_side_stream(cuda_device, monkeypa
     assert_parity(gl, want[0][1], "side-stream lse")
 
 
+def test_side_stream_grid_that_finds_no_unit_left(cuda_device, monkeypatch):
+    """Two short prompt chunks beside a long streaming kernel: the second tile grid comes too late for any of them.  What
+    follows on the stream (the copies below) still comes after the streaming kernel."""
+    import torch
+    from paper_2503_18989_b200 import runner
+    monkeypatch.setenv("HAT_SIDE_SMS", "56")
+    monkeypatch.setenv("HAT_PREFILL_KERNEL", "tc5")
+    sc = W.mixed_13b(num_prefill=2, prefill_chunk=64, max_prefill_prefix=100, num_verify=40, min_verify_prefix=1000,
+                     max_verify_prefix=6000, H=4, seed=82)
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, sc.steps[0])
+    assert ds.info["prefill_kernel"] == 1
+    s = torch.cuda.Stream(cuda_device)
+    kp, vp, want = oracle_replay(sc)
+    for _ in range(5):
+        ds.out.fill_(float("nan"))
+        ds.lse.fill_(float("nan"))
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            ds.attend(stream=s.cuda_stream)
+            out, lse = ds.out.clone(), ds.lse.clone()
+        s.synchronize()
+        assert_parity(out.cpu().numpy(), want[0][0], "out, copied on the call's stream")
+        assert_parity(lse.cpu().numpy(), want[0][1], "lse, copied on the call's stream")
+    ds.close()
+
+
 def test_the_call_can_be_captured_in_a_cuda_graph_and_replayed(cuda_device):
     """hat_chunk_attention is stream-ordered and neither allocates nor synchronises, so a caller can capture the
     launch set of a step (append, streaming kernel, merge, tile kernel) once and replay it."""
