@@ -148,8 +148,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_k_new,
                 const __grid_constant__ CUtensorMap map_v_new, int fold) {
     constexpr bool ONE = FORM != kMany;
+    static_assert(!ONE || kD == 128, "the forms with one unit a CTA store rows of 128 columns");
     constexpr uint32_t kTileBytes = tile_bytes<kD>();
-    constexpr int kHalves = kD / 64;                             // 64-column slabs of a Q tile
+    constexpr int kSlabs = kD / 64;                              // 64-column slabs of a Q tile
     constexpr uint32_t kGroupBytes = group_bytes<kD>(), kPageBytes = page_bytes<kD>();
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the swizzle pattern and the matrix descriptors assume it
@@ -270,9 +271,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 pdl_wait();                                      // up to here only the plan's own arrays were read
             }
             if (lane == 0) mbar_expect_tx(&bars->q_full, u.nq * kTileBytes);
-            if (lane < kHalves * u.nq)      // lane = kHalves * (query tile) + (column half)
-                tma_load_3d(smem_u32(q_tiles) + (lane / kHalves) * kTileBytes + (lane % kHalves) * kSlabBytes, &map_q, (lane % kHalves) * 64, u.h,
-                            u.row_base + u.row0 + (lane / kHalves) * kRows, &bars->q_full);
+            if (lane < kSlabs * u.nq)       // lane = kSlabs * (query tile) + (column half)
+                tma_load_3d(smem_u32(q_tiles) + (lane / kSlabs) * kTileBytes + (lane % kSlabs) * kSlabBytes, &map_q, (lane % kSlabs) * 64, u.h,
+                            u.row_base + u.row0 + (lane / kSlabs) * kRows, &bars->q_full);
             // tiles [0, n_plain) hold nothing of the chunk, or the call does not append
             const int n_plain = APPEND ? min(u.n_all, max(0, u.P - u.kv_begin) / kKeys) : u.n_all;
             const int c3 = u.hk << s3;
