@@ -217,6 +217,9 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
     cluster_wait();
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
+    // The two producers wait for the previous kernel's end once they have read what they can; the other roles do so here, so that
+    // their bounded waits do not run while another kernel does.
+    if (warp != 0 && warp != 11 && !a.overlap) pdl_wait();
 
     // A consumer's read of the unit queue: the unit published as number `un` (-1: none left, -2: gave up).
     auto read_unit = [&](int un, bool whole_warp) -> int {

@@ -8,9 +8,9 @@
 //   page  ceil(P/16)          the chunk's own rows, gathered: from k_new / v_new when the call appends (the pool then
 //                             need not be written first), else row by row from the pool; rows beyond the chunk are zero
 // so both kinds of call do the same arithmetic in the same order and give the same bits.
-//   warp 4      producer: waits for the end of the stream's previous kernel (no other warp touches what kernels write before
-//               the producer's data reaches it); unit after unit without draining in between, the Q tile (cp.async) and the pages, each by
-//               2 or 4 TMA boxes of 2 KiB (64 columns x 16 tokens, 128-byte swizzle), into a ring of slots on mbarriers
+//   warp 4      producer: reads its first unit's record and page ids, then waits for the end of the stream's previous kernel; unit
+//               after unit without draining in between, the Q tile (cp.async) and the pages, each by two TMA boxes (16 tokens of K and
+//               of V, 128-byte swizzle), into a ring of slots on mbarriers
 //   warps 0-3   page j of a unit belongs to warp 3 - j mod 4: mma.sync m16n8k16, fp32 accumulate, online softmax whose
 //               reference maximum only moves when it grows by more than 2^8, so the accumulator is rarely rescaled.
 //               At the end of a unit the partial results pass from warp to warp through one shared-memory buffer; a warp
@@ -176,6 +176,7 @@ attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, 
     const uint32_t g_inv = ((1u << 20) + G - 1) / G;
     auto pair_row = [&](int pair) { return G < 256 ? (int)(((uint32_t)pair * g_inv) >> 20) : pair / G; };
     bool ok = true;
+    if (warp != kWarps) tc5::pdl_wait();                          // the bounded waits below do not run while another kernel does
 
     if (warp == kWarps) {
         // ------------------------------------------------------------------ producer

@@ -198,6 +198,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     pdl_launch_dependents();
+    // The producer waits for the previous kernel's end once it has read what it can; the other roles do so here, so that their bounded
+    // waits (for what the producer requests afterwards) do not run while another kernel does.
+    if (warp != 0 && !a.overlap) pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch + TMA producer

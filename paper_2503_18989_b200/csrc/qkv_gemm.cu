@@ -257,6 +257,7 @@ qkv_gemm_kernel(const __grid_constant__ QkvArgs a, const __grid_constant__ CUten
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     pdl_launch_dependents();
+    if (warp != 0) pdl_wait();                                  // the bounded waits below do not run while another kernel does
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one lane)

@@ -310,6 +310,50 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(cuda_device, kernel,
     assert_parity(gl, want[0][1], "lse after a timed-out call")
 
 
+@pytest.mark.parametrize("kernel", ["tc5", "pair", "stream", "projection"])
+def test_waits_are_not_used_up_by_the_kernel_in_front(cuda_device, kernel, monkeypatch):
+    """A kernel that starts in the tail of the previous one begins its bounded waits when that one has ended: one unit of 60000
+    keys (about half a millisecond on one SM, the others idle), and behind it a call whose waits may take a tenth of that."""
+    import torch
+    from paper_2503_18989_b200 import binding as B, runner
+    monkeypatch.setenv("HAT_PREFILL_SPLIT_LEN", "0")
+    monkeypatch.setenv("HAT_PREFILL_KERNEL", "tc5")
+    long = _manual("fp16", 1, 128, [60000], [64], 24)
+    long_ds = runner.DeviceStep(runner.DeviceCache(long.cache, long.k_pool, long.v_pool, cuda_device), long.steps[0])
+    assert long_ds.info["num_prefill_items"] == 1
+    if kernel == "pair":
+        monkeypatch.setenv("HAT_PREFILL_KERNEL", "pair")
+    sc = _manual("fp16", 2, 128, [100], [4 if kernel == "stream" else 64], 25)
+    st = sc.steps[0]
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, st)
+    x, w = (torch.randn(n, 192, device=cuda_device).to(torch.float16) for n in (st.total_rows, 3 * 2 * 128))
+    q = torch.empty((st.total_rows, 2, 128), dtype=torch.float16, device=cuda_device)
+
+    def call():
+        if kernel == "projection":
+            B.hat_qkv_rope_append(cache.desc, ds.plan, x, 192, w, q, 10000.0, False)
+        else:
+            ds.attend()
+
+    call()
+    long_ds.attend()
+    torch.cuda.synchronize()
+    B.hat_plan_set_wait_limit(ds.plan, 100_000)
+    for _ in range(3):
+        long_ds.attend()
+        call()
+    assert B.hat_last_device_status(ds.plan) == B.HAT_OK
+    assert B.hat_last_device_status(long_ds.plan) == B.HAT_OK
+    if kernel != "projection":
+        kp, vp, want = oracle_replay(sc)
+        go, gl = ds.results()
+        assert_parity(go, want[0][0], "out")
+        assert_parity(gl, want[0][1], "lse")
+    ds.close()
+    long_ds.close()
+
+
 def test_long_prefill_request_is_cut_into_at_most_32_key_ranges(cuda_device):
     from paper_2503_18989_b200 import binding as B, runner
     sc = _manual("fp16", 1, 128, [20000], [300], 22)
