@@ -392,11 +392,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             if (ok) pay();
             tile_append::stores_done();
         }
-        if (!ok) {
-            // give copies already in flight a bounded chance to land before the CTA's shared memory is released
-            const long long t0 = clock64();
-            while (clock64() - t0 < 2000000) { }
-        }
     } else if (warp == 11) {
         // ------------------------------------------------------------------ TMA producer of the V halves (both CTAs)
         // A warp of its own: the K and the V ring then fill independently (one warp doing both waits for a V slot
@@ -499,10 +494,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
         if constexpr (APPEND) {
             if (ok) pay();
             tile_append::stores_done();
-        }
-        if (!ok) {
-            const long long t0 = clock64();
-            while (clock64() - t0 < 2000000) { }
         }
     } else if (warp == 1 && rank != 0) {
         // ------------------------------------------------------------------ CTA 1: forward "landed" to CTA 0's barriers
@@ -985,6 +976,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
     // both CTAs are done with each other's barriers, and every MMA has finished, before tensor memory is freed
     tc_fence_before();
     __syncthreads();
+    if (bars->abort_flag) settle();
     cluster_arrive();
     cluster_wait();
     if (warp == 1) {

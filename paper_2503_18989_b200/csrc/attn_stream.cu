@@ -138,21 +138,25 @@ __device__ __forceinline__ bool wait_for(uint64_t* bar, uint32_t parity, Ctl<SLO
     return true;
 }
 
+// The dynamic shared memory from its first 1024-byte boundary on: ring, Q tile, hand-over buffer, control block.
+template <int D>
+__device__ __forceinline__ Ctl<Geo<D>::SLOTS>* ctl_of(unsigned char* smem) {
+    return reinterpret_cast<Ctl<Geo<D>::SLOTS>*>(smem + Geo<D>::SLOTS * Geo<D>::SLOT + Geo<D>::Q + Geo<D>::X);
+}
+
+// The six warps' work.  A warp returns when it is done, or early when a wait gave up.
 template <bool BF16, int D>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
-attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, int total_units, int32_t* __restrict__ work_counter,
-                   int32_t* __restrict__ piece_counters, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v) {
+__device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* smem, const StreamItem* __restrict__ items, int n_sub, int total_units,
+                                             int32_t* __restrict__ work_counter, int32_t* __restrict__ piece_counters, const CUtensorMap& map_k,
+                                             const CUtensorMap& map_v) {
     using G_ = Geo<D>;
     constexpr int CH = D / 8, ON = D / 8, SLOTS = G_::SLOTS, PER = G_::PER;
     constexpr uint32_t PAGE = G_::PAGE, SLOT = G_::SLOT;
     using Ctl_ = Ctl<SLOTS>;
 
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* q_buf = smem + SLOTS * SLOT;
     float4* xbuf = reinterpret_cast<float4*>(q_buf + G_::Q);
-    Ctl_* ctl = reinterpret_cast<Ctl_*>(q_buf + G_::Q + G_::X);
+    Ctl_* ctl = ctl_of<D>(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
@@ -324,11 +328,6 @@ attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, 
             r0 = n0; r1 = n1; r2 = n2;
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
-        if (!ok) {
-            // give the copies still in flight a bounded time to land before the CTA's shared memory is released
-            const long long t0 = clock64();
-            while (clock64() - t0 < 2000000) { }
-        }
         // the last producer to finish leaves the unit counter at zero for the next call
         if (lane == 0) {
             __threadfence();
@@ -728,6 +727,18 @@ attn_stream_kernel(AttnArgs a, const StreamItem* __restrict__ items, int n_sub, 
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctl->hand[warp]);
     }
+}
+
+template <bool BF16, int D>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+attn_stream_kernel(const __grid_constant__ AttnArgs a, const StreamItem* __restrict__ items, int n_sub, int total_units, int32_t* __restrict__ work_counter,
+                   int32_t* __restrict__ piece_counters, const __grid_constant__ CUtensorMap map_k,
+                   const __grid_constant__ CUtensorMap map_v) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    stream_roles<BF16, D>(a, smem, items, n_sub, total_units, work_counter, piece_counters, map_k, map_v);
+    __syncthreads();
+    if (ctl_of<D>(smem)->abort_flag) tc5::settle();
 }
 
 template <bool BF16, int D>

@@ -355,11 +355,6 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             if (ok) pay();
             tile_append::stores_done();
         }
-        if (!ok) {
-            // give copies already in flight a bounded chance to land before the CTA's shared memory is released
-            const long long t0 = clock64();
-            while (clock64() - t0 < 2000000) { }
-        }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (one thread)
         if (lane == 0) {
@@ -794,7 +789,10 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
 
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0 && bars->abort_flag) atomicOr(status, 1);
+    if (bars->abort_flag) {
+        if (threadIdx.x == 0) atomicOr(status, 1);
+        settle();
+    }
     if constexpr (FORM == kHalves) {
         cluster_arrive();                                        // the other CTA has read what it needs of this one's shared memory
         cluster_wait();

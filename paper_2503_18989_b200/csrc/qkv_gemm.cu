@@ -283,11 +283,6 @@ qkv_gemm_kernel(const __grid_constant__ QkvArgs a, const __grid_constant__ CUten
                     tma_load_2d(dst + kABytes, &map_w, ks * kTileK, w_row, &bars->full[s]);
                 }
             }
-            if (!ok) {
-                // give copies already in flight a bounded chance to land before the CTA's shared memory is released
-                const long long t0 = clock64();
-                while (clock64() - t0 < 2000000) { }
-            }
         }
         __syncwarp();
     } else if (warp == 1 && rank != 0) {
@@ -380,6 +375,7 @@ qkv_gemm_kernel(const __grid_constant__ QkvArgs a, const __grid_constant__ CUten
 
     tc_fence_before();
     __syncthreads();
+    if (bars->abort_flag) settle();
     if constexpr (PAIR) {
         // both CTAs are done with each other's barriers, and every MMA has finished, before tensor memory is freed
         cluster_arrive();

@@ -89,6 +89,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// For a CTA that gave up a wait, once all its roles have stopped: copies and products still in flight get a bounded time (a
+// millisecond) to land before its shared and tensor memory is released.
+__device__ __forceinline__ void settle() {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000) { }
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
