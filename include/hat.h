@@ -353,15 +353,18 @@ int hat_plan_wait_verify(const hat_plan* plan);
 int hat_last_device_status(const hat_plan* plan, void* stream, int* out);
 
 /*
- * Failure detection of the tcgen05 kernels (tile attention, projection).
- * Every wait inside them (on a TMA transfer, on the tensor pipe, on another
- * warp or the other CTA of a pair) is bounded by `cycles` SM clock cycles (0
- * selects the default of 2e9, about a second); a wait that runs out sets the
- * status word above, tells the other warps of its CTA (and the other CTA of
- * its pair) to stop, and the CTA releases its tensor memory and exits.
+ * Failure detection of the kernels that wait on the device: tile attention and
+ * projection (tcgen05) and streaming attention by TMA.  Every wait inside them
+ * (on a transfer, on the tensor pipe, on another warp or the other CTA of a
+ * pair) is bounded by `cycles` SM clock cycles (0 selects the default of 2e9,
+ * about a second), counted from the end of what precedes the call on the stream;
+ * a wait that runs out sets the status word above, tells the other warps of its
+ * CTA (and the other CTA of its pair) to stop, and the CTA lets what is in flight
+ * land, releases its tensor memory and exits.
  * withhold_next_call != 0 is a self test of that path: in the next
  * hat_chunk_attention or hat_qkv_rope_append call on this plan, whichever
- * comes first, every CTA that loads skips one of its own transfers, so that
+ * comes first, every CTA that loads (of two that merge their halves, the first)
+ * skips one of its own transfers, so that
  * a wait does run out within the bound; that call's results are undefined.
  * Nothing faults or hangs.
  */

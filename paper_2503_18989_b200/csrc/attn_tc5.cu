@@ -214,6 +214,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         int sk = 0, sv = 0;                                      // ring slots of the next tile
         uint32_t pk = 1, pv = 1;                                 // parities of their "empty" barriers: the first round passes at once
         bool withhold = a.withhold;                              // self test: the first V tile never arrives, its consumers give up
+        if constexpr (FORM == kHalves) withhold = withhold && cluster_ctarank() == 0;   // (and the other CTA waits for its rows in vain)
         bool ok = true;
         // the tile before the one being requested, if this unit is the one that appends its pages: stored from its ring slots
         bool owes = false, o_whole = false, stored = false;      // stored: a slot may still be read by its store

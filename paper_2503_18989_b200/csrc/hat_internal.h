@@ -92,7 +92,7 @@ struct AttnArgs {
     int64_t     part_rows;    // partial rows the workspace holds (index checks of the debug build)
     float       scale_log2;   // sm_scale * log2(e)
     long long   wait_cycles;  // bound of every device-side wait, in SM clock cycles
-    int         withhold;     // self test: the tile kernel's producer skips its first V tile so that a wait runs out
+    int         withhold;     // self test: a producer skips one of its first transfers so that a wait runs out
     int         static_first; // a CTA's first unit is its own number, the counter gives the ones after the grid's; else all come from the counter
     int         overlap;      // the grid runs beside the stream's previous kernel (which has waited for everything before it): waits for its end only at its own
     int         tail_reset;   // the last producer of the persistent tile kernel to finish clears the unit counter for the next call

@@ -284,25 +284,47 @@ def test_host_buffer_entry_point(cuda_device):
         assert_parity(l.numpy(), want[0][1], "host entry, two in flight, lse")
 
 
-@pytest.mark.parametrize("kernel,code", [("tc5", 1), ("pair", 3)])
-def test_bounded_wait_gives_up_and_the_context_stays_usable(cuda_device, kernel, code, monkeypatch):
-    """Failure detection without a fault: the tile kernel's producer withholds one transfer, the waiting
-    warps give up after the (shortened) bound (in the CTA-pair kernel both CTAs of every pair), the status word
-    reports it, and the next call is correct."""
+# (prefix, chunk, heads): one unit a CTA; CTAs that draw several units; tiles cut in two that clusters merge; several pairs; streaming
+# units more than CTAs, some requests cut, and a chunk without a prefix
+_GIVES_UP = {
+    "one": ("tc5", 1, [1000], [128], 8),
+    "many": ("tc5", 1, [300] * 24, [200, 256, 64] * 8, 16),
+    "halves": ("tc5", 1, [300], [200], 2),
+    "pair": ("pair", 3, [300, 40, 900] * 3, [200, 512, 300] * 3, 8),
+    "stream": (None, 0, [700, 5000, 0, 33, 16] * 8, [4, 16, 3, 8, 1] * 8, 16),
+}
+
+
+@pytest.mark.parametrize("form", list(_GIVES_UP))
+@pytest.mark.parametrize("fused", [True, False])
+def test_bounded_wait_gives_up_and_the_context_stays_usable(cuda_device, form, fused, monkeypatch):
+    """Failure detection without a fault: a producer withholds one transfer, the waiting warps give up after the (shortened)
+    bound (in the CTA-pair kernel both CTAs of every pair; of two CTAs that merge their halves the second one on the first),
+    the status word reports it, and the next call is correct: every counter is back where it belongs."""
     from paper_2503_18989_b200 import binding as B, runner
-    monkeypatch.setenv("HAT_PREFILL_KERNEL", kernel)
-    sc = _manual("fp16", 2, 128, [300], [200], 21)
+    kernel, code, prefix, chunk, heads = _GIVES_UP[form]
+    if kernel:
+        monkeypatch.setenv("HAT_PREFILL_KERNEL", kernel)
+    sc = _manual("fp16", heads, 128, prefix, chunk, 21)
     st = sc.steps[0]
     cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
     ds = runner.DeviceStep(cache, st)
-    assert ds.info["prefill_kernel"] == code
+    units = ds.info["num_prefill_items"] * heads
+    if kernel:
+        assert ds.info["prefill_kernel"] == code
+        assert {"one": units <= 148 and ds.info["max_splits"] != 2, "many": units > 148, "pair": units > 74,
+                "halves": ds.info["max_splits"] == 2 and ds.workspace_bytes == 0}[form]
+    else:
+        assert ds.info["stream_kernel"] == 1 and ds.info["num_verify_items"] * heads > 2 * 148 and ds.info["max_splits"] > 1
+    if not fused:
+        ds.append()
     assert B.hat_last_device_status(ds.plan) == B.HAT_OK
     B.hat_plan_set_wait_limit(ds.plan, 20_000_000, withhold_next_call=True)      # about 10 ms
-    ds.attend(fused_append=True)
+    ds.attend(fused_append=fused)
     assert B.hat_last_device_status(ds.plan) == B.HAT_ERR_DEVICE_TIMEOUT
     assert B.hat_last_device_status(ds.plan) == B.HAT_OK                            # reading clears the word
     B.hat_plan_set_wait_limit(ds.plan, 0)
-    ds.attend(fused_append=True)                                                    # the self test was one-shot
+    ds.attend(fused_append=fused)                                                   # the self test was one-shot
     go, gl = ds.results()
     assert B.hat_last_device_status(ds.plan) == B.HAT_OK
     kp, vp, want = oracle_replay(sc)
