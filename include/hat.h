@@ -342,8 +342,8 @@ int hat_plan_verify_event(const hat_plan* plan, void** event_out);
 int hat_plan_wait_verify(const hat_plan* plan);
 
 /*
- * Read and clear the device-side status word of a plan (synchronises
- * `stream`).  *out is HAT_OK, HAT_ERR_DEVICE_BOUNDS (only a library built with
+ * Read and clear the device-side status word of a plan, behind the plan's
+ * latest call on whichever stream (synchronises `stream`).  *out is HAT_OK, HAT_ERR_DEVICE_BOUNDS (only a library built with
  * -DHAT_DEBUG_BOUNDS checks: a block-table column, page id, ring slot, TMEM column or output row was out of range;
  * the access was skipped or clamped, nothing trapped), or HAT_ERR_DEVICE_TIMEOUT if a bounded wait
  * inside a kernel gave up since the word was last read; the results of the

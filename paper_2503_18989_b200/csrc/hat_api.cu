@@ -1208,7 +1208,9 @@ int hat_last_device_status(const hat_plan* plan, void* stream, int* out) {
     if (!plan || !out || plan->host_only) return HAT_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int32_t word = 0;
-    cudaError_t e = cudaMemcpyAsync(&word, plan->dev.status, sizeof word, cudaMemcpyDeviceToHost, s);
+    // behind the plan's latest call, whose counters are among the words that are cleared
+    cudaError_t e = plan->has_last && plan->last_stream != s ? cudaStreamWaitEvent(s, plan->res.ev_done, 0) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&word, plan->dev.status, sizeof word, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(plan->dev.status, 0, plan->num_status_words * sizeof word, s);     // status, counters
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e);

@@ -332,6 +332,31 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(cuda_device, form, f
     assert_parity(gl, want[0][1], "lse after a timed-out call")
 
 
+def test_the_status_is_read_behind_the_plans_latest_call(cuda_device):
+    """Reading the status clears the plan's counters too: on another stream than the call's it waits for the call."""
+    import torch
+    from paper_2503_18989_b200 import binding as B, runner
+    sc = _manual("fp16", 4, 128, [5000, 300], [4, 200], 26)
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, sc.steps[0])
+    assert ds.info["max_splits"] > 1
+    streams = [torch.cuda.Stream(cuda_device) for _ in range(2)]
+    done = torch.cuda.Event()
+    ds.attend(stream=streams[0].cuda_stream)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(streams[0]):
+        torch.cuda._sleep(200_000_000)                              # about a tenth of a second
+        ds.attend(stream=streams[0].cuda_stream)
+        done.record()
+    assert B.hat_last_device_status(ds.plan, streams[1].cuda_stream) == B.HAT_OK
+    assert done.query(), "the status was read before the call had run"
+    go, gl = ds.results()
+    kp, vp, want = oracle_replay(sc)
+    assert_parity(go, want[0][0], "out")
+    assert_parity(gl, want[0][1], "lse")
+    ds.close()
+
+
 @pytest.mark.parametrize("kernel", ["tc5", "pair", "stream", "projection"])
 def test_waits_are_not_used_up_by_the_kernel_in_front(cuda_device, kernel, monkeypatch):
     """A kernel that starts in the tail of the previous one begins its bounded waits when that one has ended: one unit of 60000
