@@ -38,7 +38,7 @@ extern "C" {
 
 /* status codes */
 #define HAT_OK                        0
-#define HAT_ERR_INVALID_ARG          -1  /* null pointer, negative count, cu_chunk inconsistent with chunk_len */
+#define HAT_ERR_INVALID_ARG          -1  /* null pointer, negative count, cu_chunk inconsistent with chunk_len; host memory exhausted */
 #define HAT_ERR_UNSUPPORTED          -2  /* dtype, head_dim, page_size, head counts or strides outside what is built */
 #define HAT_ERR_OUT_OF_RANGE         -3  /* page id outside the pool, table too short, page written by two requests */
 #define HAT_ERR_WORKSPACE_TOO_SMALL  -4

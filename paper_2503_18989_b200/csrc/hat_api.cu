@@ -672,6 +672,10 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
 
     hat_plan* p = new (std::nothrow) hat_plan();
     if (!p) return HAT_ERR_INVALID_ARG;
+    struct Owner {
+        hat_plan* p;
+        ~Owner() { if (p) hat_plan_destroy(p); }
+    } owner{p};                                              // until the plan is handed out
     p->dtype = cache->dtype;
     p->num_pages = cache->num_pages;
     p->num_heads = batch->num_q_heads;
@@ -731,7 +735,7 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) { delete p; return cuda_fail(e); }
+        if (e != cudaSuccess) return cuda_fail(e);
     }
     // the tcgen05 tile kernels need a pool layout a TMA descriptor can express (the CTA-pair one also head_dim 128)
     bool use_tc5 = true;
@@ -783,15 +787,13 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     // launch-geometry limits: work items index gridDim.y (65535), partial rows and units are 32-bit
     const int64_t verify_count = (int64_t)(p->verify_items.size() + p->stream_items.size());
     if (verify_count > 65535 || verify_count * p->num_kv_heads * p->verify_subtiles > INT32_MAX / 2 || p->prefill_items.size() > 65535 || p->num_heads > 65535 ||
-        p->part_rows > INT32_MAX / 2 || (int64_t)p->prefill_items.size() * p->num_heads > INT32_MAX / 2) {
-        delete p;
+        p->part_rows > INT32_MAX / 2 || (int64_t)p->prefill_items.size() * p->num_heads > INT32_MAX / 2)
         return HAT_ERR_TOO_LARGE;
-    }
 
     if (!p->host_only) {
-        if (part) { *out = p; return HAT_OK; }               // uploaded with the others
+        if (part) { *out = p; owner.p = nullptr; return HAT_OK; }   // uploaded with the others
         st = upload_plans(&p, 1, &p->res);
-        if (st != HAT_OK) { hat_plan_destroy(p); return st; }
+        if (st != HAT_OK) return st;
         // Optional throughput mode for a mixed batch on the tcgen05 path (HAT_SIDE_SMS = n > 0): see the launch
         // sequence.  Off by default: it finishes the whole step sooner but the decode-phase rows later.  The side
         // stream has the highest priority so that the tile CTAs are placed before the streaming kernel's many small
@@ -805,12 +807,13 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
                 if (ee == cudaSuccess) ee = cudaStreamCreateWithPriority(&p->aux_stream, cudaStreamNonBlocking, hi);
                 if (ee == cudaSuccess) ee = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
                 if (ee == cudaSuccess) ee = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
-                if (ee != cudaSuccess) { hat_plan_destroy(p); return cuda_fail(ee); }
+                if (ee != cudaSuccess) return cuda_fail(ee);
                 p->side_sms = side;
             }
         }
     }
     *out = p;
+    owner.p = nullptr;
     return HAT_OK;
 }
 
@@ -987,7 +990,7 @@ int64_t hat_launch_count(void) { return g_launches.load(std::memory_order_relaxe
 int64_t hat_device_alloc_count(void) { return plan_res_allocs(); }
 
 int hat_plan_create(const hat_cache_desc* cache, const hat_batch_desc* batch, hat_plan** out) {
-    return create_plan(cache, batch, /*part=*/false, /*whole=*/false, out);
+    return guarded([&] { return create_plan(cache, batch, /*part=*/false, /*whole=*/false, out); });
 }
 
 int hat_plan_get_info(const hat_plan* plan, hat_plan_info* out) {
@@ -1033,8 +1036,10 @@ int hat_plan_destroy(hat_plan* plan) {
 }
 
 int hat_release_cached(void) {
-    const cudaError_t e = plan_res_trim();
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+    return guarded([] {
+        const cudaError_t e = plan_res_trim();
+        return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+    });
 }
 
 int hat_kv_append(const hat_cache_desc* cache, const hat_plan* plan, const void* k_new, const void* v_new,
@@ -1084,23 +1089,25 @@ int hat_qkv_rope_append(const hat_cache_desc* cache, const hat_plan* plan, const
     if (plan->total_rows == 0) return HAT_OK;
     if (!x || !w_qkv || !q_out || !aligned(x, 16) || !aligned(w_qkv, 16) || !aligned(q_out, 16)) return HAT_ERR_INVALID_ARG;
     plan_note_call(const_cast<hat_plan*>(plan), static_cast<cudaStream_t>(stream));
-    cudaError_t e = launch_qkv_gemm(plan, view_of(cache), cache->k_pool, cache->v_pool, x, hidden, w_qkv, q_out, theta,
-                                    interleaved != 0, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+    return guarded([&] {
+        const cudaError_t e = launch_qkv_gemm(plan, view_of(cache), cache->k_pool, cache->v_pool, x, hidden, w_qkv, q_out, theta,
+                                              interleaved != 0, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? HAT_OK : cuda_fail(e);
+    });
 }
 
 int hat_chunk_attention(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
                         const void* v_new, float* out, float* lse, float sm_scale, void* workspace,
                         size_t workspace_bytes, void* stream) {
     if (!out && plan && plan->total_rows > 0) return HAT_ERR_INVALID_ARG;
-    return run_attention(cache, plan, q, k_new, v_new, out, nullptr, lse, sm_scale, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
+    return guarded([&] { return run_attention(cache, plan, q, k_new, v_new, out, nullptr, lse, sm_scale, workspace, workspace_bytes, static_cast<cudaStream_t>(stream)); });
 }
 
 int hat_chunk_attention_out16(const hat_cache_desc* cache, const hat_plan* plan, const void* q, const void* k_new,
                               const void* v_new, void* out16, float* lse, float sm_scale, void* workspace,
                               size_t workspace_bytes, void* stream) {
     if (!out16 && plan && plan->total_rows > 0) return HAT_ERR_INVALID_ARG;
-    return run_attention(cache, plan, q, k_new, v_new, nullptr, out16, lse, sm_scale, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
+    return guarded([&] { return run_attention(cache, plan, q, k_new, v_new, nullptr, out16, lse, sm_scale, workspace, workspace_bytes, static_cast<cudaStream_t>(stream)); });
 }
 
 int hat_plan_verify_event(const hat_plan* plan, void** event_out) {
@@ -1124,7 +1131,14 @@ int hat_plan_enable_timing(hat_plan* plan, int max_calls) {
     }
     Timing* tm = new (std::nothrow) Timing();
     if (!tm) return HAT_ERR_INVALID_ARG;
-    tm->events.resize((size_t)max_calls * HAT_TIMING_SLOTS * 2);
+    if (guarded([&] {
+            tm->events.resize((size_t)max_calls * HAT_TIMING_SLOTS * 2);
+            tm->launched.assign((size_t)max_calls * HAT_TIMING_SLOTS, 0);
+            return HAT_OK;
+        }) != HAT_OK) {
+        delete tm;
+        return HAT_ERR_INVALID_ARG;
+    }
     for (size_t i = 0; i < tm->events.size(); ++i) {
         cudaError_t e = cudaEventCreate(&tm->events[i]);
         if (e != cudaSuccess) {
@@ -1133,7 +1147,6 @@ int hat_plan_enable_timing(hat_plan* plan, int max_calls) {
             return cuda_fail(e);
         }
     }
-    tm->launched.assign((size_t)max_calls * HAT_TIMING_SLOTS, 0);
     tm->max_calls = max_calls;
     plan->timing = tm;
     return HAT_OK;
@@ -1199,8 +1212,10 @@ int hat_chunk_attention_host(const hat_cache_desc* cache, const hat_plan* plan, 
     float* dout = reinterpret_cast<float*>(base + q16 + 2 * kv16);
     float* dlse = reinterpret_cast<float*>(base + q16 + 2 * kv16 + out32);
     cudaError_t e = cudaSuccess;
-    st = host_step(cache, plan, HostBuffers{q_host, k_new_host, v_new_host, out_host, lse_host}, HostBuffers{dq, dk, dv, dout, dlse}, sm_scale,
-                   workspace, workspace_bytes, static_cast<cudaStream_t>(stream), &e);
+    st = guarded([&] {
+        return host_step(cache, plan, HostBuffers{q_host, k_new_host, v_new_host, out_host, lse_host}, HostBuffers{dq, dk, dv, dout, dlse}, sm_scale,
+                         workspace, workspace_bytes, static_cast<cudaStream_t>(stream), &e);
+    });
     return st == HAT_ERR_CUDA && e != cudaSuccess ? cuda_fail(e) : st;
 }
 

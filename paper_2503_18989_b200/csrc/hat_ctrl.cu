@@ -12,7 +12,7 @@
 #include <new>
 #include <vector>
 
-#include "../../include/hat.h"
+#include "hat_internal.h"
 
 struct hat_ctrl {
     double alpha;
@@ -73,9 +73,13 @@ int hat_ctrl_create(double alpha, double bin_width, int num_bins, int max_device
     c->bin_width = bin_width;
     c->has_mu = false;
     c->mu = 0.0;
-    c->g.assign(num_bins, 0.0);
-    c->seen.assign(num_bins, 0);
-    c->dev.assign(max_devices, hat_ctrl::Device{false, 0.0, 0.0, 0.0});
+    const int st = hat::guarded([&] {
+        c->g.assign(num_bins, 0.0);
+        c->seen.assign(num_bins, 0);
+        c->dev.assign(max_devices, hat_ctrl::Device{false, 0.0, 0.0, 0.0});
+        return HAT_OK;
+    });
+    if (st != HAT_OK) { delete c; return st; }
     *out = c;
     return HAT_OK;
 }

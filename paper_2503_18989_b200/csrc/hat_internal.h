@@ -351,6 +351,11 @@ cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, c
 }
 #endif
 void set_last_cuda_error(int e);   // what hat_last_cuda_error() returns on this thread
+// What a C entry point returns: no exception crosses it.  Only host allocations throw here; they end as a null `new` does.
+template <typename F>
+int guarded(F&& f) {
+    try { return f(); } catch (...) { return HAT_ERR_INVALID_ARG; }
+}
 }  // namespace hat
 
 namespace hat {

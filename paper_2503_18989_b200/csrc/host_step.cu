@@ -35,13 +35,12 @@ bool split_requests(const hat_plan* p, std::vector<int>& first) {
     return first.size() > 1;
 }
 
-void make_parts(hat_plan* p, const hat_cache_desc* cache) {
-    std::vector<int> first;
-    p->parts_made = true;
-    if (!split_requests(p, first)) return;
+// Makes and uploads the plans; false: they are not all there.
+bool plan_parts(hat_plan* p, const hat_cache_desc* cache, std::vector<int>& first) {
     first.push_back(p->num_requests);
     std::vector<int32_t> cu;
-    bool ok = true;
+    p->parts.reserve(first.size());
+    p->part_row.reserve(first.size());
     for (size_t i = 0; i + 1 < first.size(); ++i) {
         const int r0 = first[i], n = first[i + 1] - r0;
         cu.resize(n + 1);
@@ -62,12 +61,20 @@ void make_parts(hat_plan* p, const hat_cache_desc* cache) {
             delete part;
             st = create_plan(cache, &b, /*part=*/true, /*whole=*/true, &part);
         }
-        ok = st == HAT_OK;
-        if (!ok) break;
+        if (st != HAT_OK) return false;
         p->parts.push_back(part);
         p->part_row.push_back(p->cu_chunk[r0]);
     }
-    if (ok) ok = upload_plans(p->parts.data(), p->parts.size(), &p->part_res) == HAT_OK;
+    return upload_plans(p->parts.data(), p->parts.size(), &p->part_res) == HAT_OK;
+}
+
+void make_parts(hat_plan* p, const hat_cache_desc* cache) {
+    std::vector<int> first;
+    p->parts_made = true;
+    bool several = false, ok = false;
+    guarded([&] { several = split_requests(p, first); return HAT_OK; });
+    if (!several) return;
+    guarded([&] { ok = plan_parts(p, cache, first); return HAT_OK; });
     for (hat_plan* part : p->parts) {
         part->res.ev_verify = p->part_res.ev_verify;
         part->res.ev_done = p->part_res.ev_done;
@@ -75,6 +82,7 @@ void make_parts(hat_plan* p, const hat_cache_desc* cache) {
     }
     if (!ok) {
         p->parts.clear();
+        p->part_row.clear();
         plan_res_free(p->part_res);
     }
 }

@@ -32,7 +32,7 @@ size_t block_size(size_t n) {
 
 struct Pool {
     std::mutex mu;
-    std::vector<PlanRes> idle;
+    std::vector<PlanRes> idle;        // room for kMaxIdle from the start: giving back allocates nothing
     // uploads: one at a time, complete before the next, so that one pinned buffer serves all plans
     std::mutex up_mu;
     std::vector<std::pair<int, cudaStream_t>> up_streams;   // per device
@@ -40,7 +40,7 @@ struct Pool {
     size_t up_bytes = 0;
 };
 Pool& pool() {
-    static Pool* p = new Pool();      // never destroyed: plans may outlive static destructors
+    static Pool* p = [] { Pool* q = new Pool(); q->idle.reserve(kMaxIdle); return q; }();   // never destroyed: plans may outlive static destructors
     return *p;
 }
 
@@ -123,7 +123,8 @@ cudaError_t plan_res_copy_streams(PlanRes& r) {
 cudaError_t plan_res_release(PlanRes& r, bool reusable) {
     if (!r.blob || !reusable || r.blob_bytes > kMaxIdleBytes) return plan_res_free(r);
     Pool& p = pool();
-    std::vector<PlanRes> gone;
+    PlanRes gone[kMaxIdle];
+    size_t num_gone = 0;
     {
         std::lock_guard<std::mutex> lock(p.mu);
         size_t bytes = idle_bytes(p.idle);
@@ -135,7 +136,7 @@ cudaError_t plan_res_release(PlanRes& r, bool reusable) {
                 if (cudaEventQuery(old.ev_done) != cudaSuccess) { ++i; continue; }
             }
             bytes -= old.blob_bytes;
-            gone.push_back(old);
+            gone[num_gone++] = old;
             p.idle.erase(p.idle.begin() + i);
         }
         if (queried) cudaGetLastError();                         // cudaErrorNotReady of a query is no error
@@ -145,8 +146,8 @@ cudaError_t plan_res_release(PlanRes& r, bool reusable) {
         }
     }
     cudaError_t first = plan_res_free(r);                        // nothing, if it waits in the list
-    for (PlanRes& old : gone) {
-        const cudaError_t e = plan_res_free(old);
+    for (size_t i = 0; i < num_gone; ++i) {
+        const cudaError_t e = plan_res_free(gone[i]);
         if (first == cudaSuccess) first = e;
     }
     return first;
@@ -180,6 +181,7 @@ cudaError_t plan_res_upload(PlanRes& r, const UploadPart* parts, size_t num_part
 cudaError_t plan_res_trim() {
     Pool& p = pool();
     std::vector<PlanRes> gone;
+    gone.reserve(kMaxIdle);                                      // what the list has afterwards
     {
         std::lock_guard<std::mutex> lock(p.mu);
         gone.swap(p.idle);

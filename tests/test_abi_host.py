@@ -267,3 +267,34 @@ def test_choice_of_the_tile_kernel(hat_lib):
     assert info([1000] * 8, [512] * 8, 40, dtype="fp16")["prefill_kernel"] == 1    # fp16 units of ~1400 keys: no gain on pairs
     assert info([100] * 8, [4] * 8, 40)["prefill_kernel"] == 1                 # no tile-class chunk at all
     assert info([100] * 8, [512] * 8, 40, d=64)["prefill_kernel"] == 1
+
+
+_EXHAUSTED = """
+import resource, sys
+import numpy as np
+from paper_2503_18989_b200 import binding as B
+B.lib()
+rows = 1 << 28                                  # the plan's table of rows alone takes 1 GiB
+pages = rows // 16
+table = np.arange(pages, dtype=np.int32).reshape(1, pages)
+cache = B.make_cache_desc("fp16", pages, 1, 64, 1024, 64, 1024)
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (600 << 20), resource.RLIM_INFINITY))
+for _ in range(2):
+    try:
+        B.hat_plan_create(cache, 1, [0, rows], [0], [rows], table, flags=B.HAT_PLAN_HOST_ONLY)
+    except B.HatError as e:
+        print("status", e.status)
+plan = B.hat_plan_create(cache, 1, [0, 5], [0], [5], table, flags=B.HAT_PLAN_HOST_ONLY)
+print("rows", B.hat_plan_get_info(plan).total_rows)
+"""
+
+
+def test_exhausted_host_memory_is_a_status(hat_lib):
+    """A plan whose arrays cannot be allocated: a status, not an exception across the C boundary (which ends the process)."""
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _EXHAUSTED], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr[-500:]
+    assert r.stdout.split() == ["status", "-1", "status", "-1", "rows", "5"]
