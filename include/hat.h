@@ -335,7 +335,10 @@ int hat_plan_read_timing(hat_plan* plan, float* ms, int capacity_calls, int* num
  * as soon as their out/lse rows are final; the tile kernel for the prompt chunks
  * of the same batch only takes the SMs that they leave.
  *   hat_plan_verify_event   the cudaEvent_t (as void*), e.g. for cudaStreamWaitEvent on the caller's own stream
- *                           that returns those rows to the devices; it is re-recorded by every attention call
+ *                           that returns those rows to the devices; it is re-recorded by every attention call of a
+ *                           batch that has such chunks, and counts as occurred for one that has none.  A call with host
+ *                           buffers that is processed in parts records it in the last part that has such chunks; the rows
+ *                           are then final in `staging`, and in host memory once the stream is
  *   hat_plan_wait_verify    blocks the host until the event of the latest call has occurred
  */
 int hat_plan_verify_event(const hat_plan* plan, void** event_out);

@@ -928,9 +928,9 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
         if (e != cudaSuccess) return cuda_fail(e);
         mark(2, 1);
     }
-    // a batch without such rows has nothing to announce (an event that was never recorded counts as occurred); a part's are
-    // announced with the whole batch
-    if (has_verify && !plan->is_part && (e = cudaEventRecord(plan->res.ev_verify, s)) != cudaSuccess) return cuda_fail(e);
+    // a batch without such rows has nothing to announce (an event that was never recorded counts as occurred); of the parts of a
+    // batch the last one that has some announces (the others have no event)
+    if (has_verify && plan->res.ev_verify && (e = cudaEventRecord(plan->res.ev_verify, s)) != cudaSuccess) return cuda_fail(e);
     // The tile kernels depend on nothing the streaming kernel does: they take the SMs as it leaves them.  (Not under the timing
     // recorder, which wants the kernels one after the other.)
     a.overlap = has_verify && plan->info.stream_kernel == 1 && !side && call < 0 ? 1 : 0;

@@ -75,11 +75,13 @@ void make_parts(hat_plan* p, const hat_cache_desc* cache) {
     guarded([&] { several = split_requests(p, first); return HAT_OK; });
     if (!several) return;
     guarded([&] { ok = plan_parts(p, cache, first); return HAT_OK; });
+    hat_plan* last = nullptr;                                // of the parts with drafts: announces those of the whole batch
     for (hat_plan* part : p->parts) {
-        part->res.ev_verify = p->part_res.ev_verify;
         part->res.ev_done = p->part_res.ev_done;
+        if (part->info.num_verify_items > 0) last = part;
         if (!ok) delete part;
     }
+    if (ok && last) last->res.ev_verify = p->res.ev_verify;
     if (!ok) {
         p->parts.clear();
         p->part_row.clear();
@@ -156,7 +158,6 @@ int host_step(const hat_cache_desc* cache, const hat_plan* plan, const HostBuffe
         if (i > 0 && !copy_out(p->part_row[i - 1], p->parts[i - 1]->total_rows, out)) return HAT_ERR_CUDA;
         if (!edge(s, out)) return HAT_ERR_CUDA;
     }
-    if ((e = cudaEventRecord(p->res.ev_verify, s)) != cudaSuccess) return HAT_ERR_CUDA;
     done.now();                                              // before the last copies back: they are no one's business but the caller's
     if (!copy_out(p->part_row[n - 1], p->parts[n - 1]->total_rows, out) || !edge(out, s)) return HAT_ERR_CUDA;
     return HAT_OK;

@@ -53,6 +53,38 @@ def test_parts_of_a_host_call(cuda_device, dtype, group, tree, pinned):
     ds.close()
 
 
+def test_drafts_are_announced_in_the_last_part_that_has_some(cuda_device):
+    """The verify event of a call in parts: the drafts' rows are final in staging memory when it has occurred; the parts
+    behind it hold prompt chunks only."""
+    import torch
+    from paper_2503_18989_b200 import binding as B, runner
+    H, d = 5, 128
+    sc = _batch("fp16", H, d, [700, 33] + _PREFIX[:1] + [900, 640, 1000], [4, 16] + _CHUNK[:1] + [512, 500, 512], 303)
+    st = sc.steps[0]
+    cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
+    ds = runner.DeviceStep(cache, st)
+    T = st.total_rows
+    q, k, v = (torch.from_numpy(a.view(np.int16)).pin_memory() for a in (st.q, st.k_new, st.v_new))
+    nbytes = B.hat_plan_staging_bytes(ds.plan)
+    o, l = torch.empty((T, H, d)).pin_memory(), torch.empty((T, H)).pin_memory()
+    staging = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device=cuda_device)
+    s, side = torch.cuda.Stream(cuda_device), torch.cuda.Stream(cuda_device)
+    torch.cuda.synchronize()
+    before = B.hat_launch_count()
+    B.hat_chunk_attention_host(cache.desc, ds.plan, q, k, v, o, l, 0.0, staging, nbytes, ds.workspace, ds.workspace_bytes, s.cuda_stream)
+    assert B.hat_launch_count() - before >= 4                         # several parts
+    B.hat_plan_wait_verify(ds.plan)
+    pad = lambda n: (n + 255) // 256 * 256
+    at = 3 * pad(T * H * d * 2)                                       # q, k_new, v_new of as many heads
+    with torch.cuda.stream(side):
+        rows = staging[at:at + 20 * H * d * 4].cpu().view(torch.float32).view(20, H, d).numpy()
+    torch.cuda.synchronize()
+    kp, vp, want = oracle_replay(sc)
+    assert_parity(rows, want[0][0][:20], "drafts in staging")
+    assert_parity(o.numpy(), want[0][0], "out")
+    ds.close()
+
+
 @pytest.mark.parametrize("first,second", [("host", "device"), ("device", "host"), ("host", "host")])
 def test_a_call_in_parts_and_the_plans_other_calls_are_ordered(cuda_device, first, second):
     """Two calls of one plan on two streams: the second one's kernels wait for the first, whichever of them copies from host
