@@ -998,7 +998,7 @@ cudaError_t launch_attn_pair(const hat_plan* plan, const AttnArgs& args, cudaStr
     if (!mq || !plan_pool_maps(plan, args.cache, &mk4, &mv) || !plan_tile_maps(plan, args.cache, &mk, &mv5, &fold) ||
         !plan_new_maps(plan, args.k_new, args.v_new, &mkn, &mvn, &mvh))
         return cudaErrorInvalidValue;
-    // the unit counter is zero at this point: the previous call's last CTA cleared it
+    // the unit counter is zero at this point: the last of the previous call's producers cleared it
     const int total_units = num_units >= 0 ? num_units : (int)plan->tile_units.size();
     if (total_units <= 0) return cudaSuccess;
     int32_t* counter = plan->dev.status + 1;

@@ -2,8 +2,9 @@
 //
 // Some hosts of this library run where cudaMalloc is off limits: inside a CUDA-graph capture or
 // a latency-critical serving loop whose memory was carved up at start-up, or under a framework that
-// owns the whole device heap.  hat_chunk_attention needs a plan (one cudaMalloc) and a caller-provided
-// workspace for its split-KV partial results.  The entry point in this file needs neither: the batch
+// owns the whole device heap.  hat_chunk_attention needs a plan (device memory, allocated unless
+// a destroyed plan left some) and a caller-provided workspace for its split-KV partial results.  The
+// entry point in this file needs neither: the batch
 // descriptor arrays are read straight from device memory, every request is cut into a fixed number of
 // key ranges computed from its length inside the kernel, and the partial results live in a file-scope
 // __device__ array that is part of the loaded module (HAT_STATIC_SCRATCH_BYTES on every GPU that loads

@@ -828,7 +828,7 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     int fold = 0;
     if (!mq || !plan_tile_maps(plan, args.cache, &mk, &mv, &fold) || !plan_new_maps(plan, args.k_new, args.v_new, &mkn, &mvn, &mvh))
         return cudaErrorInvalidValue;
-    // one CTA per SM draws units from a counter that is zero at this point: the previous call's last CTA cleared it
+    // one CTA per SM draws units from a counter that is zero at this point: the last of the previous call's producers cleared it
     // (reset_counter); a grid that joins another one on the same counter leaves it alone
     const int total_units = num_units >= 0 ? num_units : (int)plan->tile_units.size() - first_unit;
     if (total_units <= 0) return cudaSuccess;

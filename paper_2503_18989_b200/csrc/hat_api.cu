@@ -189,7 +189,8 @@ static bool pieces_meet_in_clusters(const hat_plan* p, int num_sms, int64_t unit
 }
 
 // Key-range length for the tile-class requests of a batch that is too small to fill the persistent tcgen05 kernel.
-// Every candidate length is priced with a small model of that kernel, in SM clock cycles measured on B200: a 128-key
+// Every candidate length is priced with a small model of the one-CTA kernel (also for batches of the pair kernel, whose 74 pairs
+// take 2350 to 2720 cycles a step: the model is only a rough guide there), in SM clock cycles measured on B200: a 128-key
 // step of a 256-row unit (two query tiles) or of a unit of at most 128 rows (two chains share it), the fixed cost of a
 // unit (its Q tiles, refilling the rings, storing its rows), and the merge pass (its launch plus reading every partial
 // row).  Units go to the CTAs longest first, as the kernel draws them.  Returns 0 for "leave every request whole".
@@ -760,8 +761,9 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
             for (int row0 = 0; row0 < C; row0 += 256)
                 if (C - row0 > 128) { ++wide_tiles; wide_keys += p->prefix_len[r] + std::min(C, row0 + 256); }
         }
-        // measured (chunks of 512 and 256 rows, 40 heads): for bf16 the pair kernel is the faster one at every batch size
-        // (1 to 8 chunks: 9 to 26 %), for fp16 from about 1.5 units per SM on (equal at 160 units, 2.5 % at 240, 16 % at 320)
+        // measured (chunks of 512 and 256 rows, 40 heads; the one-CTA kernel has since got units of 128 rows, halves merged by
+        // clusters and shorter code, so that small bf16 batches may by now be faster on it: not measured again): for bf16 the pair
+        // kernel is the faster one at every batch size (1 to 8 chunks: 9 to 26 %), for fp16 from about 1.5 units per SM on (equal at 160 units, 2.5 % at 240, 16 % at 320)
         // bf16: the units of more than 128 rows go to the pairs even when the batch also has narrower ones (those run on
         // single CTAs behind them: a ragged bf16 batch measured 0.298 + 0.118 ms that way against 0.49 on either kernel alone)
         // fp16: pairs pay off only for long units (prefix 4000: +16 %; 8 chunks of 512 at prefix 2000: +4.5 %, at 1000: -2 %; a ragged batch's wide units, ~2300 keys on average with many short ones: -3 %)

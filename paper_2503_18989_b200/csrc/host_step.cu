@@ -4,8 +4,8 @@
 // idle in one direction all the time and in both while the kernels run (636 rows x 32 heads: 294 + 95 + 190 us).  So a batch
 // with enough rows is split into parts, contiguous requests with plans of their own: part by part the rows come in on a
 // stream of the plan's, are computed on the caller's stream and go back on a third one.  The caller's stream waits for the
-// last copy back.  636 rows: 603 us in one part, 514 us in
-// six (the link moves 44 to 77 GB/s in both directions together at such sizes).
+// last copy back.  636 rows: 603 us in one part, 508 us in
+// five (the link moves 44 to 77 GB/s in both directions together at such sizes).
 #include <algorithm>
 
 #include "hat_internal.h"

@@ -13,8 +13,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 
 // Programmatic dependent launch: a kernel launched with launch_pdl starts while the stream's previous kernel still runs, once
 // every CTA of that one has called pdl_launch_dependents or ended (a kernel calls it early, a persistent grid being
-// resident by then; the streaming and pair kernels once what precedes them has ended, since kernels of the same call may run beside them).  pdl_wait returns when the previous kernel has ended and its writes are visible.  Before it a kernel
-// reads nothing but its plan's arrays, which the host completed before the launch, and writes nothing.
+// resident by then; the streaming and pair kernels once what precedes them has ended, since kernels of the same call may run
+// beside them).  pdl_wait returns when the previous kernel has ended and its writes are visible.  Before it a kernel
+// reads nothing but its plan's arrays, which the host completed before the launch, writes nothing, and starts no bounded wait.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
