@@ -360,7 +360,7 @@ int hat_last_device_status(const hat_plan* plan, void* stream, int* out);
  * projection (tcgen05) and streaming attention by TMA.  Every wait inside them
  * (on a transfer, on the tensor pipe, on another warp or the other CTA of a
  * pair) is bounded by `cycles` SM clock cycles (0 selects the default of 2e9,
- * about a second), counted from the end of what precedes the call on the stream;
+ * about a second), beside the time its kernel waited for what precedes it;
  * a wait that runs out sets the status word above, tells the other warps of its
  * CTA (and the other CTA of its pair) to stop, and the CTA lets what is in flight
  * land, releases its tensor memory and exits.

@@ -94,7 +94,7 @@ struct __align__(8) Barriers {
     uint64_t m_ready[2][4];                                 // fp16, own: warpgroup w, lane quarter q published its tile's reference maximum
     uint64_t fin_ready[2][4];                               // fp16, own: the same for the row-sum hand-over at the end of a unit
     uint64_t drain, drain2;
-    long long wait_cycles;                                  // bound of every wait below
+    volatile long long wait_cycles;                         // bound of every wait below (see waits_begin)
     uint32_t tmem_base;
     volatile int abort_flag;
     volatile int unit_slot[kUnitSlots];                     // unit index, or -1 when the work has run out
@@ -201,7 +201,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
         mbar_init(&bars->drain, 1);
         mbar_init(&bars->drain2, 1);
         bars->abort_flag = 0;
-        bars->wait_cycles = a.wait_cycles;
+        bars->wait_cycles = a.overlap ? a.wait_cycles : kNotYet;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
@@ -217,9 +217,6 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
     cluster_wait();
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
-    // The two producers wait for the previous kernel's end once they have read what they can; the other roles do so here, so that
-    // their bounded waits do not run while another kernel does.
-    if (warp != 0 && warp != 11 && !a.overlap) pdl_wait();
 
     // A consumer's read of the unit queue: the unit published as number `un` (-1: none left, -2: gave up).
     auto read_unit = [&](int un, bool whole_warp) -> int {
@@ -236,6 +233,7 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch (CTA 0) + TMA producer (both)
         bool ok = true;
+        const long long since = clock64();
         // CTA 0: draw a unit and publish it in slot un % 4 of both CTAs' queues (all lanes return it); the slot is free
         // once every reader in both CTAs has read the unit published four draws earlier
         auto publish = [&](int un) -> int {
@@ -298,7 +296,10 @@ attn_pair_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units
             };
             int page = page_of(0);
             if (un == 0) {
-                if (!a.overlap) pdl_wait();                      // up to here only the plan's own arrays were read
+                if (!a.overlap) {
+                    pdl_wait();                                  // up to here only the plan's own arrays were read
+                    if (lane == 0) waits_begin(&bars->wait_cycles, since, a.wait_cycles);
+                }
                 pdl_launch_dependents();                         // the kernel behind may be one that runs beside this one
             }
             if (rank == 0) {

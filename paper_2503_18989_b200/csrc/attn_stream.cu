@@ -121,6 +121,7 @@ template <int SLOTS> struct __align__(16) Ctl {
     uint64_t todo_full;                                          // every unit is done, the list is final
     uint64_t hand[kWarps];                                       // warp w has handed over (the last in line: to the output warp)
     volatile int abort_flag;
+    volatile long long wait_cycles;                              // bound of every wait (see tc5::waits_begin)
 };
 
 template <int SLOTS>
@@ -129,7 +130,7 @@ __device__ __forceinline__ bool wait_for(uint64_t* bar, uint32_t parity, Ctl<SLO
     const long long t0 = clock64();
     while (!mbar_try(bar, parity)) {
         if (ctl->abort_flag) return false;
-        if (clock64() - t0 > a.wait_cycles) {
+        if (clock64() - t0 > ctl->wait_cycles) {
             ctl->abort_flag = 1;
             atomicOr(a.plan.status, 1);
             return false;
@@ -168,6 +169,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
         ctl->num_todo = 0;
         for (int w = 0; w < kWarps; ++w) mbar_init(&ctl->hand[w], 1);
         ctl->abort_flag = 0;
+        ctl->wait_cycles = tc5::kNotYet;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
@@ -180,10 +182,10 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
     const uint32_t g_inv = ((1u << 20) + G - 1) / G;
     auto pair_row = [&](int pair) { return G < 256 ? (int)(((uint32_t)pair * g_inv) >> 20) : pair / G; };
     bool ok = true;
-    if (warp != kWarps) tc5::pdl_wait();                          // the bounded waits below do not run while another kernel does
 
     if (warp == kWarps) {
         // ------------------------------------------------------------------ producer
+        const long long since = clock64();
         const uint16_t* __restrict__ q = static_cast<const uint16_t*>(a.q);
         const bool fused = a.k_new != nullptr;
         // Pages are requested kBatch at a time, lanes 2 k and 2 k + 1 moving K and V of page k: a page at a time (600 cycles of
@@ -219,6 +221,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
             }
         }
         tc5::pdl_wait();                                          // up to here only the plan's own arrays were read
+        if (lane == 0) tc5::waits_begin(&ctl->wait_cycles, since, a.wait_cycles);
         // the kernel behind may be one that runs beside this one (tile kernels of the same call): what precedes both has ended
         tc5::pdl_launch_dependents();
         for (;;) {

@@ -60,7 +60,7 @@ struct __align__(8) Barriers {
     uint64_t x_ready, x_ready0;                             // split units: (reference maximum, row sum) of chain 1 are in xchg, chain 0's too
     uint64_t peer_ready[8];                                 // kHalves: the softmax warp of the same number in the other CTA has its rows ready
     uint64_t drain;
-    long long wait_cycles;                                  // bound of every wait below
+    volatile long long wait_cycles;                         // bound of every wait below (see waits_begin)
     uint32_t tmem_base;
     volatile int abort_flag;
     volatile int unit_slot[2];                              // unit index, or -1 when the work has run out
@@ -181,7 +181,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         for (int w = 0; w < 8; ++w) mbar_init(&bars->peer_ready[w], 1);
         mbar_init(&bars->drain, 1);
         bars->abort_flag = 0;
-        bars->wait_cycles = a.wait_cycles;
+        bars->wait_cycles = a.overlap ? a.wait_cycles : kNotYet;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
@@ -198,15 +198,18 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     pdl_launch_dependents();
-    // The producer waits for the previous kernel's end once it has read what it can; the other roles do so here, so that their bounded
-    // waits (for what the producer requests afterwards) do not run while another kernel does.
-    if (warp != 0 && !a.overlap) pdl_wait();
-
     if (warp == 0) {
         // ------------------------------------------------------------------ unit fetch + TMA producer
         // Lane pg + 8 g moves page pg of a tile: one box (g = 0), or its two 8-row groups where the pool's strides fold neither
         // way and for rows of k_new / v_new.  What this warp does per tile is close to what a tile costs the tensor core, so
         // the loop over plain tiles holds no more than it must (ring positions are stepped, page ids fetched a tile ahead).
+        const long long since = clock64();
+        // the previous kernel's end, once what the plan's own arrays hold has been read
+        auto front_ended = [&]() {
+            if (a.overlap) return;
+            pdl_wait();
+            if (lane == 0) waits_begin(&bars->wait_cycles, since, a.wait_cycles);
+        };
         const int pg = lane & 7, grp = lane >> 3;
         const int boxes = fold ? 8 : 16;                         // lanes that move pool pages
         const int c1 = 8 * grp, s3 = fold == 1 ? 1 : 0, s4 = fold == 2 ? 1 : 0;
@@ -255,7 +258,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             unit = __shfl_sync(0xffffffffu, unit, 0);
             if (unit < 0) {
                 // a grid that joins another one may find nothing left: its end still stands for the end of what precedes it
-                if (un == 0 && !a.overlap) pdl_wait();
+                if (un == 0) front_ended();
                 break;
             }
             const Unit u = decode_unit(a, items, unit);
@@ -271,8 +274,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             if (un > 0) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_empty, (un - 1) & 1, bars));
                 if (!ok) break;
-            } else if (!a.overlap) {
-                pdl_wait();                                      // up to here only the plan's own arrays were read
+            } else {
+                front_ended();
             }
             if (lane == 0) mbar_expect_tx(&bars->q_full, u.nq * kTileBytes);
             if (lane < kSlabs * u.nq)       // lane = kSlabs * (query tile) + (column half)

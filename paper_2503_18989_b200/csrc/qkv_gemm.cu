@@ -60,7 +60,7 @@ struct __align__(8) Barriers {
     uint64_t full[kMaxStages], empty[kMaxStages];
     uint64_t acc_full[2], acc_empty[2];
     uint64_t drain;
-    long long wait_cycles;
+    volatile long long wait_cycles;          // see waits_begin
     uint32_t tmem_base;
     volatile int abort_flag;
 };
@@ -234,7 +234,7 @@ qkv_gemm_kernel(const __grid_constant__ QkvArgs a, const __grid_constant__ CUten
         }
         mbar_init(&bars->drain, 1);
         bars->abort_flag = 0;
-        bars->wait_cycles = a.wait_cycles;
+        bars->wait_cycles = kNotYet;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
@@ -257,17 +257,18 @@ qkv_gemm_kernel(const __grid_constant__ QkvArgs a, const __grid_constant__ CUten
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     pdl_launch_dependents();
-    if (warp != 0) pdl_wait();                                  // the bounded waits below do not run while another kernel does
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one lane)
         if (lane == 0) {
             bool ok = true;
             int it = 0;                                        // stages issued so far, over all tiles
+            const long long since = clock64();
             // CTAs start as the previous kernel's run out of work: its tail brings the first stretch of w to L2 (128 rows, 13B
             // shape, with the attention behind it: 178.3 us a layer without, 176.5 with; 40 steps are no better)
             for (int ks = 0; ks < min(k_steps, kAhead); ++ks) tma_prefetch_2d(&map_w, ks * kTileK, (first_tile / a.m_tiles) * kTileN + (int)rank * G::kBRows);
             pdl_wait();                                        // nothing that kernels write was read before, and nothing written
+            waits_begin(&bars->wait_cycles, since, a.wait_cycles);
             for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
                 const int m = tile % a.m_tiles, n = tile / a.m_tiles;
                 const int x_row = PAIR ? m * 2 * kTileM + (int)rank * kTileM : m * kTileM;

@@ -90,6 +90,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// The bound of a CTA's waits, in its shared memory.  A kernel that starts in the tail of the previous one must not use it up while that one
+// runs: it is as good as infinite until the producer has waited for that end (from clock `since` on, the start of the roles) and adds
+// what that took.  (The other warps waiting for it themselves cost 0.6 us a call and more: 10 drafts and chunks 143 -> 147 us.)
+constexpr long long kNotYet = 1ll << 62;
+__device__ __forceinline__ void waits_begin(volatile long long* bound, long long since, long long limit) { *bound = clock64() - since + limit; }
+
 // For a CTA that gave up a wait, once all its roles have stopped: copies and products still in flight get a bounded time (a
 // millisecond) to land before its shared and tensor memory is released.
 __device__ __forceinline__ void settle() {
