@@ -194,7 +194,6 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
         // has the fewest.
         const int bk = lane < 2 * kBatch ? lane >> 1 : 0, is_v = lane & 1, way = kWarps - 1 - bk % kWarps;
         int issued = 0;                                           // pages requested for `way` so far
-        bool withhold = a.withhold;                               // self test: one transfer of the first pages never arrives, its consumer gives up
         int unit = blockIdx.x, un = 0;
         int hs = 0, page_id = 0;
         int4 r0, r1, r2;                                          // the unit's StreamItem; page_id: of its first 32 pages, one per lane
@@ -258,7 +257,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
                 }
                 if (lane == 0) { ctl->unit[0] = r0; ctl->unit[1] = r1; ctl->unit[2] = r2; ctl->hs = done ? -1 : hs; }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->q_full);
+                if (lane == 0 && !(a.withhold && un == 0)) mbar_arrive(&ctl->q_full);   // self test: the first Q tile never arrives
                 ++un;
             }
             if (done) break;
@@ -296,7 +295,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
                     const bool prefix = mine && page0 + j0 + bk < npre;
                     if (prefix && !is_v) mbar_expect_tx(&ctl->full[slot], SLOT);
                     __syncwarp();
-                    if (prefix && !(withhold && lane == 1)) tc5::tma_load_5d(smem_u32(smem) + slot * SLOT + is_v * PAGE, is_v ? &map_v : &map_k, 0, 0, 0, h, page, &ctl->full[slot]);
+                    if (prefix) tc5::tma_load_5d(smem_u32(smem) + slot * SLOT + is_v * PAGE, is_v ? &map_v : &map_k, 0, 0, 0, h, page, &ctl->full[slot]);
                     if (page1 > npre && j0 + kBatch >= n) {
                         // the chunk's rows, one after the other from k_new / v_new or from their slots of the pool
                         const int cslot = __shfl_sync(0xffffffffu, slot, 2 * (n - 1 - j0));
@@ -321,9 +320,8 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
                         }
                         cp_async_on(&ctl->full[cslot]);
                         __syncwarp();
-                        if (lane == 0 && !(withhold && page0 + j0 == npre)) mbar_arrive(&ctl->full[cslot]);
+                        if (lane == 0) mbar_arrive(&ctl->full[cslot]);
                     }
-                    withhold = false;
                     issued += (min(kBatch, n - j0) + way) / kWarps;
                 }
                 if (!ok) break;
