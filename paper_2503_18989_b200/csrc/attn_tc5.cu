@@ -14,8 +14,8 @@
 //               softmax in registers (reference maximum only moved when it grows by more than 2^8, so O is rarely
 //               rescaled), P written back to TMEM as the 16-bit A operand; at the end of a unit O is pulled into
 //               registers (which frees the accumulator for the next unit), divided by l and stored with the lse
-// TMEM columns: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512).  P_t(j) overwrites S_t(j) in place (16-bit pairs in
-// columns [0,64), the bf16 rounding remainder in [64,128)); S_t(j+1) is issued after P_t V(j) by the same thread, and
+// TMEM columns: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512).  P_t(j) overwrites S_t(j) in place (softmax_tile.cuh);
+// S_t(j+1) is issued after P_t V(j) by the same thread, and
 // tcgen05 executes one thread's MMAs in issue order, so no extra barrier guards the reuse.
 // A unit of at most 128 rows uses both column pairs for the SAME query tile: two chains over alternating key tiles,
 // merged by the first chain's warpgroup when the unit ends (see Unit::split).
@@ -32,6 +32,7 @@
 #include "tma_desc.h"
 #include "tc5_ptx.cuh"
 #include "out_rows.cuh"
+#include "softmax_tile.cuh"
 #include "tile_append.cuh"
 
 namespace hat {
@@ -440,10 +441,10 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         for (int ks = 0; ks < kKeys / 16; ++ks) {
                             // 16 keys = one page; inside it 64-column blocks 1 KiB apart (leading), then the next 8-key group
                             const uint64_t vdesc = vd + (uint64_t)((ks * kPageBytes) >> 4);
-                            mma_ts(to, tp + ks * 8, vdesc, idesc_o, (sidx > 0) || (ks > 0));
-                            if constexpr (BF16) mma_ts(to, tp + 64 + ks * 8, vdesc, idesc_o, true);
+                            mma_ts(to, tp + softmax_tile::weight_col(ks), vdesc, idesc_o, (sidx > 0) || (ks > 0));
+                            if constexpr (BF16) mma_ts(to, tp + softmax_tile::weight_col(ks) + 16, vdesc, idesc_o, true);
                         }
-                        tc_commit(&bars->o_done[qt]);
+                        if (sidx == u.n_t(qt) - 1) tc_commit(&bars->o_done[qt]);      // before that S(next) tells
                         if (SPLIT || qt == u.nq - 1) tc_commit(&bars->v_empty[st]);
                     };
                     if (u.n_t0 > 0) issue_s(0, 0);
@@ -509,24 +510,11 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     ++s_cnt;
                     if (!ok) break;
                     tc_fence_after();
-                    float s[kKeys];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) tmem_ld32(tm_s + c * 32, reinterpret_cast<uint32_t*>(s) + c * 32);
-                    tmem_ld_wait();
-
-                    // raw maximum (the scale is positive, so it commutes with max); four independent chains
-                    const int lim = last_key - kb;          // keys 0..lim of this tile are visible to this row
-                    if (lim < kKeys - 1) {
-#pragma unroll
-                        for (int k = 0; k < kKeys; ++k) s[k] = (k <= lim) ? s[k] : -INFINITY;
-                    }
-                    float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int k = 0; k < kKeys; k += 8) {
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) mx4[v] = fmaxf(mx4[v], fmaxf(s[k + 2 * v], s[k + 2 * v + 1]));
-                    }
-                    const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sc;
+                    softmax_tile::mask<kKeys>(tm_s, last_key - kb);   // keys 0 .. last_key - kb of this tile are visible to this row
+                    // raw maximum (the scale is positive, so it commutes with max)
+                    const float mx = softmax_tile::row_max<kKeys>(tm_s) * sc;
+                    uint32_t first[32];
+                    tmem_ld32(tm_s, first);
                     // move the reference maximum only when it grew by more than the threshold
                     float alpha = 1.f;
                     bool rescale = false;
@@ -535,39 +523,14 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         rescale = (m_used != -INFINITY);
                         m_used = mx;
                     }
-                    const float neg_ref = (m_used == -INFINITY) ? 0.f : -m_used;
-                    float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t p[16];
-                        uint32_t pl[16];
-#pragma unroll
-                        for (int k = 0; k < 32; k += 2) {
-                            const float e0 = fast_exp2(fmaf(s[c * 32 + k], sc, neg_ref));
-                            const float e1 = fast_exp2(fmaf(s[c * 32 + k + 1], sc, neg_ref));
-                            sum4[(k >> 1) & 3] += e0 + e1;
-                            p[k / 2] = pack2<BF16>(e0, e1);
-                            if constexpr (BF16) {
-                                const float r0 = e0 - __uint_as_float(p[k / 2] << 16);
-                                const float r1 = e1 - __uint_as_float(p[k / 2] & 0xffff0000u);
-                                pl[k / 2] = pack2<BF16>(r0, r1);
-                            }
-                        }
-                        tmem_st16(tm_s + c * 16, p);
-                        if constexpr (BF16) tmem_st16(tm_s + 64 + c * 16, pl);
-                    }
-                    l = l * alpha + ((sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
+                    softmax_tile::Weigh<BF16> weigh(sc, (m_used == -INFINITY) ? 0.f : -m_used);
+                    weigh.keys128(first, tm_s);
+                    l = l * alpha + weigh.total();
 
-                    // O may only be rescaled once the previous P V product has finished; waiting here every tile (it
-                    // has long completed by now) also keeps this thread's count of the barrier's phases exact
-                    if (sidx > 0) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done[qt], o_cnt & 1, bars));
-                        ++o_cnt;
-                        if (!ok) break;
-                        tc_fence_after();
-                    }
+                    // O may only be rescaled once the previous P V product has finished: it was issued, by the same thread, before
+                    // this step's S, which is here
                     if (__any_sync(0xffffffffu, rescale)) {
-#pragma unroll
+#pragma unroll 1
                         for (int c = 0; c < kD / 32; ++c) {
                             uint32_t o[32];
                             tmem_ld32(tm_o + c * 32, o);
