@@ -28,8 +28,10 @@
 // What bounds it: HBM for large batches (30 requests x 32 heads, 980 MB: 151 us = 6.5 TB/s, which is the measured copy rate; the
 // step of append, this kernel and their gap was 163 us, now 157), the start of the pipeline and the tail for medium ones (12
 // requests, 250 MB: 63 us of append, attention, merge and gaps per layer, now 46), a chain of latencies for one request
-// (4 rows x 700 tokens: 16.4 us a call, now 11.2: 1.5 us to the first request, 0.8 us HBM, 1 us a page, 1 us from warp to
-// warp, 3 us to store, count and merge).
+// (4 rows x 700 tokens: 10.9 us a call: 1 us to the Q tile, 1 us to the first page, 1.3 to 2 us of pages, 1.3 to 1.8 from warp to warp,
+// 1.3 to store and count, 3.3 to merge).
+// Batches of few units therefore run in a short form (CL > 0 below): a CTA for every unit, the warps' results combined by all warps
+// at once, the pieces of a request exchanged within a cluster: 8.0 us for that call; pick_short_cluster (hat_api.cu) says which batches.
 // Waits on the mbarriers are bounded and report through the plan's status word.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -139,14 +141,74 @@ __device__ __forceinline__ bool wait_for(uint64_t* bar, uint32_t parity, Ctl<SLO
     return true;
 }
 
+// The same for a barrier that the other CTAs of the cluster arrive on, acquiring what they wrote before.
+template <int SLOTS>
+__device__ __forceinline__ bool wait_for_cluster(uint64_t* bar, uint32_t parity, Ctl<SLOTS>* ctl, const AttnArgs& a) {
+    const long long t0 = clock64();
+    while (!tc5::mbar_try_cluster(bar, parity)) {
+        if (ctl->abort_flag) return false;
+        if (clock64() - t0 > ctl->wait_cycles) {
+            ctl->abort_flag = 1;
+            atomicOr(a.plan.status, 1);
+            return false;
+        }
+    }
+    return true;
+}
+
 // The dynamic shared memory from its first 1024-byte boundary on: ring, Q tile, hand-over buffer, control block.
 template <int D>
 __device__ __forceinline__ Ctl<Geo<D>::SLOTS>* ctl_of(unsigned char* smem) {
     return reinterpret_cast<Ctl<Geo<D>::SLOTS>*>(smem + Geo<D>::SLOTS * Geo<D>::SLOT + Geo<D>::Q + Geo<D>::X);
 }
 
-// The six warps' work.  A warp returns when it is done, or early when a wait gave up.
-template <bool BF16, int D>
+// Final rows of a unit: column chunk c (8 columns) of rows g and g + 8 of the tile, each with its maximum and row sum in ml.
+template <int D>
+struct RowStore {
+    const AttnArgs& a;
+    int H, G, h, pair0, pairs, row_base, lane;
+    template <typename F>
+    __device__ __forceinline__ void rows(const float4& ml, F&& row) const {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            if (e * 8 + (lane >> 2) >= pairs) continue;
+            const int pair = pair0 + e * 8 + (lane >> 2), i = pair / G;
+            row(e, (int64_t)(row_base + i) * H + h * G + (pair - i * G), e ? ml.y : ml.x, e ? ml.w : ml.z);
+        }
+    }
+    __device__ __forceinline__ void chunk(int c, const float4& o, int e, int64_t at, float inv) const {
+        const float v0 = (e ? o.z : o.x) * inv, v1 = (e ? o.w : o.y) * inv;
+        const int64_t to = at * D + 2 * (lane & 3) + c * 8;
+        if (a.out16 != nullptr) *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(a.out16) + to) = pack_out16(v0, v1, a.out16_bf16);
+        else *reinterpret_cast<float2*>(a.out + to) = make_float2(v0, v1);
+    }
+    __device__ __forceinline__ void lse(int64_t at, float m, float sum) const {
+        if ((lane & 3) == 0) a.lse[at] = sum > 0.f ? (m + log2f(sum)) * 0.6931471805599453f : -INFINITY;
+    }
+};
+
+// Partial results of the same rows over other keys, one after the other: maxima and sums of rows g and g + 8 (x, y and z, w).
+struct Weights { float m0, m1, l0, l1; };
+template <int N>
+__device__ __forceinline__ Weights weights_of(const float4 (&ml)[N], float (&w0)[N], float (&w1)[N]) {
+    Weights t{-INFINITY, -INFINITY, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < N; ++i) { t.m0 = fmaxf(t.m0, ml[i].x); t.m1 = fmaxf(t.m1, ml[i].y); }
+    const float f0 = t.m0 == -INFINITY ? 0.f : t.m0, f1 = t.m1 == -INFINITY ? 0.f : t.m1;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        w0[i] = fast_exp2(ml[i].x - f0); w1[i] = fast_exp2(ml[i].y - f1);
+        t.l0 += ml[i].z * w0[i]; t.l1 += ml[i].w * w1[i];
+    }
+    return t;
+}
+
+// The warps' work.  A warp returns when it is done, or early when a wait gave up.
+// CL = 0: persistent, as above.  CL > 0, the short form: as many CTAs as units, each with one: the CTAs of a cluster of CL have the pieces
+// (of equal size, the last with the chunk) of one request, K/V head and slab.  The warps' results meet in the ring slots, which nothing will refill, and are
+// combined by all warps at once; then the CTAs' through each other's shared memory, every CTA finishing D / CL columns: no chain
+// from warp to warp, no output warp, no partial rows, fence, count and merge.
+template <bool BF16, int D, int CL>
 __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* smem, const StreamItem* __restrict__ items, int n_sub, int total_units,
                                              int32_t* __restrict__ work_counter, int32_t* __restrict__ piece_counters, const CUtensorMap& map_k,
                                              const CUtensorMap& map_v) {
@@ -164,16 +226,21 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
         for (int s = 0; s < SLOTS; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         mbar_init(&ctl->q_full, 1);
         mbar_init(&ctl->q_empty, kWarps);
-        mbar_init(&ctl->x_free, 1);
+        mbar_init(&ctl->x_free, CL > 1 ? CL * kWarps : 1);
         mbar_init(&ctl->todo_full, 1);
         ctl->num_todo = 0;
-        for (int w = 0; w < kWarps; ++w) mbar_init(&ctl->hand[w], 1);
+        for (int w = 0; w < kWarps; ++w) mbar_init(&ctl->hand[w], CL > 0 ? kWarps : 1);
         ctl->abort_flag = 0;
         ctl->wait_cycles = tc5::kNotYet;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
     __syncthreads();
+    if constexpr (CL > 1) {
+        tc5::cluster_arrive();                                    // the other CTAs' barriers are initialised
+        tc5::cluster_wait();
+    }
+    const int rank = CL > 1 ? (int)tc5::cluster_ctarank() : 0;
 
     const int H = a.plan.num_heads, G = a.plan.group, Hkv = a.plan.num_kv_heads;
     const int hs_count = Hkv * n_sub;
@@ -194,7 +261,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
         // has the fewest.
         const int bk = lane < 2 * kBatch ? lane >> 1 : 0, is_v = lane & 1, way = kWarps - 1 - bk % kWarps;
         int issued = 0;                                           // pages requested for `way` so far
-        int unit = blockIdx.x, un = 0;
+        int unit = CL > 1 ? blockIdx.x / CL : blockIdx.x, un = 0;
         int hs = 0, page_id = 0;
         int4 r0, r1, r2;                                          // the unit's StreamItem; page_id: of its first 32 pages, one per lane
         auto fetch_record = [&](int u, int& hs_, int4& q0, int4& q1, int4& q2) {
@@ -208,6 +275,10 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
             return pg < min(q1.y, (q0.w + kPageSize - 1) / kPageSize) ? __ldg(t + pg) : 0;
         };
         fetch_record(unit, hs, r0, r1, r2);
+        if constexpr (CL > 1) {
+            const int pages = r1.y;
+            r1.x = pages * rank / CL; r1.y = pages * (rank + 1) / CL;
+        }
         page_id = fetch_ids(r0, r1);
         {
             // CTAs of this kernel start as those of the one before run out of work: its tail brings their first pages to L2
@@ -231,7 +302,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
             const int h = hs / n_sub, sub = hs - h * n_sub;
 #ifdef HAT_DEBUG_BOUNDS
             if (!done && (r0.x < 0 || C < 1 || C > 16 || P < 0 || row_base < 0 || row_base + C > a.plan.total_rows || page0 < 0 ||
-                          page1 <= page0 || page1 > npre + 1 || npre > a.plan.max_pages || r2.x < 1 || r2.x > kMaxSplits)) {
+                          page1 < page0 || (CL == 0 && page1 == page0) || page1 > npre + 1 || npre > a.plan.max_pages || r2.x < 1 || r2.x > kMaxSplits)) {
                 if (lane == 0) atomicOr(a.plan.status, 2);
                 ctl->abort_flag = 1;
                 ok = false;
@@ -239,6 +310,12 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
             }
 #endif
             const bool skip = !done && sub * 16 >= C * G;    // this request has fewer pairs
+            if constexpr (CL > 0) {
+                if (skip) {                                       // of every CTA of the cluster
+                    if (lane == 0) { ctl->hs = -1; mbar_arrive(&ctl->q_full); }
+                    break;
+                }
+            }
             if (!skip) {
                 if (un >= 1) ok = wait_for(&ctl->q_empty, (un - 1) & 1, ctl, a);
                 ok = __all_sync(0xffffffffu, ok);
@@ -280,7 +357,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
                 const int n = page1 - page0;
                 int ids = page_id, ids_next = 0;                  // page ids of this and the next 32 pages, one per lane
                 for (int j0 = 0; j0 < n; j0 += kBatch) {
-                    if (step < 3 && n - j0 <= 6 * kBatch) look_ahead();
+                    if (CL == 0 && step < 3 && n - j0 <= 6 * kBatch) look_ahead();
                     if ((j0 & 31) == 0) {
                         if (j0 > 0) ids = ids_next;
                         const int ahead = page0 + j0 + 32 + lane;
@@ -326,13 +403,14 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
                 }
                 if (!ok) break;
             }
+            if constexpr (CL > 0) break;
             while (step < 3) look_ahead();
             unit = next; hs = next_hs; page_id = next_id;
             r0 = n0; r1 = n1; r2 = n2;
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         // the last producer to finish leaves the unit counter at zero for the next call
-        if (lane == 0) {
+        if (CL == 0 && lane == 0) {
             __threadfence();
             if (atomicAdd(work_counter + 1, 1) == (int)gridDim.x - 1) {
                 work_counter[0] = 0;
@@ -432,7 +510,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
         }
     };
 
-    if (warp == kWarps + 1) {
+    if (CL == 0 && warp == kWarps + 1) {
         // ------------------------------------------------------------------ output, merge of cut requests
         const int g = lane >> 2, t4 = lane & 3;
         for (int un = 0;; ++un) {
@@ -509,6 +587,7 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
         ok = __all_sync(0xffffffffu, wait_for(&ctl->q_full, un & 1, ctl, a));
         if (!ok) return;
         const int hs = ctl->hs;
+        if (CL > 0 && hs < 0) return;
         if (hs < 0) {
             // the end, handed on to the output warp once it has taken the previous result
             if (warp == kWarps - 1) {
@@ -688,6 +767,74 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
 #pragma unroll
             for (int k = 0; k < ON; ++k) { o[k][0] += o[k][2]; o[k][1] += o[k][3]; }
         }
+        if constexpr (CL > 0) {
+            const auto result_of = [&](int w) { return reinterpret_cast<float4*>(smem + w * PER * SLOT) + lane; };
+            static_assert(PER * SLOT >= G_::X && ON % kWarps == 0, "a warp's result fits its ring slots");
+            float4* mine = result_of(warp);
+#pragma unroll
+            for (int k = 0; k < ON; ++k) mine[k * 32] = make_float4(o[k][0], o[k][1], o[k][2], o[k][3]);
+            mine[ON * 32] = make_float4(m[0], m[1], l[0], l[1]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->hand[0]);
+            ok = __all_sync(0xffffffffu, wait_for(&ctl->hand[0], 0, ctl, a));
+            if (!ok) return;
+            float4 ml[kWarps];
+            float w0[kWarps], w1[kWarps];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) ml[w] = result_of(w)[ON * 32];
+            const Weights t = weights_of(ml, w0, w1);
+            const float4 tml = make_float4(t.m0, t.m1, t.l0, t.l1);
+            constexpr int SHARE = ON / kWarps;                       // column chunks a warp combines
+            float4 acc[SHARE];
+#pragma unroll
+            for (int k = 0; k < SHARE; ++k) {
+                acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    const float4 v = result_of(w)[(warp * SHARE + k) * 32];
+                    acc[k].x += v.x * w0[w]; acc[k].y += v.y * w0[w]; acc[k].z += v.z * w1[w]; acc[k].w += v.w * w1[w];
+                }
+            }
+            const RowStore<D> to{a, H, G, h, pair0, pairs, row_base, lane};
+            if constexpr (CL == 1) {
+                to.rows(tml, [&](int e, int64_t at, float mx, float sum) {
+                    const float inv = sum > 0.f ? 1.f / sum : 0.f;
+#pragma unroll
+                    for (int k = 0; k < SHARE; ++k) to.chunk(warp * SHARE + k, acc[k], e, at, inv);
+                    if (warp == 0) to.lse(at, mx, sum);
+                });
+            } else {
+                float4* give = xbuf + lane;
+#pragma unroll
+                for (int k = 0; k < SHARE; ++k) give[(warp * SHARE + k) * 32] = acc[k];
+                if (warp == 0) give[ON * 32] = tml;
+                __syncwarp();
+                if (lane < CL) tc5::mbar_arrive_cluster(tc5::map_to_cta(smem_u32(&ctl->x_free), lane));
+                ok = __all_sync(0xffffffffu, wait_for_cluster(&ctl->x_free, 0, ctl, a));
+                if (!ok) return;
+                constexpr int OWN = ON / CL;                         // column chunks a CTA finishes
+                for (int k = warp; k < OWN; k += kWarps) {
+                    const int c = rank * OWN + k;
+                    float4 ml2[CL], v[CL];
+                    float u0[CL], u1[CL];
+#pragma unroll
+                    for (int i = 0; i < CL; ++i) {
+                        const uint32_t from = tc5::map_to_cta(smem_u32(give), (uint32_t)i);
+                        ml2[i] = tc5::ld_cluster_f4(from + ON * 512);
+                        v[i] = tc5::ld_cluster_f4(from + c * 512);
+                    }
+                    const Weights t2 = weights_of(ml2, u0, u1);
+                    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < CL; ++i) { r.x += v[i].x * u0[i]; r.y += v[i].y * u0[i]; r.z += v[i].z * u1[i]; r.w += v[i].w * u1[i]; }
+                    to.rows(make_float4(t2.m0, t2.m1, t2.l0, t2.l1), [&](int e, int64_t at, float mx, float sum) {
+                        to.chunk(c, r, e, at, sum > 0.f ? 1.f / sum : 0.f);
+                        if (c == 0) to.lse(at, mx, sum);
+                    });
+                }
+            }
+            return;
+        }
         const bool have = kWarps - 1 - warp < n;                    // this warp worked on the unit
         float4* x = xbuf + lane;
         if (warp > 0) ok = wait_for(&ctl->hand[warp - 1], un & 1, ctl, a);
@@ -739,9 +886,39 @@ attn_stream_kernel(const __grid_constant__ AttnArgs a, const StreamItem* __restr
                    const __grid_constant__ CUtensorMap map_v) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    stream_roles<BF16, D>(a, smem, items, n_sub, total_units, work_counter, piece_counters, map_k, map_v);
+    stream_roles<BF16, D, 0>(a, smem, items, n_sub, total_units, work_counter, piece_counters, map_k, map_v);
     __syncthreads();
     if (ctl_of<D>(smem)->abort_flag) tc5::settle();
+}
+
+constexpr int kShortThreads = kWarps * 32 + 32;       // no output warp
+
+template <bool BF16, int D, int CL>
+__global__ void __launch_bounds__(kShortThreads, kCtasPerSm)
+attn_stream_short_kernel(const __grid_constant__ AttnArgs a, const StreamItem* __restrict__ items, int n_sub, int total_units,
+                         const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    stream_roles<BF16, D, CL>(a, smem, items, n_sub, total_units, nullptr, nullptr, map_k, map_v);
+    __syncthreads();
+    if (ctl_of<D>(smem)->abort_flag) tc5::settle();
+    if constexpr (CL > 1) {
+        tc5::cluster_arrive();                                    // the other CTAs have read what they need of this one's shared memory
+        tc5::cluster_wait();
+    }
+}
+
+template <bool BF16, int D>
+cudaError_t launch_short(const hat_plan* plan, const AttnArgs& args, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t stream) {
+    using G_ = Geo<D>;
+    constexpr int smem = 1024 + G_::SLOTS * G_::SLOT + G_::Q + G_::X + (int)sizeof(Ctl<G_::SLOTS>);
+    const int cl = plan->short_cluster, units = (int)plan->short_items.size() * plan->num_kv_heads * plan->verify_subtiles;
+    auto kern = cl == 1 ? attn_stream_short_kernel<BF16, D, 1> : cl == 2 ? attn_stream_short_kernel<BF16, D, 2>
+                : cl == 4 ? attn_stream_short_kernel<BF16, D, 4> : attn_stream_short_kernel<BF16, D, 8>;
+    cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kern), smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl_clusters(cl, kern, dim3((unsigned)(units * cl)), dim3(kShortThreads), smem, stream, args, plan->dev.short_items,
+                               plan->verify_subtiles, units, mk, mv);
 }
 
 template <bool BF16, int D>
@@ -774,7 +951,7 @@ cudaError_t launch_attn_stream(const hat_plan* plan, const AttnArgs& args, cudaS
     auto go = [&](auto b, auto d) -> cudaError_t {
         constexpr bool B = decltype(b)::value;
         constexpr int D = decltype(d)::value;
-        return launch_one<B, D>(plan, args, *mk, *mv, stream);
+        return plan->short_cluster > 0 ? launch_short<B, D>(plan, args, *mk, *mv, stream) : launch_one<B, D>(plan, args, *mk, *mv, stream);
     };
     using I128 = std::integral_constant<int, 128>;
     using I64 = std::integral_constant<int, 64>;

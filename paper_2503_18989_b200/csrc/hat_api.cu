@@ -273,9 +273,9 @@ static int pick_prefill_split(const hat_plan* p, int num_sms, int* tile_rows, in
 // So requests are cut only when the longest one alone would take longer than HBM needs for the batch, and then into as
 // many pieces as the CTAs can take in one round, or in one more round than the whole requests need (16 requests x 8 K/V heads
 // x 2 slabs: 124 us whole, 95 us in 400 units, 93 us in 576, 89 us in 1000, 99 us in 1900).
-static int pick_verify_split_slabs(const hat_plan* p, int num_sms);
-static int pick_verify_split(const hat_plan* p, int num_sms) {
-    if (p->verify_subtiles > 1) return pick_verify_split_slabs(p, num_sms);
+static int pick_verify_split_slabs(const hat_plan* p, int num_sms, double* price_us);
+static int pick_verify_split(const hat_plan* p, int num_sms, double* slabs_price) {
+    if (p->verify_subtiles > 1) return pick_verify_split_slabs(p, num_sms, slabs_price);
     constexpr int kWhole = 1 << 24, kLeast = 96;       // shorter pieces than 6 pages only add to the merge
     const double tp = 0.25 * p->head_dim / 128;   // us per page of a CTA that has the SM's share of HBM to itself
     const double tb = p->head_dim * 64 / 6.45e6;                               // us per page (K and V) at the measured HBM rate
@@ -318,7 +318,7 @@ static int pick_verify_split(const hat_plan* p, int num_sms) {
 // alike, so as many as divide evenly are placed as one.  Measured, us, rule above / this, bf16: 16 requests of 1300 to 7800 tokens x 8 K/V
 // heads x 16..32 pairs 92.4 / 86.3, 10 x 16 heads 119.7 / 91.2, 12 of up to 2048 tokens 33.1 / 27.4, 16 x 8 heads x 8..64 pairs 129.2 /
 // 103.7, 8 x 8 heads 51.9 / 52.8.
-static int pick_verify_split_slabs(const hat_plan* p, int num_sms) {
+static int pick_verify_split_slabs(const hat_plan* p, int num_sms, double* price_us) {
     const double page = 0.26 * p->head_dim / 128, unit = 0.8, cut = 3.0;       // us: a page, a unit, a piece of a cut request
     const int group = p->num_heads / p->num_kv_heads;
     int alike = 1;
@@ -355,6 +355,47 @@ static int pick_verify_split_slabs(const hat_plan* p, int num_sms) {
         const double t = price(len);
         if (t < 0.98 * least) { least = t; best = len; }
         if (len == 96) break;
+    }
+    *price_us = least;
+    return best;
+}
+
+// Whether every unit of the streaming class gets a CTA of its own (the short form of the streaming kernel), and in how many pieces a request is
+// cut then: 1, 2, 4 or 8, the CTAs of a cluster; 0: the persistent kernel takes the pieces planned above.
+// A page takes a CTA 0.20 us (bf16; fp16 0.17; 64 columns 0.75 of that; 15 % more with two CTAs on an SM), start, hand-over and rows about 5, the exchange within a cluster
+// 1.4 to 2.4.  The persistent kernel needs HBM's time and 7 us or more, 12 at least (fence, count and merge of the pieces), or what the placing of
+// its slabs said and 5.  It keeps what it may do as fast: batches whose longest request is much longer than the others, which it cuts unevenly.
+// Measured, us, persistent / short, bf16: one request x 32 heads 200 tokens 9.2 / 7.0, 700 11.2 / 8.9, 3000 15.8 / 14.2, 8000 30.5 /
+// 27.8; x 8 heads of 4 700 12.8 / 7.8, 3000 20.1 / 11.8; two of 500 to 2000 x 32 15.0 / 14.2; 9 x 32 41.1 / 38.8; 64 columns: 700 x 8 9.3 / 6.0; where
+// it is not taken: 3 of up to 4096 x 32 32.2 / 33.8, one of 3000 x 40 16.3 / 18.2, 7 of up to 8192 x 8 heads of 4 39.6 / 62.8.
+static int pick_short_cluster(const hat_plan* p, int num_sms, double slabs_price) {
+    const bool d128 = p->head_dim == 128;
+    int64_t units = 0, pages = 0;
+    int longest = 0;
+    for (int r = 0; r < p->num_requests; ++r) {
+        if (p->chunk_len[r] < 1 || p->chunk_len[r] > 16) continue;
+        const int n = ceil_div(p->prefix_len[r], kPageSize) + 1;
+        units += (int64_t)p->num_kv_heads * p->verify_subtiles;
+        pages += (int64_t)n * p->num_kv_heads;
+        longest = std::max(longest, n);
+    }
+    if (units == 0) return 0;
+    const double page = (p->dtype == HAT_DTYPE_BF16 ? 0.203 : 0.168) * (d128 ? 1.0 : 0.75), hbm = (double)pages * p->head_dim * 64 / 6.45e6;
+    const double exchange[4] = {0.0, d128 ? 1.4 : 0.8, d128 ? 2.1 : 1.0, d128 ? 2.4 : 1.1};
+    int best = 0;
+    double least = p->verify_subtiles > 1 ? slabs_price + 5.0 : std::max(hbm + 7.0, d128 ? 12.0 : 10.0);
+    // with prompt chunks behind, whose CTAs take the SMs the drafts leave: fewer CTAs that end together are worth a quarter more (6 chunks
+    // and 3 drafts x 40 heads, a step 138 us with the persistent kernel, 133 in clusters of two)
+    if (p->info.num_prefill_requests > 0) least *= 1.25;
+    const bool whole = (int64_t)p->stream_items.size() * p->num_kv_heads * p->verify_subtiles == units && p->verify_subtiles == 1;
+    for (int i = 0; i < 4; ++i) {
+        const int64_t ctas = units << i;
+        // clusters of 4 and 8 do not fill every SM of a GPC: a second round would follow
+        if (ctas > 2 * (int64_t)num_sms || (i > 1 && ctas > (int64_t)num_sms * 256 / 148)) break;
+        const bool two = ctas > num_sms;
+        const double t = std::max(hbm + 6.5, (d128 ? 5.0 : 4.0) + page * (two ? 1.15 : 1.0) * ceil_div(longest, 1 << i) + exchange[i] + (two ? 1.2 : 0.0));
+        // requests that the persistent kernel would not cut are never slower with a CTA each
+        if ((hbm < 60.0 && t < (i < 3 && best == 0 ? 0.97 : 1.0) * least) || (whole && i == 0)) { least = t; best = 1 << i; }
     }
     return best;
 }
@@ -403,8 +444,9 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
     const bool stream_tma = info.stream_kernel == 1;
     p->verify_subtiles = std::max(1, ceil_div(max_verify_rows * group, 16));
     int vsplit = env_int("HAT_VERIFY_SPLIT_LEN", 0);
+    double slabs_price = 1e9;
     if (whole) vsplit = 1 << 24;
-    else if (vsplit <= 0) vsplit = pick_verify_split(p, num_sms);
+    else if (vsplit <= 0) vsplit = pick_verify_split(p, num_sms, &slabs_price);
     vsplit = std::max(kPageSize, round_up(vsplit, kPageSize));
     info.verify_split_len = vsplit;
 
@@ -460,6 +502,12 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
         }
     }
     p->num_verify_merge_rows = (int)p->merge_rows.size();
+    p->short_cluster = stream_tma && env_int("HAT_VERIFY_SPLIT_LEN", 0) <= 0 ? pick_short_cluster(p, num_sms, slabs_price) : 0;
+    if (p->short_cluster > 0)
+        for (int r = 0; r < R; ++r) {
+            const int C = p->chunk_len[r], P = p->prefix_len[r];
+            if (C >= 1 && C <= verify_max_rows) p->short_items.push_back(StreamItem{r, p->cu_chunk[r], C, P, 0, ceil_div(P, kPageSize) + 1, -1, 0, 1, 0, 0, 0});
+        }
     int cluster_merged = 0;                 // rows the one-CTA tile kernel merges itself
     auto each_tile = [&](auto&& f) {
         for (int r = 0; r < R; ++r) {
@@ -535,7 +583,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
 
 int upload_plans(hat_plan* const* plans, size_t count, PlanRes* res) {
     // the arrays of all plans, each at a 256-byte boundary, go over in one copy
-    struct Offsets { size_t cu, pl, cl, bt, rr, vi, si, pi, mr, tu, tm, st, table; };
+    struct Offsets { size_t cu, pl, cl, bt, rr, vi, si, sh, pi, mr, tu, tm, st, table; };
     std::vector<Offsets> at(count);
     std::vector<UploadPart> parts;
     size_t bytes = 0, most_status = 0;
@@ -556,7 +604,7 @@ int upload_plans(hat_plan* const* plans, size_t count, PlanRes* res) {
     for (size_t i = 0; i < count; ++i) {
         const hat_plan* p = plans[i];
         at[i] = Offsets{add(p->cu_chunk), add(p->prefix_len), add(p->chunk_len), add(p->block_table), add(p->row_req), add(p->verify_items),
-                        add(p->stream_items), add(p->prefill_items), add(p->merge_rows), add(p->tile_units), add(p->tree_mask),
+                        add(p->stream_items), add(p->short_items), add(p->prefill_items), add(p->merge_rows), add(p->tile_units), add(p->tree_mask),
                         place(status.data(), p->num_status_words * sizeof(int32_t)), 0};
     }
     // behind the arrays: room for the (cos, sin) table of rotation and projection, filled on the device when first used
@@ -586,6 +634,7 @@ int upload_plans(hat_plan* const* plans, size_t count, PlanRes* res) {
         d.row_req = reinterpret_cast<const int32_t*>(base + o.rr);
         d.verify_items = reinterpret_cast<const WorkItem*>(base + o.vi);
         d.stream_items = reinterpret_cast<const StreamItem*>(base + o.si);
+        d.short_items = reinterpret_cast<const StreamItem*>(base + o.sh);
         d.prefill_items = reinterpret_cast<const WorkItem*>(base + o.pi);
         d.merge_rows = reinterpret_cast<const MergeRow*>(base + o.mr);
         d.tile_units = reinterpret_cast<const uint32_t*>(base + o.tu);
@@ -691,6 +740,7 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     p->timing = nullptr;
     p->append_first = append_first;
     p->num_piece_counters = 0;
+    p->short_cluster = 0;
     p->num_verify_merge_rows = 0;
     p->tile_clusters = false;
     p->append_apart = false;

@@ -54,6 +54,7 @@ struct DevicePlan {
     const int32_t*  row_req;        // [T] request of each packed row
     const WorkItem* verify_items;   // mma.sync streaming kernel
     const StreamItem* stream_items; // TMA streaming kernel, longest first
+    const StreamItem* short_items;  // the same requests, whole, where every unit has a CTA of its own (see short_cluster)
     int32_t*        piece_counters; // see StreamItem::counter; zero between calls
     const WorkItem* prefill_items;
     const uint32_t* tile_units;     // tcgen05 tile kernels: unit -> prefill item (low 16 bits) | query head (high 16 bits), in draw order
@@ -229,7 +230,8 @@ struct hat_plan {
     int num_sms;
     std::vector<int32_t> cu_chunk, prefix_len, chunk_len, block_table, row_req;
     std::vector<hat::WorkItem> verify_items, prefill_items;
-    std::vector<hat::StreamItem> stream_items;
+    std::vector<hat::StreamItem> stream_items, short_items;
+    int short_cluster;          // > 0: the streaming kernel has a CTA per unit, in clusters of this many that share a request
     int num_piece_counters;
     std::vector<uint32_t> tile_units;   // (item, head) of every unit of the tcgen05 tile kernels, in the order they are drawn
     bool pair_takes_all;                // HAT_PREFILL_KERNEL=pair: every unit goes to the CTA-pair kernel, narrow ones too (tests)
