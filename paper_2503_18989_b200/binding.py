@@ -85,11 +85,13 @@ class HatError(RuntimeError):
 
 
 _lib: Optional[C.CDLL] = None
+# the calls of every layer without ctypes' cost per argument (csrc/calls.c), once the library is loaded; None: a call for ctypes
+_call_attention = _call_attention_out16 = lambda *args: None
 
 
 def lib() -> C.CDLL:
     """Load libhat.so (built by paper_2503_18989_b200.build); fails loudly if it is absent."""
-    global _lib
+    global _lib, _call_attention, _call_attention_out16
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2503_18989_b200.build` "
@@ -160,6 +162,9 @@ def lib() -> C.CDLL:
                                                   vp, vp, vp, C.c_float, vp]
         L.hat_static_key_range.restype = i32
         L.hat_static_key_range.argtypes = [i32, i32, i32, i32, i32] + [C.POINTER(i32)] * 4
+        from . import _calls
+        _calls.init(C.cast(L.hat_chunk_attention, vp).value, C.cast(L.hat_chunk_attention_out16, vp).value, Plan)
+        _call_attention, _call_attention_out16 = _calls.chunk_attention, _calls.chunk_attention_out16
         _lib = L
     return _lib
 
@@ -297,16 +302,18 @@ def hat_qkv_rope_append(cache: hat_cache_desc, plan, x, hidden: int, w_qkv, q_ou
 
 def hat_chunk_attention(cache: hat_cache_desc, plan, q, k_new, v_new, out, lse, sm_scale: float = 0.0,
                         workspace=None, workspace_bytes: int = 0, stream: int = 0) -> None:
+    from_c = _call_attention(cache, plan, q, k_new, v_new, out, lse, sm_scale, workspace, workspace_bytes, stream)
     _check(lib().hat_chunk_attention(C.byref(cache), _h(plan), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out),
                                      _ptr(lse), float(sm_scale), _ptr(workspace), int(workspace_bytes),
-                                     stream or None), "hat_chunk_attention")
+                                     stream or None) if from_c is None else from_c, "hat_chunk_attention")
 
 
 def hat_chunk_attention_out16(cache: hat_cache_desc, plan, q, k_new, v_new, out16, lse, sm_scale: float = 0.0,
                               workspace=None, workspace_bytes: int = 0, stream: int = 0) -> None:
+    from_c = _call_attention_out16(cache, plan, q, k_new, v_new, out16, lse, sm_scale, workspace, workspace_bytes, stream)
     _check(lib().hat_chunk_attention_out16(C.byref(cache), _h(plan), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out16),
                                            _ptr(lse), C.c_float(sm_scale), _ptr(workspace), workspace_bytes,
-                                           stream or None), "hat_chunk_attention_out16")
+                                           stream or None) if from_c is None else from_c, "hat_chunk_attention_out16")
 
 
 def hat_chunk_attention_host(cache: hat_cache_desc, plan, q_host, k_new_host, v_new_host, out_host, lse_host,

@@ -6,10 +6,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhat.so")
+CALLS_SRC = os.path.join(CSRC, "calls.c")
+CALLS = os.path.join(HERE, "_calls.so")          # the binding's calls as a CPython extension
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -31,10 +34,10 @@ def sources():
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
+    deps = sources() + [CALLS_SRC] + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(HERE, "..", "include", "hat.h")]
     return any(os.path.getmtime(p) > t for p in deps)
 
@@ -80,6 +83,9 @@ def _build(lib: str, obj_name: str, extra, verbose: bool) -> str:
     tmp = lib + f".tmp{os.getpid()}"
     subprocess.check_call([_nvcc(), "-shared", "-o", tmp, *objs, "-lcudart_static", "-ldl", "-lpthread", "-lrt"])
     os.replace(tmp, lib)
+    tmp = CALLS + f".tmp{os.getpid()}"
+    subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], CALLS_SRC, "-o", tmp])
+    os.replace(tmp, CALLS)
     return lib
 
 
