@@ -203,7 +203,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         // ------------------------------------------------------------------ unit fetch + TMA producer
         // Lane pg + 8 g moves page pg of a tile: one box (g = 0), or its two 8-row groups where the pool's strides fold neither
         // way and for rows of k_new / v_new.  What this warp does per tile is close to what a tile costs the tensor core, so
-        // the loop over plain tiles holds no more than it must (ring positions are stepped, page ids fetched a tile ahead).
+        // the tiles that hold nothing of the chunk have a loop of their own with no more than it must hold (ring positions are stepped, page
+        // ids fetched a tile ahead): a prompt of 2048 in eight calls 119.4 / 117.4 us, 30 ragged chunks 467 / 459.
         const long long since = clock64();
         // the previous kernel's end, once what the plan's own arrays hold has been read
         auto front_ended = [&]() {
@@ -288,36 +289,61 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             const tile_append::Chunk ck{u.P, u.C, u.row_base, u.hk};
             // of the units that read a chunk page, the last row block of the group's first query head appends it
             const bool appends = APPEND && u.h == u.hk * a.plan.group && u.row0 + a.plan.tile_rows >= u.C;
-            for (int j = 0; j < u.n_all; ++j) {
+            int j = 0;
+#pragma unroll 1
+            for (; j < n_plain; ++j) {
                 const int npages = min(8, total_pages - 8 * j);
                 const int page_next = page_of(j + 1), c4 = page << s4;
-                const bool plain = !APPEND || j < n_plain;
+                const bool pool = lane < boxes && pg < npages;
+                HAT_CHECK(sk < kStagesK && sv < kStagesV, status);
+                if (APPEND && stored) { tile_append::stores_read(); stored = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars));
+                if (!ok) break;
+                if (lane == 0) mbar_expect_tx(&bars->k_full[sk], npages * kPageBytes);
+                if (pool) tma_load_5d(smem_u32(k_ring) + sk * kTileBytes + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars));
+                if (!ok) break;
+                if (!withhold) {
+                    if (lane == 0) mbar_expect_tx(&bars->v_full[sv], npages * kPageBytes);
+                    if (pool) tma_load_5d(smem_u32(v_ring) + sv * kTileBytes + lane_off, &map_v, 0, c1, 0, c3, c4, &bars->v_full[sv]);
+                }
+                if (APPEND && owes) {                             // the previous unit's last tile
+                    pay();
+                    if (!ok) break;
+                }
+                withhold = false;
+                page = page_next;
+                step();
+            }
+            if (!ok) break;
+            if (!APPEND) continue;
+            // tiles with chunk positions
+#pragma unroll 1
+            for (; j < u.n_all; ++j) {
+                const int npages = min(8, total_pages - 8 * j);
+                const int page_next = page_of(j + 1), c4 = page << s4;
                 const uint32_t k_dst = smem_u32(k_ring) + sk * kTileBytes, v_dst = smem_u32(v_ring) + sv * kTileBytes;
                 // in a tile with chunk positions: pages of the chunk alone come from k_new / v_new; a page with both prefix and
                 // chunk rows is gathered and completes the barriers last
                 const int kb = u.kv_begin + j * kKeys, key0 = kb + pg * kPageSize, pe = (u.P - kb) / kPageSize;
-                bool edge = false, fresh = false, pool = lane < boxes && pg < npages;
-                uint32_t bytes = npages * kPageBytes;
-                if (APPEND && !plain) {
-                    edge = u.P > kb && u.P % kPageSize != 0 && pe < npages;
-                    fresh = lane < 16 && pg < npages && ck.fresh(key0);
-                    pool = pool && !ck.fresh(key0) && !(edge && pg == pe);
-                    if (edge) bytes -= kPageBytes;
-                }
+                const bool edge = u.P > kb && u.P % kPageSize != 0 && pe < npages;
+                const bool fresh = lane < 16 && pg < npages && ck.fresh(key0);
+                const bool pool = lane < boxes && pg < npages && !ck.fresh(key0) && !(edge && pg == pe);
+                const uint32_t bytes = (npages - (edge ? 1 : 0)) * kPageBytes;
                 const int row = u.row_base + key0 - u.P + 8 * grp;
                 HAT_CHECK(sk < kStagesK && sv < kStagesV, status);
                 if (APPEND && stored) { tile_append::stores_read(); stored = false; }
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->k_empty[sk], pk, bars));
                 if (!ok) break;
-                if (lane == 0) { if (APPEND && edge) mbar_expect_only(&bars->k_full[sk], bytes); else mbar_expect_tx(&bars->k_full[sk], bytes); }
+                if (lane == 0) { if (edge) mbar_expect_only(&bars->k_full[sk], bytes); else mbar_expect_tx(&bars->k_full[sk], bytes); }
                 if (pool) tma_load_5d(k_dst + lane_off, &map_k, 0, c1, 0, c3, c4, &bars->k_full[sk]);
-                if (APPEND && fresh) tma_load_4d(k_dst + lane_off, &map_k_new, 0, row, 0, u.hk, &bars->k_full[sk]);
+                if (fresh) tma_load_4d(k_dst + lane_off, &map_k_new, 0, row, 0, u.hk, &bars->k_full[sk]);
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->v_empty[sv], pv, bars));
                 if (!ok) break;
                 if (!withhold) {
-                    if (lane == 0) { if (APPEND && edge) mbar_expect_only(&bars->v_full[sv], bytes); else mbar_expect_tx(&bars->v_full[sv], bytes); }
+                    if (lane == 0) { if (edge) mbar_expect_only(&bars->v_full[sv], bytes); else mbar_expect_tx(&bars->v_full[sv], bytes); }
                     if (pool) tma_load_5d(v_dst + lane_off, &map_v, 0, c1, 0, c3, c4, &bars->v_full[sv]);
-                    if (APPEND && fresh) tma_load_4d(v_dst + lane_off, &map_v_new, 0, row, 0, u.hk, &bars->v_full[sv]);
+                    if (fresh) tma_load_4d(v_dst + lane_off, &map_v_new, 0, row, 0, u.hk, &bars->v_full[sv]);
                 }
                 if constexpr (APPEND) {
                     if (edge) {
@@ -331,7 +357,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     }
                     pay();                                       // the tile before, or the previous unit's last
                     if (!ok) break;
-                    if (appends && !plain && !withhold) {
+                    if (appends && !withhold) {
                         owes = true;
                         o_sk = sk; o_sv = sv; o_pk = pk ^ 1; o_pv = pv ^ 1; o_page = page; o_hk = u.hk;
                         o_whole = lane < boxes && pg < npages && ck.whole(key0);
