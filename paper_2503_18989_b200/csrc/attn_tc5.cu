@@ -510,8 +510,6 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
         const uint32_t tm_s = tmem + qt * 128 + lane_sel, tm_o = tmem + 256 + qt * 128 + lane_sel;
         const int wg_tid = (int)threadIdx.x - 64 - qt * 128;
         const float sc = a.scale_log2;
-        // rows are 512 bytes apart at least, so a 32-byte aligned base keeps every 32-byte store aligned
-        const bool wide_stores = !ONE && ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.part_out)) & 31) == 0;
         int kt_base = 0;                                    // K/V tiles of the units before this one
         int s_cnt = 0, o_cnt = 0, x_cnt = 0;                // completions of s_full[qt] / o_done[qt] / x_ready consumed so far
         bool ok = true;
@@ -618,24 +616,20 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                     const int64_t orow = u.part < 0 ? u.row_base + i_row : u.part + (i_row - u.row0);
                     HAT_CHECK(i_row >= u.C || (orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows)), status);
                     const uint32_t tm_a = u.split ? tmem + 256 + lane_sel : tm_o;
-                    auto load64 = [&](float (&o)[64], int c0) {
+                    auto load32 = [&](float* o, int c0) {
                         if (have0) {
                             tmem_ld32(tm_a + c0, reinterpret_cast<uint32_t*>(o));
-                            tmem_ld32(tm_a + c0 + 32, reinterpret_cast<uint32_t*>(o) + 32);
                             tmem_ld_wait();
                         } else {
 #pragma unroll
-                            for (int k = 0; k < 64; ++k) o[k] = 0.f;
+                            for (int k = 0; k < 32; ++k) o[k] = 0.f;
                         }
                         if (have1) {
+                            uint32_t o1[32];
+                            tmem_ld32(tm_a + 128 + c0, o1);      // the second chain's accumulator: next 128 columns
+                            tmem_ld_wait();
 #pragma unroll
-                            for (int c = 0; c < 64; c += 32) {
-                                uint32_t o1[32];
-                                tmem_ld32(tm_a + 128 + c0 + c, o1);      // the second chain's accumulator: next 128 columns
-                                tmem_ld_wait();
-#pragma unroll
-                                for (int k = 0; k < 32; ++k) o[c + k] = o[c + k] * w0 + __uint_as_float(o1[k]) * w1;
-                            }
+                            for (int k = 0; k < 32; ++k) o[k] = o[k] * w0 + __uint_as_float(o1[k]) * w1;
                         }
                     };
                     if constexpr (FORM == kHalves) {
@@ -643,7 +637,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         // product that read it has ended), the maximum and sum behind chain 0's
                         const uint32_t rank = cluster_ctarank();
                         float o[64], mine[32];
-                        load64(o, 64 * qt);
+                        load32(o, 64 * qt);
+                        load32(o + 32, 64 * qt + 32);
                         float4* give = reinterpret_cast<float4*>(q_tiles) + qt * (8 * kRows) + t;
                         float2* ml = reinterpret_cast<float2*>(q_tiles + kTileBytes) + (1 + qt) * kRows + t;
 #pragma unroll
@@ -677,12 +672,12 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         if (i_row < u.C && qt == 0 && rank == 0) a.lse[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
                     } else {
                         const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-                        for (int c0 = 0; c0 < kD; c0 += 64) {
-                            if (u.split && c0 != 64 * qt) continue;
-                            float o[64];
-                            load64(o, c0);
-                            out_rows::store<64, kD, true>(a, o, inv, u.part < 0, orow, u.C - i_row, u.h, c0, lane);
+#pragma unroll 1
+                        for (int c0 = 0; c0 < kD; c0 += 32) {
+                            if (u.split && c0 >> 6 != qt) continue;
+                            float o[32];
+                            load32(o, c0);
+                            out_rows::store<32, kD, true>(a, o, inv, u.part < 0, orow, u.C - i_row, u.h, c0, lane);
                         }
                         if (i_row < u.C && !(u.split && qt == 1))
                             (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
@@ -697,83 +692,55 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         if (lane == 0) mbar_arrive(&bars->x_ready);
                     }
                 } else {
-                    // pull O into registers, hand the accumulator back, then store
-                    float o[kD];
-                    if (n_mine > 0) {
-#pragma unroll
-                        for (int c = 0; c < kD / 32; ++c) tmem_ld32(tm_o + c * 32, reinterpret_cast<uint32_t*>(o) + c * 32);
-                        tmem_ld_wait();
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < kD; ++k) o[k] = 0.f;
-                    }
-                    if (u.split && u.n_t1 > 0) {
-                        // merge the second chain (disjoint keys): weights 2^(m_t - m), sums and accumulators add up
+                    // 32 columns at a time, one copy of the code for all (see softmax_tile.cuh: 30 chunks of 32 to 128 rows x 32 heads, fp16, 82 / 74 us,
+                    // bf16 97 / 83; 30 ragged chunks 459 / 451); with the last ones in registers the accumulator is handed back
+                    const bool have1 = u.split && u.n_t1 > 0;
+                    float w0 = 1.f, w1 = 0.f;
+                    if (have1) {
+                        // the second chain (disjoint keys): weights 2^(m_t - m), sums and accumulators add up
                         ok = __all_sync(0xffffffffu, mbar_wait(&bars->x_ready, x_cnt & 1, bars));
                         ++x_cnt;
                         if (!ok) break;
                         tc_fence_after();
                         const float2 other = bars->xchg[t];
                         const float m_new = fmaxf(m_used, other.x);
-                        const float w0 = (m_used == -INFINITY) ? 0.f : fast_exp2(m_used - m_new);
-                        const float w1 = (other.x == -INFINITY) ? 0.f : fast_exp2(other.x - m_new);
+                        w0 = (m_used == -INFINITY) ? 0.f : fast_exp2(m_used - m_new);
+                        w1 = (other.x == -INFINITY) ? 0.f : fast_exp2(other.x - m_new);
                         l = l * w0 + other.y * w1;
                         m_used = m_new;
-#pragma unroll
-                        for (int c = 0; c < kD / 16; ++c) {
-                            uint32_t o1[16];
-                            tmem_ld16(tm_o + 128 + c * 16, o1);      // the second chain's accumulator: next 128 columns
+                    }
+                    const float inv = l > 0.f ? 1.f / l : 0.f;
+                    const int64_t orow = u.part < 0 ? u.row_base + i_row : u.part + (i_row - u.row0);
+                    HAT_CHECK(i_row >= u.C || (orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows)), status);
+#pragma unroll 1
+                    for (int c = 0; c < kD; c += 32) {
+                        float o[32];
+                        if (n_mine > 0) {
+                            tmem_ld32(tm_o + c, reinterpret_cast<uint32_t*>(o));
                             tmem_ld_wait();
-#pragma unroll
-                            for (int k = 0; k < 16; ++k) o[c * 16 + k] = o[c * 16 + k] * w0 + __uint_as_float(o1[k]) * w1;
-                        }
-                    }
-                    if (n_mine > 0 || (u.split && u.n_t1 > 0)) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) {
-                            if (n_mine > 0) mbar_arrive(&bars->o_free[qt]);
-                            if (u.split && u.n_t1 > 0) mbar_arrive(&bars->o_free[1]);
-                        }
-                    }
-                    if (i_row < u.C) {
-                        const float inv = l > 0.f ? 1.f / l : 0.f;
-                        float* obase; float* lbase; int64_t orow;
-                        if (u.part < 0) { obase = a.out; lbase = a.lse; orow = u.row_base + i_row; }
-                        else { obase = a.part_out; lbase = a.part_lse; orow = u.part + (i_row - u.row0); }
-                        HAT_CHECK(orow >= 0 && orow < (u.part < 0 ? (int64_t)a.plan.total_rows : a.part_rows), status);
-                        float* dst = obase + (orow * H + u.h) * kD;
-                        if (u.part < 0 && a.out16 != nullptr) {
-                            // final rows in the 16-bit output type: 256 bytes per row, eight 32-byte stores
-                            uint16_t* dst16 = static_cast<uint16_t*>(a.out16) + (orow * H + u.h) * kD;
-                            const bool wide16 = (reinterpret_cast<uintptr_t>(a.out16) & 31) == 0;
-#pragma unroll
-                            for (int k = 0; k < kD; k += 16) {
-                                uint32_t w[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) w[e] = pack_out16(o[k + 2 * e] * inv, o[k + 2 * e + 1] * inv, a.out16_bf16);
-                                if (wide16) {
-                                    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
-                                                 ::"l"(dst16 + k), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-                                } else {
-                                    *reinterpret_cast<uint4*>(dst16 + k) = make_uint4(w[0], w[1], w[2], w[3]);
-                                    *reinterpret_cast<uint4*>(dst16 + k + 8) = make_uint4(w[4], w[5], w[6], w[7]);
-                                }
-                            }
-                        } else if (wide_stores) {
-                            // a thread stores its whole row; 32-byte stores fill a sector each (half as many sector writes
-                            // as 16-byte ones, and the sector rate is what bounds this part)
-#pragma unroll
-                            for (int k = 0; k < kD; k += 8)
-                                st_global_v8(dst + k, o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv, o[k + 4] * inv,
-                                             o[k + 5] * inv, o[k + 6] * inv, o[k + 7] * inv);
                         } else {
 #pragma unroll
-                            for (int k = 0; k < kD; k += 4)
-                                *reinterpret_cast<float4*>(dst + k) = make_float4(o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv);
+                            for (int k = 0; k < 32; ++k) o[k] = 0.f;
                         }
-                        lbase[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
+                        if (have1) {
+                            uint32_t o1[32];
+                            tmem_ld32(tm_o + 128 + c, o1);           // the second chain's accumulator: next 128 columns
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) o[k] = o[k] * w0 + __uint_as_float(o1[k]) * w1;
+                        }
+                        if (c == kD - 32 && (n_mine > 0 || have1)) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) {
+                                if (n_mine > 0) mbar_arrive(&bars->o_free[qt]);
+                                if (have1) mbar_arrive(&bars->o_free[1]);
+                            }
+                        }
+                        out_rows::store<32, kD, false>(a, o, inv, u.part < 0, orow, u.C - i_row, u.h, c, lane);
+                        __syncwarp();                            // rows past the chunk store nothing
                     }
+                    if (i_row < u.C) (u.part < 0 ? a.lse : a.part_lse)[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
                 }
             }
             kt_base += u.n_all;
