@@ -398,9 +398,9 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
             const uint64_t v_desc0 = smem_desc(smem_u32(v_ring), 1024, kGroupBytes);
             bool ok = true;
             int kt_base = 0;                          // K/V tiles of the units before this one
-            int p_cnt[2] = {0, 0};                    // completions of p_ready[t] consumed so far
-            int f_cnt[2] = {0, 0};                    // completions of o_free[t] consumed so far
-            bool o_busy[2] = {false, false};          // O_t holds a finished unit that its warpgroup may still be reading
+            // bit t, for tile or chain t: parity of the next completion of p_ready[t] and of o_free[t]; O_t holds a finished unit that its
+            // warpgroup may still be reading
+            uint32_t p_par = 0, f_par = 0, o_busy = 0;
             for (int un = 0; ok; ++un) {
                 const int slot = un & 1;
                 ok = mbar_wait(&bars->unit_full[slot], (un >> 1) & 1, bars);
@@ -449,15 +449,15 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                             v_ready = j;
                             if (!ok) return;
                         }
-                        if (sidx == 0 && o_busy[qt]) {
+                        if (sidx == 0 && (o_busy >> qt) & 1) {
                             // the accumulator still holds the previous unit: wait until its rows are in registers
-                            ok = mbar_wait(&bars->o_free[qt], f_cnt[qt] & 1, bars);
-                            ++f_cnt[qt];
-                            o_busy[qt] = false;
+                            ok = mbar_wait(&bars->o_free[qt], (f_par >> qt) & 1, bars);
+                            f_par ^= 1u << qt;
+                            o_busy &= ~(1u << qt);
                             if (!ok) return;
                         }
-                        ok = mbar_wait(&bars->p_ready[qt], p_cnt[qt] & 1, bars);
-                        ++p_cnt[qt];
+                        ok = mbar_wait(&bars->p_ready[qt], (p_par >> qt) & 1, bars);
+                        p_par ^= 1u << qt;
                         if (!ok) return;
                         tc_fence_after();
                         const uint64_t vd = v_desc0 + (uint64_t)(st * (kTileBytes >> 4));
@@ -473,6 +473,21 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         if (sidx == u.n_t(qt) - 1) tc_commit(&bars->o_done[qt]);      // before that S(next) tells
                         if (SPLIT || qt == u.nq - 1) tc_commit(&bars->v_empty[st]);
                     };
+                    if constexpr (ONE) {
+                        // one copy of the products for both tiles or chains: code that a CTA of one unit meets cold (eight calls of one request
+                        // 117 / 114 us; where CTAs draw units the addresses that depend on the tile cost more, 64 columns bf16 361 / 390)
+#pragma unroll 1
+                        for (int sidx = -1; sidx < max(u.n_t0, u.n_t1) && ok; ++sidx) {
+#pragma unroll 1
+                            for (int qt = 0; qt < 2 && ok; ++qt) {
+                                const int n = u.n_t(qt);
+                                if (sidx >= n) continue;
+                                if (sidx >= 0) issue_pv(qt, sidx);
+                                if (ok && sidx + 1 < n) issue_s(qt, sidx + 1);
+                            }
+                        }
+                        return;
+                    }
                     if (u.n_t0 > 0) issue_s(0, 0);
                     if (ok && u.n_t1 > 0) issue_s(1, 0);
                     for (int sidx = 0; sidx < max(u.n_t0, u.n_t1) && ok; ++sidx) {
@@ -489,8 +504,8 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 };
                 if (u.split) run_unit(std::true_type{}); else run_unit(std::false_type{});
                 // a unit in which a tile had no keys leaves that tile's earlier hand-over pending
-                if (u.n_t0 > 0) o_busy[0] = true;
-                if (u.n_t1 > 0) o_busy[1] = true;
+                if (u.n_t0 > 0) o_busy |= 1u;
+                if (u.n_t1 > 0) o_busy |= 2u;
                 kt_base += u.n_all;
             }
             if (!ok) {
