@@ -69,7 +69,7 @@ class hat_plan_info(C.Structure):
                 ("verify_split_len", C.c_int32), ("prefill_split_len", C.c_int32),
                 ("prefill_tile_rows", C.c_int32), ("prefill_kernel", C.c_int32),
                 ("workspace_bytes", C.c_int64), ("attn_flops", C.c_int64), ("kv_read_bytes", C.c_int64),
-                ("stream_kernel", C.c_int32), ("reserved", C.c_int32)]
+                ("stream_kernel", C.c_int32), ("num_pair_units", C.c_int32)]
 
     def as_dict(self):
         return {n: int(getattr(self, n)) for n, _ in self._fields_}

@@ -797,10 +797,11 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
                                        cache->stride_token, cache->stride_head);
     p->num_sms = num_sms;
     // Which tcgen05 tile kernel: the CTA-pair kernel (cta_group::2) shares every K/V tile between the two 128-row halves
-    // of a 256-row unit and is the faster one when every unit fills both halves (and, for fp16, the batch is not small);
-    // batches with 64- or 128-row chunks (half of a pair would idle) keep the one-CTA kernel.
-    // HAT_PREFILL_KERNEL = tc5 | pair | mma overrides.
+    // of a 256-row unit and is the faster one for long units; short ones, whose start and rows count for more, and batches that do
+    // not fill the pairs are faster on the one-CTA kernel, with units of 128 rows and halves merged by clusters where they are few.
+    // HAT_PREFILL_KERNEL = tc5 | pair | mixed (wide units to pairs, whatever their length) | mma overrides.
     int tile_kernel = use_tc5 ? 1 : 0;
+    bool pairs_possible = false;
     if (use_tc5 && p->head_dim == 128) {
         bool all_wide = true;
         int64_t wide_tiles = 0, wide_keys = 0;
@@ -811,21 +812,22 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
             for (int row0 = 0; row0 < C; row0 += 256)
                 if (C - row0 > 128) { ++wide_tiles; wide_keys += p->prefix_len[r] + std::min(C, row0 + 256); }
         }
-        // measured (chunks of 512 and 256 rows, 40 heads; the one-CTA kernel has since got units of 128 rows, halves merged by
-        // clusters and shorter code, so that small bf16 batches may by now be faster on it: not measured again): for bf16 the pair
-        // kernel is the faster one at every batch size (1 to 8 chunks: 9 to 26 %), for fp16 from about 1.5 units per SM on (equal at 160 units, 2.5 % at 240, 16 % at 320)
-        // bf16: the units of more than 128 rows go to the pairs even when the batch also has narrower ones (those run on
-        // single CTAs behind them: a ragged bf16 batch measured 0.298 + 0.118 ms that way against 0.49 on either kernel alone)
-        // fp16: pairs pay off only for long units (prefix 4000: +16 %; 8 chunks of 512 at prefix 2000: +4.5 %, at 1000: -2 %; a ragged batch's wide units, ~2300 keys on average with many short ones: -3 %)
+        // bf16 (its units of more than 128 rows; narrower ones of the same batch run on single CTAs behind them): a step of 128 keys and a
+        // unit take a pair 1.45 and 7 us, a CTA 3.3 and 7.5, so pairs pay from some 2200 keys on where they are evenly loaded and surely from 3000, measured (one CTA / pairs, us, 32 heads): 4 chunks of
+        // 512 at 4000 228 / 207, 8 at up to 8000 350 / 298, 8 at up to 1000 93 / 108, 8 of 200 to 600 at up to 4000 287 / 319, 30 of 256 to 512 at up to 4000 784 /
+        // 821; few units: one chunk of 256 at 1000 19.5 / 29.0, 3 of 129 to 300 53 / 66, 4 of 512 at 4000 x 8 heads 66 / 75.
+        // fp16 (only where every unit is that wide): 4 of 512 at 4000 x 40 heads 234 / 220, 8 at up to 8000 329 / 325, x 32 heads 242 / 262.
         const bool bf16 = p->dtype == HAT_DTYPE_BF16;
-        const int64_t least = bf16 ? 1 : 3 * (int64_t)num_sms / 2;
-        const bool long_units = bf16 || (wide_tiles > 0 && wide_keys / wide_tiles >= 2500);
-        if ((all_wide || bf16) && long_units && wide_tiles > 0 && wide_tiles * p->num_heads >= least) tile_kernel = 3;
+        const bool many = wide_tiles * p->num_heads >= 3 * (int64_t)num_sms / 2;
+        const bool long_units = wide_tiles > 0 && wide_keys / wide_tiles >= (bf16 ? 3000 : 4200);
+        if ((all_wide || bf16) && long_units && many) tile_kernel = 3;
+        pairs_possible = tile_kernel == 3 || (bf16 && wide_tiles > 0);
     }
     p->pair_takes_all = false;
     if (const char* k = std::getenv("HAT_PREFILL_KERNEL")) {
         if (use_tc5 && p->head_dim == 128 && std::strcmp(k, "pair") == 0) { tile_kernel = 3; p->pair_takes_all = true; }
-        else if (use_tc5 && std::strcmp(k, "tc5") == 0) tile_kernel = 1;
+        else if (use_tc5 && std::strcmp(k, "mixed") == 0 && pairs_possible) tile_kernel = 3;
+        else if (use_tc5 && std::strcmp(k, "tc5") == 0) { tile_kernel = 1; pairs_possible = false; }
     }
     // the streaming kernel takes its pages by TMA when a descriptor can be built for the pool layout
     bool stream_tma = true;
@@ -836,6 +838,8 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
                                              cache->stride_token, cache->stride_head);
     p->info.stream_kernel = stream_tma ? 1 : 0;
     schedule(p, num_sms, tile_kernel, whole);
+    if (pairs_possible) p->info.prefill_kernel = 3;          // such a batch may go to either kernel: see num_pair_units
+    p->info.num_pair_units = p->num_pair_units;
     // launch-geometry limits: work items index gridDim.y (65535), partial rows and units are 32-bit
     const int64_t verify_count = (int64_t)(p->verify_items.size() + p->stream_items.size());
     if (verify_count > 65535 || verify_count * p->num_kv_heads * p->verify_subtiles > INT32_MAX / 2 || p->prefill_items.size() > 65535 || p->num_heads > 65535 ||
@@ -994,10 +998,10 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
     } else if (!plan->prefill_items.empty()) {
         mark(1, 0);
         if (plan->info.prefill_kernel == 3) {
-            // units of more than 128 rows on CTA pairs, the others (if any) on single CTAs that take the SMs as the pairs leave them
-            e = launch_attn_pair(plan, a, s, plan->num_pair_units);
-            if (e == cudaSuccess)
-                e = launch_attn_tc5(plan, a, s, 0, true, plan->num_pair_units, -1, /*counter_word=*/3, /*overlap=*/plan->num_pair_units > 0);
+            // long units of more than 128 rows on CTA pairs, the others (if any) on single CTAs that take the SMs as the pairs leave them
+            const bool pairs = plan->num_pair_units > 0;
+            if (pairs) e = launch_attn_pair(plan, a, s, plan->num_pair_units);
+            if (e == cudaSuccess) e = launch_attn_tc5(plan, a, s, 0, true, plan->num_pair_units, -1, /*counter_word=*/3, /*overlap=*/pairs);
         } else {
             e = plan->info.prefill_kernel == 1 ? launch_attn_tc5(plan, a, s)
                                                : launch_attn_mma(plan, a, /*verify_class=*/false, s);

@@ -1,0 +1,41 @@
+"""Which units of a bf16 batch the CTA pairs take, and both tile kernels behind one another."""
+import numpy as np
+import pytest
+
+from paper_2503_18989_b200 import binding as B, workloads as W
+
+from test_stream_kernel import _batch, _check
+
+
+def _pair_units(prefix, chunk, H, dtype="bf16"):
+    rng = np.random.Generator(np.random.PCG64(3))
+    table, pages = W._place_pages(rng, np.asarray(prefix) + np.asarray(chunk), slack_pages=2)
+    c = B.make_cache_desc(dtype, pages, H, 128, H * 16 * 128, 128, 16 * 128)
+    cu = np.concatenate([[0], np.cumsum(chunk)]).astype(np.int32)
+    p = B.hat_plan_create(c, H, cu, np.asarray(prefix, np.int32), np.asarray(chunk, np.int32), table, B.HAT_PLAN_HOST_ONLY)
+    return B.hat_plan_get_info(p).as_dict()["num_pair_units"]
+
+
+def test_pairs_take_long_wide_units_of_batches_that_fill_them(hat_lib):
+    assert _pair_units([4000] * 4, [512] * 4, 32) == 8 * 32
+    assert _pair_units([4000] * 4 + [50, 700], [512] * 4 + [100, 4], 32) == 8 * 32       # narrow units and drafts stay out
+    assert _pair_units([4000] * 4, [512] * 4, 8) == 0                                    # few units
+    assert _pair_units([500] * 8, [512] * 8, 40) == 0                                    # short ones
+    assert _pair_units([4000] * 8, [512] * 8, 40, "fp16") == 16 * 40
+    assert _pair_units([3000] * 8, [512] * 8, 40, "fp16") == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kernel", ["mixed", ""])           # wide units on pairs whatever their length; as the plan picks them (none, 8 heads)
+def test_wide_and_narrow_units_of_one_batch(cuda_device, kernel, monkeypatch):
+    if kernel:
+        monkeypatch.setenv("HAT_PREFILL_KERNEL", kernel)
+    prefix = [0, 300, 1000, 37, 2000, 640, 90, 1500]
+    chunk = [512, 384, 128, 64, 300, 17, 4, 256]
+    _check(_batch("bf16", 8, 128, prefix, chunk, 83), cuda_device, repeat=10)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("chunk,prefix", [([256], [1000]), ([129], [0]), ([200, 512], [700, 33])])     # halves merged by clusters; one unit a CTA
+def test_small_bf16_batches_on_single_ctas(cuda_device, chunk, prefix):
+    _check(_batch("bf16", 8, 128, prefix, chunk, 84), cuda_device, repeat=3)
