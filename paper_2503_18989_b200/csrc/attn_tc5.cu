@@ -132,9 +132,9 @@ __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, const WorkItem* _
 // How the units lie on the CTAs.  A template parameter because the softmax loop's registers are tight: as a branch, the other
 // output form cost it 2 %.
 //   kMany    CTAs draw units
-//   kOne     no CTA has more than one unit (head_dim 128; rows of 64 columns store as fast as they are)
+//   kOne     no CTA has more than one unit (128 columns; rows of 64 store as fast as they are)
 //   kHalves  the same, and the CTAs of a cluster of two have the two key ranges of one tile of at most 128 rows: they merge them
-//            through each other's shared memory, 32 columns to a warpgroup, instead of through global memory and a launch
+//            through each other's shared memory, a quarter of the columns to a warpgroup, instead of through global memory and a launch
 //            (one request of 256 rows x 32 heads, us a call: prefix 768
 //            19.4 -> 13.4, 1792 23.9 -> 17.9, 4000 38.9 -> 32.3)
 enum Form { kMany, kOne, kHalves };
@@ -149,7 +149,7 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_k_new,
                 const __grid_constant__ CUtensorMap map_v_new, int fold) {
     constexpr bool ONE = FORM != kMany;
-    static_assert(!ONE || kD == 128, "the forms with one unit a CTA store rows of 128 columns");
+    static_assert(FORM != kOne || kD == 128, "rows of 64 columns store as fast as they are");
     constexpr uint32_t kTileBytes = tile_bytes<kD>();
     constexpr int kSlabs = kD / 64;                              // 64-column slabs of a Q tile
     constexpr uint32_t kGroupBytes = group_bytes<kD>(), kPageBytes = page_bytes<kD>();
@@ -648,17 +648,18 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         }
                     };
                     if constexpr (FORM == kHalves) {
-                        // this CTA finishes columns 64 qt + 32 rank ..; the other 32 of the warpgroup's 64 go where the Q tile was (every
-                        // product that read it has ended), the maximum and sum behind chain 0's
+                        // this CTA finishes a quarter of the columns per warpgroup; the other half of the warpgroup's half goes where the Q tile was
+                        // (every product that read it has ended), the maximum and sum behind chain 0's
+                        constexpr int HALF = kD / 2, QUARTER = kD / 4;
                         const uint32_t rank = cluster_ctarank();
-                        float o[64], mine[32];
-                        load32(o, 64 * qt);
-                        load32(o + 32, 64 * qt + 32);
-                        float4* give = reinterpret_cast<float4*>(q_tiles) + qt * (8 * kRows) + t;
+                        float o[HALF], mine[QUARTER];
+#pragma unroll
+                        for (int c = 0; c < HALF; c += 32) load32(o + c, HALF * qt + c);
+                        float4* give = reinterpret_cast<float4*>(q_tiles) + qt * (QUARTER / 4 * kRows) + t;
                         float2* ml = reinterpret_cast<float2*>(q_tiles + kTileBytes) + (1 + qt) * kRows + t;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const float* lo = o + 4 * k; const float* hi = o + 32 + 4 * k;
+                        for (int k = 0; k < QUARTER / 4; ++k) {
+                            const float* lo = o + 4 * k; const float* hi = o + QUARTER + 4 * k;
                             give[k * kRows] = rank == 0 ? make_float4(hi[0], hi[1], hi[2], hi[3]) : make_float4(lo[0], lo[1], lo[2], lo[3]);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) mine[4 * k + e] = rank == 0 ? lo[e] : hi[e];
@@ -678,12 +679,12 @@ attn_tc5_kernel(AttnArgs a, const WorkItem* __restrict__ items, int total_units,
                         m_used = m_new;
                         const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
+                        for (int k = 0; k < QUARTER / 4; ++k) {
                             const float4 v = ld_cluster_f4(from + k * kRows * 16);
                             mine[4 * k] = mine[4 * k] * wm + v.x * wo; mine[4 * k + 1] = mine[4 * k + 1] * wm + v.y * wo;
                             mine[4 * k + 2] = mine[4 * k + 2] * wm + v.z * wo; mine[4 * k + 3] = mine[4 * k + 3] * wm + v.w * wo;
                         }
-                        out_rows::store<32, kD, true>(a, mine, inv, true, orow, u.C - i_row, u.h, 64 * qt + 32 * (int)rank, lane);
+                        out_rows::store<QUARTER, kD, kD == 128>(a, mine, inv, true, orow, u.C - i_row, u.h, HALF * qt + QUARTER * (int)rank, lane);
                         if (i_row < u.C && qt == 0 && rank == 0) a.lse[orow * H + u.h] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : -INFINITY;
                     } else {
                         const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -816,11 +817,11 @@ cudaError_t launch_attn_tc5(const hat_plan* plan, const AttnArgs& args, cudaStre
     if (grid_limit > 0) ctas = std::min(ctas, grid_limit);
     const dim3 grid((unsigned)ctas);
     const bool d128 = plan->head_dim == 128;
-    const bool one = d128 && total_units <= ctas && a2.static_first;
-    if (plan->tile_clusters && !one) return cudaErrorInvalidValue;
+    const bool alone = total_units <= ctas && a2.static_first, one = d128 && alone;
+    if (plan->tile_clusters && !alone) return cudaErrorInvalidValue;
     auto form = [&](auto b, auto app) {
         constexpr bool B = decltype(b)::value, A = decltype(app)::value;
-        return !d128 ? attn_tc5_kernel<B, 64, kMany, A> : plan->tile_clusters ? attn_tc5_kernel<B, 128, kHalves, A>
+        return !d128 ? (plan->tile_clusters ? attn_tc5_kernel<B, 64, kHalves, A> : attn_tc5_kernel<B, 64, kMany, A>) : plan->tile_clusters ? attn_tc5_kernel<B, 128, kHalves, A>
                : one ? attn_tc5_kernel<B, 128, kOne, A> : attn_tc5_kernel<B, 128, kMany, A>;
     };
     using Yes = std::true_type;

@@ -183,9 +183,10 @@ static int split_len_for(int kv_end, int wanted, int granule) {
 
 // Whether the two halves of every cut tile are merged inside the one-CTA tile kernel, by clusters of two CTAs: every tile is
 // cut in two, has at most 128 rows, and the pieces are one round of the CTAs.  (Side by side with another grid on one
-// counter, HAT_SIDE_SMS, a unit has no CTA of its own.)
+// counter, HAT_SIDE_SMS, a unit has no CTA of its own.)  With 64 columns the merge behind is short, and with few CTAs it is the
+// cheaper one: prompts of 2048 in chunks of 256, launch / clusters, 32 heads fp16 140 / 118 us, bf16 147 / 127, but 8 heads 2 to 5 % more.
 static bool pieces_meet_in_clusters(const hat_plan* p, int num_sms, int64_t units, bool all_in_two, bool all_narrow) {
-    return p->head_dim == 128 && all_in_two && all_narrow && units <= num_sms / 2 * 2 && env_int("HAT_SIDE_SMS", 0) <= 0;
+    return (p->head_dim == 128 || units >= num_sms / 2) && all_in_two && all_narrow && units <= num_sms / 2 * 2 && env_int("HAT_SIDE_SMS", 0) <= 0;
 }
 
 // Key-range length for the tile-class requests of a batch that is too small to fill the persistent tcgen05 kernel.
@@ -404,9 +405,8 @@ static int pick_short_cluster(const hat_plan* p, int num_sms, double slabs_price
 // no launch and no second read, but the instructions for it crowd the kernel's loops out of the instruction cache and its producer
 // works on units with chunk pages longer; in front, it costs a launch and the bytes once more.  So in front where CTAs have
 // several units each and a unit is short work: 64 columns, or on average at most one query tile.  Measured, us inside / in front, fp16, 32
-// heads: 30 chunks of 32 to 128 rows at up to 512 90 / 77, at up to 2048 147 / 128, 64 columns 72 / 56 and 117 / 93; 30 of 64 to 512 at up to
-// 4096 365 / 368, 64 columns 311 / 296; 30 of 64 to 256 at up to 512 115 / 120; with less than two units a CTA 8 of 64 to 256 50 / 54.  The
-// CTA-pair kernel, whose loops are smaller, appends inside (30 chunks, bf16, 433 / 441).
+// heads: 30 chunks of 32 to 128 rows at up to 1024 114 / 93, 64 columns 84 / 68; 30 of 64 to 512 at up to 4096 401 / 419, 64 columns
+// 311 / 307; 8 heads, 64 columns 23.0 / 23.5.  The CTA-pair kernel, whose loops are smaller, appends inside (30 chunks, bf16, 433 / 441).
 static bool append_is_apart(const hat_plan* p, int num_sms, int tile_rows) {
     int64_t tiles = 0, rows = 0;
     for (int r = 0; r < p->num_requests; ++r)

@@ -42,8 +42,16 @@ __device__ __forceinline__ void store(const AttnArgs& a, const float (&o)[N], fl
     if (final_rows && a.out16 != nullptr) {
         uint16_t* dst = static_cast<uint16_t*>(a.out16) + (at - odd) * pitch + h * D + col + 16 * odd;
         const bool wide = (reinterpret_cast<uintptr_t>(a.out16) & 31) == 0;
+        if constexpr (N == 16) {
+            static_assert(!SWAP, "16 columns are one 32-byte store");
+            uint32_t v[8];
 #pragma unroll
-        for (int k = 0; k < N; k += 32) {
+            for (int e = 0; e < 8; ++e) v[e] = pack_out16(o[2 * e] * inv, o[2 * e + 1] * inv, a.out16_bf16);
+            store_32(dst, v, wide);
+            return;
+        }
+#pragma unroll
+        for (int k = 0; k + 32 <= N; k += 32) {
             uint32_t v[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) v[e] = pack_out16(o[k + 2 * e] * inv, o[k + 2 * e + 1] * inv, a.out16_bf16);

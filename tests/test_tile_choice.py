@@ -39,3 +39,25 @@ def test_wide_and_narrow_units_of_one_batch(cuda_device, kernel, monkeypatch):
 @pytest.mark.parametrize("chunk,prefix", [([256], [1000]), ([129], [0]), ([200, 512], [700, 33])])     # halves merged by clusters; one unit a CTA
 def test_small_bf16_batches_on_single_ctas(cuda_device, chunk, prefix):
     _check(_batch("bf16", 8, 128, prefix, chunk, 84), cuda_device, repeat=3)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("heads,chunk,prefix,split", [(25, 256, 200, 256), (25, 129, 300, 384), (40, 77, 700, 640), (37, 128, 383, 256)])
+def test_halves_of_64_columns(cuda_device, dtype, heads, chunk, prefix, split, monkeypatch):
+    """From half a round of CTAs on, clusters merge rows of 64 columns too; calls follow without a wait, and out16 is out rounded once."""
+    import torch
+    from paper_2503_18989_b200 import runner
+    monkeypatch.setenv("HAT_PREFILL_KERNEL", "tc5")
+    monkeypatch.setenv("HAT_PREFILL_TILE_ROWS", "128")
+    monkeypatch.setenv("HAT_PREFILL_SPLIT_LEN", str(split))
+    sc = _batch(dtype, heads, 64, [prefix], [chunk], 19)
+    ds = runner.DeviceStep(runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device), sc.steps[0])
+    assert ds.info["max_splits"] == 2 and ds.workspace_bytes == 0           # the clusters need none
+    ds.attend(fused_append=True)
+    ds.attend16(fused_append=True)
+    torch.cuda.synchronize()
+    kind = torch.float16 if dtype == "fp16" else torch.bfloat16
+    assert torch.equal(ds.out16.view(kind), ds.out.to(kind))
+    ds.close()
+    _check(sc, cuda_device, repeat=5)
