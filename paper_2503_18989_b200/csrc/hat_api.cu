@@ -189,6 +189,34 @@ static bool pieces_meet_in_clusters(const hat_plan* p, int num_sms, int64_t unit
     return (p->head_dim == 128 || units >= num_sms / 2) && all_in_two && all_narrow && units <= num_sms / 2 * 2 && env_int("HAT_SIDE_SMS", 0) <= 0;
 }
 
+// ns that a unit takes a CTA of the one-CTA tile kernel: its 128-key steps, two query tiles or one, and what does not depend on the keys (the
+// Q tiles, refilling the rings, the rows).  Fitted to 1, 2 and 3 rounds of equal units, 256 to 3072 keys.
+static int64_t tile_unit_ns(const hat_plan* p, int keys, int rows) {
+    const bool bf16 = p->dtype == HAT_DTYPE_BF16, d128 = p->head_dim == 128;
+    const int wide = d128 ? (bf16 ? 3100 : 2400) : (bf16 ? 2480 : 2000), narrow = d128 ? (bf16 ? 1780 : 1450) : (bf16 ? 1350 : 1020);
+    return (int64_t)ceil_div(keys, 128) * (rows > 128 ? wide : narrow) + (d128 && rows > 128 ? 6000 : 4000);
+}
+
+// When the last of n units ends that CTAs draw in order.
+template <typename F>
+static int64_t last_end(int ctas, int n, F&& ns_of) {
+    std::vector<int64_t> at(ctas, 0);                            // a heap: when each CTA is free, the first one in front
+    int64_t last = 0;
+    for (int i = 0; i < n; ++i) {
+        const int64_t t = at[0] + ns_of(i);
+        int k = 0;
+        for (int c = 1; c < ctas; c = 2 * k + 1) {
+            c += c + 1 < ctas && at[c + 1] < at[c];
+            if (at[c] >= t) break;
+            at[k] = at[c];
+            k = c;
+        }
+        at[k] = t;
+        last = std::max(last, t);
+    }
+    return last;
+}
+
 // Key-range length for the tile-class requests of a batch that is too small to fill the persistent tcgen05 kernel.
 // Every candidate length is priced with a small model of the one-CTA kernel (also for batches of the pair kernel, whose 74 pairs
 // take 2350 to 2720 cycles a step: the model is only a rough guide there), in SM clock cycles measured on B200: a 128-key
@@ -569,6 +597,27 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
                         p->tile_units.push_back((uint32_t)i | ((uint32_t)h << 16));
                     }
             if (pass == 0) p->num_pair_units = tile_kernel == 3 ? (int)p->tile_units.size() : 0;
+        }
+        // Where CTAs have few units each, the batch ends when the CTA with the most work does: then the longest units first, if that ends
+        // sooner than request by request (odd chunks, 6 x 40 heads, with rotation and drafts 134 -> 128 us a step; 2 of up to 600 rows x 32 heads fp16 64 -> 59).  With
+        // many units a CTA the blocks of a chunk keep together (20 chunks of up to 600 rows x 40 heads bf16 469 / 517).
+        const int n = (int)p->tile_units.size();
+        if (tile_kernel == 1 && !p->tile_clusters && n > num_sms && n <= 4 * num_sms) {
+            std::vector<int64_t> ns;
+            std::vector<int> by_time;
+            for (int i = 0; i < (int)p->prefill_items.size(); ++i) {
+                ns.push_back(tile_unit_ns(p, p->prefill_items[i].kv_end - p->prefill_items[i].kv_begin, rows_of(i)));
+                by_time.push_back(i);
+            }
+            std::stable_sort(by_time.begin(), by_time.end(), [&](int a, int b) { return ns[a] > ns[b]; });
+            // looked at with a quarter of the heads on a quarter of the CTAs, where that comes out even: 4 us of planning instead of 17
+            const int part = H % 4 == 0 && num_sms % 4 == 0 ? 4 : 1, heads = H / part;
+            std::vector<int64_t> by_request;
+            for (uint32_t u : p->tile_units)
+                if ((int)(u >> 16) < heads) by_request.push_back(ns[u & 0xffff]);
+            const int64_t now = last_end(num_sms / part, n / part, [&](int k) { return by_request[k]; });
+            if (100 * last_end(num_sms / part, n / part, [&](int k) { return ns[by_time[k / heads]]; }) < 98 * now)
+                for (int k = 0; k < n; ++k) p->tile_units[k] = (uint32_t)by_time[k / H] | ((uint32_t)(k % H) << 16);
         }
     }
 

@@ -61,3 +61,14 @@ def test_halves_of_64_columns(cuda_device, dtype, heads, chunk, prefix, split, m
     assert torch.equal(ds.out16.view(kind), ds.out.to(kind))
     ds.close()
     _check(sc, cuda_device, repeat=5)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,d,heads", [("fp16", 128, 25), ("bf16", 64, 40), ("fp16", 64, 16)])     # with and without heads that come in fours
+@pytest.mark.parametrize("split", [None, 384])              # as planned; pieces behind a merge launch
+def test_uneven_units_longest_first(cuda_device, dtype, d, heads, split, monkeypatch):
+    """One to four rounds of units of very different length: the order in which CTAs draw them is theirs, not the requests'."""
+    monkeypatch.setenv("HAT_PREFILL_KERNEL", "tc5")
+    if split:
+        monkeypatch.setenv("HAT_PREFILL_SPLIT_LEN", str(split))
+    _check(_batch(dtype, heads, d, [0, 1200, 40, 700, 5, 300], [300, 17, 513, 129, 64, 3], 23), cuda_device, repeat=4)
