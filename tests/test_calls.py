@@ -29,3 +29,29 @@ def test_arguments_and_errors_are_those_of_the_ctypes_call(hat_lib):
     assert B._call_attention(desc, plan, t, None, None, t, t, 0.0, None, 0, 0) == B.HAT_ERR_INVALID_ARG
     assert B._call_attention(desc, plan, "q", None, None, t, t, 0.0, None, 0, 0) is None
     assert B._call_attention(bytes(4), plan, t, None, None, t, t, 0.0, None, 0, 0) is None
+
+
+def test_what_ctypes_refuses_is_refused(hat_lib):
+    """A handle is an int, None or a Plan, the descriptor a hat_cache_desc: the memory of anything else is not read in their place."""
+    desc = B.make_cache_desc("fp16", 4, 2, 128, 16 * 2 * 128, 128, 16 * 128, 1 << 30, 1 << 30)
+    one = np.array([0], np.int32)
+    plan = B.hat_plan_create(desc, 2, np.array([0, 0], np.int32), one, one, np.zeros((1, 1), np.int32), flags=1)
+    t, room = torch.zeros(8), np.zeros(1 << 14, np.uint8)
+
+    class Other(C.Structure):
+        _fields_ = [("words", C.c_int64 * (C.sizeof(B.hat_cache_desc) // 8))]
+
+    held = B.Plan(room, None)
+    bad = {"plan": [room, torch.from_numpy(room), 0.0, held], "stream": [np.array([5]), torch.tensor([5]), 1.5],
+           "cache": [bytes(desc), bytearray(bytes(desc)), np.frombuffer(bytes(desc), np.uint8), Other(), C.addressof(desc), None]}
+    for fast, call in ((B._call_attention, B.hat_chunk_attention), (B._call_attention_out16, B.hat_chunk_attention_out16)):
+        for which, values in bad.items():
+            for x in values:
+                args = [desc, plan, t, None, None, t, t, 0.0, None, 0, 0]
+                args[{"cache": 0, "plan": 1, "stream": 10}[which]] = x
+                assert fast(*args) is None, (which, type(x))
+                with pytest.raises((TypeError, C.ArgumentError, AttributeError, ValueError)):
+                    call(*args)
+        for x in (256.0, "256", np.int64(256)):              # ctypes decides about a size that is no int
+            assert fast(desc, plan, t, None, None, t, t, 0.0, None, x, 0) is None
+    held.handle = None
