@@ -162,9 +162,13 @@ def lib() -> C.CDLL:
                                                   vp, vp, vp, C.c_float, vp]
         L.hat_static_key_range.restype = i32
         L.hat_static_key_range.argtypes = [i32, i32, i32, i32, i32] + [C.POINTER(i32)] * 4
-        from . import _calls
-        _calls.init(C.cast(L.hat_chunk_attention, vp).value, C.cast(L.hat_chunk_attention_out16, vp).value, Plan, hat_cache_desc)
-        _call_attention, _call_attention_out16 = _calls.chunk_attention, _calls.chunk_attention_out16
+        try:
+            from . import _calls
+        except ImportError:                 # not built for this interpreter: ctypes makes every call
+            pass
+        else:
+            _calls.init(C.cast(L.hat_chunk_attention, vp).value, C.cast(L.hat_chunk_attention_out16, vp).value, Plan, hat_cache_desc)
+            _call_attention, _call_attention_out16 = _calls.chunk_attention, _calls.chunk_attention_out16
         _lib = L
     return _lib
 

@@ -12,7 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhat.so")
 CALLS_SRC = os.path.join(CSRC, "calls.c")
-CALLS = os.path.join(HERE, "_calls.so")          # the binding's calls as a CPython extension
+# the binding's calls as a CPython extension, named for the interpreter it is built for; without it ctypes makes them
+CALLS = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -33,13 +34,29 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALLS):
+def _older(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
-    deps = sources() + [CALLS_SRC] + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
-        [os.path.join(HERE, "..", "include", "hat.h")]
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(p) > t for p in deps)
+
+
+HAT_H = os.path.join(HERE, "..", "include", "hat.h")
+
+
+def is_stale() -> bool:
+    return _older(LIB, sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + [HAT_H])
+
+
+def build_calls(force: bool = False) -> None:
+    """The extension, where this interpreter's headers are installed."""
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        print(f"no Python.h in {include}: the binding's calls stay with ctypes", file=sys.stderr)
+    elif force or _older(CALLS, [CALLS_SRC, HAT_H]):
+        tmp = CALLS + f".tmp{os.getpid()}"
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", include, CALLS_SRC, "-o", tmp])
+        os.replace(tmp, CALLS)
 
 
 LIB_DEBUG = os.path.join(HERE, "libhat_debug.so")
@@ -50,6 +67,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     debug=True builds libhat_debug.so with -DHAT_DEBUG_BOUNDS: device-side range checks of block-table lookups, page
     ids, ring slots, TMEM columns and output rows that report through the plan's status word instead of trapping
     (load it with HAT_LIB=debug)."""
+    build_calls(force)
     if debug:
         return _build(LIB_DEBUG, "_build_debug", ["-DHAT_DEBUG_BOUNDS"], verbose)
     if not force and not is_stale():
@@ -83,9 +101,6 @@ def _build(lib: str, obj_name: str, extra, verbose: bool) -> str:
     tmp = lib + f".tmp{os.getpid()}"
     subprocess.check_call([_nvcc(), "-shared", "-o", tmp, *objs, "-lcudart_static", "-ldl", "-lpthread", "-lrt"])
     os.replace(tmp, lib)
-    tmp = CALLS + f".tmp{os.getpid()}"
-    subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], CALLS_SRC, "-o", tmp])
-    os.replace(tmp, CALLS)
     return lib
 
 

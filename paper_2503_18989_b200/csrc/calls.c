@@ -15,7 +15,8 @@ static int address(PyObject* x, void** out) {
     if (x == Py_None) { *out = NULL; return 0; }
     PyObject* v;
     if (PyLong_Check(x)) {
-        v = Py_NewRef(x);
+        Py_INCREF(x);
+        v = x;
     } else {
         v = PyObject_CallMethodNoArgs(x, g_data_ptr);
         if (!v) {
@@ -94,8 +95,10 @@ static PyObject* init(PyObject* self, PyObject* const* a, Py_ssize_t n) {
         if (address(a[i], &f[i])) return NULL;
     g_attention = (attention_fn)(uintptr_t)f[0];
     g_attention_out16 = (attention_fn)(uintptr_t)f[1];
-    Py_XSETREF(g_plan_type, Py_NewRef(a[2]));
-    Py_XSETREF(g_cache_type, Py_NewRef(a[3]));
+    Py_INCREF(a[2]);
+    Py_INCREF(a[3]);
+    Py_XSETREF(g_plan_type, a[2]);
+    Py_XSETREF(g_cache_type, a[3]);
     Py_RETURN_NONE;
 }
 

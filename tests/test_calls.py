@@ -55,3 +55,35 @@ def test_what_ctypes_refuses_is_refused(hat_lib):
         for x in (256.0, "256", np.int64(256)):              # ctypes decides about a size that is no int
             assert fast(desc, plan, t, None, None, t, t, 0.0, None, x, 0) is None
     held.handle = None
+
+
+_WITHOUT = """
+import sys
+import numpy as np
+sys.modules["paper_2503_18989_b200._calls"] = None          # as where the interpreter has none: importing it is an ImportError
+from paper_2503_18989_b200 import binding as B
+desc = B.make_cache_desc("fp16", 4, 2, 128, 16 * 2 * 128, 128, 16 * 128, 1 << 30, 1 << 30)
+one = np.array([0], np.int32)
+plan = B.hat_plan_create(desc, 2, np.array([0, 0], np.int32), one, one, np.zeros((1, 1), np.int32), flags=1)
+for call in (B.hat_chunk_attention, B.hat_chunk_attention_out16):
+    try:
+        call(desc, plan, 1 << 20, None, None, 1 << 20, 1 << 20)
+    except B.HatError as e:
+        print("status", e.status)
+"""
+
+
+def test_without_the_extension_ctypes_makes_the_calls(hat_lib):
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _WITHOUT], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr[-500:]
+    assert r.stdout.split() == ["status", str(B.HAT_ERR_INVALID_ARG)] * 2
+
+
+def test_the_extension_is_named_for_its_interpreter(hat_lib):
+    import sysconfig
+    from paper_2503_18989_b200 import build
+    assert build.CALLS.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and "cpython" in build.CALLS
