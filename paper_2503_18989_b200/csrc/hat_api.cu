@@ -848,9 +848,9 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     // Which tcgen05 tile kernel: the CTA-pair kernel (cta_group::2) shares every K/V tile between the two 128-row halves
     // of a 256-row unit and is the faster one for long units; short ones, whose start and rows count for more, and batches that do
     // not fill the pairs are faster on the one-CTA kernel, with units of 128 rows and halves merged by clusters where they are few.
-    // HAT_PREFILL_KERNEL = tc5 | pair | mixed (wide units to pairs, whatever their length) | mma overrides.
+    // HAT_PREFILL_KERNEL = tc5 | pair | mixed (of bf16 batches, wide units to pairs, whatever their length) | mma overrides.
     int tile_kernel = use_tc5 ? 1 : 0;
-    bool pairs_possible = false;
+    bool mixed_possible = false;
     if (use_tc5 && p->head_dim == 128) {
         bool all_wide = true;
         int64_t wide_tiles = 0, wide_keys = 0;
@@ -870,13 +870,13 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
         const bool many = wide_tiles * p->num_heads >= 3 * (int64_t)num_sms / 2;
         const bool long_units = wide_tiles > 0 && wide_keys / wide_tiles >= (bf16 ? 3000 : 4200);
         if ((all_wide || bf16) && long_units && many) tile_kernel = 3;
-        pairs_possible = tile_kernel == 3 || (bf16 && wide_tiles > 0);
+        mixed_possible = bf16 && wide_tiles > 0;
     }
     p->pair_takes_all = false;
     if (const char* k = std::getenv("HAT_PREFILL_KERNEL")) {
         if (use_tc5 && p->head_dim == 128 && std::strcmp(k, "pair") == 0) { tile_kernel = 3; p->pair_takes_all = true; }
-        else if (use_tc5 && std::strcmp(k, "mixed") == 0 && pairs_possible) tile_kernel = 3;
-        else if (use_tc5 && std::strcmp(k, "tc5") == 0) { tile_kernel = 1; pairs_possible = false; }
+        else if (use_tc5 && std::strcmp(k, "mixed") == 0 && mixed_possible) tile_kernel = 3;
+        else if (use_tc5 && std::strcmp(k, "tc5") == 0) tile_kernel = 1;
     }
     // the streaming kernel takes its pages by TMA when a descriptor can be built for the pool layout
     bool stream_tma = true;
@@ -887,7 +887,6 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
                                              cache->stride_token, cache->stride_head);
     p->info.stream_kernel = stream_tma ? 1 : 0;
     schedule(p, num_sms, tile_kernel, whole);
-    if (pairs_possible) p->info.prefill_kernel = 3;          // such a batch may go to either kernel: see num_pair_units
     p->info.num_pair_units = p->num_pair_units;
     // launch-geometry limits: work items index gridDim.y (65535), partial rows and units are 32-bit
     const int64_t verify_count = (int64_t)(p->verify_items.size() + p->stream_items.size());
@@ -1048,9 +1047,8 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
         mark(1, 0);
         if (plan->info.prefill_kernel == 3) {
             // long units of more than 128 rows on CTA pairs, the others (if any) on single CTAs that take the SMs as the pairs leave them
-            const bool pairs = plan->num_pair_units > 0;
-            if (pairs) e = launch_attn_pair(plan, a, s, plan->num_pair_units);
-            if (e == cudaSuccess) e = launch_attn_tc5(plan, a, s, 0, true, plan->num_pair_units, -1, /*counter_word=*/3, /*overlap=*/pairs);
+            e = launch_attn_pair(plan, a, s, plan->num_pair_units);
+            if (e == cudaSuccess) e = launch_attn_tc5(plan, a, s, 0, true, plan->num_pair_units, -1, /*counter_word=*/3, /*overlap=*/true);
         } else {
             e = plan->info.prefill_kernel == 1 ? launch_attn_tc5(plan, a, s)
                                                : launch_attn_mma(plan, a, /*verify_class=*/false, s);

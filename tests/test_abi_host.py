@@ -242,9 +242,9 @@ def test_static_entry_point_clamps_unvalidated_lengths(hat_lib):
 
 
 def test_choice_of_the_tile_kernel(hat_lib):
-    """The CTA-pair kernel takes the units of more than 128 rows: for bf16 in every batch that has some (narrower units
-    of the same batch run on single CTAs), for fp16 only when every unit is that wide and long (2500 keys on average)
-    and there are at least 1.5 of them per SM; head_dim 64 keeps the one-CTA tcgen05 kernel."""
+    """CTA pairs take the units of more than 128 rows of batches with at least 1.5 such units per SM that are long on average: 3000
+    keys for bf16 (narrower units of the same batch run on single CTAs), 4200 for fp16, and there only when every unit is that
+    wide; head_dim 64 keeps the one-CTA tcgen05 kernel.  prefill_kernel says 3 where pairs have units, and only there."""
     def info(prefix, chunk, H, d=128, dtype="bf16"):
         rng = np.random.Generator(np.random.PCG64(3))
         table, num_pages = W._place_pages(rng, np.asarray(prefix) + np.asarray(chunk), slack_pages=2)
@@ -253,20 +253,25 @@ def test_choice_of_the_tile_kernel(hat_lib):
         p = B.hat_plan_create(c, H, cu, np.asarray(prefix, np.int32), np.asarray(chunk, np.int32), table,
                               B.HAT_PLAN_HOST_ONLY)
         return B.hat_plan_get_info(p).as_dict()
-    assert info([100] * 8, [512] * 8, 40)["prefill_kernel"] == 3              # 16 wide units x 40 heads
-    assert info([100] * 8 + [700] * 4, [512] * 8 + [4] * 4, 40)["prefill_kernel"] == 3   # short chunks do not matter
-    assert info([100] * 8, [512] * 7 + [384], 40)["prefill_kernel"] == 3       # bf16: the 128-row unit of the 384 goes to a single CTA
-    assert info([100] * 8, [512] * 7 + [400], 40)["prefill_kernel"] == 3       # 400 = 256 + 144: both halves in use
-    assert info([100] * 8, [128] * 8, 40)["prefill_kernel"] == 1               # nothing for a pair
-    assert info([100] * 8, [512] * 7 + [384], 40, dtype="fp16")["prefill_kernel"] == 1   # fp16: only batches of full units
-    assert info([100] * 2, [512] * 2, 32)["prefill_kernel"] == 3               # bf16: small batches too
-    assert info([100], [256], 8)["prefill_kernel"] == 3
-    assert info([100] * 2, [512] * 2, 32, dtype="fp16")["prefill_kernel"] == 1   # fp16: 4 x 32 = 128 units < 222
-    assert info([4000] * 3, [512] * 3, 40, dtype="fp16")["prefill_kernel"] == 3   # 6 x 40 = 240 long units
-    assert info([4000] * 8, [512] * 8, 40, dtype="fp16")["prefill_kernel"] == 3
-    assert info([1000] * 8, [512] * 8, 40, dtype="fp16")["prefill_kernel"] == 1    # fp16 units of ~1400 keys: no gain on pairs
-    assert info([100] * 8, [4] * 8, 40)["prefill_kernel"] == 1                 # no tile-class chunk at all
-    assert info([100] * 8, [512] * 8, 40, d=64)["prefill_kernel"] == 1
+    def kernel(*args, **kw):
+        got = info(*args, **kw)
+        assert (got["prefill_kernel"] == 3) == (got["num_pair_units"] > 0)
+        return got["prefill_kernel"]
+    assert kernel([3000] * 8, [512] * 8, 40) == 3                     # 16 wide units x 40 heads
+    assert kernel([3000] * 8 + [700] * 4, [512] * 8 + [4] * 4, 40) == 3   # short chunks do not matter
+    assert kernel([3000] * 8, [512] * 7 + [384], 40) == 3             # bf16: the 128-row unit of the 384 goes to a single CTA
+    assert kernel([3000] * 8, [512] * 7 + [400], 40) == 3             # 400 = 256 + 144: both halves in use
+    assert kernel([100] * 8, [512] * 8, 40) == 1                      # short units
+    assert kernel([3000] * 8, [128] * 8, 40) == 1                     # nothing for a pair
+    assert kernel([4000] * 8, [512] * 7 + [384], 40, dtype="fp16") == 1   # fp16: only batches of full units
+    assert kernel([3000] * 2, [512] * 2, 32) == 1                     # 4 x 32 = 128 units < 222
+    assert kernel([3000], [256], 8) == 1
+    assert kernel([4000] * 2, [512] * 2, 32, dtype="fp16") == 1
+    assert kernel([4000] * 3, [512] * 3, 40, dtype="fp16") == 3       # 6 x 40 = 240 long units
+    assert kernel([4000] * 8, [512] * 8, 40, dtype="fp16") == 3
+    assert kernel([3000] * 8, [512] * 8, 40, dtype="fp16") == 1       # fp16 units of ~3400 keys: no gain on pairs
+    assert kernel([100] * 8, [4] * 8, 40) == 1                        # no tile-class chunk at all
+    assert kernel([3000] * 8, [512] * 8, 40, d=64) == 1
 
 
 _EXHAUSTED = """

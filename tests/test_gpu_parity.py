@@ -701,18 +701,20 @@ def test_calls_on_one_plan_from_two_streams_are_kept_in_order(cuda_device):
     ds.close()
 
 
-def test_a_bf16_batch_with_wide_and_narrow_units_uses_both_tile_kernels(cuda_device):
-    """bf16, head_dim 128: units of more than 128 rows run on CTA pairs and the narrower units of the same batch (a
+def test_a_bf16_batch_with_wide_and_narrow_units_uses_both_tile_kernels(cuda_device, monkeypatch):
+    """bf16, head_dim 128, wide units forced to the pairs: units of more than 128 rows run on CTA pairs and the narrower units of the same batch (a
     128-row remainder of a 384-row chunk, chunks of 128 / 64 / 17 rows) on single CTAs in a second grid with its own
     unit counter; every element against the oracle, twice in a row (the counters must be back at zero), also with key
     ranges cut and merged."""
     from paper_2503_18989_b200 import binding as B, runner
     prefix = [0, 300, 1000, 37, 2000, 640, 90, 5000]
     chunk = [512, 384, 128, 64, 300, 17, 4, 256]
+    monkeypatch.setenv("HAT_PREFILL_KERNEL", "mixed")
     sc = _manual("bf16", 2, 128, prefix, chunk, 71)
     cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
     ds = runner.DeviceStep(cache, sc.steps[0])
     assert ds.info["prefill_kernel"] == 3
+    assert 0 < ds.info["num_pair_units"] < 2 * ds.info["num_prefill_items"]
     kp, vp, want = oracle_replay(sc)
     for _ in range(2):
         ds.out.fill_(float("nan")); ds.lse.fill_(float("nan"))
@@ -725,13 +727,16 @@ def test_a_bf16_batch_with_wide_and_narrow_units_uses_both_tile_kernels(cuda_dev
     ds.close()
 
 
+@pytest.mark.parametrize("kernel", ["", "mixed"])               # as the plan picks (few heads: no pairs); wide units to the pairs
 @pytest.mark.parametrize("seed,group,out16", [(1, 1, False), (2, 2, False), (3, 1, True)])
-def test_random_bf16_batches_through_whatever_kernels_the_plan_picks(cuda_device, seed, group, out16):
+def test_random_bf16_batches_through_whatever_kernels_the_plan_picks(cuda_device, seed, group, out16, kernel, monkeypatch):
     """Random bf16 batches (chunks of 1 .. 700 rows, prefixes of 0 .. 3000 tokens, some not page multiples; grouped query
-    heads; 16-bit output): whichever mix of CTA-pair, one-CTA and streaming kernels and key-range cuts the plan picks,
+    heads; 16-bit output): whichever mix of CTA-pair, one-CTA and streaming kernels and key-range cuts the plan has,
     every element against the oracle."""
     import torch
     from paper_2503_18989_b200 import binding as B, runner
+    if kernel:
+        monkeypatch.setenv("HAT_PREFILL_KERNEL", kernel)
     rs = np.random.default_rng(100 + seed)
     R = 9
     chunk = [int(c) for c in rs.choice([1, 4, 16, 17, 64, 100, 128, 129, 200, 256, 300, 384, 512, 700], R)]
@@ -739,6 +744,7 @@ def test_random_bf16_batches_through_whatever_kernels_the_plan_picks(cuda_device
     sc = _manual("bf16", 2, 128, prefix, chunk, 300 + seed, q_group=group)
     cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
     ds = runner.DeviceStep(cache, sc.steps[0])
+    assert (ds.info["num_pair_units"] > 0) == (kernel == "mixed")
     kp, vp, want = oracle_replay(sc)
     if out16:
         ds.attend16(fused_append=True)
