@@ -133,7 +133,9 @@ typedef struct hat_plan_info {
     int64_t workspace_bytes;
     int64_t attn_flops;          /* 4*d*H_q*sum_r [C_r*P_r + C_r*(C_r+1)/2] (causal count, also when a tree mask is given) */
     int64_t kv_read_bytes;       /* 2*sum_r (P_r+C_r)*H_kv*d*elem: every visible K and V row read once per K/V head */
-    int32_t stream_kernel;       /* 0 = cp.async streaming kernel, 1 = TMA streaming kernel */
+    int32_t stream_kernel;       /* 0 = cp.async streaming kernel, 1 = TMA streaming kernel, 2 to 5 = its short form for batches of few units:
+                                    every unit has a CTA or a cluster of 2, 4 or 8.  (The fields about the streaming class's pieces, merge
+                                    rows and workspace describe the cut for kernels 0 and 1; the short form writes no partial rows.) */
     int32_t num_pair_units;      /* (work item, head) units of the tile kernels that CTA pairs take */
 } hat_plan_info;
 

@@ -390,7 +390,7 @@ static int pick_verify_split_slabs(const hat_plan* p, int num_sms, double* price
 }
 
 // Whether every unit of the streaming class gets a CTA of its own (the short form of the streaming kernel), and in how many pieces a request is
-// cut then: 1, 2, 4 or 8, the CTAs of a cluster; 0: the persistent kernel takes the pieces planned above.
+// cut then: 1, 2, 4 or 8, the CTAs of a cluster; 0: the persistent kernel takes the pieces planned above.  HAT_VERIFY_CLUSTER overrides.
 // A page takes a CTA 0.20 us (bf16; fp16 0.17; 64 columns 0.75 of that; 15 % more with two CTAs on an SM), start, hand-over and rows about 5, the exchange within a cluster
 // 1.4 to 2.4.  The persistent kernel needs HBM's time and 7 us or more, 12 at least (fence, count and merge of the pieces), or what the placing of
 // its slabs said and 5.  It keeps what it may do as fast: batches whose longest request is much longer than the others, which it cuts unevenly.
@@ -409,6 +409,9 @@ static int pick_short_cluster(const hat_plan* p, int num_sms, double slabs_price
         longest = std::max(longest, n);
     }
     if (units == 0) return 0;
+    const int forced = env_int("HAT_VERIFY_CLUSTER", -1);
+    if (forced == 0) return 0;
+    if ((forced == 1 || forced == 2 || forced == 4 || forced == 8) && units * forced <= 65535) return forced;
     const double page = (p->dtype == HAT_DTYPE_BF16 ? 0.203 : 0.168) * (d128 ? 1.0 : 0.75), hbm = (double)pages * p->head_dim * 64 / 6.45e6;
     const double exchange[4] = {0.0, d128 ? 1.4 : 0.8, d128 ? 2.1 : 1.0, d128 ? 2.4 : 1.1};
     int best = 0;
@@ -469,7 +472,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
             info.num_prefill_requests++;
         }
     }
-    const bool stream_tma = info.stream_kernel == 1;
+    const bool stream_tma = info.stream_kernel != 0;
     p->verify_subtiles = std::max(1, ceil_div(max_verify_rows * group, 16));
     int vsplit = env_int("HAT_VERIFY_SPLIT_LEN", 0);
     double slabs_price = 1e9;
@@ -531,6 +534,7 @@ static void schedule(hat_plan* p, int num_sms, int tile_kernel, bool whole) {
     }
     p->num_verify_merge_rows = (int)p->merge_rows.size();
     p->short_cluster = stream_tma && env_int("HAT_VERIFY_SPLIT_LEN", 0) <= 0 ? pick_short_cluster(p, num_sms, slabs_price) : 0;
+    for (int i = 0; i < 4; ++i) if (p->short_cluster == 1 << i) info.stream_kernel = 2 + i;
     if (p->short_cluster > 0)
         for (int r = 0; r < R; ++r) {
             const int C = p->chunk_len[r], P = p->prefix_len[r];
@@ -976,7 +980,7 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
     // the attention kernels append on the way, each class its own requests' rows, unless pages are shared between a writer and
     // a reader, a class runs on the mma.sync kernels, or a kernel in front is cheaper
     const bool has_verify = plan->info.num_verify_items > 0;
-    const bool fused = k_new && !plan->append_first && !plan->append_apart && (!has_verify || plan->info.stream_kernel == 1) &&
+    const bool fused = k_new && !plan->append_first && !plan->append_apart && (!has_verify || plan->info.stream_kernel != 0) &&
                        (plan->prefill_items.empty() || plan->info.prefill_kernel != 0);
     if (k_new && !fused) {
         mark(0, 0);
@@ -1026,7 +1030,7 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
     }
     if (has_verify) {
         mark(2, 0);
-        e = plan->info.stream_kernel == 1 ? launch_attn_stream(plan, a, s)
+        e = plan->info.stream_kernel != 0 ? launch_attn_stream(plan, a, s)
                                           : launch_attn_mma(plan, a, /*verify_class=*/true, s);
         if (e == cudaSuccess && n_vm > 0) e = launch_merge(plan, a, 0, n_vm, s);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -1037,7 +1041,7 @@ int run_attention(const hat_cache_desc* cache, const hat_plan* plan, const void*
     if (has_verify && plan->res.ev_verify && (e = cudaEventRecord(plan->res.ev_verify, s)) != cudaSuccess) return cuda_fail(e);
     // The tile kernels depend on nothing the streaming kernel does: they take the SMs as it leaves them.  (Not under the timing
     // recorder, which wants the kernels one after the other.)
-    a.overlap = has_verify && plan->info.stream_kernel == 1 && !side && call < 0 ? 1 : 0;
+    a.overlap = has_verify && plan->info.stream_kernel != 0 && !side && call < 0 ? 1 : 0;
     if (side) {
         e = launch_attn_tc5(plan, a, s, plan->side_sms, /*reset_counter=*/false);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, plan->ev_join, 0);

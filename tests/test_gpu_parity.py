@@ -332,14 +332,15 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(cuda_device, form, f
     assert_parity(gl, want[0][1], "lse after a timed-out call")
 
 
-def test_the_status_is_read_behind_the_plans_latest_call(cuda_device):
+def test_the_status_is_read_behind_the_plans_latest_call(cuda_device, monkeypatch):
     """Reading the status clears the plan's counters too: on another stream than the call's it waits for the call."""
     import torch
     from paper_2503_18989_b200 import binding as B, runner
+    monkeypatch.setenv("HAT_VERIFY_CLUSTER", "0")                   # the persistent kernel counts units and pieces
     sc = _manual("fp16", 4, 128, [5000, 300], [4, 200], 26)
     cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
     ds = runner.DeviceStep(cache, sc.steps[0])
-    assert ds.info["max_splits"] > 1
+    assert ds.info["max_splits"] > 1 and ds.info["stream_kernel"] == 1
     streams = [torch.cuda.Stream(cuda_device) for _ in range(2)]
     done = torch.cuda.Event()
     ds.attend(stream=streams[0].cuda_stream)
@@ -357,7 +358,7 @@ def test_the_status_is_read_behind_the_plans_latest_call(cuda_device):
     ds.close()
 
 
-@pytest.mark.parametrize("kernel", ["tc5", "pair", "stream", "projection"])
+@pytest.mark.parametrize("kernel", ["tc5", "pair", "stream", "short", "projection"])
 def test_waits_are_not_used_up_by_the_kernel_in_front(cuda_device, kernel, monkeypatch):
     """A kernel that starts in the tail of the previous one begins its bounded waits when that one has ended: one unit of 60000
     keys (about half a millisecond on one SM, the others idle), and behind it a call whose waits may take a tenth of that."""
@@ -370,7 +371,8 @@ def test_waits_are_not_used_up_by_the_kernel_in_front(cuda_device, kernel, monke
     assert long_ds.info["num_prefill_items"] == 1
     if kernel == "pair":
         monkeypatch.setenv("HAT_PREFILL_KERNEL", "pair")
-    sc = _manual("fp16", 2, 128, [100], [4 if kernel == "stream" else 64], 25)
+    monkeypatch.setenv("HAT_VERIFY_CLUSTER", "4" if kernel == "short" else "0")
+    sc = _manual("fp16", 2, 128, [100], [4 if kernel in ("stream", "short") else 64], 25)
     st = sc.steps[0]
     cache = runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device)
     ds = runner.DeviceStep(cache, st)

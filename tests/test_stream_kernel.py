@@ -11,6 +11,11 @@ from common import assert_parity, oracle_replay
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True)
+def _persistent(monkeypatch):
+    monkeypatch.setenv("HAT_VERIFY_CLUSTER", "0")        # the short form is test_stream_short's
+
+
 def _batch(dtype, H, d, prefix, chunk, seed, group=1, layout="paged", table=None, num_pages=None):
     rng = np.random.Generator(np.random.PCG64(seed))
     if table is None:

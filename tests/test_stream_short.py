@@ -1,25 +1,58 @@
 """The streaming kernel with a CTA per unit: clusters of 1, 2, 4 and 8 CTAs that share a request, through their shared memory."""
+import numpy as np
 import pytest
 
-from paper_2503_18989_b200 import workloads as W
+from paper_2503_18989_b200 import binding as B, workloads as W
 
 from test_stream_kernel import _batch, _check
-
-pytestmark = pytest.mark.gpu
 
 # beside the longest request ones with fewer pages than a cluster has CTAs (pieces without a page), page edges, 1 to 16 rows
 PREFIX = [0, 5, 16, 17, 128]
 CHUNK = [1, 16, 3, 8, 9, 4]
+FORM = {0: 1, 1: 2, 2: 3, 4: 4, 8: 5}               # HAT_VERIFY_CLUSTER -> hat_plan_info.stream_kernel
 
 
-@pytest.mark.parametrize("dtype,d,layout", [("fp16", 128, "paged"), ("bf16", 128, "contiguous"), ("bf16", 64, "paged")])
-@pytest.mark.parametrize("heads,longest", [(2, 3000), (8, 1500), (20, 700), (32, 60)])     # 12, 48, 120 and 192 units: clusters of 8, 4, 2 and 1
-def test_clusters_and_pieces_without_pages(cuda_device, dtype, d, layout, heads, longest):
-    _check(_batch(dtype, heads, d, PREFIX + [longest], CHUNK, 60 + heads, 1, layout), cuda_device, repeat=3)
+def _form(sc):
+    st = sc.steps[0]
+    c = B.make_cache_desc(sc.cache.dtype, sc.cache.num_pages, sc.cache.num_heads, sc.cache.head_dim, 16 * sc.cache.num_heads * sc.cache.head_dim,
+                          sc.cache.head_dim, 16 * sc.cache.head_dim, 1 << 30, 1 << 30)
+    cu = np.concatenate([[0], np.cumsum(st.chunk_len)]).astype(np.int32)
+    p = B.hat_plan_create(c, st.q.shape[1], cu, st.prefix_len, st.chunk_len, st.block_table, B.HAT_PLAN_HOST_ONLY)
+    return B.hat_plan_get_info(p).as_dict()["stream_kernel"]
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,d,layout", [("fp16", 128, "paged"), ("bf16", 128, "contiguous"), ("bf16", 64, "paged"), ("fp16", 64, "contiguous")])
+@pytest.mark.parametrize("cluster", [1, 2, 4, 8])
+@pytest.mark.parametrize("heads,longest", [(2, 3000), (20, 700)])
+def test_clusters_and_pieces_without_pages(cuda_device, dtype, d, layout, heads, longest, cluster, monkeypatch):
+    monkeypatch.setenv("HAT_VERIFY_CLUSTER", str(cluster))
+    sc = _batch(dtype, heads, d, PREFIX + [longest], CHUNK, 60 + heads, 1, layout)
+    assert _form(sc) == FORM[cluster]
+    _check(sc, cuda_device, repeat=3)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype,group", [("bf16", 4), ("fp16", 3), ("bf16", 8)])           # up to 4, 3 and 8 slabs; some requests have fewer
-def test_slabs_of_grouped_heads_and_trees(cuda_device, dtype, group):
+@pytest.mark.parametrize("cluster", [1, 2, 4, 8])
+def test_slabs_of_grouped_heads_and_trees(cuda_device, dtype, group, cluster, monkeypatch):
+    monkeypatch.setenv("HAT_VERIFY_CLUSTER", str(cluster))
     sc = _batch(dtype, 2, 128, PREFIX + [2000], CHUNK, 70 + group, group)
     sc.steps[0].tree_mask = W.random_tree_masks(70 + group, CHUNK)
+    assert _form(sc) == FORM[cluster]
     _check(sc, cuda_device, repeat=3)
+
+
+def test_batches_of_few_units_get_a_cta_or_a_cluster_each(hat_lib, monkeypatch):
+    def form(heads, prefix, dtype="bf16", d=128, group=1, chunk=4):
+        return _form(_batch(dtype, heads, d, prefix, [chunk] * len(prefix), 3, group))
+    assert form(32, [200]) == FORM[2] and form(32, [700]) == FORM[4] and form(32, [700], "fp16") == FORM[4]
+    assert form(8, [700]) == FORM[8] and form(8, [700], d=64) == FORM[8]      # few heads
+    assert form(8, [700], group=4) == FORM[8]                                 # one slab of 16 (row, query head) pairs
+    assert form(32, [300] * 9) == FORM[1]                                     # requests that need not be cut
+    assert form(40, [3000]) == FORM[0] and form(32, [8000] * 12) == FORM[0]   # more units than CTAs, or as fast in pieces
+    monkeypatch.setenv("HAT_VERIFY_CLUSTER", "0")
+    assert form(32, [700]) == FORM[0]
+    monkeypatch.delenv("HAT_VERIFY_CLUSTER")
+    monkeypatch.setenv("HAT_VERIFY_SPLIT_LEN", "160")                         # a length asked for is the persistent kernel's
+    assert form(32, [700]) == FORM[0]
