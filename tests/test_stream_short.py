@@ -4,6 +4,7 @@ import pytest
 
 from paper_2503_18989_b200 import binding as B, workloads as W
 
+from common import oracle_replay
 from test_stream_kernel import _batch, _check
 
 # beside the longest request ones with fewer pages than a cluster has CTAs (pieces without a page), page edges, 1 to 16 rows
@@ -41,6 +42,30 @@ def test_slabs_of_grouped_heads_and_trees(cuda_device, dtype, group, cluster, mo
     sc.steps[0].tree_mask = W.random_tree_masks(70 + group, CHUNK)
     assert _form(sc) == FORM[cluster]
     _check(sc, cuda_device, repeat=3)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,heads,d,prefix", [("fp16", 32, 128, 700), ("bf16", 32, 128, 700), ("fp16", 32, 64, 700), ("fp16", 8, 64, 3000), ("bf16", 8, 64, 3000)])
+def test_as_close_to_64_bits_as_the_persistent_kernel(cuda_device, dtype, heads, d, prefix, monkeypatch):
+    """The plan's own choice against the persistent kernel's many short pieces, each with a reference maximum of its own.  The weights'
+    roundings are the error of `out`: it is to be no larger (0.8 to 0.9 of it was measured).  An lse is rounded to 24 bits in any case."""
+    from paper_2503_18989_b200 import runner
+    sc = _batch(dtype, heads, d, [prefix], [6], 91)
+    _, _, want = oracle_replay(sc)
+    off = {}
+    for cluster in ("0", None):
+        if cluster:
+            monkeypatch.setenv("HAT_VERIFY_CLUSTER", cluster)
+        else:
+            monkeypatch.delenv("HAT_VERIFY_CLUSTER")
+        ds = runner.DeviceStep(runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device), sc.steps[0])
+        assert ds.info["stream_kernel"] == 1 and ds.info["max_splits"] > 4 if cluster else ds.info["stream_kernel"] > 2
+        ds.attend(fused_append=True)
+        out, lse = ds.results()
+        off[cluster] = np.linalg.norm(out - want[0][0]) / np.linalg.norm(want[0][0])
+        assert np.linalg.norm(lse - want[0][1]) <= 2.0 ** -24 * np.linalg.norm(want[0][1])
+        ds.close()
+    assert off[None] <= off["0"], off
 
 
 def test_batches_of_few_units_get_a_cta_or_a_cluster_each(hat_lib, monkeypatch):
