@@ -183,7 +183,12 @@ struct RowStore {
         else *reinterpret_cast<float2*>(a.out + to) = make_float2(v0, v1);
     }
     __device__ __forceinline__ void lse(int64_t at, float m, float sum) const {
-        if ((lane & 3) == 0) a.lse[at] = sum > 0.f ? fmaf(m, 0.6931471805599453f, logf(sum)) : -INFINITY;
+        if ((lane & 3) != 0) return;
+        // ln of m and sum together, rounded once: sum = f 2^k with f near 1, whose logarithm is small, and m + k in two terms
+        const int k = (__float_as_int(sum) - 0x3f3504f3) >> 23;
+        const float f = __uint_as_float(__float_as_uint(sum) - ((uint32_t)k << 23)), mk = m + (float)k, low = (float)k - (mk - m);
+        constexpr float kLn2 = 0.6931471805599453f;
+        a.lse[at] = sum > 0.f ? fmaf(mk, kLn2, fmaf(low, kLn2, logf(f))) : -INFINITY;
     }
 };
 
