@@ -339,7 +339,8 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
                 }
                 if (lane == 0) { ctl->unit[0] = r0; ctl->unit[1] = r1; ctl->unit[2] = r2; ctl->hs = done ? -1 : hs; }
                 __syncwarp();
-                if (lane == 0 && !(a.withhold && un == 0)) mbar_arrive(&ctl->q_full);   // self test: the first Q tile never arrives
+                // self test: the first Q tile never arrives (of a cluster, its first CTA's: the others wait for that one's result in vain)
+                if (lane == 0 && !(a.withhold && un == 0 && rank == 0)) mbar_arrive(&ctl->q_full);
                 ++un;
             }
             if (done) break;
