@@ -69,13 +69,17 @@ def test_as_close_to_64_bits_as_the_persistent_kernel(cuda_device, dtype, heads,
 
 
 def test_batches_of_few_units_get_a_cta_or_a_cluster_each(hat_lib, monkeypatch):
-    def form(heads, prefix, dtype="bf16", d=128, group=1, chunk=4):
-        return _form(_batch(dtype, heads, d, prefix, [chunk] * len(prefix), 3, group))
+    def form(heads, prefix, dtype="bf16", d=128, group=1, prompts=0):
+        return _form(_batch(dtype, heads, d, prefix + [1000] * prompts, [4] * len(prefix) + [256] * prompts, 3, group))
     assert form(32, [200]) == FORM[2] and form(32, [700]) == FORM[4] and form(32, [700], "fp16") == FORM[4]
     assert form(8, [700]) == FORM[8] and form(8, [700], d=64) == FORM[8]      # few heads
     assert form(8, [700], group=4) == FORM[8]                                 # one slab of 16 (row, query head) pairs
     assert form(32, [300] * 9) == FORM[1]                                     # requests that need not be cut
     assert form(40, [3000]) == FORM[0] and form(32, [8000] * 12) == FORM[0]   # more units than CTAs, or as fast in pieces
+    # with prompt chunks behind, clusters may take somewhat more, a CTA for each uncut request may not
+    uneven = [4066, 3779, 936, 5501, 1210, 1568]
+    assert form(40, uneven, "fp16") == FORM[0] and form(40, uneven, "fp16", prompts=3) == FORM[0]
+    assert form(40, [1500]) == FORM[0] and form(40, [1500], prompts=3) == FORM[4]
     monkeypatch.setenv("HAT_VERIFY_CLUSTER", "0")
     assert form(32, [700]) == FORM[0]
     monkeypatch.delenv("HAT_VERIFY_CLUSTER")
