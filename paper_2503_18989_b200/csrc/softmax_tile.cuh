@@ -76,14 +76,15 @@ struct Weigh {
     // a tile of 128 keys whose first 32 scores are on their way to `first`
     __device__ __forceinline__ void keys128(uint32_t (&first)[32], uint32_t scores) {
         uint32_t next[32];
+        tc5::tmem_ld_wait();
 #pragma unroll 1
         for (int c = 0; c < 128; c += 64) {
-            tc5::tmem_ld_wait();
             tc5::tmem_ld32(scores + c + 32, next);
             keys32(first, scores + c);
             tc5::tmem_ld_wait();
-            if (c == 0) tc5::tmem_ld32(scores + 64, first);
+            tc5::tmem_ld32(scores + 64, first);      // the second time unused: nothing is on its way where the loop comes round
             keys32(next, scores + c + 32);
+            tc5::tmem_ld_wait();
         }
     }
     __device__ __forceinline__ float total() const {
