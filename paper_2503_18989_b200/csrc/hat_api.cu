@@ -857,32 +857,28 @@ int create_plan(const hat_cache_desc* cache, const hat_batch_desc* batch, bool p
     // not fill the pairs are faster on the one-CTA kernel, with units of 128 rows and halves merged by clusters where they are few.
     // HAT_PREFILL_KERNEL = tc5 | pair | mixed (of bf16 batches, wide units to pairs, whatever their length) | mma overrides.
     int tile_kernel = use_tc5 ? 1 : 0;
-    bool mixed_possible = false;
-    if (use_tc5 && p->head_dim == 128) {
-        bool all_wide = true;
-        int64_t wide_tiles = 0, wide_keys = 0;
+    int64_t wide_tiles = 0, wide_keys = 0;
+    if (use_tc5 && p->head_dim == 128 && p->dtype == HAT_DTYPE_BF16) {
         for (int r = 0; r < R; ++r) {
             const int C = p->chunk_len[r];
             if (C <= 16) continue;
-            if (C % 256 != 0 && C % 256 <= 128) all_wide = false;
             for (int row0 = 0; row0 < C; row0 += 256)
                 if (C - row0 > 128) { ++wide_tiles; wide_keys += p->prefix_len[r] + std::min(C, row0 + 256); }
         }
         // bf16 (its units of more than 128 rows; narrower ones of the same batch run on single CTAs behind them): a step of 128 keys and a
-        // unit take a pair 1.45 and 7 us, a CTA 3.3 and 7.5, so pairs pay from some 2200 keys on where they are evenly loaded and surely from 3000, measured (one CTA / pairs, us, 32 heads): 4 chunks of
-        // 512 at 4000 228 / 207, 8 at up to 8000 350 / 298, 8 at up to 1000 93 / 108, 8 of 200 to 600 at up to 4000 287 / 319, 30 of 256 to 512 at up to 4000 784 /
-        // 821; few units: one chunk of 256 at 1000 19.5 / 29.0, 3 of 129 to 300 53 / 66, 4 of 512 at 4000 x 8 heads 66 / 75.
-        // fp16 (only where every unit is that wide): 4 of 512 at 4000 x 40 heads 234 / 220, 8 at up to 8000 329 / 325, x 32 heads 242 / 262.
-        const bool bf16 = p->dtype == HAT_DTYPE_BF16;
+        // unit take a pair 1.45 and 7 us, a CTA 3.3 and 7.5, so pairs pay from some 2200 keys on where they are evenly loaded and surely from 3000, measured (one CTA / pairs, us, 32 heads,
+        // means of 3 batches): 4 chunks of 512 at 4000 217 / 211, 8 at 3000 351 / 310, 8 at up to 8000 404 / 392, 12 of 256 to 512 at 2000 to 8000 583 / 536; 40 heads 4 at 4000 331 / 270,
+        // 16 at 4000 1116 / 1041; below: 8 at up to 1000 93 / 108, 8 of 200 to 600 at up to 4000 287 / 319,
+        // 30 of 256 to 512 at up to 4000 784 / 821; few units: one chunk of 256 at 1000 19.5 / 29.0, 4 of 512 at 4000 x 8 heads 66 / 75.
+        // fp16, whose CTAs multiply half as much for the same exponentials, is left to single CTAs: 4 of 512 at 4000 163 / 185, 16 653 / 778, 8 at up to 8000 290 / 329, 12 of 256 to 512
+        // 431 / 483, 40 heads 16 at 4000 832 / 968; pairs gain only where the units of single CTAs end unevenly (4 of 512 at 4000 x 40 heads 242 / 237).
         const bool many = wide_tiles * p->num_heads >= 3 * (int64_t)num_sms / 2;
-        const bool long_units = wide_tiles > 0 && wide_keys / wide_tiles >= (bf16 ? 3000 : 4200);
-        if ((all_wide || bf16) && long_units && many) tile_kernel = 3;
-        mixed_possible = bf16 && wide_tiles > 0;
+        if (many && wide_keys / wide_tiles >= 3000) tile_kernel = 3;
     }
     p->pair_takes_all = false;
     if (const char* k = std::getenv("HAT_PREFILL_KERNEL")) {
         if (use_tc5 && p->head_dim == 128 && std::strcmp(k, "pair") == 0) { tile_kernel = 3; p->pair_takes_all = true; }
-        else if (use_tc5 && std::strcmp(k, "mixed") == 0 && mixed_possible) tile_kernel = 3;
+        else if (use_tc5 && std::strcmp(k, "mixed") == 0 && wide_tiles > 0) tile_kernel = 3;
         else if (use_tc5 && std::strcmp(k, "tc5") == 0) tile_kernel = 1;
     }
     // the streaming kernel takes its pages by TMA when a descriptor can be built for the pool layout
