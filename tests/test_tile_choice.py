@@ -63,11 +63,17 @@ def test_halves_of_64_columns(cuda_device, dtype, heads, chunk, prefix, split, m
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("dtype,d,heads", [("fp16", 128, 25), ("bf16", 64, 40), ("fp16", 64, 16)])     # with and without heads that come in fours
-@pytest.mark.parametrize("split", [None, 384])              # as planned; pieces behind a merge launch
+@pytest.mark.parametrize("dtype,d,heads,split", [("fp16", 128, 25, None), ("bf16", 64, 40, None), ("bf16", 128, 32, None), ("bf16", 128, 40, None),      # as planned
+                                                 ("fp16", 128, 25, 384), ("fp16", 64, 16, 384)])       # pieces behind a merge launch
 def test_uneven_units_longest_first(cuda_device, dtype, d, heads, split, monkeypatch):
-    """One to four rounds of units of very different length: the order in which CTAs draw them is theirs, not the requests'."""
+    """One to four rounds of units of very different length, in batches whose units the plan puts in an order of its own (3 to 14 % sooner by
+    its model), with heads that come in fours (the order is found on a quarter of them) and not."""
+    from paper_2503_18989_b200 import runner
     monkeypatch.setenv("HAT_PREFILL_KERNEL", "tc5")
     if split:
         monkeypatch.setenv("HAT_PREFILL_SPLIT_LEN", str(split))
-    _check(_batch(dtype, heads, d, [0, 1200, 40, 700, 5, 300], [300, 17, 513, 129, 64, 3], 23), cuda_device, repeat=4)
+    sc = _batch(dtype, heads, d, [0, 1200, 40, 700, 5, 300, 2000], [300, 17, 513, 129, 64, 3, 40], 23)
+    ds = runner.DeviceStep(runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device), sc.steps[0])
+    assert 148 < ds.info["num_prefill_items"] * heads <= 4 * 148 and ds.info["prefill_kernel"] == 1
+    ds.close()
+    _check(sc, cuda_device, repeat=4)
