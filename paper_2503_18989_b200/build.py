@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import glob
 import os
+import shlex
 import shutil
 import subprocess
 import sys
@@ -55,7 +56,7 @@ def build_calls(force: bool = False) -> None:
         print(f"no Python.h in {include}: the binding's calls stay with ctypes", file=sys.stderr)
     elif force or _older(CALLS, [CALLS_SRC, HAT_H]):
         tmp = CALLS + f".tmp{os.getpid()}"
-        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", include, CALLS_SRC, "-o", tmp])
+        subprocess.check_call([*shlex.split(os.environ.get("CC") or "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", include, CALLS_SRC, "-o", tmp])
         os.replace(tmp, CALLS)
 
 

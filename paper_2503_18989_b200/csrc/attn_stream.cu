@@ -60,6 +60,7 @@ constexpr int kTodo = 48;                   // merges put off to the end of the 
 constexpr int kBatch = 4;                   // pages requested at a time
 constexpr int kAhead = 32;                  // pages prefetched to L2 before the previous kernel's end (a lane has one page id)
 constexpr float kMoveThreshold = 8.0f;      // log2 units
+constexpr float kLargest = 3.402823466e38f;
 
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -705,7 +706,8 @@ __device__ __forceinline__ void stream_roles(const AttnArgs& a, unsigned char* s
             // around it: packed products in line cost less than the jump (700 tokens x 32 heads bf16 8.5 us, 8.8 with, 8.7 moving rarely).
             if constexpr (CL > 0) {
                 top[0] = fmaxf(top[0], mx0); top[1] = fmaxf(top[1], mx1);
-                const bool mv0 = mx0 > top[0] - kMoveThreshold, mv1 = mx1 > top[1] - kMoveThreshold;
+                // (an infinite maximum moves it too, so that such a row is NaN as in the other form)
+                const bool mv0 = mx0 > fminf(top[0] - kMoveThreshold, kLargest), mv1 = mx1 > fminf(top[1] - kMoveThreshold, kLargest);
                 const float al0 = mv0 ? fast_exp2(m[0] - mx0) : 1.f, al1 = low_rows ? al0 : mv1 ? fast_exp2(m[1] - mx1) : 1.f;
                 if (mv0) m[0] = mx0;
                 if (mv1) m[1] = mx1;

@@ -68,6 +68,36 @@ def test_as_close_to_64_bits_as_the_persistent_kernel(cuda_device, dtype, heads,
     assert off[None] <= off["0"], off
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("cluster", ["1", "4"])
+def test_infinite_and_undefined_scores_as_in_the_persistent_kernel(cuda_device, dtype, cluster, monkeypatch):
+    """An infinite component of a cached key makes a score +inf or -inf by the sign of q: rows with the former are NaN (lse -inf), rows with
+    the latter do without that key; a NaN component makes every row NaN.  In either form alike (of the persistent one, a request in one piece)."""
+    from paper_2503_18989_b200 import runner
+    sc = _batch(dtype, 4, 128, [700, 200, 300], [4, 3, 5], 95)
+    k = sc.k_pool.reshape(-1, 4, 16, 128)
+    table, inf = sc.steps[0].block_table, 0x7c00 if dtype == "fp16" else 0x7f80
+    k[table[0, 20], 1, 3, 7] = inf
+    k[table[0, 33], 2, 0, 9] = inf
+    k[table[0, 34], 2, 5, 9] = inf
+    k[table[1, 2], 0, 1, 5] = inf | 1                                             # NaN
+    got = []
+    for c in ("0", cluster):
+        monkeypatch.setenv("HAT_VERIFY_CLUSTER", c)
+        monkeypatch.setenv("HAT_VERIFY_SPLIT_LEN", "100000" if c == "0" else "0")
+        ds = runner.DeviceStep(runner.DeviceCache(sc.cache, sc.k_pool, sc.v_pool, cuda_device), sc.steps[0])
+        assert ds.info["stream_kernel"] == FORM[int(c)]
+        ds.attend(fused_append=True)
+        got.append(ds.results())
+        ds.close()
+    (o0, l0), (o1, l1) = got
+    bad = np.isnan(o0).any(axis=2)
+    assert bad[:4, 1:3].any() and not bad[:4, 1:3].all() and bad[4:7, 0].all() and bad.sum() <= 8 + 3
+    assert np.array_equal(np.isnan(o0), np.isnan(o1)) and np.array_equal(np.isinf(l0), np.isinf(l1)) and np.array_equal(np.isnan(l0), np.isnan(l1))
+    assert np.allclose(o0[~bad], o1[~bad], rtol=0, atol=2e-3) and np.allclose(l0[np.isfinite(l0)], l1[np.isfinite(l0)], rtol=0, atol=1e-5)
+
+
 def test_batches_of_few_units_get_a_cta_or_a_cluster_each(hat_lib, monkeypatch):
     def form(heads, prefix, dtype="bf16", d=128, group=1, prompts=0):
         return _form(_batch(dtype, heads, d, prefix + [1000] * prompts, [4] * len(prefix) + [256] * prompts, 3, group))
